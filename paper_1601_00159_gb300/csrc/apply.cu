@@ -42,6 +42,31 @@ __device__ __forceinline__ void store_result(pi_result_t* res, uint32_t seq, uin
     *reinterpret_cast<uint4*>(res + seq) = w;
 }
 
+// Largest ownership marker e_i before the tile at tb, by the whole CTA, for a tile whose
+// first query continues the run before it (markers grow with i, so the nearest tile that
+// has one decides; tile 0 heads the first run). Small batches only: their descent keeps no
+// tile prefixes, and a run crosses few tiles.
+__device__ uint32_t marker_before(const ApplyArgs& a, uint32_t tb, uint32_t* s_tmp) {
+    while (tb > 0) {
+        tb -= kApplyTile;
+        uint32_t agg = 0;
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {  // whole tiles of valid queries: the run reaches past them
+            const uint32_t i = tb + (uint32_t)k * kApThreads + threadIdx.x;
+            const uint32_t op = a.sp[i] >> 30;
+            const bool head = i == 0 || a.sk[i] != a.sk[i - 1];
+            agg = max(agg, (op == 1u || op == 2u) ? 2u * i + 3u : (head ? 2u * i + 2u : 0u));
+        }
+        uint32_t most;
+        block_excl_max<kApThreads>(agg, s_tmp, &most);
+        if (most) return most;
+    }
+    return 0;
+}
+
+// kSmall: a batch from k_rank_locate, whose storage-layer state is kept per query instead of
+// per distinct key.
+template <bool kSmall>
 __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
     pdl_wait();
     pdl_trigger();
@@ -86,8 +111,12 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
     // the descent's prefixes for this tile (its markers' maximum before it, the dense
     // index of its first local run head), loaded with the batch (a block barrier below
     // would keep them from being hoisted)
-    const uint32_t tpref = a.tile_pref[tile];
-    const uint32_t dbase = a.sub_pref[tile * (kApplyTile / kSubTile)];
+    uint32_t tpref = kSmall ? 0u : a.tile_pref[tile];
+    const uint32_t dbase = kSmall ? 0u : a.sub_pref[tile * (kApplyTile / kSubTile)];
+    if (kSmall) {
+        const uint32_t tb = tile * kApplyTile;
+        if (tb > 0 && tb < qv && a.sk[tb] == a.sk[tb - 1]) tpref = marker_before(a, tb, s_tmp);
+    }
     uint32_t agg = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
@@ -105,16 +134,18 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
     // dense index of each query's local run head: the tile's first one plus the local
     // heads before it in the tile (a local head is a run head or a 256-query sub-tile's
     // first query, as the descent counted them)
-    uint32_t lh = 0, nh = 0;
+    uint32_t lh = 0, nh = 0, hidx = 0;
+    if (!kSmall) {
 #pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        const uint32_t i = base + k;
-        const uint64_t prev = k ? key[k - 1] : kprev;
-        const bool local = i < qv && (i == 0 || key[k] != prev || (i % kSubTile) == 0);
-        lh |= (local ? 1u : 0u) << k;
-        nh += local ? 1u : 0u;
+        for (int k = 0; k < kItems; ++k) {
+            const uint32_t i = base + k;
+            const uint64_t prev = k ? key[k - 1] : kprev;
+            const bool local = i < qv && (i == 0 || key[k] != prev || (i % kSubTile) == 0);
+            lh |= (local ? 1u : 0u) << k;
+            nh += local ? 1u : 0u;
+        }
+        hidx = dbase + block_excl_sum<kApThreads>(nh, s_tmp, nullptr);  // dense index of the next head
     }
-    uint32_t hidx = dbase + block_excl_sum<kApThreads>(nh, s_tmp, nullptr);  // dense index of the next head
     uint32_t new_here = 0, new_mask = 0, chg_here = 0, chg_mask = 0;
     // Per query: its run head's result index, and the gathers of its prior state, all
     // issued before any store so that their latencies overlap: the run head's state, or,
@@ -128,7 +159,7 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
         const uint32_t minc = max(M, e[k]);
         M = minc;
         e[k] = minc;  // keep the inclusive value for the owners and the new-node pass
-        dres[k] = hidx + ((lh >> k) & 1u) - 1u;  // this query's run head's result
+        dres[k] = kSmall ? base + k : hidx + ((lh >> k) & 1u) - 1u;  // this query's run head's result
         hidx += (lh >> k) & 1u;
         const uint64_t prev = k ? key[k - 1] : kprev;
         const bool q = base + k < qv;
@@ -348,12 +379,11 @@ __global__ void __launch_bounds__(kThreads) k_owner_check(ApplyArgs a) {
 
 }  // namespace
 
-cudaError_t launch_apply(const ApplyArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms) {
-    (void)epoch;
-    (void)num_sms;
+cudaError_t launch_apply(const ApplyArgs& a, bool small, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     const uint32_t tiles = (a.n + kApplyTile - 1) / kApplyTile;
-    launch_dep(k_apply, tiles, kApThreads, 0, s, a);  // tile prefixes come from the descent's scan
+    if (small) launch_dep(k_apply<true>, tiles, kApThreads, 0, s, a);
+    else launch_dep(k_apply<false>, tiles, kApThreads, 0, s, a);  // tile prefixes come from the descent's scan
     ++g_launches;
     launch_dep(k_new_scan, 1, 1024, 0, s, a);
     ++g_launches;

@@ -19,6 +19,10 @@ constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the cou
 constexpr uint32_t kCtrDistinct = 14;   // BatchMeta::tile_ctr slot: the descent prologue's tile counter
 constexpr uint32_t kApplyTile = 2048;   // sorted queries per apply tile
 constexpr uint32_t kSubTile = 256;      // sorted queries per descent warp step (one apply warp)
+constexpr uint32_t kRunTile = 1024;     // queries per tile of the small batches' sort
+// Largest batch sorted that way. A query is ranked in every other tile, so the ranking's work
+// grows with the square of the batch; the radix passes' chain of launches does not grow.
+constexpr uint32_t kSmallSort = 1u << 15;
 
 // Sticky error bits in DevMeta::error.
 constexpr uint32_t kErrTimeout = 1u;  // a bounded wait gave up
@@ -631,6 +635,11 @@ struct SortBuffers {
 cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
                         BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes);
 
+// Small batches (n <= kSmallSort): every tile of kRunTile queries sorted by (key, arrival)
+// on its own, into in_k / in_p (see k_tile_sort). Counts invalid queries into bm->invalid.
+cudaError_t launch_tile_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
+                             BatchMeta* bm, cudaStream_t s);
+
 struct DescendArgs {
     const uint64_t* sk;  // sorted keys
     const uint32_t* sp;  // sorted payload (op << 30 | arrival index)
@@ -659,6 +668,10 @@ struct DescendArgs {
 // The look-back of the first kernel takes ++epoch; a.desc needs 2 words per apply tile.
 cudaError_t launch_descend(const DescendArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms,
                            cudaEvent_t before_locate = nullptr);
+// The small batches' counterpart: from the sorted tiles (tk / tp) the whole batch in sorted
+// order (ok / op), and loc / flags / val0 of every query at its sorted position.
+cudaError_t launch_rank_locate(const DescendArgs& a, const uint64_t* tk, const uint32_t* tp, uint64_t* ok, uint32_t* op,
+                               cudaStream_t s);
 
 struct ApplyArgs {
     const uint64_t* sk;
@@ -688,7 +701,9 @@ struct ApplyArgs {
     uint32_t* err;
     uint32_t* wcount;  // debug check (null when off): writes per storage node in this batch
 };
-cudaError_t launch_apply(const ApplyArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms);
+// `small`: loc / flags / val0 hold one entry per query (launch_rank_locate), and the tile
+// prefixes are not given.
+cudaError_t launch_apply(const ApplyArgs& a, bool small, cudaStream_t s);
 // Debug check of single ownership: every storage node written at most once by the
 // batch's apply (sets kErrOwner otherwise); adds the writes to DevMeta::owner_writes and
 // clears the counts.

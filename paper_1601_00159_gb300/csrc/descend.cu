@@ -489,7 +489,120 @@ __global__ void __launch_bounds__(kThreads) k_locate(DescendArgs a, int lvl) {
     }
 }
 
+// Keys <= q in the sorted K[0, n): each round reads seven evenly spaced entries at once, so
+// that n entries take about log8(n) dependent reads.
+__device__ __forceinline__ uint32_t count_le(const uint64_t* K, uint32_t n, uint64_t q) {
+    uint32_t lo = 0, len = n;  // the count lies in [lo, lo + len]
+    while (len >= 8u) {
+        uint64_t v[7];
+#pragma unroll
+        for (uint32_t j = 0; j < 7; ++j) v[j] = K[lo + (uint32_t)(((uint64_t)len * (j + 1u)) >> 3)];
+        uint32_t c = 0;  // pivots <= q: a prefix
+#pragma unroll
+        for (uint32_t j = 0; j < 7; ++j) c += v[j] <= q ? 1u : 0u;
+        const uint32_t nlo = c ? (uint32_t)(((uint64_t)len * c) >> 3) + 1u : 0u;
+        const uint32_t nhi = c < 7u ? (uint32_t)(((uint64_t)len * (c + 1u)) >> 3) : len;
+        lo += nlo;
+        len = nhi - nlo;
+    }
+    uint64_t v[7];
+#pragma unroll
+    for (uint32_t j = 0; j < 7; ++j) v[j] = j < len ? K[lo + j] : kMaxKey;
+    uint32_t c = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < 7; ++j) c += j < len && v[j] <= q ? 1u : 0u;
+    return lo + c;
+}
+
+// Small batches: the place of every query among the sorted tiles, and its storage node, for 32
+// queries per CTA (consecutive ones of a sorted tile, one per lane). An element's place is its
+// place in its tile, plus the keys of every earlier tile that are <= its own and of every later
+// tile that are smaller: one warp per other tile counts those, while the last warp searches the
+// lowest built level (it holds every key of the levels above) and the storage gap. The kernel
+// is bound by dependent reads of L2, so the chains run side by side in warps of their own and
+// every search reads seven entries a round; the lanes' keys are neighbours, so their probes
+// share sectors. Every query is looked up, equal keys as often as they come: below kSmallSort
+// queries the passes that would collect the distinct keys cost more than the look-ups they save.
+constexpr uint32_t kRankWarps = 8;
+constexpr int kRankThreads = 32 * (kRankWarps + 1);
+
+__global__ void __launch_bounds__(kRankThreads) k_rank_locate(DescendArgs a, const uint64_t* __restrict__ tk,
+                                                              const uint32_t* __restrict__ tp,
+                                                              uint64_t* __restrict__ ok, uint32_t* __restrict__ op) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ uint32_t s_pos[kRankWarps][32];
+    const DevMeta* m = a.m;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t n = a.n, i = blockIdx.x * 32u + lane;
+    const uint64_t q = i < n ? tk[i] : kMaxKey;
+    int32_t r = -1;
+    uint64_t v = 0;
+    bool exists = false, live = false;
+    if (warp < kRankWarps) {
+        const uint32_t own = i / kRunTile, tiles = (n + kRunTile - 1) / kRunTile;
+        uint32_t c = 0;
+        for (uint32_t t = warp; t < tiles; t += kRankWarps) {
+            if (t == own) {
+                c += i - own * kRunTile;
+                continue;
+            }
+            // keys <= q are keys < q + 1; invalid queries (2^64-1) stay behind every key
+            const uint64_t* T = tk + t * kRunTile;
+            const uint32_t len = min(kRunTile, n - t * kRunTile);
+            if (t < own) c += count_le(T, len, q);
+            else c += q ? count_le(T, len, q - 1u) : 0u;
+        }
+        s_pos[warp][lane] = c;
+    } else if (q != kMaxKey && *(volatile const uint32_t*)&m->error == 0) {
+        const uint32_t size = m->size, cur = m->cur, H = m->H, Lb = m->Lb;
+        const uint64_t* SK = a.st.keys[cur];
+        uint64_t kr = 0;
+        if (Lb <= H) {
+            const uint64_t* K = (m->lcur ? a.lkeys1 : a.lkeys) + m->base[Lb];
+            const uint32_t* D = (m->lcur ? a.ldown1 : a.ldown) + m->base[Lb];
+            const uint32_t c = count_le(K, m->n[Lb], q);  // the level's sentinel follows its entries
+            const uint64_t kn = K[c];
+            const uint32_t dn = D[c];
+            const uint64_t klo = c ? K[c - 1u] : 0ull;
+            const uint32_t lo = c ? D[c - 1u] : 0u;
+            r = gap_search(SK, lo, dn, klo, kn, q, size, kr, a.err);
+        } else {
+            const uint32_t c = count_le(SK, size, q);
+            r = (int32_t)c - 1;
+            kr = c ? SK[c - 1u] : 0ull;
+        }
+        exists = r >= 0 && kr == q;
+        const uint8_t meta = exists ? a.st.meta[cur][r] : (uint8_t)0;
+        v = exists ? a.st.vals[cur][r] : 0ull;
+        live = exists && !(meta & kTomb);
+    }
+    __syncthreads();
+    if (i >= n || (warp != 0 && warp != kRankWarps)) return;
+    uint32_t pos = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < kRankWarps; ++w) pos += s_pos[w][lane];
+    if (pos >= n) {
+        atomicOr(a.err, kErrBounds);
+    } else if (warp == 0) {
+        ok[pos] = q;
+        op[pos] = tp[i];
+    } else {
+        a.loc[pos] = (uint32_t)(r + 1);
+        a.flags[pos] = (uint8_t)((exists ? 1u : 0u) | (live ? 2u : 0u));
+        a.val0[pos] = live ? v : 0ull;
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_rank_locate(const DescendArgs& a, const uint64_t* tk, const uint32_t* tp, uint64_t* ok, uint32_t* op,
+                               cudaStream_t s) {
+    if (a.n == 0 || a.n > kSmallSort) return cudaErrorInvalidValue;
+    launch_dep(k_rank_locate, (a.n + 31u) / 32u, kRankThreads, 0, s, a, tk, tp, ok, op);
+    ++g_launches;
+    return cudaGetLastError();
+}
 
 cudaError_t launch_descend(const DescendArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms,
                            cudaEvent_t before_locate) {

@@ -780,6 +780,14 @@ int sort_passes(pi_index* x, uint64_t n) {
     return prefix;
 }
 
+// Whether a batch takes the small batches' front end: its tiles sorted in shared memory, then
+// one kernel for the order and the look-ups, in place of the radix passes and the
+// level-synchronous descent. Options and test flags that choose among the latter's paths
+// keep them.
+bool small_front(const pi_index* x, uint64_t n) {
+    return n <= kSmallSort && !(x->test_flags & ~PI_TEST_OWNER_CHECK) && x->sort_cfg == 0 && x->smem_top == kSmemTopMax;
+}
+
 // Enqueues one batch (Algorithm 1) with the given per-batch scratch:
 //   stream s:  pack + sort -> [wait for the previous batch's rebuild] -> descent ->
 //              ownership + apply -> merge -> layout -> meta to the mailbox ring
@@ -796,9 +804,10 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     prof_mark(x, 0, s);
     cudaMemsetAsync(bm, 0, sizeof(BatchMeta), s);
     SortBuffers sb = sort_buffers(x, sc);
-    if ((e = launch_sort(ops, keys, (uint32_t)n, sb, bm, &x->d_meta->error, s, x->num_sms, sort_passes(x, n))) !=
-        cudaSuccess)
-        return map_cuda(e);
+    const bool small = small_front(x, n);
+    e = small ? launch_tile_sort(ops, keys, (uint32_t)n, sb, bm, s)
+              : launch_sort(ops, keys, (uint32_t)n, sb, bm, &x->d_meta->error, s, x->num_sms, sort_passes(x, n));
+    if (e != cudaSuccess) return map_cuda(e);
     prof_mark(x, 1, s);
     wait_rebuild(x, s);
     prof_mark(x, 2, s);
@@ -826,7 +835,10 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     da.val0 = sc.val0;
     da.n = (uint32_t)n;
     da.err = &x->d_meta->error;
-    if ((e = launch_descend(da, ep, s, x->num_sms, prof_event(x, 10))) != cudaSuccess) return map_cuda(e);
+    if (small) prof_mark(x, 10, s);
+    e = small ? launch_rank_locate(da, sc.in_k, sc.in_p, sc.a_k, sc.a_p, s)
+              : launch_descend(da, ep, s, x->num_sms, prof_event(x, 10));
+    if (e != cudaSuccess) return map_cuda(e);
     prof_mark(x, 3, s);
     ApplyArgs aa{};
     aa.sk = sc.a_k;
@@ -855,7 +867,7 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     aa.hp = x->hp;
     aa.err = &x->d_meta->error;
     aa.wcount = x->wcount;
-    if ((e = launch_apply(aa, ep, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
+    if ((e = launch_apply(aa, small, s)) != cudaSuccess) return map_cuda(e);
     if ((e = launch_owner_check(aa, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 4, s);
     RebuildArgs ra = rebuild_args(x, bm, (uint32_t)size_ub, x->force_rebuild ? 1u : 0u);
