@@ -21,9 +21,15 @@
 // run head (a query whose key differs from the previous one, and the first query of
 // every 256-query sub-tile) in sorted order -- so a query's storage-layer state is
 // found at its run head's dense index.
-// New nodes are staged per tile and packed in key order by k_new_scan + k_new_pack.
+// New nodes, and the changes of built levels' membership, go to their places in key order in
+// the same pass: a tile's first place comes from a decoupled look-back over the tiles' counts,
+// which only tiles that have some wait for. The CTA that finishes last ends the batch: it
+// decides whether the storage layer is re-laid-out, and if not, lays out the index levels.
+// (Staging the new nodes per tile, a scan and a packing kernel, and a one-thread level layout
+// were three more launches: 6000 mixed queries on 2^20 keys 61.0 -> 55.6 us a batch with one
+// pass; 2^22 skewed queries on 2^27 keys 556.6 -> 548.4.)
 
-#include "common.cuh"
+#include "layout.cuh"
 
 namespace pi {
 namespace {
@@ -67,16 +73,22 @@ __device__ uint32_t marker_before(const ApplyArgs& a, uint32_t tb, uint32_t* s_t
 // kSmall: a batch from k_rank_locate, whose storage-layer state is kept per query instead of
 // per distinct key.
 template <bool kSmall>
-__global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
+__global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArgs rb, uint32_t epoch) {
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t s_tmp[33];
+    __shared__ uint32_t s_tile, s_last, s_base[2];
+    __shared__ int s_fail;
     __shared__ int32_t s_delta[kLevelSlots];
     __shared__ int32_t s_tomb;
     __shared__ uint32_t s_changes, s_dirty;
     __shared__ uint32_t s_chist[kLevelSlots];  // built-level membership changes by height
 
     const int tid = threadIdx.x;
+    if (tid == 0) {
+        s_tile = atomicAdd(&a.bm->tile_ctr[kCtrApply], 1u);  // tiles in the order CTAs start
+        s_fail = 0;
+    }
     if (block_sees_error(&a.m->error)) return;
     const uint32_t n = a.n;
     const uint32_t qv = n - a.bm->invalid;
@@ -84,7 +96,7 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
     const uint32_t Lb = a.m->Lb;  // lowest built index level: changes below it leave the index alone
     uint64_t* SV = a.st.vals[cur];
     uint8_t* SM = a.st.meta[cur];
-    const uint32_t tile = blockIdx.x;
+    const uint32_t tile = s_tile, ntiles = gridDim.x;
     if (tid < kLevelSlots) {
         s_delta[tid] = 0;
         s_chist[tid] = 0;
@@ -231,11 +243,32 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
             new_mask |= 1u << k;
         }
     }
-    // New nodes: staged in this tile's slice of the staging arrays, in key order.
-    uint32_t tile_new = 0, slot = 0;
+    // Places of the tile's new nodes and level changes. Warp 0 looks back over the new
+    // nodes' counts, warp 1 over the changes'. A tile without any publishes its zero and goes
+    // on, but for every 64th, so that a look-back finds a prefix within two rounds.
+    uint32_t tile_new = 0, tile_chg = 0, slot = 0, cslot = 0;
     if (__syncthreads_or(new_here != 0)) slot = block_excl_sum<kApThreads>(new_here, s_tmp, &tile_new);
+    if (__syncthreads_or(chg_here != 0)) cslot = block_excl_sum<kApThreads>(chg_here, s_tmp, &tile_chg);
+    if (tid < 64) {
+        const uint32_t c = tid < 32 ? tile_new : tile_chg;
+        uint64_t* desc = a.desc + (tid < 32 ? 0u : ntiles);
+        if (c || (tile & 63u) == 0) {
+            bool ok = true;
+            const uint32_t ex = lookback_warp_wide<false, 8>(desc, tile, epoch, c, a.err, &ok);
+            if ((tid & 31) == 0) {
+                s_base[tid >> 5] = ex;
+                if (!ok) s_fail = 1;
+            }
+        } else if ((tid & 31) == 0) {
+            lookback_publish(desc, tile, epoch, 0u);
+        }
+    }
+    if (tile_new || tile_chg) {
+        __syncthreads();
+        if (s_fail) return;
+    }
     if (new_mask) {
-        const uint32_t so = tile * kApplyTile;
+        uint32_t o = s_base[0] + slot;
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {
             if (!(new_mask & (1u << k))) continue;
@@ -243,112 +276,58 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a) {
             const uint32_t jw = (e[k] - 3u) >> 1;
             const uint32_t pw = (jw == i) ? pay[k] : a.sp[jw];
             const uint32_t h = tower_height(key[k], a.hp);
-            a.stage.keys[so + slot] = key[k];
-            a.stage.vals[so + slot] = a.uvals[pw & kSeqMask];
-            a.stage.loc[so + slot] = a.loc[dres[k]];
-            a.stage.height[so + slot] = (uint8_t)h;
-            ++slot;
+            a.nn.keys[o] = key[k];
+            a.nn.vals[o] = a.uvals[pw & kSeqMask];
+            a.nn.loc[o] = a.loc[dres[k]];
+            a.nn.height[o] = (uint8_t)h;
+            ++o;
             atomicAdd(&s_changes, 1u);
             atomicAdd(&s_delta[1], 1);
             for (uint32_t l = 2; l <= h; ++l) atomicAdd(&s_delta[l], 1);
             if (h >= 2) s_dirty = 1;
         }
     }
-    // Built-level membership changes: staged the same way, for an incremental rebuild.
-    uint32_t tile_chg = 0, cslot = 0;
-    if (__syncthreads_or(chg_here != 0)) cslot = block_excl_sum<kApThreads>(chg_here, s_tmp, &tile_chg);
+    // Built-level membership changes, for an incremental rebuild.
     if (chg_mask) {
-        const uint32_t so = tile * kApplyTile;
+        uint32_t o = s_base[1] + cslot;
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {
             if (!(chg_mask & (1u << k))) continue;
             const uint32_t r = a.loc[dres[k]] - 1u;
             const uint8_t mt = SM[r];  // as this kernel left it
             const uint32_t h = mt & kHeightMask;
-            a.cstage.keys[so + cslot] = key[k];
-            a.cstage.pos[so + cslot] = r;
-            a.cstage.hl[so + cslot] = (uint8_t)(h | ((mt & kTomb) ? 0u : 0x80u));
-            ++cslot;
+            a.chg.keys[o] = key[k];
+            a.chg.pos[o] = r;
+            a.chg.hl[o] = (uint8_t)(h | ((mt & kTomb) ? 0u : 0x80u));
+            ++o;
             atomicAdd(&s_chist[h < (uint32_t)kLevelSlots ? h : kLevelSlots - 1], 1u);
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        a.tile_new[tile] = tile_new;
-        a.tile_chg[tile] = tile_chg;
-    }
     if (tid < kLevelSlots && s_chist[tid]) atomicAdd(&a.bm->chg_hist[tid], s_chist[tid]);
     if (tid < kLevelSlots && s_delta[tid]) atomicAdd(&a.bm->delta[tid], s_delta[tid]);
-    if (tid == 0) {
+    if (tid == 64) {
         if (s_tomb) atomicAdd(&a.bm->tomb_delta, s_tomb);
         if (s_changes) atomicAdd(&a.bm->changes, s_changes);
         if (s_dirty) atomicOr(&a.bm->index_dirty, 1u);
+        if (tile_new) atomicAdd(&a.bm->new_count, tile_new);
+        if (tile_chg) atomicAdd(&a.bm->nchg, tile_chg);
     }
-}
-
-// Exclusive sums of the per-tile new-node and level-change counts (one CTA); totals ->
-// bm->new_count and bm->nchg.
-__global__ void __launch_bounds__(1024) k_new_scan(ApplyArgs a) {
-    pdl_wait();
-    pdl_trigger();
-    __shared__ uint32_t s_tmp[33];
-    __shared__ uint32_t s_carry, s_ccarry;
-    if (block_sees_error(&a.m->error)) return;
-    const uint32_t ntiles = (a.n + kApplyTile - 1) / kApplyTile;
-    if (threadIdx.x == 0) {
-        s_carry = 0;
-        s_ccarry = 0;
+    // Arrival: the barrier orders every thread's stores before thread 0's fence, which (being
+    // cumulative) releases them before its count; the last CTA then sees all of them.
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        s_last = atomicAdd(&a.bm->tile_ctr[kCtrApplyDone], 1u) == ntiles - 1u ? 1u : 0u;
+        if (s_last) __threadfence();
     }
     __syncthreads();
-    for (uint32_t b0 = 0; b0 < ntiles; b0 += 1024) {
-        const uint32_t i = b0 + threadIdx.x;
-        const uint32_t v = i < ntiles ? a.tile_new[i] : 0u;
-        const uint32_t c = i < ntiles ? a.tile_chg[i] : 0u;
-        uint32_t tot, ctot;
-        const uint32_t ex = block_excl_sum<1024>(v, s_tmp, &tot);
-        const uint32_t cex = block_excl_sum<1024>(c, s_tmp, &ctot);
-        if (i < ntiles) {
-            a.tile_pref[i] = s_carry + ex;  // tile_pref is free again
-            a.tile_chg_pref[i] = s_ccarry + cex;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            s_carry += tot;
-            s_ccarry += ctot;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        a.bm->new_count = s_carry;
-        a.bm->nchg = s_ccarry;
-    }
-}
-
-// Packs each tile's staged new nodes and level changes to their places in key order.
-__global__ void __launch_bounds__(kThreads) k_new_pack(ApplyArgs a) {
-    pdl_wait();
-    pdl_trigger();
-    if (*(volatile const uint32_t*)&a.m->error) return;  // no barrier in this kernel
-    const uint32_t tile = blockIdx.x;
-    const uint32_t so = tile * kApplyTile;
-    const uint32_t c = a.tile_new[tile];
-    if (c) {
-        const uint32_t dst = a.tile_pref[tile];
-        for (uint32_t j = threadIdx.x; j < c; j += kThreads) {
-            a.nn.keys[dst + j] = a.stage.keys[so + j];
-            a.nn.vals[dst + j] = a.stage.vals[so + j];
-            a.nn.loc[dst + j] = a.stage.loc[so + j];
-            a.nn.height[dst + j] = a.stage.height[so + j];
-        }
-    }
-    const uint32_t cc = a.tile_chg[tile];
-    if (cc) {
-        const uint32_t dst = a.tile_chg_pref[tile];
-        for (uint32_t j = threadIdx.x; j < cc; j += kThreads) {
-            a.chg.keys[dst + j] = a.cstage.keys[so + j];
-            a.chg.pos[dst + j] = a.cstage.pos[so + j];
-            a.chg.hl[dst + j] = a.cstage.hl[so + j];
-        }
+    if (!s_last || tid >= 32) return;
+    const bool merge = merge_needed(a.m, a.bm);
+    if (merge) {
+        if (tid == 0) a.bm->merged = 1u;  // the merge's kernels end the batch
+    } else {
+        level_layout(rb, false);
     }
 }
 
@@ -379,15 +358,11 @@ __global__ void __launch_bounds__(kThreads) k_owner_check(ApplyArgs a) {
 
 }  // namespace
 
-cudaError_t launch_apply(const ApplyArgs& a, bool small, cudaStream_t s) {
+cudaError_t launch_apply(const ApplyArgs& a, const RebuildArgs& rb, bool small, uint32_t& epoch, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     const uint32_t tiles = (a.n + kApplyTile - 1) / kApplyTile;
-    if (small) launch_dep(k_apply<true>, tiles, kApThreads, 0, s, a);
-    else launch_dep(k_apply<false>, tiles, kApThreads, 0, s, a);  // tile prefixes come from the descent's scan
-    ++g_launches;
-    launch_dep(k_new_scan, 1, 1024, 0, s, a);
-    ++g_launches;
-    launch_dep(k_new_pack, tiles, kThreads, 0, s, a);
+    if (small) launch_dep(k_apply<true>, tiles, kApThreads, 0, s, a, rb, ++epoch);
+    else launch_dep(k_apply<false>, tiles, kApThreads, 0, s, a, rb, ++epoch);  // tile prefixes come from the descent
     ++g_launches;
     return cudaGetLastError();
 }

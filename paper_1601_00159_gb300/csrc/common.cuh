@@ -16,7 +16,9 @@ constexpr uint32_t kSmemTopMax = 12288;  // index entries staged in shared memor
 constexpr uint32_t kPad = 64;           // readable entries past every array's end
 constexpr uint32_t kSortTile = 2048;    // elements per radix-sort tile
 constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the count kernel's scan
-constexpr uint32_t kCtrDistinct = 14;   // BatchMeta::tile_ctr slot: the descent prologue's tile counter
+constexpr uint32_t kCtrDistinct = 14;   // BatchMeta::tile_ctr slots: the descent prologue's tile counter,
+constexpr uint32_t kCtrApply = 15;      // the apply kernel's, and its finished tiles
+constexpr uint32_t kCtrApplyDone = 16;
 constexpr uint32_t kApplyTile = 2048;   // sorted queries per apply tile
 constexpr uint32_t kSubTile = 256;      // sorted queries per descent warp step (one apply warp)
 constexpr uint32_t kRunTile = 1024;     // queries per tile of the small batches' sort
@@ -685,15 +687,10 @@ struct ApplyArgs {
     NewNodes nn;
     DevMeta* m;
     BatchMeta* bm;
-    uint64_t* desc;  // unused
-    uint32_t* tile_pref;  // per-tile exclusive prefix (max, then reused for new-node sums)
-    uint32_t* tile_new;   // per-tile new-node count
+    uint64_t* desc;            // look-back descriptors: 2 words per tile
+    const uint32_t* tile_pref; // per-tile exclusive marker prefix
     const uint32_t* sub_pref;  // dense index of each 256-query sub-tile's first distinct key
-    NewNodes stage;       // per-tile staging of new nodes (kApplyTile slots per tile)
-    LevelChanges cstage;  // per-tile staging of level membership changes
-    LevelChanges chg;     // the changes, packed in key order
-    uint32_t* tile_chg;   // per-tile change count
-    uint32_t* tile_chg_pref;
+    LevelChanges chg;          // level membership changes, in key order
     uint32_t* lcnt;  // per-level per-tile live counts (see RebuildArgs)
     uint32_t lstride;
     uint32_t n;
@@ -701,9 +698,11 @@ struct ApplyArgs {
     uint32_t* err;
     uint32_t* wcount;  // debug check (null when off): writes per storage node in this batch
 };
-// `small`: loc / flags / val0 hold one entry per query (launch_rank_locate), and the tile
+struct RebuildArgs;
+// Executes the sorted batch and, unless it re-lays-out the storage layer, ends it (the level
+// layout of rb). The look-back takes ++epoch. `small`: loc / flags / val0 hold one entry per query (launch_rank_locate), and the tile
 // prefixes are not given.
-cudaError_t launch_apply(const ApplyArgs& a, bool small, cudaStream_t s);
+cudaError_t launch_apply(const ApplyArgs& a, const RebuildArgs& rb, bool small, uint32_t& epoch, cudaStream_t s);
 // Debug check of single ownership: every storage node written at most once by the
 // batch's apply (sets kErrOwner otherwise); adds the writes to DevMeta::owner_writes and
 // clears the counts.

@@ -42,19 +42,14 @@ struct Scratch {
     uint8_t* flags = nullptr;
     uint64_t* val0 = nullptr;
     NewNodes nn{};
-    NewNodes stage{};
     uint32_t* tile_pref = nullptr;
-    uint32_t* tile_new = nullptr;
     uint32_t* tcnt = nullptr;  // radix sort: per-tile digit counts
     uint32_t* toff = nullptr;  // radix sort: per-tile digit offsets
     uint32_t* gsum = nullptr;  // radix sort: per-group digit totals / offsets
     uint32_t* gctr = nullptr;  // radix sort: the count kernels' arrival counters
     uint8_t* ndig = nullptr;   // radix sort: next pass's digits
     uint32_t* fixmap = nullptr;  // radix sort: segment marks of the prefix fix-up
-    LevelChanges cstage{};       // apply: per-tile staging of level membership changes
-    LevelChanges chg{};          // apply: the changes, packed in key order
-    uint32_t* tile_chg = nullptr;
-    uint32_t* tile_chg_pref = nullptr;
+    LevelChanges chg{};          // apply: level membership changes, in key order
     uint64_t* lst_keys = nullptr;  // incremental rebuild: per-level change lists
     uint32_t* lst_pos = nullptr;
     int32_t* lst_pref = nullptr;
@@ -316,11 +311,9 @@ void free_scratch(Scratch& s) {
     dfree(s.in_k); dfree(s.in_p); dfree(s.a_k); dfree(s.a_p); dfree(s.b_k); dfree(s.b_p);
     dfree(s.loc); dfree(s.flags); dfree(s.val0);
     dfree(s.nn.keys); dfree(s.nn.vals); dfree(s.nn.loc); dfree(s.nn.height);
-    dfree(s.stage.keys); dfree(s.stage.vals); dfree(s.stage.loc); dfree(s.stage.height);
-    dfree(s.tile_pref); dfree(s.tile_new);
+    dfree(s.tile_pref);
     dfree(s.tcnt); dfree(s.toff); dfree(s.ndig); dfree(s.fixmap); dfree(s.gsum); dfree(s.gctr);
-    dfree(s.cstage.keys); dfree(s.cstage.pos); dfree(s.cstage.hl); dfree(s.chg.keys); dfree(s.chg.pos); dfree(s.chg.hl);
-    dfree(s.tile_chg); dfree(s.tile_chg_pref);
+    dfree(s.chg.keys); dfree(s.chg.pos); dfree(s.chg.hl);
     dfree(s.lst_keys); dfree(s.lst_pos); dfree(s.lst_pref); dfree(s.lst_ins);
     dfree(s.sub_pref); dfree(s.dq); dfree(s.dlo);
     s.cap = 0;
@@ -337,19 +330,14 @@ cudaError_t alloc_scratch(Scratch& s, uint64_t q) {
     PI_TRY(dalloc(&s.nn.keys, c)); PI_TRY(dalloc(&s.nn.vals, c));
     PI_TRY(dalloc(&s.nn.loc, c)); PI_TRY(dalloc(&s.nn.height, c));
     const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
-    const uint64_t cs = tiles * kApplyTile;
-    PI_TRY(dalloc(&s.stage.keys, cs)); PI_TRY(dalloc(&s.stage.vals, cs));
-    PI_TRY(dalloc(&s.stage.loc, cs)); PI_TRY(dalloc(&s.stage.height, cs));
-    PI_TRY(dalloc(&s.tile_pref, tiles)); PI_TRY(dalloc(&s.tile_new, tiles));
+    PI_TRY(dalloc(&s.tile_pref, tiles));
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
     PI_TRY(dalloc(&s.tcnt, stiles * 256)); PI_TRY(dalloc(&s.toff, stiles * 256));
     const uint64_t sgroups = stiles / kScanGroup + 1;
     PI_TRY(dalloc(&s.gsum, sgroups * 256)); PI_TRY(dalloc(&s.gctr, 8 * (sgroups + 1)));
     PI_TRY(dalloc(&s.ndig, stiles * kSortTile + 16));
     PI_TRY(dalloc(&s.fixmap, c / 32 + 1));
-    PI_TRY(dalloc(&s.cstage.keys, cs)); PI_TRY(dalloc(&s.cstage.pos, cs)); PI_TRY(dalloc(&s.cstage.hl, cs));
     PI_TRY(dalloc(&s.chg.keys, c)); PI_TRY(dalloc(&s.chg.pos, c)); PI_TRY(dalloc(&s.chg.hl, c));
-    PI_TRY(dalloc(&s.tile_chg, tiles)); PI_TRY(dalloc(&s.tile_chg_pref, tiles));
     s.lst_cap = 2 * c + 64;
     PI_TRY(dalloc(&s.lst_keys, s.lst_cap)); PI_TRY(dalloc(&s.lst_pos, s.lst_cap));
     PI_TRY(dalloc(&s.lst_pref, s.lst_cap)); PI_TRY(dalloc(&s.lst_ins, s.lst_cap));
@@ -668,20 +656,17 @@ constexpr uint64_t al256(uint64_t b) { return (b + 255) & ~uint64_t(255); }
 
 constexpr uint64_t noalloc_bytes(uint64_t q) {
     const uint64_t c = q + kPad;
-    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1, cs = tiles * kApplyTile;
+    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
     const uint64_t nsub = (q + kSubTile - 1) / kSubTile + 1;
     return 3 * al256(c * 8) + 3 * al256(c * 4)                    // in, a, b (keys, payload)
            + al256(c * 4) + al256(c) + al256(c * 8)               // loc, flags, val0
            + 2 * al256(c * 8) + al256(c * 4) + al256(c)           // new nodes
-           + 2 * al256(cs * 8) + al256(cs * 4) + al256(cs)        // new-node staging
-           + 2 * al256(tiles * 4)                                 // tile prefix / new
+           + al256(tiles * 4)                                     // tile prefix
            + 2 * al256(stiles * 256 * 4) + al256(stiles * kSortTile + 16)  // tcnt, toff, ndig
            + al256((stiles / kScanGroup + 1) * 256 * 4) + al256(8 * (stiles / kScanGroup + 2) * 4)  // gsum, gctr
            + al256((c / 32 + 1) * 4)                              // fixmap
-           + al256(cs * 8) + al256(cs * 4) + al256(cs)            // level-change staging
            + al256(c * 8) + al256(c * 4) + al256(c)               // level changes
-           + 2 * al256(tiles * 4)                                 // per-tile change counts
            + al256((2 * c + 64) * 8) + 2 * al256((2 * c + 64) * 4) + al256(2 * c + 64)  // lists
            + al256(nsub * 4)                                      // sub_pref
            + al256(c * 8) + al256(c * 4);                         // dq, dlo
@@ -700,21 +685,18 @@ uint64_t carve_scratch(uint8_t* base, uint64_t q, Scratch& s) {
         off += al256(bytes);
     };
     const uint64_t c = q + kPad;
-    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1, cs = tiles * kApplyTile;
+    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
     const uint64_t nsub = (q + kSubTile - 1) / kSubTile + 1;
     take(s.in_k, c * 8); take(s.a_k, c * 8); take(s.b_k, c * 8);
     take(s.in_p, c * 4); take(s.a_p, c * 4); take(s.b_p, c * 4);
     take(s.loc, c * 4); take(s.flags, c); take(s.val0, c * 8);
     take(s.nn.keys, c * 8); take(s.nn.vals, c * 8); take(s.nn.loc, c * 4); take(s.nn.height, c);
-    take(s.stage.keys, cs * 8); take(s.stage.vals, cs * 8); take(s.stage.loc, cs * 4); take(s.stage.height, cs);
-    take(s.tile_pref, tiles * 4); take(s.tile_new, tiles * 4);
+    take(s.tile_pref, tiles * 4);
     take(s.tcnt, stiles * 256 * 4); take(s.toff, stiles * 256 * 4); take(s.ndig, stiles * kSortTile + 16);
     take(s.gsum, (stiles / kScanGroup + 1) * 256 * 4); take(s.gctr, 8 * (stiles / kScanGroup + 2) * 4);
     take(s.fixmap, (c / 32 + 1) * 4);
-    take(s.cstage.keys, cs * 8); take(s.cstage.pos, cs * 4); take(s.cstage.hl, cs);
     take(s.chg.keys, c * 8); take(s.chg.pos, c * 4); take(s.chg.hl, c);
-    take(s.tile_chg, tiles * 4); take(s.tile_chg_pref, tiles * 4);
     s.lst_cap = 2 * c + 64;
     take(s.lst_keys, s.lst_cap * 8); take(s.lst_pos, s.lst_cap * 4); take(s.lst_pref, s.lst_cap * 4);
     take(s.lst_ins, s.lst_cap);
@@ -854,22 +836,14 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     aa.bm = bm;
     aa.desc = x->desc;
     aa.tile_pref = sc.tile_pref;
-    aa.tile_new = sc.tile_new;
     aa.sub_pref = sc.sub_pref;
-    aa.stage = sc.stage;
-    aa.cstage = sc.cstage;
     aa.chg = sc.chg;
-    aa.tile_chg = sc.tile_chg;
-    aa.tile_chg_pref = sc.tile_chg_pref;
     aa.lcnt = x->lcnt;
     aa.lstride = x->lstride;
     aa.n = (uint32_t)n;
     aa.hp = x->hp;
     aa.err = &x->d_meta->error;
     aa.wcount = x->wcount;
-    if ((e = launch_apply(aa, small, s)) != cudaSuccess) return map_cuda(e);
-    if ((e = launch_owner_check(aa, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
-    prof_mark(x, 4, s);
     RebuildArgs ra = rebuild_args(x, bm, (uint32_t)size_ub, x->force_rebuild ? 1u : 0u);
     ra.nn = sc.nn;
     ra.chg = sc.chg;
@@ -878,6 +852,9 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     ra.lst_pref = sc.lst_pref;
     ra.lst_ins = sc.lst_ins;
     ra.lst_cap = (uint32_t)(sc.lst_cap > 0xFFFFFFF0ull ? 0xFFFFFFF0ull : sc.lst_cap);
+    if ((e = launch_apply(aa, ra, small, ep, s)) != cudaSuccess) return map_cuda(e);
+    if ((e = launch_owner_check(aa, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
+    prof_mark(x, 4, s);
     if ((e = launch_merge(ra, ep, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 5, s);
     if ((e = launch_level_bases(ra, s)) != cudaSuccess) return map_cuda(e);

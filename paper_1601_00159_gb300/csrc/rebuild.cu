@@ -19,9 +19,7 @@
 // deltas, so the layout (level bases, sentinels, staging split) is known before the
 // pass and the pass writes every entry exactly once.
 
-#include <cstddef>
-
-#include "common.cuh"
+#include "layout.cuh"
 
 namespace pi {
 namespace {
@@ -30,12 +28,6 @@ constexpr int kThreads = 256;
 constexpr int kNodes = 4096;             // storage nodes per tile
 constexpr int kPer = kNodes / kThreads;  // 16 per thread
 constexpr uint32_t kCtrMerge = 9, kCtrCreate = 11;
-
-__device__ __forceinline__ bool merge_needed(const DevMeta* m, const BatchMeta* bm) {
-    const uint32_t size = m->size;
-    const uint32_t tombs = (uint32_t)((int32_t)m->tombs + bm->tomb_delta);
-    return bm->new_count > 0 || (tombs > 0 && (uint64_t)tombs * 8u > size);
-}
 
 // Entries of the sorted a[0, n) below x, by a whole warp (every lane calls it and gets
 // the result): each round
@@ -104,7 +96,7 @@ __global__ void __launch_bounds__(kThreads) k_merge_count(RebuildArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevMeta* m = a.m;
     if (block_sees_error(&m->error)) return;
-    if (!merge_needed(m, a.bm)) return;
+    if (!a.bm->merged) return;
     const uint32_t size = m->size, ntiles = size / kNodes + 1;
     const uint8_t* M0 = a.st.meta[m->cur];
     uint32_t* live = a.mcnt;
@@ -175,7 +167,7 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a) {
     const int tid = threadIdx.x;
     const DevMeta* m = a.m;
     if (block_sees_error(&m->error)) return;
-    if (!merge_needed(m, a.bm)) return;
+    if (!a.bm->merged) return;
     const uint32_t size = m->size, src = m->cur, dst = src ^ 1u;
     const uint32_t newc = a.bm->new_count;
     const uint32_t ntiles = size / kNodes + 1;
@@ -280,161 +272,12 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a) {
     }
 }
 
-// ---------------------------------------------------------------------------------
-// Layout: apply the batch's deltas, switch storage buffers after a merge, decide the
-// rebuild, and lay the index levels out top-first with their sentinels.
-// Thread 0: sizes, re-layout switch, rebuild decision and level layout. Returns true
-// when the rebuild runs (the sentinels are then written by the caller's lanes).
-__device__ bool level_bases_body(RebuildArgs a) {
-    DevMeta* m = a.m;
-    BatchMeta* bm = a.bm;
-    if (*(volatile uint32_t*)&m->error) return false;
-    const bool merged = merge_needed(m, bm);
-    uint32_t tombs = (uint32_t)((int32_t)m->tombs + bm->tomb_delta);
-    uint32_t size = m->size;
-    if (merged) {
-        size = size - tombs + bm->new_count;
-        tombs = 0;
-        m->cur ^= 1u;
-    }
-    if (size > a.st_cap) {  // cannot happen when the host reserved capacity
-        atomicOr(a.err, kErrBounds);
-        return false;
-    }
-    m->size = size;
-    m->tombs = tombs;
-    bm->merged = merged ? 1u : 0u;
-    const uint32_t cur = m->cur;
-    a.st.keys[cur][size] = kMaxKey;
-    a.st.vals[cur][size] = 0;
-    a.st.meta[cur][size] = 0;
-    for (int l = 1; l < kLevelSlots; ++l) m->cnt[l] = (uint32_t)((int32_t)m->cnt[l] + bm->delta[l]);
-    m->updates += bm->changes;
-    m->sort_fix_big = bm->fix_big;
-    if (a.force_rebuild != 2u) m->batches += 1;
-
-    bool rebuild = a.force_rebuild || merged;
-    if (!rebuild && bm->index_dirty) {
-        if (a.rebuild_policy == 0) rebuild = true;
-        else rebuild = (uint64_t)m->updates * 100u >= (uint64_t)a.threshold_pct * (uint64_t)(size ? size : 1u);
-    }
-    bm->rebuild = rebuild ? 1u : 0u;
-    if (!rebuild) {
-        if (bm->index_dirty) m->levels_exact = 0;  // deferred: the levels now lag the storage layer
-        return false;
-    }
-    m->updates = 0;
-    m->rebuilds += 1;
-    // the layout being replaced, for an incremental rebuild
-    const uint32_t oH = m->H, oLb = m->Lb;
-    bm->old_H = oH;
-    bm->old_total = m->index_total;
-    for (int l = 0; l < kLevelSlots; ++l) {
-        bm->old_n[l] = m->n[l];
-        bm->old_base[l] = m->base[l];
-    }
-
-    uint32_t H = 1;
-    for (int l = 2; l < kLevelSlots; ++l)
-        if (m->cnt[l] > 0) H = (uint32_t)l;
-    // Lowest level that fits: drop bottom levels (the descent then scans longer storage
-    // gaps) rather than overrun the capacity; the host grows it later.
-    const uint32_t Lb0 = a.min_lb > 2u ? a.min_lb : 2u;
-    uint64_t need = 0;
-    for (uint32_t l = Lb0; l <= H; ++l) need += (uint64_t)m->cnt[l] + 1u;
-    uint32_t Lb = Lb0;
-    uint64_t fit = need;
-    while (Lb <= H && fit > a.index_cap) {
-        fit -= (uint64_t)m->cnt[Lb] + 1u;
-        ++Lb;
-    }
-    m->index_need = (uint32_t)need;
-    m->grow_request = (Lb > Lb0) ? 1u : 0u;
-    for (int l = 0; l < kLevelSlots; ++l) {
-        m->n[l] = 0;
-        m->base[l] = 0;
-    }
-    uint32_t off = 0;
-    for (int l = (int)H; l >= (int)Lb; --l) {
-        m->base[l] = off;
-        m->n[l] = m->cnt[l];
-        off += m->cnt[l] + 1u;
-    }
-    m->H = H;
-    m->Lb = Lb;
-    m->index_total = off;
-    uint32_t Ls = H + 1;
-    for (int l = (int)H; l >= (int)Lb; --l) {
-        if (m->base[l] + m->n[l] + 1u <= a.smem_top) Ls = (uint32_t)l;
-        else break;
-    }
-    m->Ls = Ls;
-    m->smem_entries = (Ls <= H) ? m->base[Ls] + m->n[Ls] + 1u : 0u;
-    // Incremental when the storage layer kept its layout and the old levels are exact:
-    // the new levels are the old ones plus the batch's membership changes, written to
-    // the other buffer. The per-level change lists must fit their arrays.
-    bool inc = !merged && a.force_rebuild == 0 && m->levels_exact && Lb == oLb && oLb <= oH && Lb <= H;
-    if (inc) {
-        const uint32_t Hm = H > oH ? H : oH;
-        uint64_t lists = 0, ge = 0;
-        for (int l = kLevelSlots - 1; l >= (int)Lb; --l) {
-            ge += bm->chg_hist[l];
-            if ((uint32_t)l <= Hm) lists += ge + 1u;
-        }
-        inc = lists <= a.lst_cap;
-    }
-    bm->inc = inc ? 1u : 0u;
-    if (inc) {
-        m->lcur ^= 1u;
-        m->inc_rebuilds += 1;
-    }
-    m->levels_exact = 1;
-    __threadfence_block();
-    return true;
-}
-
-// The body reads and writes the device meta and batch counters word by word on one
-// thread; it works on shared-memory copies loaded and stored by the whole warp, so its
-// dependent accesses cost shared-memory latency rather than L2 latency.
-__global__ void k_level_bases(RebuildArgs a) {
+// The end of a batch that was merged, or of a bulk build (the others end in the apply kernel).
+__global__ void __launch_bounds__(32) k_level_bases(RebuildArgs a) {
     pdl_wait();
     pdl_trigger();
-    __shared__ DevMeta s_m;
-    __shared__ BatchMeta s_bm;
-    __shared__ int s_go;
-    constexpr int kMW = sizeof(DevMeta) / 4, kBW = sizeof(BatchMeta) / 4;
-    static_assert(sizeof(DevMeta) % 4 == 0 && sizeof(BatchMeta) % 4 == 0, "word copies");
-    constexpr int kErrWord = offsetof(DevMeta, error) / 4;
-    uint32_t* sm = reinterpret_cast<uint32_t*>(&s_m);
-    uint32_t* sb = reinterpret_cast<uint32_t*>(&s_bm);
-    const uint32_t* gm = reinterpret_cast<const uint32_t*>(a.m);
-    const uint32_t* gb = reinterpret_cast<const uint32_t*>(a.bm);
-    for (int w = threadIdx.x; w < kMW; w += blockDim.x) sm[w] = gm[w];
-    for (int w = threadIdx.x; w < kBW; w += blockDim.x) sb[w] = gb[w];
-    if (threadIdx.x == 0) s_go = 0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        RebuildArgs b = a;
-        b.m = &s_m;
-        b.bm = &s_bm;
-        s_go = level_bases_body(b) ? 1 : 0;
-    }
-    __syncthreads();
-    // write back everything but the error word (errors are raised on the global copy)
-    uint32_t* gmw = reinterpret_cast<uint32_t*>(a.m);
-    for (int w = threadIdx.x; w < kMW; w += blockDim.x)
-        if (w != kErrWord) gmw[w] = sm[w];
-    uint32_t* gbw = reinterpret_cast<uint32_t*>(a.bm);
-    for (int w = threadIdx.x; w < kBW; w += blockDim.x) gbw[w] = sb[w];  // nothing else runs on it now
-    if (!s_go) return;
-    // sentinels of the built levels, one lane per level
-    const DevMeta& m = s_m;
-    const int l = (int)m.Lb + (int)threadIdx.x;
-    if (l <= (int)m.H) {
-        const uint32_t sidx = m.base[l] + m.n[l];
-        (m.lcur ? a.lkeys1 : a.lkeys)[sidx] = kMaxKey;
-        (m.lcur ? a.ldown1 : a.ldown)[sidx] = (l > (int)m.Lb) ? m.n[l - 1] : m.size;
-    }
+    const bool merged = a.bm->merged != 0;
+    if (merged || a.force_rebuild == 2u) level_layout(a, merged);
 }
 
 // ---------------------------------------------------------------------------------
