@@ -160,7 +160,6 @@ struct pi_index {
     uint64_t* desc = nullptr;
     uint64_t desc_words = 0;
     uint32_t* lcnt = nullptr;  // per-level per-tile live counts: 32 rows x lstride
-    uint32_t* mcnt = nullptr;  // merge: per-tile live counts and their prefix, 2 x lstride
     uint32_t* wcount = nullptr;  // PI_TEST_OWNER_CHECK: writes per storage node in a batch
     uint64_t wcap = 0;
     uint32_t* loff = nullptr;  // rebuild offsets, same shape
@@ -276,10 +275,8 @@ cudaError_t ensure_tile_cnt(pi_index* x, uint64_t st_cap) {
     if (stride <= x->lstride) return cudaSuccess;
     dfree(x->lcnt);
     dfree(x->loff);
-    dfree(x->mcnt);
     cudaError_t e = dalloc(&x->lcnt, 32 * stride);
     if (e == cudaSuccess) e = dalloc(&x->loff, 32 * stride);
-    if (e == cudaSuccess) e = dalloc(&x->mcnt, 2 * stride);
     if (e == cudaSuccess) e = cudaMemset(x->lcnt, 0, 32 * stride * sizeof(uint32_t));
     x->lstride = (e == cudaSuccess) ? (uint32_t)stride : 0u;
     x->force_rebuild = true;
@@ -436,7 +433,7 @@ void destroy(pi_index* x) {
     if (x->ev_last) cudaEventDestroy(x->ev_last);
     free_storage(x->st);
     dfree(x->lkeys); dfree(x->ldown); dfree(x->lkeys1); dfree(x->ldown1);
-    dfree(x->desc); dfree(x->lcnt); dfree(x->loff); dfree(x->mcnt); dfree(x->wcount); dfree(x->d_meta); dfree(x->d_bm); dfree(x->d_dofs); dfree(x->d_count);
+    dfree(x->desc); dfree(x->lcnt); dfree(x->loff); dfree(x->wcount); dfree(x->d_meta); dfree(x->d_bm); dfree(x->d_dofs); dfree(x->d_count);
     if (x->h_mbox) cudaFreeHost(x->h_mbox);
     if (x->ev_applied) cudaEventDestroy(x->ev_applied);
     if (x->ev_rebuilt) cudaEventDestroy(x->ev_rebuilt);
@@ -634,7 +631,6 @@ RebuildArgs rebuild_args(pi_index* x, BatchMeta* bm, uint32_t size_ub, uint32_t 
     r.desc = x->desc;
     r.lcnt = x->lcnt;
     r.loff = x->loff;
-    r.mcnt = x->mcnt;
     r.lstride = x->lstride;
     r.index_cap = (uint32_t)(x->idx_cap > 0xFFFFFFF0ull ? 0xFFFFFFF0ull : x->idx_cap);
     r.size_ub = size_ub;
@@ -857,7 +853,6 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     prof_mark(x, 4, s);
     if ((e = launch_merge(ra, ep, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 5, s);
-    if ((e = launch_level_bases(ra, s)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 6, s);
     const uint64_t slot = x->issued % kRing;
     if (x->issued - x->seen >= kRing) {  // the slot is still unread: wait for its batch
@@ -1046,8 +1041,7 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         cudaMemsetAsync(x->d_bm, 0, sizeof(BatchMeta), s);
         RebuildArgs ra = rebuild_args(x, x->d_bm, (uint32_t)hm.size, 2u);
         uint32_t ep = next_epochs(x, 4, s);
-        if ((e = launch_merge(ra, ep, s, x->num_sms)) != cudaSuccess) break;
-        if ((e = launch_level_bases(ra, s)) != cudaSuccess) break;
+        if ((e = launch_level_layout(ra, s)) != cudaSuccess) break;
         if ((e = launch_rebuild(ra, ep, s, x->num_sms)) != cudaSuccess) break;
         x->epoch = ep;
         if ((e = read_meta(x, s, &x->known)) != cudaSuccess) break;
