@@ -108,7 +108,7 @@ def tuned_plain(keys):
 
 # The sources of the single-index batch path (the kernels a capture of the skewed
 # workload measures, and the host code that launches them).
-BATCH_PATH_SOURCES = ("common.cuh", "layout.cuh", "sort.cu", "descend.cu", "apply.cu", "rebuild.cu", "relevel.cu", "pi.cu")
+BATCH_PATH_SOURCES = ("common.cuh", "layout.cuh", "sort.cu", "descend.cu", "apply.cu", "rebuild.cu", "relevel.cuh", "pi.cu")
 
 
 def source_digest():
@@ -1050,7 +1050,7 @@ def run_ours(args, ws, rank, local):
     rebuilds_region = info1["rebuilds"] - info0["rebuilds"]
     entries = sum(sizes[lowest:])
     if rebuilds_region and inc_region == rebuilds_region:
-        wkernel, wbytes = "k_relevel_write", 24 * entries
+        wkernel, wbytes = "k_rebuild_write", 24 * entries
         wmodel = "12 B read + 12 B written per built index entry (incremental rebuild)"
     else:
         wkernel, wbytes = "k_rebuild_write", 9 * info1["size"] + 12 * entries

@@ -740,7 +740,6 @@ struct RebuildArgs {
     uint8_t* lst_ins;
     uint32_t lst_cap;        // entries the lists hold (an incremental rebuild needs them all)
 };
-cudaError_t launch_relevel(const RebuildArgs& a, cudaStream_t s, int num_sms);
 cudaError_t launch_merge(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms);
 cudaError_t launch_level_layout(const RebuildArgs& a, cudaStream_t s);
 // ---------------------------------------------------------------------------------

@@ -22,6 +22,7 @@
 #include <cstddef>
 
 #include "layout.cuh"
+#include "relevel.cuh"
 
 namespace pi {
 namespace {
@@ -369,18 +370,23 @@ __global__ void __launch_bounds__(256) k_rebuild_count(RebuildArgs a) {
 // Per built level, exclusive scan of the tile counts over tiles. Grid: (chunks, levels);
 // each CTA scans kScanChunk tiles (4 per thread) and gets the prefix of the chunks
 // before it by a warp-wide decoupled look-back (the chain is a few chunks long). The
-// level's last chunk checks the total against the level size.
+// level's last chunk checks the total against the level size. In an incremental rebuild
+// the first CTA of each row builds a level's change list instead.
 constexpr uint32_t kScanChunk = 4096;
 
-__global__ void __launch_bounds__(1024) k_rebuild_scan(RebuildArgs a, uint32_t epoch) {
+__global__ void __launch_bounds__(1024) k_rebuild_prep(RebuildArgs a, uint32_t epoch) {
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t s_tmp[33];
     __shared__ uint32_t s_prefix;
     __shared__ int s_ok;
     const DevMeta* m = a.m;
+    if (!a.bm->rebuild) return;
     if (block_sees_error(&m->error)) return;
-    if (!a.bm->rebuild || a.bm->inc) return;  // an incremental rebuild needs no tile offsets
+    if (a.bm->inc) {  // an incremental rebuild needs its change lists, not tile offsets
+        if (blockIdx.x == 0) relevel::lists(a, blockIdx.y, s_tmp);
+        return;
+    }
     const uint32_t H = m->H, Lb = m->Lb, size = m->size;
     const uint32_t l = Lb + blockIdx.y;
     if (H < Lb || size == 0 || l > H) return;
@@ -448,21 +454,38 @@ constexpr uint32_t kWarpNodes = kNodes / 8;  // 512 nodes per warp
 //     (coalesced stores), and compacts the list in place to the members of level
 //     Lb + 1, keeping each one's index in level Lb for its down pointer; the next
 //     levels repeat step 3 on the shrinking list.
-__global__ void __launch_bounds__(kThreads) k_rebuild_write(RebuildArgs a) {
+// An incremental rebuild writes from the previous levels instead (relevel.cuh). One kernel
+// for both, since the host cannot know which a batch needs and a launch that only exits costs
+// it 3 us (the rebuild was five launches: 1000 lookups 47.6 -> 40.4 us a batch, 6000 mixed
+// queries 55.6 -> 50.7). Six CTAs per SM at 40 registers measured best over both kinds.
+union WriteSmem {
+    struct {
+        uint8_t meta[kMetaBytes];
+        uint32_t list[8 * kWarpNodes];
+        uint32_t wcnt[8][32];
+    } full;
+    relevel::WriteSmem inc;
+};
+
+__global__ void __launch_bounds__(kThreads, 6) k_rebuild_write(RebuildArgs a) {
     pdl_wait();
     pdl_trigger();
-    extern __shared__ __align__(16) uint8_t s_dyn[];
-    uint8_t* s_meta = s_dyn;                                              // kNodes + 16
-    uint32_t* s_list = reinterpret_cast<uint32_t*>(s_dyn + kMetaBytes);   // 8 x 512
+    __shared__ __align__(16) WriteSmem s_u;
     __shared__ __align__(8) uint64_t s_bar;
-    __shared__ uint32_t s_wcnt[8][32];
     __shared__ uint32_t s_base[kLevelSlots], s_n[kLevelSlots];
     __shared__ int s_ok;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevMeta* m = a.m;
-    if (a.bm->inc || !a.bm->rebuild) return;  // the incremental path writes the levels instead
+    if (!a.bm->rebuild) return;
     if (block_sees_error(&m->error)) return;
+    if (a.bm->inc) {
+        relevel::write(a, blockIdx.x, gridDim.x, s_u.inc);
+        return;
+    }
+    uint8_t* s_meta = s_u.full.meta;
+    uint32_t* s_list = s_u.full.list;
+    auto& s_wcnt = s_u.full.wcnt;
     const uint32_t H = m->H, Lb = m->Lb, size = m->size, cur = m->cur;
     if (H < Lb || size == 0) return;
     uint64_t* LK = m->lcur ? a.lkeys1 : a.lkeys;  // the index layer's buffer in use
@@ -743,26 +766,23 @@ cudaError_t launch_level_layout(const RebuildArgs& a, cudaStream_t s) {
 
 cudaError_t launch_rebuild_prep(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms) {
     const uint32_t tiles = (a.size_ub + kNodes - 1) / kNodes + 1;
-    const uint32_t cb = (tiles + 7) / 8, ccap = (uint32_t)num_sms * 4u;
-    launch_dep(k_rebuild_count, cb < ccap ? cb : ccap, 256, 0, s, a);  // exits at once unless recounting
-    ++g_launches;
+    if (a.force_rebuild) {  // the counts are recounted (unless the batch merged)
+        const uint32_t cb = (tiles + 7) / 8, ccap = (uint32_t)num_sms * 4u;
+        launch_dep(k_rebuild_count, cb < ccap ? cb : ccap, 256, 0, s, a);
+        ++g_launches;
+    }
     const uint32_t chunks = (tiles + kScanChunk - 1) / kScanChunk;
-    launch_dep(k_rebuild_scan, dim3(chunks, kLevelSlots - 2), 1024, 0, s, a, ++epoch);
+    launch_dep(k_rebuild_prep, dim3(chunks, kLevelSlots - 2), 1024, 0, s, a, ++epoch);
     ++g_launches;
     return cudaGetLastError();
 }
 
 cudaError_t launch_rebuild_write(const RebuildArgs& a, cudaStream_t s, int num_sms) {
-    static bool attr_set = false;
-    const int dyn = (int)(kMetaBytes + 8 * kWarpNodes * 4);
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_rebuild_write, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    const uint32_t tiles = (a.size_ub + kNodes - 1) / kNodes + 1;
-    const uint32_t cap = (uint32_t)num_sms * 8u;  // persistent: the CTAs resident at once
-    launch_dep(k_rebuild_write, tiles < cap ? tiles : cap, kThreads, dyn, s, a);
+    const uint32_t cap = (uint32_t)num_sms * 6u;  // the CTAs resident at once
+    // per tile of the storage layer, or of the levels and their changes (fewer but for change
+    // lists, which a batch's queries bound)
+    const uint32_t tiles = (a.size_ub + kNodes - 1) / kNodes + 1 + a.lst_cap / (2u * 256u) + kLevelSlots;
+    launch_dep(k_rebuild_write, tiles < cap ? tiles : cap, kThreads, 0, s, a);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -4,9 +4,9 @@
 // lowest built level; every other key keeps its storage position. The rebuild then reads
 // the old levels (the buffer not in use after the layout step flipped DevMeta::lcur) and
 // writes the new ones, instead of scanning the storage layer and gathering member keys:
-//   k_relevel_lists   one CTA per level l: the batch's changes of height >= l, in key
+//   lists (k_rebuild_prep)   one CTA per level l: the batch's changes of height >= l, in key
 //                     order, with the running count (inserts - deletes) before each;
-//   k_relevel_write   every old entry moves by the running count of its level's list
+//   write (k_rebuild_write)  every old entry moves by the running count of its level's list
 //                     before its key (or goes, if deleted); its down pointer into level
 //                     l - 1 moves by that level's running count; every insert lands at
 //                     (old entries below its key) + (running count before it).
@@ -14,13 +14,15 @@
 // live keys of height >= l in key order, with the position of the same key one level
 // down (or in the storage layer, at the lowest built level).
 
+#pragma once
+
 #include "common.cuh"
 
 namespace pi {
-namespace {
+namespace relevel {
 
 constexpr int kT = 256;
-constexpr uint32_t kItems = 8;
+constexpr uint32_t kItems = 4;
 constexpr uint32_t kTile = kT * kItems;  // old entries per tile
 constexpr uint32_t kSlice = 512;         // list entries staged in shared memory per tile and level
 
@@ -60,17 +62,13 @@ __device__ __forceinline__ uint32_t lb_keys(const uint64_t* K, uint32_t n, uint6
     return lo;
 }
 
-__global__ void __launch_bounds__(1024) k_relevel_lists(RebuildArgs a) {
-    pdl_wait();
-    pdl_trigger();
-    __shared__ uint32_t s_tmp[33];
+// Level Lb + row's change list, by a CTA of 1024 threads.
+__device__ void lists(const RebuildArgs& a, uint32_t row, uint32_t* s_tmp) {
     __shared__ uint32_t s_off;
     const DevMeta* m = a.m;
     BatchMeta* bm = a.bm;
-    if (block_sees_error(&m->error)) return;
-    if (!bm->inc) return;
     const uint32_t Lb = m->Lb, Hm = m->H > bm->old_H ? m->H : bm->old_H;
-    const uint32_t l = Lb + blockIdx.x;
+    const uint32_t l = Lb + row;
     if (l > Hm) return;
     if (threadIdx.x == 0) {
         uint32_t off = 0;
@@ -176,18 +174,18 @@ __device__ __forceinline__ uint32_t slice_rank(const uint64_t* sk, uint32_t len,
     return lo;
 }
 
-__global__ void __launch_bounds__(kT, 4) k_relevel_write(RebuildArgs a) {
-    pdl_wait();
-    pdl_trigger();
-    __shared__ uint32_t s_apref[kLevelSlots + 1], s_bpref[kLevelSlots + 1];
-    __shared__ uint32_t s_ta, s_tb;
-    __shared__ uint64_t s_k0[kSlice], s_k1[kSlice];
-    __shared__ int32_t s_p0[kSlice + 1], s_p1[kSlice + 1];
-    __shared__ uint32_t s_j0, s_len0, s_j1, s_len1;
+// The shared memory of the writer, in the rebuild kernel's dynamic block.
+struct WriteSmem {
+    uint64_t k0[kSlice], k1[kSlice];
+    int32_t p0[kSlice + 1], p1[kSlice + 1];
+    uint32_t apref[kLevelSlots + 1], bpref[kLevelSlots + 1];
+    uint32_t ta, tb, j0, len0, j1, len1;
+};
+
+// The new levels, by CTAs `cta` of `ctas`, kT threads each.
+__device__ void write(const RebuildArgs& a, uint32_t cta, uint32_t ctas, WriteSmem& s) {
     const DevMeta* m = a.m;
     const BatchMeta* bm = a.bm;
-    if (block_sees_error(&m->error)) return;
-    if (!bm->inc) return;
     const uint32_t Lb = m->Lb, H = m->H, oH = bm->old_H, Hm = H > oH ? H : oH;
     const uint64_t* OK = m->lcur ? a.lkeys : a.lkeys1;  // the previous buffer
     const uint32_t* OD = m->lcur ? a.ldown : a.ldown1;
@@ -197,26 +195,26 @@ __global__ void __launch_bounds__(kT, 4) k_relevel_write(RebuildArgs a) {
     if (tid == 0) {
         uint32_t t = 0;
         for (uint32_t l = Lb; l <= Hm + 1u && l <= (uint32_t)kLevelSlots; ++l) {
-            s_bpref[l] = t;
+            s.bpref[l] = t;
             if (l <= Hm) t += (bm->lst_n[l] + kT - 1u) / kT;
         }
-        s_tb = t;
+        s.tb = t;
         t = 0;
         for (uint32_t l = Lb; l <= Hm + 1u && l <= (uint32_t)kLevelSlots; ++l) {
-            s_apref[l] = t;
+            s.apref[l] = t;
             if (l <= oH) t += (bm->old_n[l] + kTile - 1u) / kTile;
         }
-        s_ta = t;
+        s.ta = t;
     }
     __syncthreads();
-    const uint32_t TA = s_ta, TB = s_tb;
+    const uint32_t TA = s.ta, TB = s.tb;
     // The inserts come first: their searches are long chains of dependent loads, which
     // then overlap with the streaming of the old entries on the other CTAs.
-    for (uint32_t t = blockIdx.x; t < TA + TB; t += gridDim.x) {
+    for (uint32_t t = cta; t < TA + TB; t += ctas) {
         if (t < TB) {
             uint32_t l = Lb;
-            while (l < Hm && s_bpref[l + 1] <= t) ++l;
-            const uint32_t c = (t - s_bpref[l]) * kT + (uint32_t)tid;
+            while (l < Hm && s.bpref[l + 1] <= t) ++l;
+            const uint32_t c = (t - s.bpref[l]) * kT + (uint32_t)tid;
             const uint32_t off0 = bm->lst_off[l];
             if (c < bm->lst_n[l] && a.lst_ins[off0 + c]) {
                 const uint64_t key = a.lst_keys[off0 + c];
@@ -241,20 +239,20 @@ __global__ void __launch_bounds__(kT, 4) k_relevel_write(RebuildArgs a) {
         // a tile of old entries of level l (warp-contiguous: entry i0 + k * kT + tid)
         const uint32_t ta = t - TB;
         uint32_t l = Lb;
-        while (l < oH && s_apref[l + 1] <= ta) ++l;
-        const uint32_t i0 = (ta - s_apref[l]) * kTile;
+        while (l < oH && s.apref[l + 1] <= ta) ++l;
+        const uint32_t i0 = (ta - s.apref[l]) * kTile;
         const uint32_t on = bm->old_n[l];
         const uint32_t i1 = i0 + kTile < on ? i0 + kTile : on;
         const uint32_t ob = bm->old_base[l];
         const uint64_t kmin = OK[ob + i0], kmax = OK[ob + i1 - 1u];
         const uint32_t off0 = bm->lst_off[l], n0 = bm->lst_n[l];
-        const bool st0 = stage_slice(a, off0, n0, kmin, kmax, s_k0, s_p0, &s_j0, &s_len0);
+        const bool st0 = stage_slice(a, off0, n0, kmin, kmax, s.k0, s.p0, &s.j0, &s.len0);
         bool st1 = true;
         uint32_t off1 = 0, n1 = 0;
         if (l > Lb) {
             off1 = bm->lst_off[l - 1];
             n1 = bm->lst_n[l - 1];
-            st1 = stage_slice(a, off1, n1, kmin, kmax, s_k1, s_p1, &s_j1, &s_len1);
+            st1 = stage_slice(a, off1, n1, kmin, kmax, s.k1, s.p1, &s.j1, &s.len1);
         }
         __syncthreads();
         const uint32_t nb = m->base[l], nl = m->n[l];
@@ -275,9 +273,9 @@ __global__ void __launch_bounds__(kT, 4) k_relevel_write(RebuildArgs a) {
             bool hit;
             int32_t shift;
             if (st0) {
-                const uint32_t x = slice_rank(s_k0, s_len0, key);
-                hit = x < s_len0 && s_k0[x] == key;
-                shift = s_p0[x];
+                const uint32_t x = slice_rank(s.k0, s.len0, key);
+                hit = x < s.len0 && s.k0[x] == key;
+                shift = s.p0[x];
             } else {
                 const uint32_t j = lb_keys(a.lst_keys + off0, n0, key);
                 hit = j < n0 && a.lst_keys[off0 + j] == key;
@@ -286,7 +284,7 @@ __global__ void __launch_bounds__(kT, 4) k_relevel_write(RebuildArgs a) {
             if (hit) continue;  // the key was deleted (an existing entry is never an insert)
             const uint32_t out = i + (uint32_t)shift;
             if (l > Lb) {
-                const int32_t s1 = st1 ? s_p1[slice_rank(s_k1, s_len1, key)]
+                const int32_t s1 = st1 ? s.p1[slice_rank(s.k1, s.len1, key)]
                                        : a.lst_pref[off1 + lb_keys(a.lst_keys + off1, n1, key)];
                 nd += (uint32_t)s1;
             }
@@ -301,14 +299,5 @@ __global__ void __launch_bounds__(kT, 4) k_relevel_write(RebuildArgs a) {
     }
 }
 
-}  // namespace
-
-cudaError_t launch_relevel(const RebuildArgs& a, cudaStream_t s, int num_sms) {
-    launch_dep(k_relevel_lists, kLevelSlots, 1024, 0, s, a);
-    ++g_launches;
-    launch_dep(k_relevel_write, (uint32_t)num_sms * 4u, kT, 0, s, a);  // the CTAs resident at once
-    ++g_launches;
-    return cudaGetLastError();
-}
-
+}  // namespace relevel
 }  // namespace pi
