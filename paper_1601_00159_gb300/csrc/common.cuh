@@ -739,6 +739,8 @@ struct RebuildArgs {
     int32_t* lst_pref;       // entries' running (inserts - deletes) before them; one extra at the end
     uint8_t* lst_ins;
     uint32_t lst_cap;        // entries the lists hold (an incremental rebuild needs them all)
+    DevMeta* mbox;           // the batch's slot of the host's mailbox ring (mapped host memory)
+    BatchMeta* bm_next;      // the next batch's counters, cleared when this one ends
 };
 cudaError_t launch_merge(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms);
 cudaError_t launch_level_layout(const RebuildArgs& a, cudaStream_t s);

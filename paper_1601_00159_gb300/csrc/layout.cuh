@@ -131,4 +131,20 @@ __device__ __forceinline__ void level_layout(const RebuildArgs& a, bool merged) 
     }
 }
 
+// The last step of a batch, by one warp: the device meta goes to the batch's mailbox slot, which
+// the host reads once the batch's event has completed, and the next batch's counters are
+// cleared (their previous user, the rebuild of the batch before this one, has finished: this
+// batch's descent waited for it). In the kernel these cost no copy or memset on the stream.
+__device__ __forceinline__ void post_batch(const RebuildArgs& a) {
+    const uint32_t lane = threadIdx.x & 31u;
+    constexpr uint32_t kMetaWords = sizeof(DevMeta) / 4, kBatchWords = sizeof(BatchMeta) / 4;
+    static_assert(sizeof(DevMeta) % 4 == 0 && sizeof(BatchMeta) % 4 == 0, "word copies");
+    __syncwarp();
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(a.m);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(a.mbox);
+    uint32_t* nxt = reinterpret_cast<uint32_t*>(a.bm_next);
+    for (uint32_t w = lane; w < kMetaWords; w += 32u) dst[w] = __ldcg(&src[w]);
+    for (uint32_t w = lane; w < kBatchWords; w += 32u) nxt[w] = 0u;
+}
+
 }  // namespace pi

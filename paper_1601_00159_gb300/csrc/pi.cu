@@ -165,8 +165,8 @@ struct pi_index {
     uint32_t* loff = nullptr;  // rebuild offsets, same shape
     uint32_t lstride = 0;
     uint32_t epoch = 1;
-    // Ring of mailboxes: batch b copies the device meta to slot b % kRing and records
-    // ev[b % kRing]; the newest completed slot bounds the host's view of the sizes.
+    // Ring of mailboxes: batch b's last kernel writes the device meta to slot b % kRing, and
+    // ev[b % kRing] marks the batch's end; the newest completed slot bounds the host's view of the sizes.
     DevMeta* h_mbox = nullptr;  // pinned, kRing slots
     cudaEvent_t ev[64] = {};
     uint64_t ring_n[64] = {};   // queries of the batch in each slot
@@ -176,6 +176,7 @@ struct pi_index {
     uint64_t pending_n = 0;  // queries issued after that snapshot
     uint64_t extra_n = 0;    // queries of batching-form calls since the last full sync
     bool force_rebuild = false;
+    bool bm_clear = false;   // the next batch's counters are zero (the last batch cleared them)
     // With small_mode 1, small batches (Q <= kSmallBatch on at most kSmallIndex nodes) run
     // through a one-index batching set whose batch takes a thread-block cluster: one
     // launch instead of the level-synchronous pipeline's tens. Created on first use.
@@ -193,7 +194,7 @@ struct pi_index {
     // own stream, overlapping the next batch's sort; the next batch's descent waits for
     // it (ev_rebuilt), and so does every other use of the index state.
     cudaStream_t rs = nullptr;
-    cudaEvent_t ev_applied = nullptr, ev_rebuilt = nullptr;
+    cudaEvent_t ev_rebuilt = nullptr;
     bool rebuild_pending = false;
     // The index's last operation (a batch, a range search or a batching-form call) ends
     // at last_ev on last_stream; an entry point on another stream first waits for it.
@@ -435,7 +436,6 @@ void destroy(pi_index* x) {
     dfree(x->lkeys); dfree(x->ldown); dfree(x->lkeys1); dfree(x->ldown1);
     dfree(x->desc); dfree(x->lcnt); dfree(x->loff); dfree(x->wcount); dfree(x->d_meta); dfree(x->d_bm); dfree(x->d_dofs); dfree(x->d_count);
     if (x->h_mbox) cudaFreeHost(x->h_mbox);
-    if (x->ev_applied) cudaEventDestroy(x->ev_applied);
     if (x->ev_rebuilt) cudaEventDestroy(x->ev_rebuilt);
     if (x->rs) cudaStreamDestroy(x->rs);
     for (auto& e : x->ev)
@@ -466,21 +466,17 @@ cudaError_t read_meta(pi_index* x, cudaStream_t s, DevMeta* out) {
 
 constexpr uint64_t kRing = 64;
 
-// Non-blocking: adopt the newest completed batch's mailbox.
+// Non-blocking: adopt the newest completed batch's mailbox. Batches complete in order, so the
+// events are asked from the oldest on: one that is not ready, and one per batch since.
 void refresh_known(pi_index* x) {
     uint64_t newest = x->seen;
-    for (uint64_t b = x->issued; b > x->seen; --b) {
-        if (cudaEventQuery(x->ev[(b - 1) % kRing]) == cudaSuccess) {
-            newest = b;
-            break;
-        }
+    while (newest < x->issued && cudaEventQuery(x->ev[newest % kRing]) == cudaSuccess) {
+        x->pending_n -= x->ring_n[newest % kRing];
+        ++newest;
     }
     if (newest == x->seen) return;
     x->known = x->h_mbox[(newest - 1) % kRing];
     x->seen = newest;
-    uint64_t p = 0;
-    for (uint64_t b = newest; b < x->issued; ++b) p += x->ring_n[b % kRing];
-    x->pending_n = p;
 }
 
 // Makes `s` wait for the background rebuild still in flight, if any (no host sync).
@@ -493,9 +489,9 @@ void order_after_last(pi_index* x, cudaStream_t s) {
     if (x->has_last && x->last_stream != s) cudaStreamWaitEvent(s, x->last_ev, 0);
 }
 
-void mark_last(pi_index* x, cudaStream_t s) {
-    cudaEventRecord(x->ev_last, s);
-    x->last_ev = x->ev_last;
+void mark_last(pi_index* x, cudaStream_t s, cudaEvent_t recorded = nullptr) {
+    if (!recorded) cudaEventRecord(x->ev_last, s);
+    x->last_ev = recorded ? recorded : x->ev_last;
     x->last_stream = s;
     x->has_last = true;
 }
@@ -780,7 +776,8 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     uint32_t ep = next_epochs(x, 16, s);
     if (x->prof && x->pused == kProfSlots) prof_fold(x);
     prof_mark(x, 0, s);
-    cudaMemsetAsync(bm, 0, sizeof(BatchMeta), s);
+    if (!x->bm_clear) cudaMemsetAsync(bm, 0, sizeof(BatchMeta), s);  // else the batch before cleared it
+    x->bm_clear = false;
     SortBuffers sb = sort_buffers(x, sc);
     const bool small = small_front(x, n);
     e = small ? launch_tile_sort(ops, keys, (uint32_t)n, sb, bm, s)
@@ -848,22 +845,23 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     ra.lst_pref = sc.lst_pref;
     ra.lst_ins = sc.lst_ins;
     ra.lst_cap = (uint32_t)(sc.lst_cap > 0xFFFFFFF0ull ? 0xFFFFFFF0ull : sc.lst_cap);
+    const uint64_t slot = x->issued % kRing;
+    if (x->issued - x->seen >= kRing) {  // the slot is still unread: wait for its batch
+        cudaEventSynchronize(x->ev[slot]);
+        refresh_known(x);
+    }
+    ra.mbox = &x->h_mbox[slot];
+    ra.bm_next = x->d_bm + ((x->issued + 1u) & 1u);
     if ((e = launch_apply(aa, ra, small, ep, s)) != cudaSuccess) return map_cuda(e);
     if ((e = launch_owner_check(aa, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 4, s);
     if ((e = launch_merge(ra, ep, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 5, s);
     prof_mark(x, 6, s);
-    const uint64_t slot = x->issued % kRing;
-    if (x->issued - x->seen >= kRing) {  // the slot is still unread: wait for its batch
-        cudaEventSynchronize(x->ev[slot]);
-        refresh_known(x);
-    }
-    cudaMemcpyAsync(&x->h_mbox[slot], x->d_meta, sizeof(DevMeta), cudaMemcpyDeviceToHost, s);
+    // the batch's end: the mailbox is written, results are complete
     cudaEventRecord(x->ev[slot], s);
     // the rebuild, in the background
-    cudaEventRecord(x->ev_applied, s);
-    cudaStreamWaitEvent(x->rs, x->ev_applied, 0);
+    cudaStreamWaitEvent(x->rs, x->ev[slot], 0);
     prof_mark(x, 7, x->rs);
     if ((e = launch_rebuild_prep(ra, ep, x->rs, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 8, x->rs);
@@ -874,9 +872,11 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     if (x->prof) x->pused++;
     x->epoch = ep;
     x->force_rebuild = false;
+    x->bm_clear = true;
     x->ring_n[slot] = n;
     x->issued++;
     x->pending_n += n;
+    mark_last(x, s, x->ev[slot]);
     return map_cuda(cudaGetLastError());
 }
 
@@ -886,7 +886,6 @@ int enqueue_batch(pi_index* x, const Scratch& sc, const uint8_t* ops, const uint
     g_ktimer = x->kt;
     const int r = enqueue_batch_body(x, sc, ops, keys, values, n, results, size_ub, s);
     g_ktimer = nullptr;
-    if (r == PI_OK) mark_last(x, s);
     x->launches += g_launches - l0;
     return r;
 }
@@ -980,7 +979,6 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         if ((e = dalloc(&x->d_meta, 1)) != cudaSuccess) break;
         if ((e = dalloc(&x->d_bm, 2)) != cudaSuccess) break;
         if ((e = cudaStreamCreateWithFlags(&x->rs, cudaStreamNonBlocking)) != cudaSuccess) break;
-        if ((e = cudaEventCreateWithFlags(&x->ev_applied, cudaEventDisableTiming)) != cudaSuccess) break;
         if ((e = cudaEventCreateWithFlags(&x->ev_rebuilt, cudaEventDisableTiming)) != cudaSuccess) break;
         if ((e = cudaEventCreateWithFlags(&x->ev_last, cudaEventDisableTiming)) != cudaSuccess) break;
         if ((e = dalloc(&x->d_dofs, 8 * 256)) != cudaSuccess) break;
@@ -1184,6 +1182,7 @@ int pi_range_search(pi_index_t* x, const uint64_t* lo, const uint64_t* hi, uint6
     cudaMemcpyAsync(x->r_bounds, lo, n * 8, cudaMemcpyDeviceToDevice, s);
     cudaMemcpyAsync(x->r_bounds + n, hi, n * 8, cudaMemcpyDeviceToDevice, s);
     BatchMeta* bm = x->d_bm + (x->issued & 1u);  // the other block may still be read by the rebuild
+    x->bm_clear = false;
     cudaMemsetAsync(bm, 0, sizeof(BatchMeta), s);
     const Scratch& sc = x->sc;
     SortBuffers sb = sort_buffers(x, sc);
@@ -1433,6 +1432,7 @@ int pi_export(pi_index_t* x, uint64_t* keys_out, uint64_t* vals_out, uint64_t ca
     if (e != cudaSuccess) return map_cuda(e);
     if (int rc = sticky_error(x->known)) return rc;
     cudaMemsetAsync(x->d_count, 0, sizeof(uint32_t), s);
+    x->bm_clear = false;  // block 0 may be the next batch's
     cudaMemsetAsync(&x->d_bm->tile_ctr[12], 0, sizeof(uint32_t), s);
     uint32_t ep = next_epochs(x, 2, s);
     e = launch_export_live(x->st, x->d_meta, keys_out, vals_out, cap, x->d_count, x->desc, &x->d_bm->tile_ctr[12], ep,
@@ -1890,6 +1890,7 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
         x->issued++;
         x->pending_n += b[0].n;
         x->force_rebuild = true;  // the plain path recounts its per-tile level counts
+        x->bm_clear = false;      // the counters' parity moved on
         x->launches += mx->launches;
         x->routed++;
         mark_last(x, s);

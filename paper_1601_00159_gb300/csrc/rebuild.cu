@@ -99,13 +99,19 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
     __shared__ int s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevMeta* m = a.m;
-    if (!a.bm->merged) return;
+    if (!a.bm->merged) {  // the apply kernel ended the batch, or an error did
+        if (blockIdx.x == 0 && warp == 0) post_batch(a);
+        return;
+    }
     if (tid == 0) {
         s_cta = atomicAdd(&a.bm->tile_ctr[kCtrMerge], 1u);
         s_fail = 0;
     }
     if (tid < 2 * kLevelSlots) (&s_cnt[0][0])[tid] = 0;
-    if (block_sees_error(&m->error)) return;
+    if (block_sees_error(&m->error)) {
+        if (blockIdx.x == 0 && warp == 0) post_batch(a);
+        return;
+    }
     const uint32_t size = m->size, src = m->cur, dst = src ^ 1u;
     const uint32_t newc = a.bm->new_count, cta = s_cta, G = gridDim.x;
     const bool flagged = (int32_t)m->tombs + a.bm->tomb_delta != 0;
@@ -189,7 +195,10 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
         }
     }
     __syncthreads();
-    if (s_fail) return;
+    if (s_fail) {  // this CTA will not arrive, so the batch has no last one
+        if (warp == 0) post_batch(a);
+        return;
+    }
     uint32_t lbase = s_pref;  // live old nodes before the chunk
     for (uint32_t c = c0; c < c1; ++c) {
         const uint32_t ck = (c - c0) % kCuts;
@@ -304,7 +313,10 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
         if (s_last) __threadfence();
     }
     __syncthreads();
-    if (s_last && warp == 0) level_layout(a, true);
+    if (s_last && warp == 0) {
+        level_layout(a, true);
+        post_batch(a);
+    }
 }
 
 // The level layout of a bulk build (a batch's is done by the kernel that ends the batch).
