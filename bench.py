@@ -108,7 +108,7 @@ def tuned_plain(keys):
 
 # The sources of the single-index batch path (the kernels a capture of the skewed
 # workload measures, and the host code that launches them).
-BATCH_PATH_SOURCES = ("common.cuh", "layout.cuh", "sort.cu", "descend.cu", "apply.cu", "rebuild.cu", "relevel.cuh", "pi.cu")
+BATCH_PATH_SOURCES = ("common.cuh", "layout.cuh", "search.cuh", "sort.cu", "descend.cu", "apply.cu", "rebuild.cu", "relevel.cuh", "pi.cu")
 
 
 def source_digest():

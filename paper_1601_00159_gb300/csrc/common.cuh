@@ -781,20 +781,21 @@ struct MultiArgs {
     DevMeta* mirror;          // copy of every processed index's meta, by index (may be null)
 };
 
-// Range search: both bounds of n queries, sorted and descended as 2n point lookups.
+// Range search of n queries.
 struct RangeArgs {
-    const uint64_t* sk;       // sorted bounds
-    const uint32_t* sp;       // their payload: bound index (lo of query b, or hi of query b - n)
-    const uint32_t* loc;      // per distinct bound: storage nodes with key <= it
-    const uint8_t* flags;     // per distinct bound: bit 0 = a node with this key exists
-    const uint32_t* sub_pref; // descent sub-tile prefixes of the distinct bounds
+    const uint64_t* lo;       // bounds, in arrival order
+    const uint64_t* hi;
+    const uint64_t* lkeys;    // index layer, both buffers
+    const uint32_t* ldown;
+    const uint64_t* lkeys1;
+    const uint32_t* ldown1;
+    uint32_t* done;           // CTAs finished (0 between calls)
     const DevMeta* m;
-    const BatchMeta* bm;
     Storage st;
     uint32_t* start;          // [n] first node with key >= lo
     uint32_t* end;            // [n] first node with key > hi
     uint32_t* cnt;            // [n] live nodes in [start, end)
-    uint64_t* bsum;           // [n / 256 + 1] per-CTA sums, then their prefix
+    uint64_t* bsum;           // [range_blocks] per-CTA sums, then their prefix
     uint64_t* offsets;        // [n + 1] output (caller's)
     uint64_t* keys_out;       // [cap] output (caller's)
     uint64_t* vals_out;
@@ -802,7 +803,8 @@ struct RangeArgs {
     uint32_t n;
     uint32_t* err;
 };
-cudaError_t launch_range(const RangeArgs& a, cudaStream_t s);
+cudaError_t launch_range(const RangeArgs& a, cudaStream_t s, int num_sms);
+uint32_t range_blocks(uint32_t n, int num_sms);  // CTAs of its kernels
 
 uint64_t multi_scratch_bytes(uint32_t qcap);
 // A kernel variant: warps per CTA, radix digit bits, CTAs per batch (cluster; <= 1: one).

@@ -27,7 +27,7 @@
 // lanes (the SIMD-compare analogue of Section 3.2.1); otherwise each lane scans its own
 // gap four keys (and downs) per round. Both end at the level's sentinel.
 
-#include "common.cuh"
+#include "search.cuh"
 
 namespace pi {
 namespace {
@@ -383,60 +383,6 @@ __global__ void __launch_bounds__(kThreads) k_level(DescendArgs a, int l) {
     }
 }
 
-// Largest p in [slo - 1, shi) with K[p] <= q, for a storage gap with K[shi] > q and,
-// when slo > 0 or has_lo, K[slo] <= q; -1 when q is below every key. The gap's keys
-// lie between klo = K[slo] and khi = K[shi], so the answer is looked for first in the
-// 64-byte line of 8 keys around the linear estimate slo + (q - klo) / (khi - klo) *
-// (shi - slo): for keys spread evenly over the gap that line usually holds it. From
-// there the search moves line by line towards the answer, so it stays exact for any
-// key distribution.
-__device__ __forceinline__ int32_t gap_search(const uint64_t* K, uint32_t slo, uint32_t shi, uint64_t klo,
-                                              uint64_t khi, uint64_t q, uint32_t lim, uint64_t& k_out, uint32_t* err) {
-    uint32_t est = slo;
-    if (shi > slo + 1u && khi != kMaxKey && khi > klo) {
-        const float f = __ull2float_rz(q - klo) / __ull2float_rn(khi - klo);  // in [0, 1]
-        est = slo + (uint32_t)(f * (float)(shi - slo));
-        if (est >= shi) est = shi - 1u;
-    }
-    uint32_t c = est & ~7u;
-    int dir = 0;
-    const uint32_t max_lines = (shi - slo) / 8u + 3u;
-    for (uint32_t it = 0;; ++it) {
-        if (c > lim || it > max_lines) {
-            atomicOr(err, kErrBounds);
-            return -1;
-        }
-        const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(K + c);
-        uint64_t kk[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const ulonglong2 v = kp[j];
-            kk[2 * j] = v.x;
-            kk[2 * j + 1] = v.y;
-        }
-        uint32_t gt = 0;  // bit j: K[c + j] > q (a suffix of the line, the keys being sorted)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) gt |= (kk[j] > q ? 1u : 0u) << j;
-        if (gt == 0xFFu) {  // the answer is before this line
-            if (dir > 0) return (int32_t)c - 1;  // (k_out was set on the previous line)
-            if (c == 0) return -1;
-            dir = -1;
-            c -= 8u;
-        } else if (gt == 0u) {  // the answer is at the end of this line or after it
-            k_out = kk[7];
-            if (dir < 0) return (int32_t)c + 7;
-            dir = 1;
-            c += 8u;
-        } else {
-            const int f = __ffs(gt) - 1;  // >= 1
-#pragma unroll
-            for (int j = 1; j < 8; ++j)
-                if (j == f) k_out = kk[j - 1];
-            return (int32_t)c + f - 1;
-        }
-    }
-}
-
 // The storage layer: the node with the largest key <= q (exists if equal) and its state.
 // `lvl` is the lowest index level that can be built. When it is built and not pinned in
 // shared memory (the usual case), it has no launch of its own: it is searched here, which
@@ -489,31 +435,6 @@ __global__ void __launch_bounds__(kThreads) k_locate(DescendArgs a, int lvl) {
     }
 }
 
-// Keys <= q in the sorted K[0, n): each round reads seven evenly spaced entries at once, so
-// that n entries take about log8(n) dependent reads.
-__device__ __forceinline__ uint32_t count_le(const uint64_t* K, uint32_t n, uint64_t q) {
-    uint32_t lo = 0, len = n;  // the count lies in [lo, lo + len]
-    while (len >= 8u) {
-        uint64_t v[7];
-#pragma unroll
-        for (uint32_t j = 0; j < 7; ++j) v[j] = K[lo + (uint32_t)(((uint64_t)len * (j + 1u)) >> 3)];
-        uint32_t c = 0;  // pivots <= q: a prefix
-#pragma unroll
-        for (uint32_t j = 0; j < 7; ++j) c += v[j] <= q ? 1u : 0u;
-        const uint32_t nlo = c ? (uint32_t)(((uint64_t)len * c) >> 3) + 1u : 0u;
-        const uint32_t nhi = c < 7u ? (uint32_t)(((uint64_t)len * (c + 1u)) >> 3) : len;
-        lo += nlo;
-        len = nhi - nlo;
-    }
-    uint64_t v[7];
-#pragma unroll
-    for (uint32_t j = 0; j < 7; ++j) v[j] = j < len ? K[lo + j] : kMaxKey;
-    uint32_t c = 0;
-#pragma unroll
-    for (uint32_t j = 0; j < 7; ++j) c += j < len && v[j] <= q ? 1u : 0u;
-    return lo + c;
-}
-
 // Small batches: the place of every query among the sorted tiles, and its storage node, for 32
 // queries per CTA (consecutive ones of a sorted tile, one per lane). An element's place is its
 // place in its tile, plus the keys of every earlier tile that are <= its own and of every later
@@ -555,23 +476,9 @@ __global__ void __launch_bounds__(kRankThreads) k_rank_locate(DescendArgs a, con
         }
         s_pos[warp][lane] = c;
     } else if (q != kMaxKey && *(volatile const uint32_t*)&m->error == 0) {
-        const uint32_t size = m->size, cur = m->cur, H = m->H, Lb = m->Lb;
-        const uint64_t* SK = a.st.keys[cur];
+        const uint32_t cur = m->cur;
         uint64_t kr = 0;
-        if (Lb <= H) {
-            const uint64_t* K = (m->lcur ? a.lkeys1 : a.lkeys) + m->base[Lb];
-            const uint32_t* D = (m->lcur ? a.ldown1 : a.ldown) + m->base[Lb];
-            const uint32_t c = count_le(K, m->n[Lb], q);  // the level's sentinel follows its entries
-            const uint64_t kn = K[c];
-            const uint32_t dn = D[c];
-            const uint64_t klo = c ? K[c - 1u] : 0ull;
-            const uint32_t lo = c ? D[c - 1u] : 0u;
-            r = gap_search(SK, lo, dn, klo, kn, q, size, kr, a.err);
-        } else {
-            const uint32_t c = count_le(SK, size, q);
-            r = (int32_t)c - 1;
-            kr = c ? SK[c - 1u] : 0ull;
-        }
+        r = storage_search(m, a.st.keys[cur], a.lkeys, a.ldown, a.lkeys1, a.ldown1, q, kr, a.err);
         exists = r >= 0 && kr == q;
         const uint8_t meta = exists ? a.st.meta[cur][r] : (uint8_t)0;
         v = exists ? a.st.vals[cur][r] : 0ull;

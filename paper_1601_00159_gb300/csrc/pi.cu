@@ -131,12 +131,12 @@ struct pi_index {
     uint32_t sort_cfg = 0;            // pi_config_t.sort_passes
     uint64_t launches = 0;            // kernels launched by the batch entry points
     uint32_t full_sort_left = 0;      // batches still sorted with all eight passes
-    // range search: both bounds back to back, per-query storage slices and counts
-    uint64_t* r_bounds = nullptr;
+    // range search: per-query storage slices and counts, per-CTA sums
     uint32_t* r_start = nullptr;
     uint32_t* r_end = nullptr;
     uint32_t* r_cnt = nullptr;
     uint64_t* r_bsum = nullptr;
+    uint32_t* r_done = nullptr;
     uint64_t r_cap = 0;
     DevMeta* d_meta = nullptr;
     BatchMeta* d_bm = nullptr;  // two per-batch counter blocks, alternating between batches
@@ -419,7 +419,7 @@ void destroy(pi_index* x) {
     }
     delete x->kt;
     free_scratch(x->sc);
-    dfree(x->r_bounds); dfree(x->r_start); dfree(x->r_end); dfree(x->r_cnt); dfree(x->r_bsum);
+    dfree(x->r_start); dfree(x->r_end); dfree(x->r_cnt); dfree(x->r_bsum); dfree(x->r_done);
     for (auto& g : x->stg) {
         dfree(g.ops); dfree(g.keys); dfree(g.vals); dfree(g.res);
     }
@@ -1165,67 +1165,29 @@ int pi_range_search(pi_index_t* x, const uint64_t* lo, const uint64_t* hi, uint6
     refresh_known(x);
     if (int rc = sticky_error(x->known)) return rc;
     order_after_last(x, s);
-    const uint64_t nb = 2 * n;
-    // sort and descent scratch for the 2n bounds (grows like a batch's)
-    if (nb > x->sc.cap && (e = grow_scratch(x, nb, s)) != cudaSuccess) return map_cuda(e);
     if (n > x->r_cap) {
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return map_cuda(e);
-        dfree(x->r_bounds); dfree(x->r_start); dfree(x->r_end); dfree(x->r_cnt); dfree(x->r_bsum);
+        dfree(x->r_start); dfree(x->r_end); dfree(x->r_cnt); dfree(x->r_bsum); dfree(x->r_done);
         x->r_cap = 0;
-        if ((e = dalloc(&x->r_bounds, nb)) != cudaSuccess || (e = dalloc(&x->r_start, n)) != cudaSuccess ||
-            (e = dalloc(&x->r_end, n)) != cudaSuccess || (e = dalloc(&x->r_cnt, n)) != cudaSuccess ||
-            (e = dalloc(&x->r_bsum, n / 256 + 2)) != cudaSuccess)
+        if ((e = dalloc(&x->r_start, n)) != cudaSuccess || (e = dalloc(&x->r_end, n)) != cudaSuccess ||
+            (e = dalloc(&x->r_cnt, n)) != cudaSuccess ||
+            (e = dalloc(&x->r_bsum, n / 256 + 8 * (uint64_t)x->num_sms + 8)) != cudaSuccess ||
+            (e = dalloc(&x->r_done, 1)) != cudaSuccess ||
+            (e = cudaMemsetAsync(x->r_done, 0, sizeof(uint32_t), s)) != cudaSuccess)
             return map_cuda(e);
         x->r_cap = n;
     }
     const uint64_t l0 = g_launches;
-    cudaMemcpyAsync(x->r_bounds, lo, n * 8, cudaMemcpyDeviceToDevice, s);
-    cudaMemcpyAsync(x->r_bounds + n, hi, n * 8, cudaMemcpyDeviceToDevice, s);
-    BatchMeta* bm = x->d_bm + (x->issued & 1u);  // the other block may still be read by the rebuild
-    x->bm_clear = false;
-    cudaMemsetAsync(bm, 0, sizeof(BatchMeta), s);
-    const Scratch& sc = x->sc;
-    SortBuffers sb = sort_buffers(x, sc);
-    if ((e = launch_sort(nullptr, x->r_bounds, (uint32_t)nb, sb, bm, &x->d_meta->error, s, x->num_sms,
-                         sort_passes(x, nb))) != cudaSuccess)
-        return map_cuda(e);
     wait_rebuild(x, s);
-    DescendArgs da{};
-    da.sk = sc.a_k;
-    da.sp = sc.a_p;
-    da.tile_pref = sc.tile_pref;
-    da.sub_pref = sc.sub_pref;
-    da.desc = x->desc;
-    da.dq = sc.dq;
-    da.dlo = sc.dlo;
-    // the lowest buildable level is never walked by the prologue: the storage locate
-    // searches it itself (it needs that level's gap ends)
-    da.top_launched = std::max(top_launched_for(x), (int)x->min_lb);
-    da.bottom_launched = (int)x->min_lb;
-    da.m = x->d_meta;
-    da.bm = bm;
-    da.lkeys = x->lkeys;
-    da.ldown = x->ldown;
-    da.lkeys1 = x->lkeys1;
-    da.ldown1 = x->ldown1;
-    da.st = x->st;
-    da.loc = sc.loc;
-    da.flags = sc.flags;
-    da.val0 = sc.val0;
-    da.n = (uint32_t)nb;
-    da.err = &x->d_meta->error;
-    uint32_t ep = next_epochs(x, 4, s);
-    e = launch_descend(da, ep, s, x->num_sms);
-    x->epoch = ep;
-    if (e != cudaSuccess) return map_cuda(e);
     RangeArgs ra{};
-    ra.sk = sc.a_k;
-    ra.sp = sc.a_p;
-    ra.loc = sc.loc;
-    ra.flags = sc.flags;
-    ra.sub_pref = sc.sub_pref;
+    ra.lo = lo;
+    ra.hi = hi;
+    ra.lkeys = x->lkeys;
+    ra.ldown = x->ldown;
+    ra.lkeys1 = x->lkeys1;
+    ra.ldown1 = x->ldown1;
+    ra.done = x->r_done;
     ra.m = x->d_meta;
-    ra.bm = bm;
     ra.st = x->st;
     ra.start = x->r_start;
     ra.end = x->r_end;
@@ -1237,7 +1199,7 @@ int pi_range_search(pi_index_t* x, const uint64_t* lo, const uint64_t* hi, uint6
     ra.cap = cap;
     ra.n = (uint32_t)n;
     ra.err = &x->d_meta->error;
-    e = launch_range(ra, s);
+    e = launch_range(ra, s, x->num_sms);
     x->launches += g_launches - l0;
     if (e == cudaSuccess) mark_last(x, s);
     return map_cuda(e);
