@@ -14,7 +14,8 @@ constexpr uint8_t kTomb = 0x80;      // meta bit 7: the delete flag F_del (Algor
 constexpr uint8_t kHeightMask = 0x3F;
 constexpr uint32_t kSmemTopMax = 12288;  // index entries staged in shared memory (148 KB with their downs)
 constexpr uint32_t kPad = 64;           // readable entries past every array's end
-constexpr uint32_t kSortTile = 2048;    // elements per radix-sort tile
+constexpr uint32_t kSortTile = 2048;    // elements per radix-sort tile (the smaller of two sizes)
+constexpr uint32_t kSortHist = 9 * 256; // digit counts of a radix sort
 constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the count kernel's scan
 constexpr uint32_t kCtrDistinct = 14;   // BatchMeta::tile_ctr slots: the descent prologue's tile counter,
 constexpr uint32_t kCtrApply = 15;      // the apply kernel's, and its finished tiles
@@ -620,8 +621,10 @@ struct SortBuffers {
     uint32_t* a_p;
     uint64_t* b_k;
     uint32_t* b_p;
-    uint32_t* dofs;  // [256] digit bases (first output slot of each digit) of the current pass
-    uint64_t* desc;  // [tiles][256] look-back descriptors
+    uint32_t* hist;      // [kSortHist] digit counts of the passes
+    uint32_t* desc[2];   // [tiles][256] look-back words, alternating between passes
+    // larger batches, without look-back:
+    uint32_t* dofs;      // [256] digit bases (first output slot of each digit) of the current pass
     uint32_t* tcnt;      // [tiles][256] per-tile digit counts of the current pass
     uint32_t* toff;      // [tiles][256] per-tile digit offsets within the tile's group
     uint32_t* gsum;      // [groups][256] per-group digit totals, then the groups' offsets
@@ -634,8 +637,9 @@ struct SortBuffers {
 // ops may be NULL (all searches). Counts invalid queries into bm->invalid.
 // At most max_passes (1..8) digit passes run, on the most significant bytes that vary;
 // when more bytes vary, runs of equal sorted bytes are then ordered by the rest.
+// *hist_clear: whether sb.hist is zero already; on return, whether the sort leaves it so.
 cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
-                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes);
+                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear);
 
 // Small batches (n <= kSmallSort): every tile of kRunTile queries sorted by (key, arrival)
 // on its own, into in_k / in_p (see k_tile_sort). Counts invalid queries into bm->invalid.

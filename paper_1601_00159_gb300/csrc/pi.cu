@@ -43,9 +43,8 @@ struct Scratch {
     uint64_t* val0 = nullptr;
     NewNodes nn{};
     uint32_t* tile_pref = nullptr;
-    uint32_t* tcnt = nullptr;  // radix sort: per-tile digit counts
-    uint32_t* toff = nullptr;  // radix sort: per-tile digit offsets
-    uint32_t* gsum = nullptr;  // radix sort: per-group digit totals / offsets
+    uint32_t* sdesc[2] = {};   // radix sort: per-tile look-back words, or digit counts and offsets
+    uint32_t* gsum = nullptr;  // radix sort of large batches: per-group digit totals / offsets
     uint32_t* gctr = nullptr;  // radix sort: the count kernels' arrival counters
     uint8_t* ndig = nullptr;   // radix sort: next pass's digits
     uint32_t* fixmap = nullptr;  // radix sort: segment marks of the prefix fix-up
@@ -140,7 +139,8 @@ struct pi_index {
     uint64_t r_cap = 0;
     DevMeta* d_meta = nullptr;
     BatchMeta* d_bm = nullptr;  // two per-batch counter blocks, alternating between batches
-    uint32_t* d_dofs = nullptr;
+    uint32_t* d_hist = nullptr;  // radix sort: digit counts
+    bool hist_clear = false;     // they are zero (the last sort cleared them)
     uint32_t* d_count = nullptr;
     Storage st{};
     uint64_t st_cap = 0;  // nodes per buffer, padding excluded
@@ -310,7 +310,8 @@ void free_scratch(Scratch& s) {
     dfree(s.loc); dfree(s.flags); dfree(s.val0);
     dfree(s.nn.keys); dfree(s.nn.vals); dfree(s.nn.loc); dfree(s.nn.height);
     dfree(s.tile_pref);
-    dfree(s.tcnt); dfree(s.toff); dfree(s.ndig); dfree(s.fixmap); dfree(s.gsum); dfree(s.gctr);
+    dfree(s.sdesc[0]); dfree(s.sdesc[1]); dfree(s.fixmap);
+    dfree(s.gsum); dfree(s.gctr); dfree(s.ndig);
     dfree(s.chg.keys); dfree(s.chg.pos); dfree(s.chg.hl);
     dfree(s.lst_keys); dfree(s.lst_pos); dfree(s.lst_pref); dfree(s.lst_ins);
     dfree(s.sub_pref); dfree(s.dq); dfree(s.dlo);
@@ -330,7 +331,7 @@ cudaError_t alloc_scratch(Scratch& s, uint64_t q) {
     const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
     PI_TRY(dalloc(&s.tile_pref, tiles));
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
-    PI_TRY(dalloc(&s.tcnt, stiles * 256)); PI_TRY(dalloc(&s.toff, stiles * 256));
+    PI_TRY(dalloc(&s.sdesc[0], stiles * 256)); PI_TRY(dalloc(&s.sdesc[1], stiles * 256));
     const uint64_t sgroups = stiles / kScanGroup + 1;
     PI_TRY(dalloc(&s.gsum, sgroups * 256)); PI_TRY(dalloc(&s.gctr, 8 * (sgroups + 1)));
     PI_TRY(dalloc(&s.ndig, stiles * kSortTile + 16));
@@ -434,7 +435,7 @@ void destroy(pi_index* x) {
     if (x->ev_last) cudaEventDestroy(x->ev_last);
     free_storage(x->st);
     dfree(x->lkeys); dfree(x->ldown); dfree(x->lkeys1); dfree(x->ldown1);
-    dfree(x->desc); dfree(x->lcnt); dfree(x->loff); dfree(x->wcount); dfree(x->d_meta); dfree(x->d_bm); dfree(x->d_dofs); dfree(x->d_count);
+    dfree(x->desc); dfree(x->lcnt); dfree(x->loff); dfree(x->wcount); dfree(x->d_meta); dfree(x->d_bm); dfree(x->d_hist); dfree(x->d_count);
     if (x->h_mbox) cudaFreeHost(x->h_mbox);
     if (x->ev_rebuilt) cudaEventDestroy(x->ev_rebuilt);
     if (x->rs) cudaStreamDestroy(x->rs);
@@ -446,10 +447,10 @@ void destroy(pi_index* x) {
 SortBuffers sort_buffers(pi_index* x, const Scratch& s) {
     SortBuffers sb;
     sb.in_k = s.in_k; sb.in_p = s.in_p; sb.a_k = s.a_k; sb.a_p = s.a_p; sb.b_k = s.b_k; sb.b_p = s.b_p;
-    sb.dofs = x->d_dofs;
-    sb.desc = x->desc;
-    sb.tcnt = s.tcnt;
-    sb.toff = s.toff;
+    sb.hist = x->d_hist;
+    sb.desc[0] = sb.tcnt = s.sdesc[0];
+    sb.desc[1] = sb.toff = s.sdesc[1];
+    sb.dofs = x->d_hist + kSortHist;
     sb.gsum = s.gsum;
     sb.gctr = s.gctr;
     sb.ndig = s.ndig;
@@ -655,8 +656,7 @@ constexpr uint64_t noalloc_bytes(uint64_t q) {
            + al256(c * 4) + al256(c) + al256(c * 8)               // loc, flags, val0
            + 2 * al256(c * 8) + al256(c * 4) + al256(c)           // new nodes
            + al256(tiles * 4)                                     // tile prefix
-           + 2 * al256(stiles * 256 * 4) + al256(stiles * kSortTile + 16)  // tcnt, toff, ndig
-           + al256((stiles / kScanGroup + 1) * 256 * 4) + al256(8 * (stiles / kScanGroup + 2) * 4)  // gsum, gctr
+           + 2 * al256(stiles * 256 * 4)                          // sort look-back words
            + al256((c / 32 + 1) * 4)                              // fixmap
            + al256(c * 8) + al256(c * 4) + al256(c)               // level changes
            + al256((2 * c + 64) * 8) + 2 * al256((2 * c + 64) * 4) + al256(2 * c + 64)  // lists
@@ -685,8 +685,7 @@ uint64_t carve_scratch(uint8_t* base, uint64_t q, Scratch& s) {
     take(s.loc, c * 4); take(s.flags, c); take(s.val0, c * 8);
     take(s.nn.keys, c * 8); take(s.nn.vals, c * 8); take(s.nn.loc, c * 4); take(s.nn.height, c);
     take(s.tile_pref, tiles * 4);
-    take(s.tcnt, stiles * 256 * 4); take(s.toff, stiles * 256 * 4); take(s.ndig, stiles * kSortTile + 16);
-    take(s.gsum, (stiles / kScanGroup + 1) * 256 * 4); take(s.gctr, 8 * (stiles / kScanGroup + 2) * 4);
+    take(s.sdesc[0], stiles * 256 * 4); take(s.sdesc[1], stiles * 256 * 4);
     take(s.fixmap, (c / 32 + 1) * 4);
     take(s.chg.keys, c * 8); take(s.chg.pos, c * 4); take(s.chg.hl, c);
     s.lst_cap = 2 * c + 64;
@@ -781,7 +780,8 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     SortBuffers sb = sort_buffers(x, sc);
     const bool small = small_front(x, n);
     e = small ? launch_tile_sort(ops, keys, (uint32_t)n, sb, bm, s)
-              : launch_sort(ops, keys, (uint32_t)n, sb, bm, &x->d_meta->error, s, x->num_sms, sort_passes(x, n));
+              : launch_sort(ops, keys, (uint32_t)n, sb, bm, &x->d_meta->error, s, x->num_sms, sort_passes(x, n),
+                          &x->hist_clear);
     if (e != cudaSuccess) return map_cuda(e);
     prof_mark(x, 1, s);
     wait_rebuild(x, s);
@@ -981,7 +981,7 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         if ((e = cudaStreamCreateWithFlags(&x->rs, cudaStreamNonBlocking)) != cudaSuccess) break;
         if ((e = cudaEventCreateWithFlags(&x->ev_rebuilt, cudaEventDisableTiming)) != cudaSuccess) break;
         if ((e = cudaEventCreateWithFlags(&x->ev_last, cudaEventDisableTiming)) != cudaSuccess) break;
-        if ((e = dalloc(&x->d_dofs, 8 * 256)) != cudaSuccess) break;
+        if ((e = dalloc(&x->d_hist, kSortHist + 256)) != cudaSuccess) break;
         if ((e = dalloc(&x->d_count, 1)) != cudaSuccess) break;
         cudaMemsetAsync(x->d_meta, 0, sizeof(DevMeta), s);
         cudaMemsetAsync(x->d_bm, 0, 2 * sizeof(BatchMeta), s);
@@ -995,8 +995,8 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
             if ((e = alloc_scratch(tmp, n)) != cudaSuccess) break;
             SortBuffers sb = sort_buffers(x, tmp);
             uint32_t ep = next_epochs(x, 16, s);
-            if ((e = launch_sort(nullptr, keys, (uint32_t)n, sb, x->d_bm, &x->d_meta->error, s, x->num_sms, 8)) !=
-                cudaSuccess)
+            if ((e = launch_sort(nullptr, keys, (uint32_t)n, sb, x->d_bm, &x->d_meta->error, s, x->num_sms, 8,
+                                 &x->hist_clear)) != cudaSuccess)
                 break;
             x->epoch = ep;
             BatchMeta hbm;

@@ -1,14 +1,13 @@
 // K0 + K1: validate/pack the query set and sort it by key (Definition 3: the queries
 // of a query set are ordered by key; Section 4.2: the sort can use data parallelism).
 //
-// LSD radix sort with 8-bit digits. Every pass is three launches over tiles of 2048
-// elements, so no tile ever waits for another:
-//   count:   the tile's digit histogram (tile-major rows of 256 counters);
-//   scan:    one CTA per digit turns that digit's column into global offsets
-//            (digit base from the up-front histograms + prefix over tiles);
-//   scatter: ranks the tile's elements stably within the tile and writes them to
-//            offset + rank, staged in shared memory so each digit's run is written
-//            contiguously.
+// LSD radix sort with 8-bit digits over tiles of 2048 or 4096 elements. A tile ranks its elements
+// stably and writes them staged in shared memory, so each digit's run is written
+// contiguously. Where a tile's digits go comes, up to kSweepMost queries, from a decoupled
+// look-back inside the pass (Merrill and Garland 2016; Adinets and Merrill, "Onesweep", 2022): one
+// launch per pass, the digit counts over the whole batch having been counted by the kernel
+// before. Larger batches count each tile's digits in a kernel of its own before each pass, whose
+// last CTAs scan the counts, so that no tile waits for another.
 // A pass whose byte is the same in every key is skipped (byte-wise min/max in the pack
 // kernel). The sort is stable, so equal keys stay in arrival order: the order is
 // (key, arrival index), the reading of Definition 3 for duplicate keys.
@@ -31,12 +30,50 @@
 namespace pi {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;             // the fix-up's CTAs
 constexpr int kItems = 8;
-constexpr int kTile = kThreads * kItems;  // kSortTile
+constexpr int kTile = kThreads * kItems;
 constexpr int kWarps = kThreads / 32;
 constexpr int kWarpSpan = 32 * kItems;    // 256 consecutive elements per warp
-static_assert(kTile == kSortTile, "tile size shared with the host's descriptor sizing");
+static_assert(kTile == kSortTile, "tile size shared with the host's sizing");
+
+// The first digit of a full-width batch: its four most significant bytes vary, and the passes
+// start at the lowest of them. The pack kernel counts this byte; other plans count theirs
+// in the plan kernel.
+constexpr uint32_t kUsualByte = 4;
+constexpr uint32_t kUsualRow = 8;         // its row of the counts (rows 0 .. 7: the passes')
+constexpr uint32_t kSweepMost = 1u << 20;   // largest batch whose passes look back (see k_sort_count)
+constexpr uint32_t kLargeTiles = 1u << 19;  // from here on, their tiles hold 4096 elements instead of 2048
+
+__device__ __forceinline__ uint32_t usual_digit(uint64_t k) { return (uint32_t)(k >> (8u * kUsualByte)) & 255u; }
+
+// Adds the digits of a thread's nv <= kN consecutive elements to the block's counts, each run
+// of equal digits with one shared-memory atomic, and one per warp when the whole warp holds
+// one digit, so that a hot key's run costs no contention. The whole warp calls it.
+template <int kN>
+__device__ __forceinline__ void count_digits(const uint32_t (&d)[kN], uint32_t nv, uint32_t* h) {
+    uint32_t cur = d[0], run = nv ? 1u : 0u;
+    bool single = true;
+#pragma unroll
+    for (int k = 1; k < kN; ++k) {
+        if ((uint32_t)k >= nv) break;
+        if (d[k] == cur) {
+            ++run;
+        } else {
+            single = false;
+            atomicAdd(&h[cur], run);
+            cur = d[k];
+            run = 1;
+        }
+    }
+    const uint32_t d0 = __shfl_sync(0xffffffffu, cur, 0);
+    if (__all_sync(0xffffffffu, single && cur == d0)) {  // the warp holds one digit
+        const uint32_t tot = __reduce_add_sync(0xffffffffu, run);
+        if ((threadIdx.x & 31u) == 0 && tot) atomicAdd(&h[d0], tot);
+    } else if (run) {
+        atomicAdd(&h[cur], run);
+    }
+}
 
 // K0: validate and pack. Also finds, per key byte, whether it is the same in every
 // valid key (byte-wise min and max), which decides the radix passes that can be skipped.
@@ -60,43 +97,62 @@ struct PackAcc {
     }
 };
 
+template <bool kSweep>
 __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, const uint64_t* __restrict__ keys,
                                               uint32_t n, uint64_t* __restrict__ sk, uint32_t* __restrict__ sp,
-                                              uint32_t* __restrict__ fixmap, BatchMeta* bm) {
+                                              uint32_t* __restrict__ fixmap, uint32_t* __restrict__ desc,
+                                              uint32_t ndesc, uint32_t* __restrict__ hist, BatchMeta* bm) {
     pdl_wait();
     pdl_trigger();
+    __shared__ uint32_t s_hist[256];
+    if (kSweep) {
+        s_hist[threadIdx.x] = 0;
+        __syncthreads();
+    }
     const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
+    if (kSweep)
+        for (uint32_t w = gt; w < ndesc; w += gs) desc[w] = 0;  // the first pass's look-back words
     for (uint32_t w = gt; w < (n + 31u) / 32u; w += gs) fixmap[w] = 0;  // segment marks of the prefix fix-up
     PackAcc acc;
     const bool vec = ((reinterpret_cast<uintptr_t>(keys) & 15u) | (reinterpret_cast<uintptr_t>(ops) & 3u)) == 0;
     uint32_t tail = 0;  // first query left to the scalar loop
     if (vec) {
         const uint32_t n4 = n / 4u;
-        for (uint32_t g = gt; g < n4; g += gs) {
-            const uint32_t i = 4u * g;
-            const ulonglong2 k01 = reinterpret_cast<const ulonglong2*>(keys + i)[0];
-            const ulonglong2 k23 = reinterpret_cast<const ulonglong2*>(keys + i)[1];
-            const uint32_t o4 = ops ? *reinterpret_cast<const uint32_t*>(ops + i) : 0u;
-            const uint32_t o0 = o4 & 255u, o1 = (o4 >> 8) & 255u, o2 = (o4 >> 16) & 255u, o3 = o4 >> 24;
-            ulonglong2 s01, s23;
-            s01.x = acc.take(k01.x, o0);
-            s01.y = acc.take(k01.y, o1);
-            s23.x = acc.take(k23.x, o2);
-            s23.y = acc.take(k23.y, o3);
-            reinterpret_cast<ulonglong2*>(sk + i)[0] = s01;
-            reinterpret_cast<ulonglong2*>(sk + i)[1] = s23;
-            uint4 p;
-            p.x = ((o0 & 3u) << 30) | i;
-            p.y = ((o1 & 3u) << 30) | (i + 1u);
-            p.z = ((o2 & 3u) << 30) | (i + 2u);
-            p.w = ((o3 & 3u) << 30) | (i + 3u);
-            *reinterpret_cast<uint4*>(sp + i) = p;
+        for (uint32_t g0 = gt - (threadIdx.x & 31u); g0 < n4; g0 += gs) {  // whole warps
+            const uint32_t g = g0 + (threadIdx.x & 31u), i = 4u * g;
+            uint32_t dg[4] = {0, 0, 0, 0};
+            if (g < n4) {
+                const ulonglong2 k01 = reinterpret_cast<const ulonglong2*>(keys + i)[0];
+                const ulonglong2 k23 = reinterpret_cast<const ulonglong2*>(keys + i)[1];
+                const uint32_t o4 = ops ? *reinterpret_cast<const uint32_t*>(ops + i) : 0u;
+                const uint32_t o0 = o4 & 255u, o1 = (o4 >> 8) & 255u, o2 = (o4 >> 16) & 255u, o3 = o4 >> 24;
+                ulonglong2 s01, s23;
+                s01.x = acc.take(k01.x, o0);
+                s01.y = acc.take(k01.y, o1);
+                s23.x = acc.take(k23.x, o2);
+                s23.y = acc.take(k23.y, o3);
+                reinterpret_cast<ulonglong2*>(sk + i)[0] = s01;
+                reinterpret_cast<ulonglong2*>(sk + i)[1] = s23;
+                uint4 p;
+                p.x = ((o0 & 3u) << 30) | i;
+                p.y = ((o1 & 3u) << 30) | (i + 1u);
+                p.z = ((o2 & 3u) << 30) | (i + 2u);
+                p.w = ((o3 & 3u) << 30) | (i + 3u);
+                *reinterpret_cast<uint4*>(sp + i) = p;
+                dg[0] = usual_digit(s01.x);
+                dg[1] = usual_digit(s01.y);
+                dg[2] = usual_digit(s23.x);
+                dg[3] = usual_digit(s23.y);
+            }
+            if (kSweep) count_digits(dg, g < n4 ? 4u : 0u, s_hist);
         }
         tail = 4u * n4;
     }
     for (uint32_t i = tail + gt; i < n; i += gs) {
         const uint32_t op = ops ? ops[i] : 0u;
-        sk[i] = acc.take(keys[i], op);
+        const uint64_t k = acc.take(keys[i], op);
+        if (kSweep) atomicAdd(&s_hist[usual_digit(k)], 1u);
+        sk[i] = k;
         sp[i] = ((op & 3u) << 30) | i;
     }
     uint32_t invalid = acc.invalid;
@@ -126,6 +182,7 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, c
         }
     }
     __syncthreads();
+    if (kSweep && s_hist[threadIdx.x]) atomicAdd(&hist[kUsualRow * 256u + threadIdx.x], s_hist[threadIdx.x]);
     // one global atomic per byte per CTA
     if (threadIdx.x < 8) atomicMax(&bm->bmax[threadIdx.x], s_red[threadIdx.x]);
     else if (threadIdx.x < 16) atomicMax(&bm->bnmin[threadIdx.x - 8], s_red[threadIdx.x]);
@@ -141,15 +198,226 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, c
 // max_passes of them (the prefix). The fix-up then orders each segment of equal prefix
 // bytes by the full key; its long-segment path sorts by every other byte that can
 // differ inside a segment (rdig).
-__global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, BatchMeta* bm, uint32_t* gctr, uint32_t max_passes) {
+template <bool kSweep>
+__global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, BatchMeta* bm, uint32_t max_passes) {
     pdl_wait();
     pdl_trigger();
-    const int b = threadIdx.x;
-    const uint32_t ngroups = ((n + kTile - 1) / kTile + kScanGroup - 1) / kScanGroup;
-    for (uint32_t i = b; i < 8u * (ngroups + 1u); i += 256) gctr[i] = 0;  // the count kernels' arrivals
-    if (b == 0) plan_digits(bm->bmax, bm->bnmin, bm->invalid, n, max_passes, bm->plan);
+    __shared__ SortPlan s_plan;
+    __shared__ uint32_t s_hist[256];
+    if (!kSweep) {  // one CTA
+        const uint32_t ngroups = ((n + kTile - 1) / kTile + kScanGroup - 1) / kScanGroup;
+        for (uint32_t i = threadIdx.x; i < 8u * (ngroups + 1u); i += 256) sb.gctr[i] = 0;  // the counts' arrivals
+    }
+    if (threadIdx.x == 0) {
+        plan_digits(bm->bmax, bm->bnmin, bm->invalid, n, max_passes, s_plan);
+        if (blockIdx.x == 0) bm->plan = s_plan;
+    }
+    s_hist[threadIdx.x] = 0;
+    __syncthreads();
+    if (!kSweep || s_plan.digit[0] == kUsualByte) return;  // counted with the packing
+    const uint32_t shift = 8u * s_plan.digit[0];
+    for (uint32_t base = blockIdx.x * 2048u; base < n; base += gridDim.x * 2048u) {
+        const uint32_t i0 = base + threadIdx.x * 8u;
+        const uint32_t nv = i0 < n ? min(8u, n - i0) : 0u;
+        uint32_t dg[8];
+        if (nv == 8u) {
+            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(sb.in_k + i0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const ulonglong2 v = p[k];
+                dg[2 * k] = (uint32_t)(v.x >> shift) & 255u;
+                dg[2 * k + 1] = (uint32_t)(v.y >> shift) & 255u;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) dg[k] = (uint32_t)k < nv ? (uint32_t)(sb.in_k[i0 + k] >> shift) & 255u : 0u;
+        }
+        count_digits(dg, nv, s_hist);
+    }
+    __syncthreads();
+    if (s_hist[threadIdx.x]) atomicAdd(&sb.hist[threadIdx.x], s_hist[threadIdx.x]);
 }
 
+// Look-back word of one digit of one tile: flag (2 bits) | count (30). 0: not published yet.
+// Words are cleared between uses: a pass clears its tiles' words of the other buffer for the
+// next pass, and the pack kernel those of the first.
+constexpr uint32_t kWordAgg = 1u << 30, kWordPrefix = 2u << 30, kWordMask = kWordAgg - 1u;
+
+__device__ __forceinline__ uint32_t ld_relaxed32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Sum of one digit's counts over the tiles before `tile`: 16 tiles' words per round, which the
+// threads of the digits read as rows. A wait that gives up records kErrTimeout and returns
+// false.
+__device__ __forceinline__ bool digit_lookback(const uint32_t* words, uint32_t tile, uint32_t* err, uint32_t& sum) {
+    constexpr int kWin = 16;
+    uint32_t excl = 0, spins = 0;
+    int64_t t = (int64_t)tile - 1;
+    while (t >= 0) {
+        uint32_t w[kWin];
+#pragma unroll
+        for (int i = 0; i < kWin; ++i) w[i] = t - i >= 0 ? ld_relaxed32(words + (size_t)(t - i) * 256) : kWordPrefix;
+        bool stop = false, stall = false;
+        int used = 0;
+#pragma unroll
+        for (int i = 0; i < kWin; ++i) {
+            if (stop || stall) continue;
+            if (w[i] == 0) {
+                stall = true;
+                continue;
+            }
+            excl += w[i] & kWordMask;
+            ++used;
+            stop = (w[i] & kWordPrefix) != 0;
+        }
+        if (stop) break;
+        t -= used;
+        if (stall) {
+            ++spins;
+            if (spins > kSpinLimit) {
+                atomicOr(err, kErrTimeout);
+                return false;
+            }
+            if ((spins & 1023u) == 0 && *(volatile uint32_t*)err) return false;
+            if (spins > 32) __nanosleep(100);
+        }
+    }
+    sum = excl;
+    return true;
+}
+
+// One pass: tiles of kPassThreads x kI elements. Bound by issue slots and shared memory in the
+// ranking (nine ballots and an atomic per element row); the look-back's wait overlaps the
+// other CTA of the SM. Larger tiles mean fewer look-backs in flight, smaller ones more CTAs for
+// batches that would leave SMs idle.
+constexpr int kPassThreads = 512;
+constexpr int kPassWarps = kPassThreads / 32;
+template <int kI>
+constexpr int pass_smem() {
+    return kPassThreads * kI * (int)(sizeof(uint64_t) + sizeof(uint32_t)) + kPassWarps * 256 * 4;
+}
+
+template <int kI>
+__global__ void __launch_bounds__(kPassThreads, 2) k_sort_pass(uint32_t j, uint32_t n, SortBuffers sb, BatchMeta* bm,
+                                                               uint32_t* err) {
+    pdl_wait();
+    pdl_trigger();
+    constexpr uint32_t kT = kPassThreads * kI;
+    const SortPlan& P = bm->plan;
+    if (j >= P.npass) return;
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    uint64_t* s_key = reinterpret_cast<uint64_t*>(s_dyn);
+    uint32_t* s_pay = reinterpret_cast<uint32_t*>(s_dyn + kT * sizeof(uint64_t));
+    uint32_t(*s_whist)[256] = reinterpret_cast<uint32_t(*)[256]>(s_dyn + kT * 12u);
+    __shared__ uint32_t s_gbase[256], s_tstart[256], s_next[256];
+    __shared__ uint32_t s_tmp[33], s_tile;
+    __shared__ int s_fail;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        s_tile = atomicAdd(&bm->tile_ctr[j], 1u);
+        s_fail = 0;
+    }
+    for (int i = tid; i < kPassWarps * 64; i += kPassThreads)
+        reinterpret_cast<uint4*>(&s_whist[0][0])[i] = make_uint4(0, 0, 0, 0);
+    if (tid < 256) s_next[tid] = 0;
+    const uint32_t shift = 8u * P.digit[j];
+    const uint64_t* src_k = P.src[j] == 0 ? sb.in_k : (P.src[j] == 1 ? sb.a_k : sb.b_k);
+    const uint32_t* src_p = P.src[j] == 0 ? sb.in_p : (P.src[j] == 1 ? sb.a_p : sb.b_p);
+    uint64_t* dst_k = P.dst[j] == 1 ? sb.a_k : sb.b_k;
+    uint32_t* dst_p = P.dst[j] == 1 ? sb.a_p : sb.b_p;
+    const uint32_t row = j == 0 && P.digit[0] == kUsualByte ? kUsualRow : j;
+    const uint32_t all = tid < 256 ? sb.hist[row * 256u + (uint32_t)tid] : 0u;  // the batch's count of digit tid
+    uint32_t* words = j & 1u ? sb.desc[1] : sb.desc[0];
+    uint32_t* other = j & 1u ? sb.desc[0] : sb.desc[1];
+    __syncthreads();
+    const uint32_t tile = s_tile, tbase = tile * kT, tn = min(kT, n - tbase);
+
+    uint64_t key[kI];
+    uint32_t pay[kI], dig[kI], rank[kI];
+#pragma unroll
+    for (int k = 0; k < kI; ++k) {
+        const uint32_t li = (uint32_t)(warp * 32 * kI + k * 32 + lane);
+        const bool v = li < tn;
+        key[k] = v ? src_k[tbase + li] : 0ull;
+        pay[k] = v ? src_p[tbase + li] : 0u;
+        dig[k] = v ? (uint32_t)((key[k] >> shift) & 255u) : 256u;
+    }
+    const uint32_t dbase = block_excl_sum<kPassThreads>(all, s_tmp, nullptr);  // the digit's first output slot
+    warp_digit_ranks<kI, 8>(dig, rank, s_whist[warp]);
+    __syncthreads();
+    // Thread d < 256 owns digit d: the tile's count is published, and each warp's first rank.
+    uint32_t total = 0;
+    if (tid < 256) {
+#pragma unroll
+        for (int w = 0; w < kPassWarps; ++w) {
+            const uint32_t c = s_whist[w][tid];
+            s_whist[w][tid] = total;
+            total += c;
+        }
+        atomicExch(&words[(size_t)tile * 256 + tid], (tile == 0 ? kWordPrefix : kWordAgg) | total);
+        other[(size_t)tile * 256 + tid] = 0;  // for the next pass
+    }
+    const uint32_t tstart = block_excl_sum<kPassThreads>(total, s_tmp, nullptr);
+    if (tid < 256) s_tstart[tid] = tstart;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kI; ++k) {
+        const uint32_t d = dig[k];
+        if (d < 256u) {
+            const uint32_t pos = s_tstart[d] + s_whist[warp][d] + rank[k];
+            s_key[pos] = key[k];
+            s_pay[pos] = pay[k];
+        }
+    }
+    if (tid < 256) {
+        uint32_t before = 0;
+        if (tile > 0) {
+            if (!digit_lookback(words + tid, tile, err, before)) s_fail = 1;
+            atomicExch(&words[(size_t)tile * 256 + tid], kWordPrefix | (before + total));
+        }
+        s_gbase[tid] = dbase + before - tstart;  // output slot = this + place in the tile
+    }
+    __syncthreads();
+    if (s_fail) return;
+    const bool next = j + 1 < P.npass;
+    const uint32_t nshift = next ? 8u * P.digit[j + 1] : 0u;
+    for (uint32_t s0 = 0; s0 < tn; s0 += kPassThreads) {
+        const uint32_t s = s0 + (uint32_t)tid;
+        const bool in = s < tn;
+        const uint64_t k = in ? s_key[s] : 0ull;
+        if (in) {
+            const uint32_t g = s_gbase[(uint32_t)(k >> shift) & 255u] + s;
+            if (g < n) {
+                dst_k[g] = k;
+                dst_p[g] = s_pay[s];
+            } else {
+                atomicOr(err, kErrBounds);
+            }
+        }
+        if (next) {  // the next pass's digit counts; a hot key's run is one atomic per warp
+            const uint32_t nd = in ? (uint32_t)(k >> nshift) & 255u : 256u;
+            const uint32_t d0 = __shfl_sync(0xffffffffu, nd, 0);
+            if (__all_sync(0xffffffffu, nd == d0)) {
+                if (lane == 0 && d0 < 256u) atomicAdd(&s_next[d0], 32u);
+            } else if (in) {
+                atomicAdd(&s_next[nd], 1u);
+            }
+        }
+    }
+    if (next) {
+        __syncthreads();
+        if (tid < 256 && s_next[tid]) atomicAdd(&sb.hist[(j + 1u) * 256u + (uint32_t)tid], s_next[tid]);
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// Batches above kSweepMost: a counting and a scattering kernel per pass. With hundreds of tiles
+// in flight the look-back costs more than a launch that reads one digit byte per element:
+// 2^22 queries on 2^27 keys took 571 us a batch with k_sort_pass and 544 with these two; at 2^20
+// queries k_sort_pass is ahead (428 against 432), and at 10^5 by 21 of 99 us.
 __device__ __forceinline__ const uint64_t* pass_src_keys(const SortPlan& P, uint32_t j, const SortBuffers& sb) {
     return P.src[j] == 0 ? sb.in_k : (P.src[j] == 1 ? sb.a_k : sb.b_k);
 }
@@ -164,31 +432,6 @@ __device__ __forceinline__ const uint64_t* pass_src_keys(const SortPlan& P, uint
 // Each thread counts 8 consecutive elements and adds each run of equal digits with one
 // shared-memory atomic (one per warp when the whole warp holds one digit), so a run of a
 // hot key costs no atomic contention. The scans load 16 rows per round trip.
-__device__ __forceinline__ void count_digits(const uint32_t (&d)[8], uint32_t nv, uint32_t* h) {
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t cur = d[0], run = nv ? 1u : 0u;
-    bool single = true;
-#pragma unroll
-    for (int k = 1; k < 8; ++k) {
-        if ((uint32_t)k >= nv) break;
-        if (d[k] == cur) {
-            ++run;
-        } else {
-            single = false;
-            atomicAdd(&h[cur], run);
-            cur = d[k];
-            run = 1;
-        }
-    }
-    const uint32_t d0 = __shfl_sync(0xffffffffu, cur, 0);
-    if (__all_sync(0xffffffffu, single && cur == d0)) {  // the warp holds one digit
-        const uint32_t tot = __reduce_add_sync(0xffffffffu, run);
-        if (lane == 0 && tot) atomicAdd(&h[d0], tot);
-    } else if (run) {
-        atomicAdd(&h[cur], run);
-    }
-}
-
 // Exclusive running sum, per digit (thread d), over `rows` rows of 256 counters starting
 // at `in`: writes each row's prefix to `out` (may equal `in`) and returns the total.
 __device__ __forceinline__ uint32_t scan_rows(const uint32_t* in, uint32_t* out, uint32_t rows) {
@@ -284,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_sort_count(uint32_t j, uint32_t
 }
 
 
-__global__ void __launch_bounds__(kThreads, 4) k_sort_pass(uint32_t j, uint32_t n, SortBuffers sb,
+__global__ void __launch_bounds__(kThreads, 4) k_sort_scatter(uint32_t j, uint32_t n, SortBuffers sb,
                                                            BatchMeta* bm, uint32_t* err) {
     pdl_wait();
     pdl_trigger();
@@ -370,10 +613,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_pass(uint32_t j, uint32_t 
 // different keys. A position i whose key differs from key i-1 but whose prefix does not
 // lies inside such a segment; the segment's start is found by a galloping search back
 // from i followed by a binary search, both over the prefix order.
-__global__ void __launch_bounds__(256) k_sort_find(uint32_t n, SortBuffers sb, const BatchMeta* bm) {
+__global__ void __launch_bounds__(256) k_sort_find(uint32_t n, SortBuffers sb, const BatchMeta* bm, bool sweep) {
     pdl_wait();
     pdl_trigger();
     const SortPlan& P = bm->plan;
+    if (sweep && blockIdx.x == 0)  // the passes are done with the counts: zero for the next sort
+        for (uint32_t w = threadIdx.x; w < kSortHist; w += 256u) sb.hist[w] = 0;
     if (!P.fix) return;
     const uint64_t pm = P.pmask;
     const uint64_t* __restrict__ ak = sb.a_k;
@@ -781,37 +1026,74 @@ cudaError_t launch_tile_sort(const uint8_t* ops, const uint64_t* keys, uint32_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
-                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes) {
-    if (n == 0) return cudaSuccess;
-    if (max_passes < 1 || max_passes > 8) return cudaErrorInvalidValue;
-    int grid = min((int)((n + 255) / 256), num_sms * 8);
-    launch_dep(k_pack, grid, 256, 0, s, ops, keys, n, sb.in_k, sb.in_p, sb.fixmap, bm);
-    ++g_launches;
-    launch_dep(k_sort_plan, 1, 256, 0, s, n, bm, sb.gctr, (uint32_t)max_passes);
-    ++g_launches;
+namespace {
+
+template <int kI>
+cudaError_t launch_passes(uint32_t n, const SortBuffers& sb, BatchMeta* bm, uint32_t* err, cudaStream_t s,
+                          int max_passes) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k_sort_pass<kI>, cudaFuncAttributeMaxDynamicSharedMemorySize, pass_smem<kI>());
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    const uint32_t tiles = (n + kPassThreads * kI - 1) / (kPassThreads * kI);
+    for (uint32_t j = 0; j < (uint32_t)max_passes; ++j) {
+        launch_dep(k_sort_pass<kI>, tiles, kPassThreads, pass_smem<kI>(), s, j, n, sb, bm, err);
+        ++g_launches;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace
+
+static cudaError_t launch_count_passes(uint32_t n, const SortBuffers& sb, BatchMeta* bm, uint32_t* err, cudaStream_t s,
+                                       int max_passes) {
     static bool attr_set = false;
     const int dyn = kTile * (int)(sizeof(uint64_t) + sizeof(uint32_t));
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        cudaError_t e = cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     const uint32_t tiles = (n + kTile - 1) / kTile;
-    launch_dep(k_sort_count, tiles, kThreads, 0, s, 0, n, sb, bm);
-    ++g_launches;
     for (uint32_t j = 0; j < (uint32_t)max_passes; ++j) {
-        launch_dep(k_sort_pass, tiles, kThreads, dyn, s, j, n, sb, bm, err);
+        launch_dep(k_sort_count, tiles, kThreads, 0, s, j, n, sb, bm);
         ++g_launches;
-        if (j + 1 < (uint32_t)max_passes) {
-            launch_dep(k_sort_count, tiles, kThreads, 0, s, j + 1, n, sb, bm);
-            ++g_launches;
-        }
+        launch_dep(k_sort_scatter, tiles, kThreads, dyn, s, j, n, sb, bm, err);
+        ++g_launches;
     }
+    return cudaSuccess;
+}
+
+cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
+                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear) {
+    if (n == 0) return cudaSuccess;
+    if (max_passes < 1 || max_passes > 8) return cudaErrorInvalidValue;
+    const bool sweep = n <= kSweepMost, large = n >= kLargeTiles;
+    const int grid = min((int)((n + 255) / 256), num_sms * 8);
+    cudaError_t e = cudaSuccess;
+    if (sweep) {
+        if (!*hist_clear && (e = cudaMemsetAsync(sb.hist, 0, kSortHist * sizeof(uint32_t), s)) != cudaSuccess) return e;
+        *hist_clear = false;
+        const uint32_t tile = (uint32_t)kPassThreads * (large ? 8u : 4u), words = (n + tile - 1) / tile * 256u;
+        launch_dep(k_pack<true>, grid, 256, 0, s, ops, keys, n, sb.in_k, sb.in_p, sb.fixmap, sb.desc[0], words, sb.hist, bm);
+        launch_dep(k_sort_plan<true>, min((int)((n + 2047) / 2048), num_sms * 4), 256, 0, s, n, sb, bm, (uint32_t)max_passes);
+        g_launches += 2;
+        e = large ? launch_passes<8>(n, sb, bm, err, s, max_passes) : launch_passes<4>(n, sb, bm, err, s, max_passes);
+    } else {
+        launch_dep(k_pack<false>, grid, 256, 0, s, ops, keys, n, sb.in_k, sb.in_p, sb.fixmap, (uint32_t*)nullptr, 0u,
+                   (uint32_t*)nullptr, bm);
+        launch_dep(k_sort_plan<false>, 1, 256, 0, s, n, sb, bm, (uint32_t)max_passes);
+        g_launches += 2;
+        e = launch_count_passes(n, sb, bm, err, s, max_passes);
+    }
+    if (e != cudaSuccess) return e;
     if (max_passes < 8) {  // with eight passes every byte is sorted: nothing to fix
         const int fgrid = min((int)((n + 1023) / 1024), num_sms * 8);
-        launch_dep(k_sort_find, fgrid, 256, 0, s, n, sb, bm);
+        launch_dep(k_sort_find, fgrid, 256, 0, s, n, sb, bm, sweep);
         ++g_launches;
+        if (sweep) *hist_clear = true;
         launch_dep(k_sort_fix, (n + kFixSlice - 1) / kFixSlice, kThreads, 0, s, n, sb, bm);
         ++g_launches;
     }
