@@ -73,9 +73,10 @@ typedef struct {
                                     re-laid-out or the updates since the last rebuild
                                     exceed rebuild_threshold_pct percent of its size. */
     uint32_t rebuild_threshold_pct; /* policy 1 only; default 15 (Section 6) */
-    uint32_t smem_top_entries;   /* cap on the index entries staged in shared memory by the
-                                    descent (default and maximum 12288); smaller values
-                                    pin fewer top levels */
+    uint32_t smem_top_entries;   /* cap on the top levels' entries that count as pinned in
+                                    pi_info's smem_low_level (default and maximum 12288).
+                                    Results do not depend on it. A value below the maximum
+                                    keeps small batches on the path of large ones. */
     uint64_t storage_capacity;   /* initial storage-layer capacity, in nodes */
     uint64_t index_capacity;     /* initial index-layer capacity, in entries */
     uint32_t test_flags;         /* PI_TEST_*: alternative code paths for tests; 0 in use */
@@ -110,8 +111,8 @@ typedef struct {
                                     test_flags or with the deferred rebuild policy. */
 } pi_config_t;
 
-/* test_flags bit: give only the lowest index level a launch of its own in the
- * level-synchronous descent, so every other level takes the in-kernel walk. */
+/* test_flags bit: the descent searches every key from the top of the lowest built level, without
+ * shared-memory windows. */
 #define PI_TEST_WALK_LEVELS 1u
 /* test_flags bit: sort every batch with all eight radix passes (no prefix fix-up). */
 #define PI_TEST_SORT_FULL 2u
@@ -184,7 +185,7 @@ int pi_execute_batch_host(pi_index_t* idx, const uint8_t* ops_host, const uint64
  * allocator (cudaMalloc/cudaFree can synchronise the device, which a latency-bound
  * serving loop cannot afford) and code running where a memory budget is fixed up front.
  * The per-batch scratch of up to PI_NOALLOC_MAX_BATCH queries comes from one
- * file-scope device array of a fixed size (about 8.5 MB), held by
+ * file-scope device array of a fixed size (about 7.8 MB), held by
  * every GPU that loads the library until the process exits; this call allocates nothing.
  *   - n > PI_NOALLOC_MAX_BATCH returns PI_ERR_INVALID_ARG.
  *   - A batch that could need the storage layer to grow returns PI_ERR_OOM with the
@@ -236,7 +237,7 @@ typedef struct {
     uint32_t top_level;      /* H: highest level holding a key (1 if only storage) */
     uint32_t bottom_built;   /* lowest materialised index level (pi_config_t.lowest_level,
                                 raised when the index layer overflows its capacity) */
-    uint32_t smem_low_level; /* lowest level staged in shared memory by the descent */
+    uint32_t smem_low_level; /* lowest level whose entries and those above fit smem_top_entries */
     uint32_t promote_shift;  /* b, with P = 2^-b */
     uint64_t level_size[34]; /* level_size[l] = live keys with height >= l, l = 1..33 */
     uint64_t storage_capacity;
@@ -301,10 +302,10 @@ int pi_export_storage(pi_index_t* idx, uint64_t* keys_out, uint8_t* meta_out, ui
  * Stage timing, for measurement (no counterpart in the paper). While enabled, each
  * pi_execute_batch records CUDA events between the pipeline's stages, on the stream
  * each stage runs on:
- *   0 pack + radix sort (K0, K1)        4 level layout (K6b)
+ *   0 pack + radix sort (K0, K1)        4 unused (about 0: the layout is part of 3)
  *   1 descent + storage locate (K2, K3) 5 index-layer rebuild (K6c; background stream)
- *   2 ownership + apply (K4, K5)        6 the rebuild's writer kernels alone (part of 5)
- *   3 storage merge (K6a)               7 the storage-locate kernel alone (part of 1)
+ *   2 ownership + apply (K4, K5)        6 the rebuild's writer kernel alone (part of 5)
+ *   3 storage merge, level layout (K6)  7 the descent's kernel alone (part of 1)
  * The descent's stage excludes its wait for the previous batch's rebuild.
  * pi_profile(idx, 1) starts (and clears) the accumulation; pi_profile(idx, 0) stops it.
  * pi_profile_read synchronises `stream` and writes the summed milliseconds per stage to

@@ -15,29 +15,32 @@
 //    state to the storage node (value, delete flag), or emits a new node when the key
 //    is not in the storage layer and ends up present (Algorithm 4, insertNode).
 //
-// The max-scan is split across kernels so no tile of k_apply ever waits on another:
-// the descent's first kernel already walks the sorted batch and leaves each 2048-query
-// tile's exclusive max prefix of e (tile_pref); k_apply is then fully data-parallel. The descent stored one result per distinct key -- per local
-// run head (a query whose key differs from the previous one, and the first query of
-// every 256-query sub-tile) in sorted order -- so a query's storage-layer state is
-// found at its run head's dense index.
+// The descent left the storage-layer state at each local run head (a query whose key differs
+// from the previous one, and the first query of every 128-query block) and each block's
+// largest e. A warp takes a block and scans it on its own: the nearest local head before a
+// query, by its number, has its state, and a block that continues a run looks back over the blocks' (then the
+// tiles') marks for the run's last write, 256 of them a step. So no warp waits for another
+// until the counts of the tile: with block-wide scans, barriers were the largest stall.
 // New nodes, and the changes of built levels' membership, go to their places in key order in
 // the same pass: a tile's first place comes from a decoupled look-back over the tiles' counts,
-// which only tiles that have some wait for. The CTA that finishes last ends the batch: it
-// decides whether the storage layer is re-laid-out, and if not, lays out the index levels.
-// (Staging the new nodes per tile, a scan and a packing kernel, and a one-thread level layout
-// were three more launches: 6000 mixed queries on 2^20 keys 61.0 -> 55.6 us a batch with one
-// pass; 2^22 skewed queries on 2^27 keys 556.6 -> 548.4.)
+// which only tiles that have some wait for. Half of the kernel's time is its scattered 16-byte
+// result stores (2^22 searches: 84 us, and 43 with the results stored in order), the rest its
+// chain of dependent reads, so the owners' reads are issued with the results' at each step of
+// the chain: 2^22 skewed queries with 10% updates 117 -> 97 us.
+// (Staging the new nodes per tile, a scan and a packing kernel were two more launches.)
 
-#include "layout.cuh"
+#include "common.cuh"
 
 namespace pi {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kApThreads = 512;                  // k_apply: two CTAs per SM at 64 registers
-constexpr int kItems = kApplyTile / kApThreads;  // 4 sorted queries per thread
+constexpr int kApThreads = 256;         // k_apply: four CTAs per SM at 64 registers
+constexpr int kItems = 4;               // sorted queries per thread
+constexpr uint32_t kTile = kApThreads * kItems;
+static_assert(kApplyTile % kTile == 0 && kTile >= kDescendTile, "the descent's tiles hold whole blocks");
 constexpr uint32_t kSeqMask = (1u << 30) - 1u;
+static_assert(kApplyBlock == 32u * kItems, "a warp's queries");
 
 __device__ __forceinline__ void store_result(pi_result_t* res, uint32_t seq, uint64_t v, uint32_t st) {
     uint4 w;
@@ -50,11 +53,11 @@ __device__ __forceinline__ void store_result(pi_result_t* res, uint32_t seq, uin
 
 // Largest ownership marker e_i before the tile at tb, by the whole CTA, for a tile whose
 // first query continues the run before it (markers grow with i, so the nearest tile that
-// has one decides; tile 0 heads the first run). Small batches only: their descent keeps no
-// tile prefixes, and a run crosses few tiles.
-__device__ uint32_t marker_before(const ApplyArgs& a, uint32_t tb, uint32_t* s_tmp) {
+// has one decides; tile 0 heads the first run). Small batches only: they have no marks, and a
+// run crosses few tiles.
+__device__ uint32_t marker_before_tile(const ApplyArgs& a, uint32_t tb, uint32_t* s_tmp) {
     while (tb > 0) {
-        tb -= kApplyTile;
+        tb -= kTile;
         uint32_t agg = 0;
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {  // whole tiles of valid queries: the run reaches past them
@@ -70,24 +73,61 @@ __device__ uint32_t marker_before(const ApplyArgs& a, uint32_t tb, uint32_t* s_t
     return 0;
 }
 
-// kSmall: a batch from k_rank_locate, whose storage-layer state is kept per query instead of
-// per distinct key.
+// The nearest nonzero of marks[0, n), from the end, by a whole warp; *seen is how many entries
+// were looked at when it gave up after `steps` steps.
+__device__ __forceinline__ uint32_t last_mark(const uint32_t* marks, uint32_t n, uint32_t steps, uint32_t* seen) {
+    constexpr int kPer = 8;
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t done = 0;
+    for (uint32_t st = 0; st < steps && done < n; ++st, done += 32u * kPer) {
+        uint32_t most = 0;  // markers grow with their place, so the largest is the nearest
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const uint32_t x = done + 32u * (uint32_t)u + lane;
+            most = max(most, x < n ? marks[n - 1u - x] : 0u);
+        }
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (most) return most;
+    }
+    *seen = min(done, n);
+    return 0;
+}
+
+// Largest marker before block blk, which continues the run before it.
+__device__ __forceinline__ uint32_t marker_before_block(const ApplyArgs& a, uint32_t blk) {
+    uint32_t seen = 0;
+    const uint32_t mk = last_mark(a.blk_mark, blk, a.tile_mark ? 1u : 0xffffffffu, &seen);
+    if (mk || !a.tile_mark) return mk;
+    // the tile of the last block not looked at, and all before it (a tile's other blocks hold none)
+    const uint32_t left = blk - seen;
+    return last_mark(a.tile_mark, (left + kApplyTile / kApplyBlock - 1u) / (kApplyTile / kApplyBlock), 0xffffffffu, &seen);
+}
+
+// kSmall: a batch from k_rank_locate, whose storage-layer state is kept at every query, and which
+// comes without marks.
 template <bool kSmall>
-__global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArgs rb, uint32_t epoch) {
+__global__ void __launch_bounds__(kApThreads, 4) k_apply(ApplyArgs a, uint32_t epoch) {
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t s_tmp[33];
-    __shared__ uint32_t s_tile, s_last, s_base[2];
+    __shared__ uint32_t s_tile, s_base[2], s_warp[kApThreads / 32];
     __shared__ int s_fail;
     __shared__ int32_t s_delta[kLevelSlots];
     __shared__ int32_t s_tomb;
     __shared__ uint32_t s_changes, s_dirty;
     __shared__ uint32_t s_chist[kLevelSlots];  // built-level membership changes by height
 
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < kLevelSlots) {
+        s_delta[tid] = 0;
+        s_chist[tid] = 0;
+    }
     if (tid == 0) {
         s_tile = atomicAdd(&a.bm->tile_ctr[kCtrApply], 1u);  // tiles in the order CTAs start
         s_fail = 0;
+        s_tomb = 0;
+        s_changes = 0;
+        s_dirty = 0;
     }
     if (block_sees_error(&a.m->error)) return;
     const uint32_t n = a.n;
@@ -97,39 +137,44 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
     uint64_t* SV = a.st.vals[cur];
     uint8_t* SM = a.st.meta[cur];
     const uint32_t tile = s_tile, ntiles = gridDim.x;
-    if (tid < kLevelSlots) {
-        s_delta[tid] = 0;
-        s_chist[tid] = 0;
-    }
-    if (tid == 0) {
-        s_tomb = 0;
-        s_changes = 0;
-        s_dirty = 0;
-    }
-    const uint32_t base = tile * kApplyTile + tid * kItems;
+    const uint32_t blk = tile * (kTile / kApplyBlock) + (uint32_t)warp;
+    const uint32_t base = blk * kApplyBlock + (uint32_t)lane * kItems;
 
     uint64_t key[kItems];
     uint32_t pay[kItems];
-    uint32_t e[kItems];
-    uint32_t dres[kItems];
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        const uint32_t i = base + k;
-        key[k] = i < qv ? a.sk[i] : kMaxKey;
-        pay[k] = i < n ? a.sp[i] : 0u;
+    {  // 16-byte loads; the arrays are padded past the batch
+        ulonglong2 k01 = {kMaxKey, kMaxKey}, k23 = {kMaxKey, kMaxKey};
+        uint4 p = {0, 0, 0, 0};
+        if (base < n) {
+            k01 = reinterpret_cast<const ulonglong2*>(a.sk + base)[0];
+            k23 = reinterpret_cast<const ulonglong2*>(a.sk + base)[1];
+            p = *reinterpret_cast<const uint4*>(a.sp + base);
+        }
+        key[0] = base < qv ? k01.x : kMaxKey;
+        key[1] = base + 1u < qv ? k01.y : kMaxKey;
+        key[2] = base + 2u < qv ? k23.x : kMaxKey;
+        key[3] = base + 3u < qv ? k23.y : kMaxKey;
+        pay[0] = p.x;
+        pay[1] = p.y;
+        pay[2] = p.z;
+        pay[3] = p.w;
     }
-    const uint64_t kprev = (base > 0 && base - 1 < qv) ? a.sk[base - 1] : kMaxKey;
-    const uint64_t knext = (base + kItems < qv) ? a.sk[base + kItems] : kMaxKey;
-    // the descent's prefixes for this tile (its markers' maximum before it, the dense
-    // index of its first local run head), loaded with the batch (a block barrier below
-    // would keep them from being hoisted)
-    uint32_t tpref = kSmall ? 0u : a.tile_pref[tile];
-    const uint32_t dbase = kSmall ? 0u : a.sub_pref[tile * (kApplyTile / kSubTile)];
+    uint64_t kprev = __shfl_up_sync(0xffffffffu, key[kItems - 1], 1);
+    if (lane == 0) kprev = (base > 0 && base - 1 < qv) ? a.sk[base - 1] : kMaxKey;
+    uint64_t knext = __shfl_down_sync(0xffffffffu, key[0], 1);
+    if (lane == 31) knext = (base + kItems < qv) ? a.sk[base + kItems] : kMaxKey;
+    // the marker before the block, wanted where it continues a run
+    uint32_t mark = 0;
+    const uint32_t head0 = !kSmall && blk * kApplyBlock < n ? a.blk_head[blk] : 0u;
     if (kSmall) {
-        const uint32_t tb = tile * kApplyTile;
-        if (tb > 0 && tb < qv && a.sk[tb] == a.sk[tb - 1]) tpref = marker_before(a, tb, s_tmp);
+        const uint32_t tb = tile * kTile;
+        if (tb > 0 && tb < qv && a.sk[tb] == a.sk[tb - 1]) mark = marker_before_tile(a, tb, s_tmp);
+    } else if (__shfl_sync(0xffffffffu, base < qv && base > 0 && kprev == key[0], 0)) {
+        mark = marker_before_block(a, blk);
     }
-    uint32_t agg = 0;
+    // M: the largest marker before each query; dres: the nearest local head at or before it
+    uint32_t e[kItems], dres[kItems];
+    uint32_t agg = 0, heads = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
         const uint32_t i = base + k;
@@ -140,49 +185,64 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
         const bool write = valid && (op == 1u || op == 2u);
         e[k] = write ? 2u * i + 3u : (head ? 2u * i + 2u : 0u);
         agg = max(agg, e[k]);
+        heads += head || (valid && i % kApplyBlock == 0) ? 1u : 0u;
+        dres[k] = heads;
     }
-    const uint32_t texcl = block_excl_max<kApThreads>(agg, s_tmp, nullptr);
-    uint32_t M = max(tpref, texcl);
-    // dense index of each query's local run head: the tile's first one plus the local
-    // heads before it in the tile (a local head is a run head or a 256-query sub-tile's
-    // first query, as the descent counted them)
-    uint32_t lh = 0, nh = 0, hidx = 0;
-    if (!kSmall) {
+    uint32_t M;
+    if (kSmall) {
+        M = max(mark, block_excl_max<kApThreads>(agg, s_tmp, nullptr));
+    } else {
+        uint32_t x = agg, h = heads;
 #pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            const uint32_t i = base + k;
-            const uint64_t prev = k ? key[k - 1] : kprev;
-            const bool local = i < qv && (i == 0 || key[k] != prev || (i % kSubTile) == 0);
-            lh |= (local ? 1u : 0u) << k;
-            nh += local ? 1u : 0u;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o), z = __shfl_up_sync(0xffffffffu, h, o);
+            if (lane >= o) {
+                x = max(x, y);
+                h += z;
+            }
         }
-        hidx = dbase + block_excl_sum<kApThreads>(nh, s_tmp, nullptr);  // dense index of the next head
+        x = __shfl_up_sync(0xffffffffu, x, 1);
+        M = lane ? max(mark, x) : mark;
+        const uint32_t dtile = a.tile_mark ? kApplyTile : kDescendTile;
+        h += head0 + base / dtile * dtile - heads - 1u;  // (wraps for a block past the valid queries: not used)
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) dres[k] += h;
     }
     uint32_t new_here = 0, new_mask = 0, chg_here = 0, chg_mask = 0;
-    // Per query: its run head's result index, and the gathers of its prior state, all
-    // issued before any store so that their latencies overlap: the run head's state, or,
-    // when an earlier query of its run wrote (the marker names it), that query's payload.
-    uint32_t fromw = 0, insw = 0, flx = 0;  // bit k: from an earlier write; that write inserts; flags
+    // Per query, all gathers of a step issued before any store so that their latencies overlap:
+    // the run head's state, or, when an earlier query of its run wrote (the marker names it),
+    // that query's payload; for the run's owner (its last query, if the run writes) the
+    // storage place and the payload of the run's last write.
+    uint32_t fromw = 0, insw = 0, flx = 0, own = 0;  // bit k: from an earlier write; that write inserts; flags; owner
     uint64_t val[kItems];
-    uint32_t pj[kItems];
+    uint32_t pj[kItems], pw[kItems], at[kItems];
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
+        const uint32_t i = base + k;
+        if (kSmall) dres[k] = i;
         const uint32_t mex = M;
         const uint32_t minc = max(M, e[k]);
         M = minc;
-        e[k] = minc;  // keep the inclusive value for the owners and the new-node pass
-        dres[k] = kSmall ? base + k : hidx + ((lh >> k) & 1u) - 1u;  // this query's run head's result
-        hidx += (lh >> k) & 1u;
-        const uint64_t prev = k ? key[k - 1] : kprev;
-        const bool q = base + k < qv;
-        const bool fw = q && (base + k != 0 && key[k] == prev) && (mex & 1u);
+        const uint64_t prev = k ? key[k - 1] : kprev, next = (k + 1 < kItems) ? key[k + 1] : knext;
+        const bool q = i < qv;
+        const bool fw = q && (i != 0 && key[k] == prev) && (mex & 1u);
+        const bool ow = q && next != key[k] && (minc & 1u);
+        const uint32_t jw = (minc - 3u) >> 1;
         fromw |= (fw ? 1u : 0u) << k;
+        own |= (ow ? 1u : 0u) << k;
         flx |= (q ? (uint32_t)a.flags[dres[k]] : 0u) << (2 * k);
         val[k] = q ? a.val0[dres[k]] : 0ull;
         pj[k] = fw ? a.sp[(mex - 3u) >> 1] : 0u;
+        at[k] = ow ? a.loc[dres[k]] : 0u;
+        pw[k] = !ow ? 0u : (jw == i ? pay[k] : a.sp[jw]);
     }
+    uint64_t nv[kItems];  // the owner's new value
+    uint32_t mt[kItems];  // its node's state byte
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
+        const bool ow = (own >> k) & 1u, exists = (flx >> (2 * k)) & 1u;
+        nv[k] = ow && (pw[k] >> 30) == 1u ? a.uvals[pw[k] & kSeqMask] : 0ull;
+        mt[k] = ow && exists ? SM[at[k] - 1u] : 0u;
         if (!((fromw >> k) & 1u)) {
             if (!((flx >> (2 * k + 1)) & 1u)) val[k] = 0ull;  // the run head's key is not live
             continue;
@@ -200,30 +260,18 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
             store_result(a.results, seq, 0ull, PI_R_INVALID);
             continue;
         }
-        const uint32_t dj = dres[k];
         const bool exists = (flx >> (2 * k)) & 1u, live0 = (flx >> (2 * k + 1)) & 1u;
         const bool pl = ((fromw >> k) & 1u) ? ((insw >> k) & 1u) != 0 : live0;
         store_result(a.results, seq, val[k], pl ? PI_R_PRESENT : PI_R_ABSENT);
-
-        const uint64_t next = (k + 1 < kItems) ? key[k + 1] : knext;
-        const bool last = next != key[k];
-        const uint32_t minc = e[k];
-        if (!last || !(minc & 1u)) continue;  // not the owner, or the run never writes
-        const uint32_t jw = (minc - 3u) >> 1;
-        const uint32_t pw = (jw == i) ? pay[k] : a.sp[jw];
-        const bool fin_live = (pw >> 30) == 1u;
+        if (!((own >> k) & 1u)) continue;
+        const bool fin_live = (pw[k] >> 30) == 1u;
         if (exists) {
-            const uint32_t r = a.loc[dj] - 1u;
+            const uint32_t r = at[k] - 1u;
             if (a.wcount) atomicAdd(&a.wcount[r], 1u);
-            const uint8_t mt = SM[r];
-            const uint32_t h = mt & kHeightMask;
-            if (fin_live) {
-                SV[r] = a.uvals[pw & kSeqMask];
-                SM[r] = (uint8_t)h;
-            } else {
-                SM[r] = (uint8_t)(h | kTomb);
-            }
+            const uint32_t h = mt[k] & kHeightMask;
+            if (fin_live) SV[r] = nv[k];
             if (fin_live != live0) {
+                SM[r] = (uint8_t)(h | (fin_live ? 0u : kTomb));
                 atomicAdd(&s_tomb, fin_live ? -1 : 1);
                 atomicAdd(&s_changes, 1u);
                 atomicAdd(&s_delta[1], fin_live ? 1 : -1);
@@ -236,6 +284,7 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
                     s_dirty = 1;
                     chg_here++;
                     chg_mask |= 1u << k;
+                    mt[k] = h | (fin_live ? 0x80u : 0u);  // as the change list has it
                 }
             }
         } else if (fin_live) {
@@ -246,39 +295,46 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
     // Places of the tile's new nodes and level changes. Warp 0 looks back over the new
     // nodes' counts, warp 1 over the changes'. A tile without any publishes its zero and goes
     // on, but for every 64th, so that a look-back finds a prefix within two rounds.
-    uint32_t tile_new = 0, tile_chg = 0, slot = 0, cslot = 0;
-    if (__syncthreads_or(new_here != 0)) slot = block_excl_sum<kApThreads>(new_here, s_tmp, &tile_new);
-    if (__syncthreads_or(chg_here != 0)) cslot = block_excl_sum<kApThreads>(chg_here, s_tmp, &tile_chg);
+    uint32_t both = new_here | (chg_here << 16), incl = both;  // a tile's counts stay below 2^16
+    if (__any_sync(0xffffffffu, both != 0)) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    const uint32_t wc = lane < kApThreads / 32 ? s_warp[lane] : 0u;
+    const uint32_t tot = __reduce_add_sync(0xffffffffu, wc);
+    const uint32_t wb = __reduce_add_sync(0xffffffffu, lane < warp ? wc : 0u) + incl - both;
+    const uint32_t tile_new = tot & 0xFFFFu, tile_chg = tot >> 16;
     if (tid < 64) {
         const uint32_t c = tid < 32 ? tile_new : tile_chg;
         uint64_t* desc = a.desc + (tid < 32 ? 0u : ntiles);
         if (c || (tile & 63u) == 0) {
             bool ok = true;
             const uint32_t ex = lookback_warp_wide<false, 8>(desc, tile, epoch, c, a.err, &ok);
-            if ((tid & 31) == 0) {
+            if (lane == 0) {
                 s_base[tid >> 5] = ex;
                 if (!ok) s_fail = 1;
             }
-        } else if ((tid & 31) == 0) {
+        } else if (lane == 0) {
             lookback_publish(desc, tile, epoch, 0u);
         }
     }
-    if (tile_new || tile_chg) {
-        __syncthreads();
-        if (s_fail) return;
-    }
+    if (!tot && !s_changes) return;  // block-uniform: no node came, went or changed its state
+    __syncthreads();
+    if (s_fail) return;
     if (new_mask) {
-        uint32_t o = s_base[0] + slot;
+        uint32_t o = s_base[0] + (wb & 0xFFFFu);
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {
             if (!(new_mask & (1u << k))) continue;
-            const uint32_t i = base + k;
-            const uint32_t jw = (e[k] - 3u) >> 1;
-            const uint32_t pw = (jw == i) ? pay[k] : a.sp[jw];
             const uint32_t h = tower_height(key[k], a.hp);
             a.nn.keys[o] = key[k];
-            a.nn.vals[o] = a.uvals[pw & kSeqMask];
-            a.nn.loc[o] = a.loc[dres[k]];
+            a.nn.vals[o] = nv[k];
+            a.nn.loc[o] = at[k];
             a.nn.height[o] = (uint8_t)h;
             ++o;
             atomicAdd(&s_changes, 1u);
@@ -289,16 +345,14 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
     }
     // Built-level membership changes, for an incremental rebuild.
     if (chg_mask) {
-        uint32_t o = s_base[1] + cslot;
+        uint32_t o = s_base[1] + (wb >> 16);
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {
             if (!(chg_mask & (1u << k))) continue;
-            const uint32_t r = a.loc[dres[k]] - 1u;
-            const uint8_t mt = SM[r];  // as this kernel left it
-            const uint32_t h = mt & kHeightMask;
+            const uint32_t h = mt[k] & kHeightMask;
             a.chg.keys[o] = key[k];
-            a.chg.pos[o] = r;
-            a.chg.hl[o] = (uint8_t)(h | ((mt & kTomb) ? 0u : 0x80u));
+            a.chg.pos[o] = at[k] - 1u;
+            a.chg.hl[o] = (uint8_t)mt[k];
             ++o;
             atomicAdd(&s_chist[h < (uint32_t)kLevelSlots ? h : kLevelSlots - 1], 1u);
         }
@@ -312,22 +366,6 @@ __global__ void __launch_bounds__(kApThreads, 2) k_apply(ApplyArgs a, RebuildArg
         if (s_dirty) atomicOr(&a.bm->index_dirty, 1u);
         if (tile_new) atomicAdd(&a.bm->new_count, tile_new);
         if (tile_chg) atomicAdd(&a.bm->nchg, tile_chg);
-    }
-    // Arrival: the barrier orders every thread's stores before thread 0's fence, which (being
-    // cumulative) releases them before its count; the last CTA then sees all of them.
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(&a.bm->tile_ctr[kCtrApplyDone], 1u) == ntiles - 1u ? 1u : 0u;
-        if (s_last) __threadfence();
-    }
-    __syncthreads();
-    if (!s_last || tid >= 32) return;
-    const bool merge = merge_needed(a.m, a.bm);
-    if (merge) {
-        if (tid == 0) a.bm->merged = 1u;  // the merge's kernels end the batch
-    } else {
-        level_layout(rb, false);
     }
 }
 
@@ -358,11 +396,11 @@ __global__ void __launch_bounds__(kThreads) k_owner_check(ApplyArgs a) {
 
 }  // namespace
 
-cudaError_t launch_apply(const ApplyArgs& a, const RebuildArgs& rb, bool small, uint32_t& epoch, cudaStream_t s) {
+cudaError_t launch_apply(const ApplyArgs& a, bool small, uint32_t& epoch, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
-    const uint32_t tiles = (a.n + kApplyTile - 1) / kApplyTile;
-    if (small) launch_dep(k_apply<true>, tiles, kApThreads, 0, s, a, rb, ++epoch);
-    else launch_dep(k_apply<false>, tiles, kApThreads, 0, s, a, rb, ++epoch);  // tile prefixes come from the descent
+    const uint32_t tiles = (a.n + kTile - 1) / kTile;
+    if (small) launch_dep(k_apply<true>, tiles, kApThreads, 0, s, a, ++epoch);
+    else launch_dep(k_apply<false>, tiles, kApThreads, 0, s, a, ++epoch);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -17,11 +17,9 @@ constexpr uint32_t kPad = 64;           // readable entries past every array's e
 constexpr uint32_t kSortTile = 2048;    // elements per radix-sort tile (the smaller of two sizes)
 constexpr uint32_t kSortHist = 9 * 256; // digit counts of a radix sort
 constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the count kernel's scan
-constexpr uint32_t kCtrDistinct = 14;   // BatchMeta::tile_ctr slots: the descent prologue's tile counter,
-constexpr uint32_t kCtrApply = 15;      // the apply kernel's, and its finished tiles
-constexpr uint32_t kCtrApplyDone = 16;
+constexpr uint32_t kCtrApply = 15;      // BatchMeta::tile_ctr slot: the apply kernel's tile counter
 constexpr uint32_t kApplyTile = 2048;   // sorted queries per apply tile
-constexpr uint32_t kSubTile = 256;      // sorted queries per descent warp step (one apply warp)
+constexpr uint32_t kApplyBlock = 128;   // sorted queries per apply warp
 constexpr uint32_t kRunTile = 1024;     // queries per tile of the small batches' sort
 // Largest batch sorted that way. A query is ranked in every other tile, so the ranking's work
 // grows with the square of the batch; the radix passes' chain of launches does not grow.
@@ -134,7 +132,7 @@ struct BatchMeta {
     uint32_t index_dirty;        // level membership changed
     uint32_t rebuild;            // the rebuild runs in this batch
     uint32_t changes;            // storage nodes whose liveness changed or that were added
-    uint32_t distinct;           // distinct keys of the batch (local run heads)
+    uint32_t size0, tombs0;      // DevMeta's size and tombs as the batch found them
     uint32_t bmax[8];            // per key byte: its maximum over the batch
     uint32_t bnmin[8];           // per key byte: 255 - its minimum over the batch
     uint32_t fix_big;            // queries in key-prefix segments longer than one warp
@@ -207,6 +205,14 @@ __device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p) {
 // on average with stores, 3.1 us with exchanges).
 __device__ __forceinline__ void publish(uint64_t* p, uint64_t v) {
     atomicExch(reinterpret_cast<unsigned long long*>(p), (unsigned long long)v);
+}
+// Four consecutive 64-bit words with one 32-byte load (p 32-byte aligned): a lane's access to a
+// line of its own costs the L1 one look-up instead of two.
+__device__ __forceinline__ void ld_256(const uint64_t* p, uint64_t (&v)[4]) {
+    asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
+                 : "l"(p)
+                 : "memory");
 }
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -649,14 +655,9 @@ cudaError_t launch_tile_sort(const uint8_t* ops, const uint64_t* keys, uint32_t 
 struct DescendArgs {
     const uint64_t* sk;  // sorted keys
     const uint32_t* sp;  // sorted payload (op << 30 | arrival index)
-    uint32_t* tile_pref; // per-apply-tile exclusive max prefix of the run markers e_i
-    uint32_t* sub_pref;  // dense index of each sub-tile's first distinct key
-    uint64_t* desc;      // look-back descriptors: 2 words per apply tile
-    uint64_t* dq;        // dense distinct keys
-    uint32_t* dlo;       // their current start position on the level being searched
-    int top_launched;    // highest index level given its own launch (see launch_descend);
-                         // at least bottom_launched
-    int bottom_launched; // lowest level that can be built: searched by the storage locate
+    uint32_t* blk_head;  // per 128-query block: its first local run head's number in the descent's tile
+    uint32_t* blk_mark;  // per block: the largest run marker e_i in it (0: none)
+    uint32_t* tile_mark; // per apply tile; null: the batch takes no windows, and there are none
     const DevMeta* m;
     BatchMeta* bm;
     const uint64_t* lkeys;   // index-layer buffer 0 (DevMeta::lcur picks the one in use)
@@ -664,16 +665,19 @@ struct DescendArgs {
     const uint64_t* lkeys1;  // buffer 1
     const uint32_t* ldown1;
     Storage st;
-    uint32_t* loc;
+    uint32_t* loc;           // storage place and state of the local run heads, from each tile's start on
     uint8_t* flags;
     uint64_t* val0;
     uint32_t n;
     uint32_t* err;
 };
-// before_locate (may be null) is recorded on s just before the storage-locate kernel.
-// The look-back of the first kernel takes ++epoch; a.desc needs 2 words per apply tile.
-cudaError_t launch_descend(const DescendArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms,
-                           cudaEvent_t before_locate = nullptr);
+// Whether a batch of n queries on a lowest built level of `entries` entries takes windows of the
+// level. A tile per CTA needs enough tiles for every SM, and the average tile's stretch has to
+// leave room in a window.
+constexpr uint64_t kWindowBatch = 1u << 19;
+bool descend_windows(uint64_t n, uint64_t entries);
+constexpr uint32_t kDescendTile = 256;  // queries of a descent tile without windows (with: kApplyTile)
+cudaError_t launch_descend(const DescendArgs& a, cudaStream_t s);
 // The small batches' counterpart: from the sorted tiles (tk / tp) the whole batch in sorted
 // order (ok / op), and loc / flags / val0 of every query at its sorted position.
 cudaError_t launch_rank_locate(const DescendArgs& a, const uint64_t* tk, const uint32_t* tp, uint64_t* ok, uint32_t* op,
@@ -692,8 +696,9 @@ struct ApplyArgs {
     DevMeta* m;
     BatchMeta* bm;
     uint64_t* desc;            // look-back descriptors: 2 words per tile
-    const uint32_t* tile_pref; // per-tile exclusive marker prefix
-    const uint32_t* sub_pref;  // dense index of each 256-query sub-tile's first distinct key
+    const uint32_t* blk_head;  // from the descent (not for small batches)
+    const uint32_t* blk_mark;
+    const uint32_t* tile_mark;
     LevelChanges chg;          // level membership changes, in key order
     uint32_t* lcnt;  // per-level per-tile live counts (see RebuildArgs)
     uint32_t lstride;
@@ -702,11 +707,9 @@ struct ApplyArgs {
     uint32_t* err;
     uint32_t* wcount;  // debug check (null when off): writes per storage node in this batch
 };
-struct RebuildArgs;
-// Executes the sorted batch and, unless it re-lays-out the storage layer, ends it (the level
-// layout of rb). The look-back takes ++epoch. `small`: loc / flags / val0 hold one entry per query (launch_rank_locate), and the tile
-// prefixes are not given.
-cudaError_t launch_apply(const ApplyArgs& a, const RebuildArgs& rb, bool small, uint32_t& epoch, cudaStream_t s);
+// The look-back takes ++epoch. `small`: loc / flags / val0 hold every query's state
+// (launch_rank_locate), and there are no marks.
+cudaError_t launch_apply(const ApplyArgs& a, bool small, uint32_t& epoch, cudaStream_t s);
 // Debug check of single ownership: every storage node written at most once by the
 // batch's apply (sets kErrOwner otherwise); adds the writes to DevMeta::owner_writes and
 // clears the counts.

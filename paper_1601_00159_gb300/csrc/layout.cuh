@@ -7,12 +7,10 @@
 namespace pi {
 
 // Whether the batch re-lays-out the storage layer: new nodes must be placed, or delete-flagged
-// nodes exceed 1/8 of it. Read with every counter of the batch in place; afterwards
-// BatchMeta::merged holds the answer.
-__device__ __forceinline__ bool merge_needed(const DevMeta* m, const BatchMeta* bm) {
-    const uint32_t size = __ldcg(&m->size);
-    const uint32_t tombs = (uint32_t)((int32_t)__ldcg(&m->tombs) + __ldcg(&bm->tomb_delta));
-    return __ldcg(&bm->new_count) > 0 || (tombs > 0 && (uint64_t)tombs * 8u > size);
+// nodes exceed 1/8 of it. Only reads what stays as it is while the batch ends.
+__device__ __forceinline__ bool merge_needed(const BatchMeta* bm) {
+    const uint32_t tombs = (uint32_t)((int32_t)bm->tombs0 + bm->tomb_delta);
+    return bm->new_count > 0 || (tombs > 0 && (uint64_t)tombs * 8u > bm->size0);
 }
 
 __device__ __forceinline__ uint64_t suffix_sum64(uint64_t v, uint32_t lane) {

@@ -42,7 +42,6 @@ struct Scratch {
     uint8_t* flags = nullptr;
     uint64_t* val0 = nullptr;
     NewNodes nn{};
-    uint32_t* tile_pref = nullptr;
     uint32_t* sdesc[2] = {};   // radix sort: per-tile look-back words, or digit counts and offsets
     uint32_t* gsum = nullptr;  // radix sort of large batches: per-group digit totals / offsets
     uint32_t* gctr = nullptr;  // radix sort: the count kernels' arrival counters
@@ -54,9 +53,9 @@ struct Scratch {
     int32_t* lst_pref = nullptr;
     uint8_t* lst_ins = nullptr;
     uint64_t lst_cap = 0;
-    uint32_t* sub_pref = nullptr;
-    uint64_t* dq = nullptr;    // descent: dense distinct keys
-    uint32_t* dlo = nullptr;   // descent: per-key start position
+    uint32_t* blk_head = nullptr;   // descent: per 128-query block, its first head's number
+    uint32_t* blk_mark = nullptr;   // descent: markers per block and per apply tile
+    uint32_t* tile_mark = nullptr;
 };
 
 // pi_profile level 2: the two events around every kernel launch of the batch entry
@@ -249,7 +248,7 @@ int map_cuda(cudaError_t e) {
 // Look-back descriptors needed for q queries and a storage capacity of s nodes.
 uint64_t desc_need(uint64_t q, uint64_t s) {
     uint64_t a = 0;                                    // (the sort needs none)
-    uint64_t b = 2 * ((q + 2047) / 2048);    // apply
+    uint64_t b = 2 * ((q + 1023) / 1024);    // apply
     uint64_t c = (s / 4096 + 2) * 32;        // merge, export
     if (c < 32 * 64) c = 32 * 64;            // rebuild level scan: 64 chunks x 32 levels
     uint64_t m = a > b ? a : b;
@@ -309,12 +308,11 @@ void free_scratch(Scratch& s) {
     dfree(s.in_k); dfree(s.in_p); dfree(s.a_k); dfree(s.a_p); dfree(s.b_k); dfree(s.b_p);
     dfree(s.loc); dfree(s.flags); dfree(s.val0);
     dfree(s.nn.keys); dfree(s.nn.vals); dfree(s.nn.loc); dfree(s.nn.height);
-    dfree(s.tile_pref);
     dfree(s.sdesc[0]); dfree(s.sdesc[1]); dfree(s.fixmap);
     dfree(s.gsum); dfree(s.gctr); dfree(s.ndig);
     dfree(s.chg.keys); dfree(s.chg.pos); dfree(s.chg.hl);
     dfree(s.lst_keys); dfree(s.lst_pos); dfree(s.lst_pref); dfree(s.lst_ins);
-    dfree(s.sub_pref); dfree(s.dq); dfree(s.dlo);
+    dfree(s.blk_head); dfree(s.blk_mark); dfree(s.tile_mark);
     s.cap = 0;
 }
 
@@ -329,7 +327,6 @@ cudaError_t alloc_scratch(Scratch& s, uint64_t q) {
     PI_TRY(dalloc(&s.nn.keys, c)); PI_TRY(dalloc(&s.nn.vals, c));
     PI_TRY(dalloc(&s.nn.loc, c)); PI_TRY(dalloc(&s.nn.height, c));
     const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
-    PI_TRY(dalloc(&s.tile_pref, tiles));
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
     PI_TRY(dalloc(&s.sdesc[0], stiles * 256)); PI_TRY(dalloc(&s.sdesc[1], stiles * 256));
     const uint64_t sgroups = stiles / kScanGroup + 1;
@@ -340,9 +337,8 @@ cudaError_t alloc_scratch(Scratch& s, uint64_t q) {
     s.lst_cap = 2 * c + 64;
     PI_TRY(dalloc(&s.lst_keys, s.lst_cap)); PI_TRY(dalloc(&s.lst_pos, s.lst_cap));
     PI_TRY(dalloc(&s.lst_pref, s.lst_cap)); PI_TRY(dalloc(&s.lst_ins, s.lst_cap));
-    const uint64_t nsub = (q + kSubTile - 1) / kSubTile + 1;
-    PI_TRY(dalloc(&s.sub_pref, nsub));
-    PI_TRY(dalloc(&s.dq, c)); PI_TRY(dalloc(&s.dlo, c));
+    PI_TRY(dalloc(&s.blk_head, tiles * (kApplyTile / kApplyBlock)));
+    PI_TRY(dalloc(&s.blk_mark, tiles * (kApplyTile / kApplyBlock))); PI_TRY(dalloc(&s.tile_mark, tiles));
 #undef PI_TRY
     s.cap = q;
     return cudaSuccess;
@@ -596,23 +592,12 @@ cudaError_t grow_scratch(pi_index* x, uint64_t n, cudaStream_t s) {
     return ensure_desc(x, desc_need(q, x->st_cap));
 }
 
-// The descent walks the levels below the pinned ones inside its top kernel, one key
-// per thread, as long as they are small (about 24 MB of entries: L2-resident); the
-// levels below get one launch each. Taken from the host's last view of the index; any
-// split gives the same result.
-constexpr uint64_t kWalkEntries = 2u << 20;
-
-int top_launched_for(const pi_index* x) {
+// Whether a batch's descent takes windows of the lowest built level, by the host's last view of
+// the index: either way gives the same result.
+bool windows_for(const pi_index* x, uint64_t n) {
     const DevMeta& k = x->known;
-    if (x->test_flags & PI_TEST_WALK_LEVELS) return 2;
-    if (k.Ls < 3 || k.Ls > (uint32_t)x->hp.hmax + 1) return x->hp.hmax;
-    uint64_t cum = 0;
-    int l = (int)k.Ls - 1;
-    while (l >= 2 && cum + k.n[l] <= kWalkEntries) {
-        cum += k.n[l];
-        --l;
-    }
-    return l < 2 ? 2 : l;
+    const uint64_t entries = k.Lb <= k.H && k.Lb < (uint32_t)kLevelSlots ? k.n[k.Lb] : k.size;
+    return descend_windows(n, entries) && !(x->test_flags & PI_TEST_WALK_LEVELS);
 }
 
 RebuildArgs rebuild_args(pi_index* x, BatchMeta* bm, uint32_t size_ub, uint32_t force) {
@@ -651,17 +636,14 @@ constexpr uint64_t noalloc_bytes(uint64_t q) {
     const uint64_t c = q + kPad;
     const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
-    const uint64_t nsub = (q + kSubTile - 1) / kSubTile + 1;
     return 3 * al256(c * 8) + 3 * al256(c * 4)                    // in, a, b (keys, payload)
            + al256(c * 4) + al256(c) + al256(c * 8)               // loc, flags, val0
            + 2 * al256(c * 8) + al256(c * 4) + al256(c)           // new nodes
-           + al256(tiles * 4)                                     // tile prefix
            + 2 * al256(stiles * 256 * 4)                          // sort look-back words
            + al256((c / 32 + 1) * 4)                              // fixmap
            + al256(c * 8) + al256(c * 4) + al256(c)               // level changes
            + al256((2 * c + 64) * 8) + 2 * al256((2 * c + 64) * 4) + al256(2 * c + 64)  // lists
-           + al256(nsub * 4)                                      // sub_pref
-           + al256(c * 8) + al256(c * 4);                         // dq, dlo
+           + 2 * al256(tiles * (kApplyTile / kApplyBlock) * 4) + al256(tiles * 4);  // heads, marks
 }
 
 constexpr uint64_t kNoAllocBytes = noalloc_bytes(PI_NOALLOC_MAX_BATCH);
@@ -679,20 +661,18 @@ uint64_t carve_scratch(uint8_t* base, uint64_t q, Scratch& s) {
     const uint64_t c = q + kPad;
     const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
     const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
-    const uint64_t nsub = (q + kSubTile - 1) / kSubTile + 1;
     take(s.in_k, c * 8); take(s.a_k, c * 8); take(s.b_k, c * 8);
     take(s.in_p, c * 4); take(s.a_p, c * 4); take(s.b_p, c * 4);
     take(s.loc, c * 4); take(s.flags, c); take(s.val0, c * 8);
     take(s.nn.keys, c * 8); take(s.nn.vals, c * 8); take(s.nn.loc, c * 4); take(s.nn.height, c);
-    take(s.tile_pref, tiles * 4);
     take(s.sdesc[0], stiles * 256 * 4); take(s.sdesc[1], stiles * 256 * 4);
     take(s.fixmap, (c / 32 + 1) * 4);
     take(s.chg.keys, c * 8); take(s.chg.pos, c * 4); take(s.chg.hl, c);
     s.lst_cap = 2 * c + 64;
     take(s.lst_keys, s.lst_cap * 8); take(s.lst_pos, s.lst_cap * 4); take(s.lst_pref, s.lst_cap * 4);
     take(s.lst_ins, s.lst_cap);
-    take(s.sub_pref, nsub * 4);
-    take(s.dq, c * 8); take(s.dlo, c * 4);
+    take(s.blk_head, tiles * (kApplyTile / kApplyBlock) * 4);
+    take(s.blk_mark, tiles * (kApplyTile / kApplyBlock) * 4); take(s.tile_mark, tiles * 4);
     s.cap = q;
     return off;
 }
@@ -789,15 +769,9 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     DescendArgs da{};
     da.sk = sc.a_k;
     da.sp = sc.a_p;
-    da.tile_pref = sc.tile_pref;
-    da.sub_pref = sc.sub_pref;
-    da.desc = x->desc;
-    da.dq = sc.dq;
-    da.dlo = sc.dlo;
-    // the lowest buildable level is never walked by the prologue: the storage locate
-    // searches it itself (it needs that level's gap ends)
-    da.top_launched = std::max(top_launched_for(x), (int)x->min_lb);
-    da.bottom_launched = (int)x->min_lb;
+    da.blk_head = sc.blk_head;
+    da.blk_mark = sc.blk_mark;
+    da.tile_mark = windows_for(x, n) ? sc.tile_mark : nullptr;
     da.m = x->d_meta;
     da.bm = bm;
     da.lkeys = x->lkeys;
@@ -810,9 +784,8 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     da.val0 = sc.val0;
     da.n = (uint32_t)n;
     da.err = &x->d_meta->error;
-    if (small) prof_mark(x, 10, s);
-    e = small ? launch_rank_locate(da, sc.in_k, sc.in_p, sc.a_k, sc.a_p, s)
-              : launch_descend(da, ep, s, x->num_sms, prof_event(x, 10));
+    prof_mark(x, 10, s);
+    e = small ? launch_rank_locate(da, sc.in_k, sc.in_p, sc.a_k, sc.a_p, s) : launch_descend(da, s);
     if (e != cudaSuccess) return map_cuda(e);
     prof_mark(x, 3, s);
     ApplyArgs aa{};
@@ -828,8 +801,9 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     aa.m = x->d_meta;
     aa.bm = bm;
     aa.desc = x->desc;
-    aa.tile_pref = sc.tile_pref;
-    aa.sub_pref = sc.sub_pref;
+    aa.blk_head = sc.blk_head;
+    aa.blk_mark = sc.blk_mark;
+    aa.tile_mark = da.tile_mark;
     aa.chg = sc.chg;
     aa.lcnt = x->lcnt;
     aa.lstride = x->lstride;
@@ -852,7 +826,7 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     }
     ra.mbox = &x->h_mbox[slot];
     ra.bm_next = x->d_bm + ((x->issued + 1u) & 1u);
-    if ((e = launch_apply(aa, ra, small, ep, s)) != cudaSuccess) return map_cuda(e);
+    if ((e = launch_apply(aa, small, ep, s)) != cudaSuccess) return map_cuda(e);
     if ((e = launch_owner_check(aa, s, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 4, s);
     if ((e = launch_merge(ra, ep, s, x->num_sms)) != cudaSuccess) return map_cuda(e);

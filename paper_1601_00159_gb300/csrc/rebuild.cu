@@ -80,7 +80,8 @@ __device__ __forceinline__ uint64_t block_excl_sum64(uint64_t v, uint64_t* tmp, 
 // come from these), so nothing reads the new meta bytes again for them. A tile's counts are
 // cleared by the CTA whose chunks reach the tile's start, before that CTA publishes: outputs
 // never lie beyond their place in the sequence, so whoever adds to a tile has looked back past
-// that publication. The CTA that finishes last lays out the levels.
+// that publication. The CTA that finishes last lays out the levels; a batch that needs no merge
+// has that done by the first CTA.
 // Bound by HBM: 17 B read and 17 B written per node. Measured, a batch: 78,000 keys appended to
 // 4 M nodes 807 -> 234 us (the merge 642 -> 89); 2^18 keys spread over 17.3 M nodes 439 -> 418 us
 // (the count it takes along was 31 us of the rebuild).
@@ -99,8 +100,11 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
     __shared__ int s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevMeta* m = a.m;
-    if (!a.bm->merged) {  // the apply kernel ended the batch, or an error did
-        if (blockIdx.x == 0 && warp == 0) post_batch(a);
+    if (!merge_needed(a.bm)) {  // the storage layer stays: this only ends the batch
+        if (blockIdx.x == 0 && warp == 0) {
+            level_layout(a, false);
+            post_batch(a);
+        }
         return;
     }
     if (tid == 0) {
