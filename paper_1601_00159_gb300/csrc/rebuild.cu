@@ -32,35 +32,6 @@ constexpr int kNodes = 4096;             // storage nodes per tile
 constexpr int kPer = kNodes / kThreads;  // 16 per thread
 constexpr uint32_t kCtrMerge = 9, kCtrMergeDone = 10, kCtrCreate = 11;
 
-// Block-wide exclusive sum of 64-bit values (kThreads threads); total in *total.
-__device__ __forceinline__ uint64_t block_excl_sum64(uint64_t v, uint64_t* tmp, uint64_t* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint64_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) tmp[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        const uint64_t w = lane < kThreads / 32 ? tmp[lane] : 0ull;
-        uint64_t t = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        if (lane < kThreads / 32) tmp[lane] = t - w;
-        if (lane == kThreads / 32 - 1) tmp[32] = t;
-    }
-    __syncthreads();
-    const uint64_t r = tmp[warp] + x - v;
-    if (total) *total = tmp[32];
-    __syncthreads();
-    return r;
-}
-
 // ---------------------------------------------------------------------------------
 // Merge: old live nodes + new nodes -> the other storage buffer, in key order. A new node with
 // loc = x goes right before old node x.
@@ -73,29 +44,46 @@ __device__ __forceinline__ uint64_t block_excl_sum64(uint64_t v, uint64_t* tmp, 
 //   1. its cuts, all at once by its warps, and the live nodes among its old ones (no read when
 //      nothing is delete-flagged); a look-back over the CTAs, numbered in the order they
 //      start, gives its first output place;
-//   2. per chunk, a blocked pass (16 positions per thread) over the meta bytes and the new
-//      nodes' insertion points gives every position its output offset, and a striped pass
-//      copies the live nodes with coalesced loads and stores.
+//   2. per chunk, whose old nodes arrive in shared memory by TMA bulk copies two chunks ahead,
+//      a blocked pass over the state bytes and the new nodes' insertion points gives every
+//      position its output offset, and a striped pass writes the live nodes, coalesced.
 // The pass also counts, per output tile, the nodes of each built level (the rebuild's offsets
 // come from these), so nothing reads the new meta bytes again for them. A tile's counts are
 // cleared by the CTA whose chunks reach the tile's start, before that CTA publishes: outputs
 // never lie beyond their place in the sequence, so whoever adds to a tile has looked back past
 // that publication. The CTA that finishes last lays out the levels; a batch that needs no merge
 // has that done by the first CTA.
-// Bound by HBM: 17 B read and 17 B written per node. Measured, a batch: 78,000 keys appended to
-// 4 M nodes 807 -> 234 us (the merge 642 -> 89); 2^18 keys spread over 17.3 M nodes 439 -> 418 us
-// (the count it takes along was 31 us of the rebuild).
-constexpr uint32_t kChunk = kNodes - 32;  // 15 positions of alignment and the slot after the last fit a tile
-constexpr uint32_t kCuts = 64;            // cuts found at once
+// Bound by HBM: 17 B read and 17 B written per node. With plain loads, issued and waited for
+// within the chunk, the copy ran at 42% of the memory rate, its warps waiting for loads and at
+// barriers; the copies ahead take the loads out of the chunk, and three barriers are left in it,
+// whose waits the other three CTAs of the SM fill. 2^18 new keys spread over 17.3 M nodes 187 ->
+// 140 us (100 at the copy rate); 78,000 keys appended to 4.2 M 89 -> 58.
+constexpr uint32_t kMergeTile = 1280;              // positions of a chunk's tile
+constexpr uint32_t kChunk = kMergeTile - 32;       // 15 positions of alignment and the slot after the last fit
+constexpr uint32_t kCuts = 256;                    // cuts found at once
+constexpr int kMergePer = (int)kMergeTile / kThreads;
+constexpr int kStages = 2;
 
-__global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoch) {
+struct MergeStage {
+    uint64_t keys[kMergeTile];
+    uint64_t vals[kMergeTile];
+    uint8_t meta[kMergeTile];
+};
+struct MergeSmem {
+    MergeStage st[kStages];
+    // per position: its new nodes' last one in the chunk, plus one; then live old nodes before it |
+    // new nodes at or before it << 16
+    // (two, so that one is cleared while the other is read)
+    uint32_t off[2][kMergeTile];
+};
+
+__global__ void __launch_bounds__(kThreads, 4) k_merge(RebuildArgs a, uint32_t epoch) {
     pdl_wait();
     pdl_trigger();
-    // per position: new nodes inserted there; then live old nodes before it | new nodes at or
-    // before it << 16
-    __shared__ __align__(16) uint32_t s_off[kNodes];
-    __shared__ uint64_t s_tmp[33];
-    __shared__ uint32_t s_cut[kCuts + 1], s_cnt[2][kLevelSlots], s_warp[kThreads / 32];
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    MergeSmem& S = *reinterpret_cast<MergeSmem*>(s_dyn);
+    __shared__ __align__(8) uint64_t s_bar[kStages];
+    __shared__ uint32_t s_cut[kCuts + 1], s_cnt[2][kLevelSlots], s_warp[kThreads / 32], s_new[kThreads / 32];
     __shared__ uint32_t s_cta, s_pref, s_last;
     __shared__ int s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -110,6 +98,7 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
     if (tid == 0) {
         s_cta = atomicAdd(&a.bm->tile_ctr[kCtrMerge], 1u);
         s_fail = 0;
+        for (int k = 0; k < kStages; ++k) mbar_init(&s_bar[k], 1);
     }
     if (tid < 2 * kLevelSlots) (&s_cnt[0][0])[tid] = 0;
     if (block_sees_error(&m->error)) {
@@ -152,6 +141,18 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
             if (lane == 0) s_cut[k] = lo;
         }
     };
+    // one thread: the old nodes of chunk c, whose cut is s_cut[k], into its stage
+    auto fetch = [&](uint32_t c, uint32_t k) {
+        const uint32_t xal = (min(c * kChunk, W) - s_cut[k]) & ~15u;
+        MergeStage& T = S.st[(c - c0) % kStages];
+        uint64_t* bar = &s_bar[(c - c0) % kStages];
+        mbar_arrive_expect_tx(bar, kMergeTile * 17u);
+        // the storage arrays are padded by more than a tile past the last node
+        bulk_g2s(T.keys, K0 + xal, kMergeTile * 8u, bar);
+        bulk_g2s(T.vals, V0 + xal, kMergeTile * 8u, bar);
+        bulk_g2s(T.meta, M0 + xal, kMergeTile, bar);
+    };
+    uint32_t live = 0;
     if (c1 > c0) {
         // the CTA's old positions [x0, x1)
         const uint32_t nc = min(kCuts, c1 - c0);
@@ -159,33 +160,50 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
         __syncthreads();
         const uint32_t x0 = d0 - s_cut[0];
         uint32_t x1 = d1 - s_cut[nc];
-        if (c1 - c0 > kCuts) {  // the last cut lies past the first group (found again below)
+        if (c1 - c0 > kCuts) {  // the last cut lies past the first group
+            const uint32_t first = s_cut[0];
             __syncthreads();
             find_cuts(c1, 1u);
             __syncthreads();
             x1 = d1 - s_cut[0];
+            __syncthreads();
+            if (tid == 0) s_cut[0] = first;
+            __syncthreads();
         }
-        uint32_t live = 0;
+        if (tid == 0)  // the first chunks arrive while the CTA counts and looks back
+            for (uint32_t k = 0; k < (uint32_t)kStages && c0 + k < c1; ++k) fetch(c0 + k, k);
         if (flagged) {
-            for (uint32_t b = (x0 & ~15u) + 16u * (uint32_t)tid; b < x1; b += 16u * kThreads) {
-                const uint4 mw = *reinterpret_cast<const uint4*>(M0 + b);
-                const uint32_t words[4] = {mw.x, mw.y, mw.z, mw.w};
+            for (uint32_t b = (x0 & ~15u) + 16u * (uint32_t)tid; b < x1; b += 64u * kThreads) {
+                uint4 mw[4];
 #pragma unroll
-                for (int k = 0; k < kPer; ++k) {
-                    const uint32_t mt = (words[k >> 2] >> (8 * (k & 3))) & 0xFFu;
-                    live += (b + k >= x0 && b + k < x1 && !(mt & kTomb)) ? 1u : 0u;
+                for (int u = 0; u < 4; ++u) {  // (bytes past x1 count as flagged)
+                    const uint32_t p = b + 16u * kThreads * (uint32_t)u;
+                    mw[u] = p < x1 ? *reinterpret_cast<const uint4*>(M0 + p) : make_uint4(~0u, ~0u, ~0u, ~0u);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t p = b + 16u * kThreads * (uint32_t)u;
+                    const uint32_t words[4] = {mw[u].x, mw[u].y, mw[u].z, mw[u].w};
+                    if (p >= x0 && p + 16u <= x1) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) live += (uint32_t)__popc(~words[k] & 0x80808080u);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            const uint32_t mt = (words[k >> 2] >> (8 * (k & 3))) & 0xFFu;
+                            live += (p + k >= x0 && p + k < x1 && !(mt & kTomb)) ? 1u : 0u;
+                        }
+                    }
                 }
             }
         } else if (tid == 0) {
             live = x1 - x0;
         }
-        live = __reduce_add_sync(0xffffffffu, live);
-        if (lane == 0) s_warp[warp] = live;
-    } else if (lane == 0) {
-        s_warp[warp] = 0u;
     }
+    live = __reduce_add_sync(0xffffffffu, live);
+    if (lane == 0) s_warp[warp] = live;
     __syncthreads();  // (also orders every thread's clears before warp 0's fence)
-    uint32_t live = 0;
+    live = 0;
 #pragma unroll
     for (int w = 0; w < kThreads / 32; ++w) live += s_warp[w];
     if (warp == 0) {
@@ -199,115 +217,165 @@ __global__ void __launch_bounds__(kThreads) k_merge(RebuildArgs a, uint32_t epoc
         }
     }
     __syncthreads();
-    if (s_fail) {  // this CTA will not arrive, so the batch has no last one
-        if (warp == 0) post_batch(a);
-        return;
-    }
     uint32_t lbase = s_pref;  // live old nodes before the chunk
-    for (uint32_t c = c0; c < c1; ++c) {
+    uint32_t landed = 0;      // chunks whose copies have been waited for
+#pragma unroll
+    for (int k = 0; k < kMergePer; ++k) S.off[0][(uint32_t)tid + k * kThreads] = 0u;
+    __syncthreads();
+    uint32_t fl_tile = 0;
+    bool fl = false;
+    auto flush = [&]() {  // the counts of the last chunk's two output tiles
+        if (!fl || tid >= 2 * kLevelSlots) return;
+        const uint32_t side = tid >= kLevelSlots ? 1u : 0u, l = (uint32_t)tid - side * kLevelSlots;
+        const uint32_t v = s_cnt[side][l];
+        if (v) {
+            atomicAdd(&a.lcnt[(size_t)(l - 2) * a.lstride + fl_tile + side], v);
+            s_cnt[side][l] = 0;
+        }
+    };
+    for (uint32_t c = c0; c < c1 && !s_fail; ++c) {
         const uint32_t ck = (c - c0) % kCuts;
-        if (ck == 0 && (c != c0 || c1 - c0 > kCuts)) {
+        if (ck == 0 && c != c0) {  // the next group's cuts; nothing is in flight here
             __syncthreads();
             find_cuts(c, min(kCuts, c1 - c) + 1u);
+            __syncthreads();
+            if (tid == 0)
+                for (uint32_t k = 0; k < (uint32_t)kStages && c + k < c1; ++k) fetch(c + k, k);
         }
-        for (uint32_t w = (uint32_t)tid; w < kNodes / 4; w += kThreads)
-            reinterpret_cast<uint4*>(s_off)[w] = make_uint4(0, 0, 0, 0);
-        __syncthreads();
+        uint32_t* off = S.off[(c - c0) & 1u];
+        uint32_t* off_next = S.off[((c - c0) & 1u) ^ 1u];
+        MergeStage& T = S.st[(c - c0) % kStages];
         const uint32_t da = c * kChunk, db = min(da + kChunk, W);
         const uint32_t ja = s_cut[ck], jb = s_cut[ck + 1], xa = da - ja, xb = db - jb;
         const uint32_t xal = xa & ~15u, sh = xa - xal, end = xb - xal;  // positions [sh, end) of the tile at xal
-        // the storage arrays are padded by a whole tile, so the 16-byte meta load stays in bounds
-        const uint32_t b0 = (uint32_t)tid * kPer;
-        const uint4 mw = *reinterpret_cast<const uint4*>(M0 + xal + b0);
-        // new nodes per insertion position, in [sh, end]
-        for (uint32_t j = ja + (uint32_t)tid; j < jb; j += kThreads) {
-            const uint32_t x = a.nn.loc[j] - xal;
-            if (x >= sh && x <= end) atomicAdd(&s_off[x], 1u);
-            else atomicOr(a.err, kErrBounds);
-        }
-        __syncthreads();
-        const uint32_t words[4] = {mw.x, mw.y, mw.z, mw.w};
-        uint32_t live_bits = 0, lc = 0, nc = 0;
-        uint32_t nat[kPer];
+        // the chunk's new nodes, kMergePer per thread: their insertion points, and whether each is
+        // the last one there
+        uint32_t nx[kMergePer], last = 0;
 #pragma unroll
-        for (int k = 0; k < kPer; ++k) {
-            const uint32_t mt = (words[k >> 2] >> (8 * (k & 3))) & 0xFFu;
-            const bool lv = b0 + k >= sh && b0 + k < end && !(mt & kTomb);
+        for (int k = 0; k < kMergePer; ++k) {
+            const uint32_t j = ja + (uint32_t)tid + k * kThreads;
+            nx[k] = j < jb ? a.nn.loc[j] - xal : ~0u;
+            if (j < jb && (j + 1u == jb || a.nn.loc[j + 1u] - xal != nx[k])) last |= 1u << k;
+            if (j < jb && (nx[k] < sh || nx[k] > end)) {
+                atomicOr(a.err, kErrBounds);
+                nx[k] = ~0u;
+            }
+        }
+        if (!mbar_wait_bounded(&s_bar[(c - c0) % kStages], ((c - c0) / kStages) & 1u, a.err)) s_fail = 1;
+#pragma unroll
+        for (int k = 0; k < kMergePer; ++k)
+            if (((last >> k) & 1u) && nx[k] != ~0u) off[nx[k]] = (uint32_t)tid + k * kThreads + 1u;
+        __syncthreads();
+        if (s_fail) break;
+        ++landed;
+        // every thread has left the chunk before: its stage and offsets are free
+        if (tid == 0 && ck > 0 && c + 1u < c1 && ck + 1u < kCuts) fetch(c + 1u, ck + 1u);
+#pragma unroll
+        for (int k = 0; k < kMergePer; ++k) off_next[(uint32_t)tid + k * kThreads] = 0u;
+        flush();  // the chunk before's counts; this one's are added two barriers later
+        const uint32_t b0 = (uint32_t)tid * kMergePer;
+        uint32_t live_bits = 0, nat[kMergePer], lc = 0, nm = 0;
+#pragma unroll
+        for (int k = 0; k < kMergePer; ++k) {
+            const bool lv = b0 + k >= sh && b0 + k < end && !(T.meta[b0 + k] & kTomb);
             live_bits |= (lv ? 1u : 0u) << k;
             lc += lv ? 1u : 0u;
-            nat[k] = s_off[b0 + k];
-            nc += nat[k];
+            nm = max(nm, off[b0 + k]);
+            nat[k] = nm;
         }
-        uint64_t tot;
-        const uint64_t ex = block_excl_sum64((uint64_t)lc | ((uint64_t)nc << 32), s_tmp, &tot);
-        {
-            uint32_t rl = (uint32_t)ex, rn = (uint32_t)(ex >> 32);
+        uint32_t il = lc, in = nm;  // sums of live nodes, maxima of the new nodes' numbers
 #pragma unroll
-            for (int k = 0; k < kPer; ++k) {
-                rn += nat[k];
-                s_off[b0 + k] = rl | (rn << 16);
-                rl += (live_bits >> k) & 1u;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, il, o), z = __shfl_up_sync(0xffffffffu, in, o);
+            if (lane >= o) {
+                il += y;
+                in = max(in, z);
             }
+        }
+        if (lane == 31) {
+            s_warp[warp] = il;
+            s_new[warp] = in;
+        }
+        uint32_t el = il - lc, en = __shfl_up_sync(0xffffffffu, in, 1);
+        if (lane == 0) en = 0;
+        __syncthreads();
+        uint32_t tot = 0;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) {
+            if (w < warp) {
+                el += s_warp[w];
+                en = max(en, s_new[w]);
+            }
+            tot += s_warp[w];
+        }
+#pragma unroll
+        for (int k = 0; k < kMergePer; ++k) {
+            off[b0 + k] = el | (max(en, nat[k]) << 16);
+            el += (live_bits >> k) & 1u;
         }
         __syncthreads();
         const uint32_t out = lbase + ja, tile0 = out / kNodes;
-        lbase += (uint32_t)tot;
+        lbase += tot;
         auto count = [&](uint32_t h, uint32_t o) {  // a node of a built level, at output o
             const uint32_t side = o / kNodes - tile0;  // a chunk's outputs lie in two tiles
             for (uint32_t l = lmin; l <= h; ++l) atomicAdd(&s_cnt[side & 1u][l], 1u);
         };
-        // striped pass: old live nodes, coalesced; four positions per round, their loads
-        // issued together (the source buffer is read-only here)
-        for (uint32_t p0 = (uint32_t)tid; p0 < end; p0 += 4u * kThreads) {
-            uint32_t mt[4];
-            uint64_t kv[4], vv[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t p = p0 + (uint32_t)u * kThreads;
-                const bool in = p >= sh && p < end;
-                mt[u] = in ? (uint32_t)__ldg(M0 + xal + p) : (uint32_t)kTomb;
-                kv[u] = in ? __ldg(K0 + xal + p) : 0ull;
-                vv[u] = in ? __ldg(V0 + xal + p) : 0ull;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (mt[u] & kTomb) continue;
-                const uint32_t v = s_off[p0 + (uint32_t)u * kThreads];
-                const uint32_t o = out + (v & 0xFFFFu) + (v >> 16);
-                if (o >= a.st_cap) {
-                    atomicOr(a.err, kErrBounds);
-                    continue;
-                }
-                K1[o] = kv[u];
-                V1[o] = vv[u];
-                M1[o] = (uint8_t)mt[u];
-                if (mt[u] >= lmin) count(mt[u], o);
-            }
-        }
-        // the chunk's new nodes, before the old node at their position
-        for (uint32_t j = ja + (uint32_t)tid; j < jb; j += kThreads) {
-            const uint32_t x = a.nn.loc[j] - xal;
-            if (x < sh || x > end) continue;  // recorded above
-            const uint32_t o = out + (s_off[x] & 0xFFFFu) + (j - ja);
+        for (int k = 0; k < kMergePer; ++k) {
+            const uint32_t p = (uint32_t)tid + k * kThreads;
+            const uint32_t mt = T.meta[p];
+            if (p < sh || p >= end || (mt & kTomb)) continue;
+            const uint32_t v = off[p];
+            const uint32_t o = out + (v & 0xFFFFu) + (v >> 16);
             if (o >= a.st_cap) {
                 atomicOr(a.err, kErrBounds);
                 continue;
             }
-            const uint32_t h = a.nn.height[j];
-            K1[o] = a.nn.keys[j];
-            V1[o] = a.nn.vals[j];
-            M1[o] = (uint8_t)h;
-            if (h >= lmin) count(h, o);
+            K1[o] = T.keys[p];
+            V1[o] = T.vals[p];
+            M1[o] = (uint8_t)mt;
+            if (mt >= lmin) count(mt, o);
         }
-        __syncthreads();
-        if (tid < 2 * kLevelSlots) {
-            const uint32_t side = tid >= kLevelSlots ? 1u : 0u, l = (uint32_t)tid - side * kLevelSlots;
-            const uint32_t v = s_cnt[side][l];
-            if (v) {
-                atomicAdd(&a.lcnt[(size_t)(l - 2) * a.lstride + tile0 + side], v);
-                s_cnt[side][l] = 0;
+        // the chunk's new nodes, before the old node at their position, their loads issued together
+        if (jb > ja) {
+            uint64_t kv[kMergePer], vv[kMergePer];
+            uint32_t hv[kMergePer];
+#pragma unroll
+            for (int k = 0; k < kMergePer; ++k) {
+                const uint32_t j = ja + (uint32_t)tid + k * kThreads;
+                const bool in = nx[k] != ~0u;
+                kv[k] = in ? a.nn.keys[j] : 0ull;
+                vv[k] = in ? a.nn.vals[j] : 0ull;
+                hv[k] = in ? a.nn.height[j] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < kMergePer; ++k) {
+                if (nx[k] == ~0u) continue;
+                const uint32_t o = out + (off[nx[k]] & 0xFFFFu) + (uint32_t)tid + k * kThreads;
+                if (o >= a.st_cap) {
+                    atomicOr(a.err, kErrBounds);
+                    continue;
+                }
+                K1[o] = kv[k];
+                V1[o] = vv[k];
+                M1[o] = (uint8_t)hv[k];
+                if (hv[k] >= lmin) count(hv[k], o);
             }
         }
+        // (s_cnt's adds: flushed after the next chunk's first barrier)
+        fl_tile = tile0;
+        fl = true;
+    }
+    __syncthreads();
+    flush();
+    if (s_fail) {  // this CTA will not arrive, so the batch has no last one; its copies land first
+        if (tid == 0)
+            for (uint32_t k = 0; k < (uint32_t)kStages && c0 + landed + k < c1; ++k) {
+                const uint32_t f = landed + k;
+                mbar_wait_bounded(&s_bar[f % kStages], (f / kStages) & 1u, a.err);
+            }
+        if (warp == 0) post_batch(a);
+        return;
     }
     if (tid == 0 && c1 > c0 && lbase - s_pref != live) atomicOr(a.err, kErrBounds);  // the two counts agree
     __syncthreads();  // every store of the CTA before its arrival is counted
@@ -767,9 +835,15 @@ __global__ void k_wait_selftest(uint64_t* desc, uint32_t* err) {
 }  // namespace
 
 cudaError_t launch_merge(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MergeSmem));
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
     const uint32_t chunks = a.size_ub / kChunk + 1;
-    const uint32_t cap = (uint32_t)num_sms * 5u;  // the CTAs resident at once
-    launch_dep(k_merge, chunks < cap ? chunks : cap, kThreads, 0, s, a, ++epoch);
+    const uint32_t cap = (uint32_t)num_sms * 4u;  // the CTAs resident at once
+    launch_dep(k_merge, chunks < cap ? chunks : cap, kThreads, sizeof(MergeSmem), s, a, ++epoch);
     ++g_launches;
     return cudaGetLastError();
 }
