@@ -16,6 +16,7 @@ constexpr uint32_t kSmemTopMax = 12288;  // index entries staged in shared memor
 constexpr uint32_t kPad = 64;           // readable entries past every array's end
 constexpr uint32_t kSortTile = 2048;    // elements per radix-sort tile (the smaller of two sizes)
 constexpr uint32_t kSortHist = 9 * 256; // digit counts of a radix sort
+constexpr uint32_t kSweepMost = 1u << 20;  // largest batch whose radix passes look back (see k_sort_count)
 constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the count kernel's scan
 constexpr uint32_t kCtrApply = 15;      // BatchMeta::tile_ctr slot: the apply kernel's tile counter
 constexpr uint32_t kApplyTile = 2048;   // sorted queries per apply tile
@@ -644,8 +645,12 @@ struct SortBuffers {
 // At most max_passes (1..8) digit passes run, on the most significant bytes that vary;
 // when more bytes vary, runs of equal sorted bytes are then ordered by the rest.
 // *hist_clear: whether sb.hist is zero already; on return, whether the sort leaves it so.
+// Without long_too, runs of more than 32 elements that need the rest are left and counted.
 cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
-                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear);
+                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear,
+                        bool long_too = true);
+// Orders the long segments that a sort without long_too has left (bm->fix_big counts their positions).
+cudaError_t launch_sort_long(uint32_t n, const SortBuffers& sb, BatchMeta* bm, cudaStream_t s);
 
 // Small batches (n <= kSmallSort): every tile of kRunTile queries sorted by (key, arrival)
 // on its own, into in_k / in_p (see k_tile_sort). Counts invalid queries into bm->invalid.

@@ -32,6 +32,7 @@ constexpr uint64_t kMinStorage = 1u << 16;
 
 struct Scratch {
     uint64_t cap = 0;  // queries
+    uint8_t* slab = nullptr;  // the allocation that the arrays are carved from (null: not owned)
     uint64_t* in_k = nullptr;
     uint32_t* in_p = nullptr;
     uint64_t* a_k = nullptr;
@@ -274,9 +275,8 @@ cudaError_t ensure_tile_cnt(pi_index* x, uint64_t st_cap) {
     const uint64_t stride = st_cap / 4096 + 2;
     if (stride <= x->lstride) return cudaSuccess;
     dfree(x->lcnt);
-    dfree(x->loff);
-    cudaError_t e = dalloc(&x->lcnt, 32 * stride);
-    if (e == cudaSuccess) e = dalloc(&x->loff, 32 * stride);
+    cudaError_t e = dalloc(&x->lcnt, 64 * stride);  // the offsets follow the counts
+    x->loff = e == cudaSuccess ? x->lcnt + 32 * stride : nullptr;
     if (e == cudaSuccess) e = cudaMemset(x->lcnt, 0, 32 * stride * sizeof(uint32_t));
     x->lstride = (e == cudaSuccess) ? (uint32_t)stride : 0u;
     x->force_rebuild = true;
@@ -304,67 +304,143 @@ uint32_t next_epochs(pi_index* x, uint32_t count, cudaStream_t s) {
     return x->epoch;
 }
 
+// The scratch of batches of up to q queries is one device allocation (an allocation or a release
+// costs the host far more than its use of one), carved in this order: first what the sort
+// needs, which is all that a bulk build takes.
+constexpr uint64_t al256(uint64_t b) { return (b + 255) & ~uint64_t(255); }
+
+constexpr uint64_t sort_bytes(uint64_t q) {
+    const uint64_t c = q + kPad, tiles = (q + kSortTile - 1) / kSortTile + 1, groups = tiles / kScanGroup + 1;
+    return 3 * al256(c * 8) + 3 * al256(c * 4)                    // in, a, b (keys, payload)
+           + 2 * al256(tiles * 256 * 4)                           // look-back words / digit counts, offsets
+           + al256((c / 32 + 1) * 4)                              // fixmap
+           + (q > kSweepMost ? al256(groups * 256 * 4) + al256(8 * (groups + 1) * 4) + al256(tiles * kSortTile + 16)
+                             : 0);                                // gsum, gctr, ndig
+}
+
+constexpr uint64_t scratch_bytes(uint64_t q) {
+    const uint64_t c = q + kPad, tiles = (q + kApplyTile - 1) / kApplyTile + 1;
+    return sort_bytes(q) + al256(c * 4) + al256(c) + al256(c * 8)  // loc, flags, val0
+           + 2 * al256(c * 8) + al256(c * 4) + al256(c)            // new nodes
+           + al256(c * 8) + al256(c * 4) + al256(c)                // level changes
+           + al256((2 * c + 64) * 8) + 2 * al256((2 * c + 64) * 4) + al256(2 * c + 64)  // lists
+           + 2 * al256(tiles * (kApplyTile / kApplyBlock) * 4) + al256(tiles * 4);      // heads, marks
+}
+
+struct Carver {
+    uint8_t* base;
+    uint64_t off = 0;
+    template <typename T>
+    void take(T*& p, uint64_t bytes) {
+        p = reinterpret_cast<T*>(base + off);
+        off += al256(bytes);
+    }
+};
+
+void carve_sort(Carver& v, uint64_t q, Scratch& s) {
+    const uint64_t c = q + kPad, tiles = (q + kSortTile - 1) / kSortTile + 1, groups = tiles / kScanGroup + 1;
+    v.take(s.in_k, c * 8); v.take(s.a_k, c * 8); v.take(s.b_k, c * 8);
+    v.take(s.in_p, c * 4); v.take(s.a_p, c * 4); v.take(s.b_p, c * 4);
+    v.take(s.sdesc[0], tiles * 256 * 4); v.take(s.sdesc[1], tiles * 256 * 4);
+    v.take(s.fixmap, (c / 32 + 1) * 4);
+    if (q > kSweepMost) {
+        v.take(s.gsum, groups * 256 * 4); v.take(s.gctr, 8 * (groups + 1) * 4); v.take(s.ndig, tiles * kSortTile + 16);
+    }
+}
+
+// Carves `base`; returns the bytes used (scratch_bytes(q)).
+uint64_t carve_scratch(uint8_t* base, uint64_t q, Scratch& s) {
+    Carver v{base};
+    const uint64_t c = q + kPad, tiles = (q + kApplyTile - 1) / kApplyTile + 1;
+    carve_sort(v, q, s);
+    v.take(s.loc, c * 4); v.take(s.flags, c); v.take(s.val0, c * 8);
+    v.take(s.nn.keys, c * 8); v.take(s.nn.vals, c * 8); v.take(s.nn.loc, c * 4); v.take(s.nn.height, c);
+    v.take(s.chg.keys, c * 8); v.take(s.chg.pos, c * 4); v.take(s.chg.hl, c);
+    s.lst_cap = 2 * c + 64;
+    v.take(s.lst_keys, s.lst_cap * 8); v.take(s.lst_pos, s.lst_cap * 4); v.take(s.lst_pref, s.lst_cap * 4);
+    v.take(s.lst_ins, s.lst_cap);
+    v.take(s.blk_head, tiles * (kApplyTile / kApplyBlock) * 4); v.take(s.blk_mark, tiles * (kApplyTile / kApplyBlock) * 4);
+    v.take(s.tile_mark, tiles * 4);
+    s.cap = q;
+    return v.off;
+}
+
 void free_scratch(Scratch& s) {
-    dfree(s.in_k); dfree(s.in_p); dfree(s.a_k); dfree(s.a_p); dfree(s.b_k); dfree(s.b_p);
-    dfree(s.loc); dfree(s.flags); dfree(s.val0);
-    dfree(s.nn.keys); dfree(s.nn.vals); dfree(s.nn.loc); dfree(s.nn.height);
-    dfree(s.sdesc[0]); dfree(s.sdesc[1]); dfree(s.fixmap);
-    dfree(s.gsum); dfree(s.gctr); dfree(s.ndig);
-    dfree(s.chg.keys); dfree(s.chg.pos); dfree(s.chg.hl);
-    dfree(s.lst_keys); dfree(s.lst_pos); dfree(s.lst_pref); dfree(s.lst_ins);
-    dfree(s.blk_head); dfree(s.blk_mark); dfree(s.tile_mark);
-    s.cap = 0;
+    dfree(s.slab);
+    s = Scratch{};
 }
 
 cudaError_t alloc_scratch(Scratch& s, uint64_t q) {
-    cudaError_t e = cudaSuccess;
-    const uint64_t c = q + kPad;
-#define PI_TRY(expr) do { e = (expr); if (e != cudaSuccess) { free_scratch(s); return e; } } while (0)
-    PI_TRY(dalloc(&s.in_k, c)); PI_TRY(dalloc(&s.in_p, c));
-    PI_TRY(dalloc(&s.a_k, c)); PI_TRY(dalloc(&s.a_p, c));
-    PI_TRY(dalloc(&s.b_k, c)); PI_TRY(dalloc(&s.b_p, c));
-    PI_TRY(dalloc(&s.loc, c)); PI_TRY(dalloc(&s.flags, c)); PI_TRY(dalloc(&s.val0, c));
-    PI_TRY(dalloc(&s.nn.keys, c)); PI_TRY(dalloc(&s.nn.vals, c));
-    PI_TRY(dalloc(&s.nn.loc, c)); PI_TRY(dalloc(&s.nn.height, c));
-    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
-    const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
-    PI_TRY(dalloc(&s.sdesc[0], stiles * 256)); PI_TRY(dalloc(&s.sdesc[1], stiles * 256));
-    const uint64_t sgroups = stiles / kScanGroup + 1;
-    PI_TRY(dalloc(&s.gsum, sgroups * 256)); PI_TRY(dalloc(&s.gctr, 8 * (sgroups + 1)));
-    PI_TRY(dalloc(&s.ndig, stiles * kSortTile + 16));
-    PI_TRY(dalloc(&s.fixmap, c / 32 + 1));
-    PI_TRY(dalloc(&s.chg.keys, c)); PI_TRY(dalloc(&s.chg.pos, c)); PI_TRY(dalloc(&s.chg.hl, c));
-    s.lst_cap = 2 * c + 64;
-    PI_TRY(dalloc(&s.lst_keys, s.lst_cap)); PI_TRY(dalloc(&s.lst_pos, s.lst_cap));
-    PI_TRY(dalloc(&s.lst_pref, s.lst_cap)); PI_TRY(dalloc(&s.lst_ins, s.lst_cap));
-    PI_TRY(dalloc(&s.blk_head, tiles * (kApplyTile / kApplyBlock)));
-    PI_TRY(dalloc(&s.blk_mark, tiles * (kApplyTile / kApplyBlock))); PI_TRY(dalloc(&s.tile_mark, tiles));
-#undef PI_TRY
-    s.cap = q;
+    uint8_t* slab = nullptr;
+    const cudaError_t e = dalloc(&slab, scratch_bytes(q));
+    if (e != cudaSuccess) return e;
+    if (carve_scratch(slab, q, s) != scratch_bytes(q)) {
+        dfree(slab);
+        return cudaErrorUnknown;
+    }
+    s.slab = slab;
     return cudaSuccess;
 }
 
-void free_storage(Storage& st) {
-    for (int i = 0; i < 2; ++i) {
-        dfree(st.keys[i]); dfree(st.vals[i]); dfree(st.meta[i]);
-    }
+// The sort's part alone, for a bulk build.
+cudaError_t alloc_sort_scratch(Scratch& s, uint64_t q) {
+    uint8_t* slab = nullptr;
+    const cudaError_t e = dalloc(&slab, sort_bytes(q));
+    if (e != cudaSuccess) return e;
+    Carver v{slab};
+    carve_sort(v, q, s);
+    s.slab = slab;
+    return cudaSuccess;
 }
 
 // Storage arrays are padded by a whole 4096-node tile plus kPad entries, so that tile
-// loads of the last (partial) tile and read-ahead past the sentinel stay in bounds.
+// loads of the last (partial) tile and read-ahead past the sentinel stay in bounds. Both
+// buffers are one allocation, which starts at keys[0].
 uint64_t storage_alloc(uint64_t cap) { return cap + 4096 + kPad; }
 
+void free_storage(Storage& st) {
+    dfree(st.keys[0]);
+    st = Storage{};
+}
+
 cudaError_t alloc_storage(Storage& st, uint64_t cap) {
-    cudaError_t e;
     const uint64_t c = storage_alloc(cap);
+    uint8_t* slab = nullptr;
+    cudaError_t e = dalloc(&slab, 4 * al256(c * 8) + 2 * al256(c));
+    if (e != cudaSuccess) return e;
+    Carver v{slab};
     for (int i = 0; i < 2; ++i) {
-        if ((e = dalloc(&st.keys[i], c)) != cudaSuccess) break;
-        if ((e = dalloc(&st.vals[i], c)) != cudaSuccess) break;
-        if ((e = dalloc(&st.meta[i], c)) != cudaSuccess) break;
-        cudaMemset(st.meta[i], 0, c);
+        v.take(st.keys[i], c * 8);
+        v.take(st.vals[i], c * 8);
     }
+    for (int i = 0; i < 2; ++i) v.take(st.meta[i], c);
+    e = cudaMemset(st.meta[0], 0, 2 * al256(c));
     if (e != cudaSuccess) free_storage(st);
     return e;
+}
+
+// The index layer's arrays, both buffers, in one allocation, which starts at lkeys.
+struct IndexArrays {
+    uint64_t *k0 = nullptr, *k1 = nullptr;
+    uint32_t *d0 = nullptr, *d1 = nullptr;
+};
+
+cudaError_t alloc_index(IndexArrays& x, uint64_t cap) {
+    const uint64_t c = cap + kPad;
+    uint8_t* slab = nullptr;
+    cudaError_t e = dalloc(&slab, 2 * al256(c * 8) + 2 * al256(c * 4));
+    if (e != cudaSuccess) return e;
+    Carver v{slab};
+    v.take(x.k0, c * 8); v.take(x.k1, c * 8);
+    v.take(x.d0, c * 4); v.take(x.d1, c * 4);
+    return cudaSuccess;
+}
+
+void use_index(pi_index* x, const IndexArrays& n) {
+    x->lkeys = n.k0;
+    x->ldown = n.d0;
+    x->lkeys1 = n.k1;
+    x->ldown1 = n.d1;
 }
 
 constexpr uint32_t kProfSlots = 2048;
@@ -430,8 +506,8 @@ void destroy(pi_index* x) {
     if (x->ds) cudaStreamDestroy(x->ds);
     if (x->ev_last) cudaEventDestroy(x->ev_last);
     free_storage(x->st);
-    dfree(x->lkeys); dfree(x->ldown); dfree(x->lkeys1); dfree(x->ldown1);
-    dfree(x->desc); dfree(x->lcnt); dfree(x->loff); dfree(x->wcount); dfree(x->d_meta); dfree(x->d_bm); dfree(x->d_hist); dfree(x->d_count);
+    dfree(x->lkeys);
+    dfree(x->desc); dfree(x->lcnt); dfree(x->wcount); dfree(x->d_meta);
     if (x->h_mbox) cudaFreeHost(x->h_mbox);
     if (x->ev_rebuilt) cudaEventDestroy(x->ev_rebuilt);
     if (x->rs) cudaStreamDestroy(x->rs);
@@ -541,36 +617,26 @@ cudaError_t grow_storage(pi_index* x, uint64_t need, cudaStream_t s) {
 
 cudaError_t grow_index(pi_index* x, uint64_t need, cudaStream_t s) {
     uint64_t cap = need + need / 4 + 4096;
-    uint64_t *nk = nullptr, *nk1 = nullptr;
-    uint32_t *nd = nullptr, *nd1 = nullptr;
-    cudaError_t e = dalloc(&nk, cap + kPad);
-    if (e == cudaSuccess) e = dalloc(&nd, cap + kPad);
-    if (e == cudaSuccess) e = dalloc(&nk1, cap + kPad);
-    if (e == cudaSuccess) e = dalloc(&nd1, cap + kPad);
-    if (e != cudaSuccess) {
-        dfree(nk); dfree(nd); dfree(nk1); dfree(nd1);
-        return e;
-    }
+    IndexArrays na;
+    cudaError_t e = alloc_index(na, cap);
+    if (e != cudaSuccess) return e;
     // the levels in use move to buffer 0 of the new arrays (called with `known` current)
     const uint64_t used = x->known.index_total;
     const uint64_t* ok = x->known.lcur ? x->lkeys1 : x->lkeys;
     const uint32_t* od = x->known.lcur ? x->ldown1 : x->ldown;
     if (ok && used) {
-        cudaMemcpyAsync(nk, ok, used * 8, cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(nd, od, used * 4, cudaMemcpyDeviceToDevice, s);
+        cudaMemcpyAsync(na.k0, ok, used * 8, cudaMemcpyDeviceToDevice, s);
+        cudaMemcpyAsync(na.d0, od, used * 4, cudaMemcpyDeviceToDevice, s);
     }
     const uint32_t zero = 0;
     cudaMemcpyAsync(&x->d_meta->lcur, &zero, sizeof(zero), cudaMemcpyHostToDevice, s);
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
-        dfree(nk); dfree(nd); dfree(nk1); dfree(nd1);
+        dfree(na.k0);
         return e;
     }
-    dfree(x->lkeys); dfree(x->ldown); dfree(x->lkeys1); dfree(x->ldown1);
-    x->lkeys = nk;
-    x->ldown = nd;
-    x->lkeys1 = nk1;
-    x->ldown1 = nd1;
+    dfree(x->lkeys);
+    use_index(x, na);
     x->known.lcur = 0;
     x->idx_cap = cap;
     x->force_rebuild = true;
@@ -629,53 +695,11 @@ RebuildArgs rebuild_args(pi_index* x, BatchMeta* bm, uint32_t size_ub, uint32_t 
 // ---------------------------------------------------------------------------------
 // Allocation-free batches (pi_execute_batch_noalloc): the per-batch scratch of up to
 // PI_NOALLOC_MAX_BATCH queries lives in one file-scope device array, carved into the
-// same buffers alloc_scratch() would allocate, in this order.
-constexpr uint64_t al256(uint64_t b) { return (b + 255) & ~uint64_t(255); }
-
-constexpr uint64_t noalloc_bytes(uint64_t q) {
-    const uint64_t c = q + kPad;
-    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
-    const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
-    return 3 * al256(c * 8) + 3 * al256(c * 4)                    // in, a, b (keys, payload)
-           + al256(c * 4) + al256(c) + al256(c * 8)               // loc, flags, val0
-           + 2 * al256(c * 8) + al256(c * 4) + al256(c)           // new nodes
-           + 2 * al256(stiles * 256 * 4)                          // sort look-back words
-           + al256((c / 32 + 1) * 4)                              // fixmap
-           + al256(c * 8) + al256(c * 4) + al256(c)               // level changes
-           + al256((2 * c + 64) * 8) + 2 * al256((2 * c + 64) * 4) + al256(2 * c + 64)  // lists
-           + 2 * al256(tiles * (kApplyTile / kApplyBlock) * 4) + al256(tiles * 4);  // heads, marks
-}
-
-constexpr uint64_t kNoAllocBytes = noalloc_bytes(PI_NOALLOC_MAX_BATCH);
+// same buffers as an index's own scratch.
+constexpr uint64_t kNoAllocBytes = scratch_bytes(PI_NOALLOC_MAX_BATCH);
 
 // Shared by every call on a device; each GPU that loads the library holds it until exit.
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes];
-
-// Carves `base` like noalloc_bytes(q); returns the bytes used.
-uint64_t carve_scratch(uint8_t* base, uint64_t q, Scratch& s) {
-    uint64_t off = 0;
-    auto take = [&](auto*& ptr, uint64_t bytes) {
-        ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(base + off);
-        off += al256(bytes);
-    };
-    const uint64_t c = q + kPad;
-    const uint64_t tiles = (q + kApplyTile - 1) / kApplyTile + 1;
-    const uint64_t stiles = (q + kSortTile - 1) / kSortTile + 1;
-    take(s.in_k, c * 8); take(s.a_k, c * 8); take(s.b_k, c * 8);
-    take(s.in_p, c * 4); take(s.a_p, c * 4); take(s.b_p, c * 4);
-    take(s.loc, c * 4); take(s.flags, c); take(s.val0, c * 8);
-    take(s.nn.keys, c * 8); take(s.nn.vals, c * 8); take(s.nn.loc, c * 4); take(s.nn.height, c);
-    take(s.sdesc[0], stiles * 256 * 4); take(s.sdesc[1], stiles * 256 * 4);
-    take(s.fixmap, (c / 32 + 1) * 4);
-    take(s.chg.keys, c * 8); take(s.chg.pos, c * 4); take(s.chg.hl, c);
-    s.lst_cap = 2 * c + 64;
-    take(s.lst_keys, s.lst_cap * 8); take(s.lst_pos, s.lst_cap * 4); take(s.lst_pref, s.lst_cap * 4);
-    take(s.lst_ins, s.lst_cap);
-    take(s.blk_head, tiles * (kApplyTile / kApplyBlock) * 4);
-    take(s.blk_mark, tiles * (kApplyTile / kApplyBlock) * 4); take(s.tile_mark, tiles * 4);
-    s.cap = q;
-    return off;
-}
 
 // Per device: the array's device address, looked up once with that device current, and
 // the hand-over between calls on different indices. A batch's index-layer rebuild runs
@@ -866,6 +890,9 @@ int enqueue_batch(pi_index* x, const Scratch& sc, const uint8_t* ops, const uint
 
 }  // namespace
 
+// Positions in long prefix segments up to which a bulk build orders them segment by segment.
+constexpr uint32_t kCreateLong = 1u << 15;
+
 extern "C" {
 
 int pi_last_error(void) { return g_last_error; }
@@ -950,13 +977,20 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
             if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) break;
         if (e != cudaSuccess) break;
         if ((e = cudaMallocHost(reinterpret_cast<void**>(&x->h_mbox), kRing * sizeof(DevMeta))) != cudaSuccess) break;
-        if ((e = dalloc(&x->d_meta, 1)) != cudaSuccess) break;
-        if ((e = dalloc(&x->d_bm, 2)) != cudaSuccess) break;
+        {  // the small device state, one allocation that starts at d_meta
+            uint8_t* slab = nullptr;
+            if ((e = dalloc(&slab, al256(sizeof(DevMeta)) + al256(2 * sizeof(BatchMeta)) + al256((kSortHist + 256) * 4) + 256)) !=
+                cudaSuccess)
+                break;
+            Carver v{slab};
+            v.take(x->d_meta, sizeof(DevMeta));
+            v.take(x->d_bm, 2 * sizeof(BatchMeta));
+            v.take(x->d_hist, (kSortHist + 256) * 4);
+            v.take(x->d_count, 256);
+        }
         if ((e = cudaStreamCreateWithFlags(&x->rs, cudaStreamNonBlocking)) != cudaSuccess) break;
         if ((e = cudaEventCreateWithFlags(&x->ev_rebuilt, cudaEventDisableTiming)) != cudaSuccess) break;
         if ((e = cudaEventCreateWithFlags(&x->ev_last, cudaEventDisableTiming)) != cudaSuccess) break;
-        if ((e = dalloc(&x->d_hist, kSortHist + 256)) != cudaSuccess) break;
-        if ((e = dalloc(&x->d_count, 1)) != cudaSuccess) break;
         cudaMemsetAsync(x->d_meta, 0, sizeof(DevMeta), s);
         cudaMemsetAsync(x->d_bm, 0, 2 * sizeof(BatchMeta), s);
         if ((e = alloc_storage(x->st, st_cap)) != cudaSuccess) break;
@@ -966,16 +1000,28 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         if ((e = ensure_desc(x, desc_need(n, st_cap))) != cudaSuccess) break;
         // 1. sort (key, arrival) and keep the last of every key run
         if (n > 0) {
-            if ((e = alloc_scratch(tmp, n)) != cudaSuccess) break;
+            if ((e = alloc_sort_scratch(tmp, n)) != cudaSuccess) break;
             SortBuffers sb = sort_buffers(x, tmp);
             uint32_t ep = next_epochs(x, 16, s);
-            if ((e = launch_sort(nullptr, keys, (uint32_t)n, sb, x->d_bm, &x->d_meta->error, s, x->num_sms, 8,
-                                 &x->hist_clear)) != cudaSuccess)
-                break;
-            x->epoch = ep;
+            // Four passes on the most significant varying bytes order all but prefix collisions,
+            // and of those the short ones are ordered with them. Long ones (keys that share
+            // leading bytes, or a repeated key beside another of its prefix) are counted first:
+            // one CTA would order each, so many of them take the other passes instead.
             BatchMeta hbm;
-            if ((e = cudaMemcpyAsync(&hbm, x->d_bm, sizeof(BatchMeta), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
-            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
+            auto sort_pairs = [&](int passes, bool long_too) {
+                if ((e = launch_sort(nullptr, keys, (uint32_t)n, sb, x->d_bm, &x->d_meta->error, s, x->num_sms, passes,
+                                     &x->hist_clear, long_too)) != cudaSuccess)
+                    return false;
+                if ((e = cudaMemcpyAsync(&hbm, x->d_bm, sizeof(BatchMeta), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return false;
+                return (e = cudaStreamSynchronize(s)) == cudaSuccess;
+            };
+            if (!sort_pairs(4, false)) break;
+            x->epoch = ep;
+            if (!hbm.invalid && hbm.fix_big > kCreateLong) {
+                if ((e = cudaMemsetAsync(x->d_bm, 0, sizeof(BatchMeta), s)) != cudaSuccess || !sort_pairs(8, true)) break;
+            } else if (hbm.fix_big) {
+                if ((e = launch_sort_long((uint32_t)n, sb, x->d_bm, s)) != cudaSuccess) break;
+            }
             if (hbm.invalid) {
                 rc = PI_ERR_INVALID_ARG;
                 break;
@@ -1003,10 +1049,9 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
             if (hm.cnt[l]) need += (uint64_t)hm.cnt[l] + 1;
         uint64_t icap = need + need / 4 + 4096;
         if (cfg && cfg->index_capacity) icap = cfg->index_capacity;
-        if ((e = dalloc(&x->lkeys, icap + kPad)) != cudaSuccess) break;
-        if ((e = dalloc(&x->ldown, icap + kPad)) != cudaSuccess) break;
-        if ((e = dalloc(&x->lkeys1, icap + kPad)) != cudaSuccess) break;
-        if ((e = dalloc(&x->ldown1, icap + kPad)) != cudaSuccess) break;
+        IndexArrays la;
+        if ((e = alloc_index(la, icap)) != cudaSuccess) break;
+        use_index(x, la);
         x->idx_cap = icap;
         // 2. lay out and build the index layer
         cudaMemsetAsync(x->d_bm, 0, sizeof(BatchMeta), s);
@@ -1367,6 +1412,10 @@ int pi_export(pi_index_t* x, uint64_t* keys_out, uint64_t* vals_out, uint64_t ca
     cudaError_t e = sync_known(x, s);
     if (e != cudaSuccess) return map_cuda(e);
     if (int rc = sticky_error(x->known)) return rc;
+    if (cap == 0) {  // only the count, which the host has just read
+        *n_out_host = x->known.cnt[1];
+        return PI_OK;
+    }
     cudaMemsetAsync(x->d_count, 0, sizeof(uint32_t), s);
     x->bm_clear = false;  // block 0 may be the next batch's
     cudaMemsetAsync(&x->d_bm->tile_ctr[12], 0, sizeof(uint32_t), s);

@@ -42,7 +42,6 @@ static_assert(kTile == kSortTile, "tile size shared with the host's sizing");
 // in the plan kernel.
 constexpr uint32_t kUsualByte = 4;
 constexpr uint32_t kUsualRow = 8;         // its row of the counts (rows 0 .. 7: the passes')
-constexpr uint32_t kSweepMost = 1u << 20;   // largest batch whose passes look back (see k_sort_count)
 constexpr uint32_t kLargeTiles = 1u << 19;  // from here on, their tiles hold 4096 elements instead of 2048
 
 __device__ __forceinline__ uint32_t usual_digit(uint64_t k) { return (uint32_t)(k >> (8u * kUsualByte)) & 255u; }
@@ -803,7 +802,7 @@ __device__ void cta_segment_smem(uint32_t s, uint32_t e, const SortPlan& P, cons
 // positions) and takes the segments that start there. A warp orders a segment of at
 // most 32 queries: rank = queries with a smaller key, or the same key and an earlier
 // position. Longer segments are queued for the whole CTA.
-__global__ void __launch_bounds__(kThreads) k_sort_fix(uint32_t n, SortBuffers sb, BatchMeta* bm) {
+__global__ void __launch_bounds__(kThreads) k_sort_fix(uint32_t n, SortBuffers sb, BatchMeta* bm, bool long_too) {
     pdl_wait();
     pdl_trigger();
     const SortPlan& P = bm->plan;
@@ -899,6 +898,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_fix(uint32_t n, SortBuffers s
             }
         }
         __syncthreads();
+        if (!long_too) continue;
         if (s_end - s <= (uint32_t)kTile)
             cta_segment_smem(s, s_end, P, sb, reinterpret_cast<uint64_t*>(s_list), s_pay, s_whist, s_base, s_tmp);
         else
@@ -1067,7 +1067,8 @@ static cudaError_t launch_count_passes(uint32_t n, const SortBuffers& sb, BatchM
 }
 
 cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
-                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear) {
+                        BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear,
+                        bool long_too) {
     if (n == 0) return cudaSuccess;
     if (max_passes < 1 || max_passes > 8) return cudaErrorInvalidValue;
     const bool sweep = n <= kSweepMost, large = n >= kLargeTiles;
@@ -1094,9 +1095,16 @@ cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, co
         launch_dep(k_sort_find, fgrid, 256, 0, s, n, sb, bm, sweep);
         ++g_launches;
         if (sweep) *hist_clear = true;
-        launch_dep(k_sort_fix, (n + kFixSlice - 1) / kFixSlice, kThreads, 0, s, n, sb, bm);
+        launch_dep(k_sort_fix, (n + kFixSlice - 1) / kFixSlice, kThreads, 0, s, n, sb, bm, long_too);
         ++g_launches;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sort_long(uint32_t n, const SortBuffers& sb, BatchMeta* bm, cudaStream_t s) {
+    // the short segments are in order already: ordering them again changes nothing
+    launch_dep(k_sort_fix, (n + kFixSlice - 1) / kFixSlice, kThreads, 0, s, n, sb, bm, true);
+    ++g_launches;
     return cudaGetLastError();
 }
 
