@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstddef>
 #include <cstring>
+#include <deque>
 #include <mutex>
 #include <string>
 #include <new>
@@ -169,12 +170,18 @@ struct pi_index {
     // ev[b % kRing] marks the batch's end; the newest completed slot bounds the host's view of the sizes.
     DevMeta* h_mbox = nullptr;  // pinned, kRing slots
     cudaEvent_t ev[64] = {};
-    uint64_t ring_n[64] = {};   // queries of the batch in each slot
+    uint64_t ring_op[64] = {};  // the operation that each slot's batch is
     uint64_t issued = 0;        // batches issued
     uint64_t seen = 0;          // batches whose mailbox has been read (a prefix)
     DevMeta known{};       // last mailbox snapshot
-    uint64_t pending_n = 0;  // queries issued after that snapshot
-    uint64_t extra_n = 0;    // queries of batching-form calls since the last full sync
+    // Operations (batches and batching-form calls) are numbered; `known` is the device meta after
+    // operation known_op, and the later ones may add as many nodes as they have queries.
+    struct Op {
+        uint64_t id, n;
+    };
+    std::deque<Op> ops;      // those after known_op
+    uint64_t op_count = 0, known_op = 0;
+    uint64_t pending_n = 0;  // their queries
     bool force_rebuild = false;
     bool bm_clear = false;   // the next batch's counters are zero (the last batch cleared them)
     // With small_mode 1, small batches (Q <= kSmallBatch on at most kSmallIndex nodes) run
@@ -539,16 +546,31 @@ cudaError_t read_meta(pi_index* x, cudaStream_t s, DevMeta* out) {
 
 constexpr uint64_t kRing = 64;
 
+// Numbers an operation of n queries that is being issued.
+uint64_t note_op(pi_index* x, uint64_t n) {
+    x->ops.push_back({++x->op_count, n});
+    x->pending_n += n;
+    return x->op_count;
+}
+
+// Takes the device meta as operation `op` left it, unless a later operation's is known already.
+void adopt(pi_index* x, const DevMeta& m, uint64_t op) {
+    if (op <= x->known_op) return;
+    x->known = m;
+    x->known_op = op;
+    while (!x->ops.empty() && x->ops.front().id <= op) {
+        x->pending_n -= x->ops.front().n;
+        x->ops.pop_front();
+    }
+}
+
 // Non-blocking: adopt the newest completed batch's mailbox. Batches complete in order, so the
 // events are asked from the oldest on: one that is not ready, and one per batch since.
 void refresh_known(pi_index* x) {
     uint64_t newest = x->seen;
-    while (newest < x->issued && cudaEventQuery(x->ev[newest % kRing]) == cudaSuccess) {
-        x->pending_n -= x->ring_n[newest % kRing];
-        ++newest;
-    }
+    while (newest < x->issued && cudaEventQuery(x->ev[newest % kRing]) == cudaSuccess) ++newest;
     if (newest == x->seen) return;
-    x->known = x->h_mbox[(newest - 1) % kRing];
+    adopt(x, x->h_mbox[(newest - 1) % kRing], x->ring_op[(newest - 1) % kRing]);
     x->seen = newest;
 }
 
@@ -577,8 +599,9 @@ cudaError_t sync_known(pi_index* x, cudaStream_t s) {
     if (e == cudaSuccess) {
         for (uint64_t b = x->seen; b < x->issued; ++b) cudaEventSynchronize(x->ev[b % kRing]);
         x->seen = x->issued;
+        x->known_op = x->op_count;
+        x->ops.clear();
         x->pending_n = 0;
-        x->extra_n = 0;
     }
     return e;
 }
@@ -871,9 +894,8 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     x->epoch = ep;
     x->force_rebuild = false;
     x->bm_clear = true;
-    x->ring_n[slot] = n;
+    x->ring_op[slot] = note_op(x, n);
     x->issued++;
-    x->pending_n += n;
     mark_last(x, s, x->ev[slot]);
     return map_cuda(cudaGetLastError());
 }
@@ -1098,7 +1120,7 @@ int pi_execute_batch(pi_index_t* x, const uint8_t* ops, const uint64_t* keys, co
     if (int rc = sticky_error(x->known)) return rc;
     // capacities (grow rarely; growing synchronises the stream)
     if (n > x->sc.cap && (e = grow_scratch(x, n, s)) != cudaSuccess) return map_cuda(e);
-    uint64_t size_ub = (uint64_t)x->known.size + x->pending_n + x->extra_n + n;
+    uint64_t size_ub = (uint64_t)x->known.size + x->pending_n + n;
     if (size_ub > x->st_cap) {
         if ((e = sync_known(x, s)) != cudaSuccess) return map_cuda(e);
         if (int rc = sticky_error(x->known)) return rc;
@@ -1240,7 +1262,7 @@ int pi_execute_batch_noalloc(pi_index_t* x, const uint8_t* ops, const uint64_t* 
     order_after_last(x, s);
     refresh_known(x);
     if (int rc = sticky_error(x->known)) return rc;
-    uint64_t size_ub = (uint64_t)x->known.size + x->pending_n + x->extra_n + n;
+    uint64_t size_ub = (uint64_t)x->known.size + x->pending_n + n;
     if (size_ub > x->st_cap) {
         if ((e = sync_known(x, s)) != cudaSuccess) return map_cuda(e);
         if (int rc = sticky_error(x->known)) return rc;
@@ -1494,7 +1516,11 @@ struct pi_multi {
     std::vector<MIndex> h_idx;
     pi_multi_config_t cfg{};
     MIndex* d_idx = nullptr;
+    // The indices' metas as the last call left them, and pinned copies of them per call parity,
+    // with the operation that the call was for each of its indices
     DevMeta* d_mirror = nullptr;
+    DevMeta* h_mirror[2] = {};
+    std::vector<std::pair<uint32_t, uint64_t>> call_ops[2];
     uint8_t* d_q = nullptr;
     uint8_t* h_q[2] = {};
     uint64_t q_bytes = 0;
@@ -1543,11 +1569,20 @@ void multi_free_graphs(pi_multi* mx) {
     mx->graph_valid = false;
 }
 
+// Takes over what the call of parity p, which has finished, left of its indices.
+void multi_adopt(pi_multi* mx, int p) {
+    for (const auto& c : mx->call_ops[p]) adopt(mx->idx[c.first], mx->h_mirror[p][c.first], c.second);
+    mx->call_ops[p].clear();
+}
+
 void multi_destroy(pi_multi* mx) {
     if (!mx) return;
     cudaSetDevice(mx->device);
-    for (int p = 0; p < 2; ++p)
+    for (uint64_t k = 0; k < 2; ++k) {  // the older call first
+        const int p = (int)((mx->calls + k) & 1u);
         if (mx->q_free[p]) cudaEventSynchronize(mx->q_free[p]);
+        multi_adopt(mx, p);
+    }
     for (pi_index* x : mx->idx)  // the calls are complete: forget the set's event
         if (x->last_ev == mx->ev_done) x->has_last = false;
     if (mx->ev_done) cudaEventDestroy(mx->ev_done);
@@ -1556,6 +1591,8 @@ void multi_destroy(pi_multi* mx) {
     dfree(mx->d_mirror);
     dfree(mx->d_q);
     for (auto& h : mx->h_q)
+        if (h) cudaFreeHost(h);
+    for (auto& h : mx->h_mirror)
         if (h) cudaFreeHost(h);
     for (auto& sc : mx->scratch) dfree(sc);
     for (auto& e : mx->q_free)
@@ -1610,6 +1647,7 @@ cudaError_t multi_build_graphs(pi_multi* mx) {
             cudaEventRecord(mx->evj[c], mx->ls[c]);
             cudaStreamWaitEvent(mx->cs, mx->evj[c], 0);
         }
+        cudaMemcpyAsync(mx->h_mirror[p], mx->d_mirror, count * sizeof(DevMeta), cudaMemcpyDeviceToHost, mx->cs);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(mx->cs, &g);
         if (e == cudaSuccess && le != cudaSuccess) e = le;
@@ -1698,6 +1736,7 @@ pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi
         for (int p = 0; p < 2; ++p) {
             if ((e = cudaMallocHost(reinterpret_cast<void**>(&mx->h_q[p]), mx->q_bytes)) != cudaSuccess) break;
             std::memset(mx->h_q[p], 0, mx->q_bytes);
+            if ((e = cudaMallocHost(reinterpret_cast<void**>(&mx->h_mirror[p]), count * sizeof(DevMeta))) != cudaSuccess) break;
             if ((e = cudaEventCreateWithFlags(&mx->q_free[p], cudaEventDisableTiming)) != cudaSuccess) break;
         }
         if (e != cudaSuccess) break;
@@ -1763,32 +1802,35 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
         seen[q.index] = 1;
     }
     cudaError_t e;
+    // The call before the last has to have finished (its queue buffer is reused): from it, and
+    // from the last one if that has finished too, the host takes its indices' sizes.
+    const int p = (int)(mx->calls & 1u);
+    if ((e = cudaEventSynchronize(mx->q_free[p])) != cudaSuccess) return map_cuda(e);
+    multi_adopt(mx, p);
+    if (cudaEventQuery(mx->q_free[p ^ 1]) == cudaSuccess) multi_adopt(mx, p ^ 1);
     // Capacities: every index must hold its batch's new keys without growing in the
-    // kernel. Growing (rare) synchronises the stream, as in pi_execute_batch.
+    // kernel. Growing (rare) synchronises the stream, as in pi_execute_batch; an index that
+    // comes near gets room for the calls that may be in flight, so that the next calls need
+    // no synchronisation to be sure of it.
     bool idx_changed = false;
     for (uint32_t i = 0; i < nb; ++i) {
         pi_index* x = mx->idx[b[i].index];
         refresh_known(x);
         if (int rc = sticky_error(x->known)) return rc;
         const uint64_t n = b[i].n;
-        uint64_t size_ub = (uint64_t)x->known.size + x->pending_n + x->extra_n + n;
-        bool grew = false;
+        uint64_t size_ub = (uint64_t)x->known.size + x->pending_n + n;
         if (size_ub > x->st_cap || x->known.grow_request) {
             if ((e = sync_known(x, s)) != cudaSuccess) return map_cuda(e);
             if (int rc = sticky_error(x->known)) return rc;
             size_ub = (uint64_t)x->known.size + n;
             if (size_ub > PI_MAX_KEYS) return PI_ERR_INVALID_ARG;
-            if (size_ub > x->st_cap) {
-                if ((e = grow_storage(x, size_ub, s)) != cudaSuccess) return map_cuda(e);
-                grew = true;
-            }
+            const uint64_t room = std::min<uint64_t>(size_ub + 2 * n, PI_MAX_KEYS);
+            if (room > x->st_cap && (e = grow_storage(x, room, s)) != cudaSuccess && size_ub > x->st_cap) return map_cuda(e);
             if (x->known.grow_request && x->known.index_need + 64ull > x->idx_cap) {
                 if ((e = grow_index(x, x->known.index_need, s)) != cudaSuccess) return map_cuda(e);
-                grew = true;
             }
             x->known.grow_request = 0;
         }
-        (void)grew;
         // The single-index path may have grown this index's arrays since the set last
         // looked (a plain batch with new keys): the device table must hold the arrays in
         // use, never freed ones.
@@ -1810,7 +1852,7 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
     for (uint32_t i = 0; i < nb; ++i) {
         if (b[i].n == 0) continue;
         const pi_index* x = mx->idx[b[i].index];
-        const uint64_t nodes = (uint64_t)x->known.size + x->pending_n + x->extra_n;
+        const uint64_t nodes = (uint64_t)x->known.size + x->pending_n;
         const int c = class_of(mx, nodes);
         per[c].push_back({nodes + 8 * b[i].n, i});
         if (b[i].n > need_q[c]) need_q[c] = (uint32_t)b[i].n;
@@ -1834,8 +1876,6 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
         rebuild_graphs = true;
     }
     if (rebuild_graphs && (e = multi_build_graphs(mx)) != cudaSuccess) return map_cuda(e);
-    const int p = (int)(mx->calls & 1u);
-    if ((e = cudaEventSynchronize(mx->q_free[p])) != cudaSuccess) return map_cuda(e);
     uint32_t* hdr = reinterpret_cast<uint32_t*>(mx->h_q[p]);
     MItem* items = reinterpret_cast<MItem*>(mx->h_q[p] + kQHeader);
     for (uint32_t c = 0; c < PI_MULTI_MAX_CLASSES; ++c) {
@@ -1871,9 +1911,8 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
         }
         cudaMemcpyAsync(&x->h_mbox[slot], x->d_meta, sizeof(DevMeta), cudaMemcpyDeviceToHost, s);
         cudaEventRecord(x->ev[slot], s);
-        x->ring_n[slot] = b[0].n;
+        x->ring_op[slot] = note_op(x, b[0].n);
         x->issued++;
-        x->pending_n += b[0].n;
         x->force_rebuild = true;  // the plain path recounts its per-tile level counts
         x->bm_clear = false;      // the counters' parity moved on
         x->launches += mx->launches;
@@ -1883,7 +1922,7 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
     }
     for (uint32_t i = 0; i < nb; ++i) {
         pi_index* x = mx->idx[b[i].index];
-        x->extra_n += b[i].n;
+        if (b[i].n) mx->call_ops[p].push_back({b[i].index, note_op(x, b[i].n)});
         x->force_rebuild = true;  // the plain path recounts its per-tile level counts
         x->last_ev = mx->ev_done;  // recorded once for the call, below
         x->last_stream = s;
