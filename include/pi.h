@@ -185,7 +185,7 @@ int pi_execute_batch_host(pi_index_t* idx, const uint8_t* ops_host, const uint64
  * allocator (cudaMalloc/cudaFree can synchronise the device, which a latency-bound
  * serving loop cannot afford) and code running where a memory budget is fixed up front.
  * The per-batch scratch of up to PI_NOALLOC_MAX_BATCH queries comes from one
- * file-scope device array of a fixed size (about 7.8 MB), held by
+ * file-scope device array of a fixed size (about 7.4 MB), held by
  * every GPU that loads the library until the process exits; this call allocates nothing.
  *   - n > PI_NOALLOC_MAX_BATCH returns PI_ERR_INVALID_ARG.
  *   - A batch that could need the storage layer to grow returns PI_ERR_OOM with the

@@ -175,16 +175,36 @@ def load_library(path: str = LIB_PATH):
     return lib
 
 
-def _stream_handle(stream=None):
+# torch, imported on first use (the module itself does not need it). A call of the smallest
+# batches is bound by host time, so the calls look nothing up twice.
+_torch = None
+
+
+def _load_torch():
+    global _torch
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    _torch = torch
+    return torch
+
+
+def _stream_handle(stream=None):
+    if stream is None:
+        stream = (_torch or _load_torch()).cuda.current_stream()
+    return ctypes.c_void_p(stream.cuda_stream)
 
 
 def _check_dev(t, dtype, name):
-    import torch
     if not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous CUDA tensor of {dtype}")
+
+
+def _check_batch(torch, ops, keys, vals):
+    i64 = torch.int64
+    if not (ops.is_cuda and keys.is_cuda and vals.is_cuda and ops.dtype == torch.uint8 and keys.dtype == i64 and
+            vals.dtype == i64 and ops.is_contiguous() and keys.is_contiguous() and vals.is_contiguous()):
+        _check_dev(ops, torch.uint8, "ops")
+        _check_dev(keys, i64, "keys")
+        _check_dev(vals, i64, "vals")
 
 
 def _chk(rc: int, what: str):
@@ -250,11 +270,9 @@ class Index:
     def execute(self, ops, keys, vals, results=None, stream=None):
         """pi_execute_batch on device tensors; returns results as int64 [n, 2]:
         column 0 = value bits, column 1 = status (low 32 bits)."""
-        import torch
+        torch = _torch or _load_torch()
         n = ops.numel()
-        _check_dev(ops, torch.uint8, "ops")
-        _check_dev(keys, torch.int64, "keys")
-        _check_dev(vals, torch.int64, "vals")
+        _check_batch(torch, ops, keys, vals)
         if keys.numel() != n or vals.numel() != n:
             raise ValueError("ops, keys and vals differ in length")
         if results is None:
@@ -266,10 +284,8 @@ class Index:
 
     def execute_noalloc(self, ops, keys, vals, results, stream=None):
         """pi_execute_batch_noalloc: device tensors; `results` (int64 [n, 2]) must exist."""
-        import torch
-        _check_dev(ops, torch.uint8, "ops")
-        _check_dev(keys, torch.int64, "keys")
-        _check_dev(vals, torch.int64, "vals")
+        torch = _torch or _load_torch()
+        _check_batch(torch, ops, keys, vals)
         _check_dev(results, torch.int64, "results")
         rc = self.lib.pi_execute_batch_noalloc(self._h, ops.data_ptr(), keys.data_ptr(), vals.data_ptr(),
                                                ops.numel(), results.data_ptr(), _stream_handle(stream))

@@ -66,7 +66,7 @@ struct SortPlan {
     uint64_t pmask;   // the key bytes the passes sort
     uint32_t npass;
     uint32_t digit[8];
-    uint32_t src[8];  // 0 = packed input, 1 = buffer A, 2 = buffer B
+    uint32_t src[8];  // 0 = the caller's queries, 1 = buffer A, 2 = buffer B
     uint32_t dst[8];
     uint32_t fix;     // 1: segments of equal pmask bytes still need ordering by the full key
     uint32_t nr;      // the other bytes that can differ inside a segment, ascending in rdig
@@ -622,8 +622,10 @@ __device__ __forceinline__ uint32_t block_excl_max(uint32_t v, uint32_t* warp_tm
 // ---------------------------------------------------------------------------------
 // Host-side launch wrappers (defined in the .cu files).
 struct SortBuffers {
-    uint64_t* in_k;  // packed keys (written by the pack kernel)
-    uint32_t* in_p;  // packed payload: op << 30 | arrival index
+    const uint8_t* ops;    // the caller's queries (launch_sort sets them; ops may be null: all searches)
+    const uint64_t* keys;
+    uint64_t* in_k;  // small batches: the tiles of queries, each sorted on its own
+    uint32_t* in_p;  // payload: op << 30 | arrival index
     uint64_t* a_k;
     uint32_t* a_p;
     uint64_t* b_k;

@@ -318,7 +318,8 @@ constexpr uint64_t al256(uint64_t b) { return (b + 255) & ~uint64_t(255); }
 
 constexpr uint64_t sort_bytes(uint64_t q) {
     const uint64_t c = q + kPad, tiles = (q + kSortTile - 1) / kSortTile + 1, groups = tiles / kScanGroup + 1;
-    return 3 * al256(c * 8) + 3 * al256(c * 4)                    // in, a, b (keys, payload)
+    const uint64_t in = std::min<uint64_t>(q, kSmallSort) + kPad;
+    return al256(in * 8) + al256(in * 4) + 2 * al256(c * 8) + 2 * al256(c * 4)  // in, a, b (keys, payload)
            + 2 * al256(tiles * 256 * 4)                           // look-back words / digit counts, offsets
            + al256((c / 32 + 1) * 4)                              // fixmap
            + (q > kSweepMost ? al256(groups * 256 * 4) + al256(8 * (groups + 1) * 4) + al256(tiles * kSortTile + 16)
@@ -346,8 +347,9 @@ struct Carver {
 
 void carve_sort(Carver& v, uint64_t q, Scratch& s) {
     const uint64_t c = q + kPad, tiles = (q + kSortTile - 1) / kSortTile + 1, groups = tiles / kScanGroup + 1;
-    v.take(s.in_k, c * 8); v.take(s.a_k, c * 8); v.take(s.b_k, c * 8);
-    v.take(s.in_p, c * 4); v.take(s.a_p, c * 4); v.take(s.b_p, c * 4);
+    const uint64_t in = std::min<uint64_t>(q, kSmallSort) + kPad;
+    v.take(s.in_k, in * 8); v.take(s.a_k, c * 8); v.take(s.b_k, c * 8);
+    v.take(s.in_p, in * 4); v.take(s.a_p, c * 4); v.take(s.b_p, c * 4);
     v.take(s.sdesc[0], tiles * 256 * 4); v.take(s.sdesc[1], tiles * 256 * 4);
     v.take(s.fixmap, (c / 32 + 1) * 4);
     if (q > kSweepMost) {

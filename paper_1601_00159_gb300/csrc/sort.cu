@@ -8,8 +8,7 @@
 // launch per pass, the digit counts over the whole batch having been counted by the kernel
 // before. Larger batches count each tile's digits in a kernel of its own before each pass, whose
 // last CTAs scan the counts, so that no tile waits for another.
-// A pass whose byte is the same in every key is skipped (byte-wise min/max in the pack
-// kernel). The sort is stable, so equal keys stay in arrival order: the order is
+// A pass whose byte is the same in every key is skipped (byte-wise min/max in the scan). The sort is stable, so equal keys stay in arrival order: the order is
 // (key, arrival index), the reading of Definition 3 for duplicate keys.
 //
 // Prefix passes. When more bytes vary than the caller's pass budget (4 for batches),
@@ -38,7 +37,7 @@ constexpr int kWarpSpan = 32 * kItems;    // 256 consecutive elements per warp
 static_assert(kTile == kSortTile, "tile size shared with the host's sizing");
 
 // The first digit of a full-width batch: its four most significant bytes vary, and the passes
-// start at the lowest of them. The pack kernel counts this byte; other plans count theirs
+// start at the lowest of them. The scan counts this byte; other plans count theirs
 // in the plan kernel.
 constexpr uint32_t kUsualByte = 4;
 constexpr uint32_t kUsualRow = 8;         // its row of the counts (rows 0 .. 7: the passes')
@@ -74,13 +73,14 @@ __device__ __forceinline__ void count_digits(const uint32_t (&d)[kN], uint32_t n
     }
 }
 
-// K0: validate and pack. Also finds, per key byte, whether it is the same in every
-// valid key (byte-wise min and max), which decides the radix passes that can be skipped.
-// Four consecutive queries per thread and step (16-byte key loads, one 4-byte load of
-// their op codes, vector stores) when the caller's arrays are aligned for it, so that
-// every thread keeps several loads in flight; the byte-wise extremes are kept four bytes
-// to a word with SIMD min/max.
-struct PackAcc {
+// K0: one read of the caller's queries that finds, per key byte, whether it is the same in every
+// valid key (byte-wise min and max), which decides the radix passes that can be skipped, and
+// counts the invalid queries. Nothing is written: the first pass reads the caller's arrays again
+// and packs as it goes (writing the packed queries here and reading them back cost 12 us of 2^22
+// queries). Four consecutive queries per thread and step (16-byte key loads, one 4-byte load of
+// their op codes) when the arrays are aligned for it, so that every thread keeps several loads
+// in flight; the byte-wise extremes are kept four bytes to a word with SIMD min/max.
+struct ScanAcc {
     uint32_t invalid = 0;
     uint32_t mxl = 0, mxh = 0;                  // byte-wise max of the valid keys (low, high word)
     uint32_t mnl = 0xFFFFFFFFu, mnh = 0xFFFFFFFFu;  // byte-wise min
@@ -97,9 +97,8 @@ struct PackAcc {
 };
 
 template <bool kSweep>
-__global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, const uint64_t* __restrict__ keys,
-                                              uint32_t n, uint64_t* __restrict__ sk, uint32_t* __restrict__ sp,
-                                              uint32_t* __restrict__ fixmap, uint32_t* __restrict__ desc,
+__global__ void __launch_bounds__(256) k_scan(const uint8_t* __restrict__ ops, const uint64_t* __restrict__ keys,
+                                              uint32_t n, uint32_t* __restrict__ fixmap, uint32_t* __restrict__ desc,
                                               uint32_t ndesc, uint32_t* __restrict__ hist, BatchMeta* bm) {
     pdl_wait();
     pdl_trigger();
@@ -112,7 +111,7 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, c
     if (kSweep)
         for (uint32_t w = gt; w < ndesc; w += gs) desc[w] = 0;  // the first pass's look-back words
     for (uint32_t w = gt; w < (n + 31u) / 32u; w += gs) fixmap[w] = 0;  // segment marks of the prefix fix-up
-    PackAcc acc;
+    ScanAcc acc;
     const bool vec = ((reinterpret_cast<uintptr_t>(keys) & 15u) | (reinterpret_cast<uintptr_t>(ops) & 3u)) == 0;
     uint32_t tail = 0;  // first query left to the scalar loop
     if (vec) {
@@ -125,23 +124,10 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, c
                 const ulonglong2 k23 = reinterpret_cast<const ulonglong2*>(keys + i)[1];
                 const uint32_t o4 = ops ? *reinterpret_cast<const uint32_t*>(ops + i) : 0u;
                 const uint32_t o0 = o4 & 255u, o1 = (o4 >> 8) & 255u, o2 = (o4 >> 16) & 255u, o3 = o4 >> 24;
-                ulonglong2 s01, s23;
-                s01.x = acc.take(k01.x, o0);
-                s01.y = acc.take(k01.y, o1);
-                s23.x = acc.take(k23.x, o2);
-                s23.y = acc.take(k23.y, o3);
-                reinterpret_cast<ulonglong2*>(sk + i)[0] = s01;
-                reinterpret_cast<ulonglong2*>(sk + i)[1] = s23;
-                uint4 p;
-                p.x = ((o0 & 3u) << 30) | i;
-                p.y = ((o1 & 3u) << 30) | (i + 1u);
-                p.z = ((o2 & 3u) << 30) | (i + 2u);
-                p.w = ((o3 & 3u) << 30) | (i + 3u);
-                *reinterpret_cast<uint4*>(sp + i) = p;
-                dg[0] = usual_digit(s01.x);
-                dg[1] = usual_digit(s01.y);
-                dg[2] = usual_digit(s23.x);
-                dg[3] = usual_digit(s23.y);
+                dg[0] = usual_digit(acc.take(k01.x, o0));
+                dg[1] = usual_digit(acc.take(k01.y, o1));
+                dg[2] = usual_digit(acc.take(k23.x, o2));
+                dg[3] = usual_digit(acc.take(k23.y, o3));
             }
             if (kSweep) count_digits(dg, g < n4 ? 4u : 0u, s_hist);
         }
@@ -151,8 +137,6 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, c
         const uint32_t op = ops ? ops[i] : 0u;
         const uint64_t k = acc.take(keys[i], op);
         if (kSweep) atomicAdd(&s_hist[usual_digit(k)], 1u);
-        sk[i] = k;
-        sp[i] = ((op & 3u) << 30) | i;
     }
     uint32_t invalid = acc.invalid;
     uint32_t mx[8], mn[8];  // mn holds max of (255 - byte), so zero is the identity
@@ -197,6 +181,40 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t* __restrict__ ops, c
 // max_passes of them (the prefix). The fix-up then orders each segment of equal prefix
 // bytes by the full key; its long-segment path sorts by every other byte that can
 // differ inside a segment (rdig).
+// Query i of the caller, as the sort takes it: invalid queries get the key 2^64-1.
+__device__ __forceinline__ void load_query(const SortBuffers& sb, uint32_t i, uint64_t& key, uint32_t& pay) {
+    const uint32_t op = sb.ops ? sb.ops[i] : 0u;
+    const uint64_t k = sb.keys[i];
+    key = op <= 2u ? k : kMaxKey;
+    pay = ((op & 3u) << 30) | i;
+}
+
+// Digits of the caller's queries i0 .. i0 + nv - 1 (nv <= 8, i0 a multiple of 8), with 16-byte key
+// loads and an 8-byte load of the op codes when the arrays are aligned for them.
+__device__ __forceinline__ void query_digits(const SortBuffers& sb, uint32_t i0, uint32_t nv, uint32_t shift,
+                                             uint32_t (&dg)[8]) {
+    const bool vec = ((reinterpret_cast<uintptr_t>(sb.keys) & 15u) | (reinterpret_cast<uintptr_t>(sb.ops) & 7u)) == 0;
+    if (vec && nv == 8u) {
+        const ulonglong2* p = reinterpret_cast<const ulonglong2*>(sb.keys + i0);
+        const uint2 o = sb.ops ? *reinterpret_cast<const uint2*>(sb.ops + i0) : make_uint2(0u, 0u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const ulonglong2 v = p[k];
+            const uint32_t w = (k < 2 ? o.x : o.y) >> (16 * (k & 1));
+            dg[2 * k] = (w & 255u) <= 2u ? (uint32_t)(v.x >> shift) & 255u : 255u;
+            dg[2 * k + 1] = ((w >> 8) & 255u) <= 2u ? (uint32_t)(v.y >> shift) & 255u : 255u;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            uint64_t key = 0;
+            uint32_t pay;
+            if ((uint32_t)k < nv) load_query(sb, i0 + k, key, pay);
+            dg[k] = (uint32_t)(key >> shift) & 255u;
+        }
+    }
+}
+
 template <bool kSweep>
 __global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, BatchMeta* bm, uint32_t max_passes) {
     pdl_wait();
@@ -213,24 +231,13 @@ __global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, B
     }
     s_hist[threadIdx.x] = 0;
     __syncthreads();
-    if (!kSweep || s_plan.digit[0] == kUsualByte) return;  // counted with the packing
+    if (!kSweep || s_plan.digit[0] == kUsualByte) return;  // counted by the scan
     const uint32_t shift = 8u * s_plan.digit[0];
     for (uint32_t base = blockIdx.x * 2048u; base < n; base += gridDim.x * 2048u) {
         const uint32_t i0 = base + threadIdx.x * 8u;
         const uint32_t nv = i0 < n ? min(8u, n - i0) : 0u;
         uint32_t dg[8];
-        if (nv == 8u) {
-            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(sb.in_k + i0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const ulonglong2 v = p[k];
-                dg[2 * k] = (uint32_t)(v.x >> shift) & 255u;
-                dg[2 * k + 1] = (uint32_t)(v.y >> shift) & 255u;
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) dg[k] = (uint32_t)k < nv ? (uint32_t)(sb.in_k[i0 + k] >> shift) & 255u : 0u;
-        }
+        query_digits(sb, i0, nv, shift, dg);
         count_digits(dg, nv, s_hist);
     }
     __syncthreads();
@@ -239,7 +246,7 @@ __global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, B
 
 // Look-back word of one digit of one tile: flag (2 bits) | count (30). 0: not published yet.
 // Words are cleared between uses: a pass clears its tiles' words of the other buffer for the
-// next pass, and the pack kernel those of the first.
+// next pass, and the scan those of the first.
 constexpr uint32_t kWordAgg = 1u << 30, kWordPrefix = 2u << 30, kWordMask = kWordAgg - 1u;
 
 __device__ __forceinline__ uint32_t ld_relaxed32(const uint32_t* p) {
@@ -323,8 +330,9 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_sort_pass(uint32_t j, uint3
         reinterpret_cast<uint4*>(&s_whist[0][0])[i] = make_uint4(0, 0, 0, 0);
     if (tid < 256) s_next[tid] = 0;
     const uint32_t shift = 8u * P.digit[j];
-    const uint64_t* src_k = P.src[j] == 0 ? sb.in_k : (P.src[j] == 1 ? sb.a_k : sb.b_k);
-    const uint32_t* src_p = P.src[j] == 0 ? sb.in_p : (P.src[j] == 1 ? sb.a_p : sb.b_p);
+    const bool caller = P.src[j] == 0;  // the first pass reads the caller's queries
+    const uint64_t* src_k = P.src[j] == 1 ? sb.a_k : sb.b_k;
+    const uint32_t* src_p = P.src[j] == 1 ? sb.a_p : sb.b_p;
     uint64_t* dst_k = P.dst[j] == 1 ? sb.a_k : sb.b_k;
     uint32_t* dst_p = P.dst[j] == 1 ? sb.a_p : sb.b_p;
     const uint32_t row = j == 0 && P.digit[0] == kUsualByte ? kUsualRow : j;
@@ -340,8 +348,16 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_sort_pass(uint32_t j, uint3
     for (int k = 0; k < kI; ++k) {
         const uint32_t li = (uint32_t)(warp * 32 * kI + k * 32 + lane);
         const bool v = li < tn;
-        key[k] = v ? src_k[tbase + li] : 0ull;
-        pay[k] = v ? src_p[tbase + li] : 0u;
+        key[k] = 0ull;
+        pay[k] = 0u;
+        if (v) {
+            if (caller) {
+                load_query(sb, tbase + li, key[k], pay[k]);
+            } else {
+                key[k] = src_k[tbase + li];
+                pay[k] = src_p[tbase + li];
+            }
+        }
         dig[k] = v ? (uint32_t)((key[k] >> shift) & 255u) : 256u;
     }
     const uint32_t dbase = block_excl_sum<kPassThreads>(all, s_tmp, nullptr);  // the digit's first output slot
@@ -417,16 +433,13 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_sort_pass(uint32_t j, uint3
 // in flight the look-back costs more than a launch that reads one digit byte per element:
 // 2^22 queries on 2^27 keys took 571 us a batch with k_sort_pass and 544 with these two; at 2^20
 // queries k_sort_pass is ahead (428 against 432), and at 10^5 by 21 of 99 us.
-__device__ __forceinline__ const uint64_t* pass_src_keys(const SortPlan& P, uint32_t j, const SortBuffers& sb) {
-    return P.src[j] == 0 ? sb.in_k : (P.src[j] == 1 ? sb.a_k : sb.b_k);
-}
 
 // Digit histogram of every tile for pass j, then its scan, by the CTAs that finish
 // last (no CTA waits for another): the last CTA of each group of kScanGroup tiles turns
 // the group's counts into offsets within the group (toff) and the group's digit totals
 // (gsum); the last group to finish turns those totals into the groups' offsets, in
 // place, and the digit totals into digit bases (dofs). A tile's first output slot for
-// digit d is then dofs[d] + gsum[group][d] + toff[tile][d]. Pass 0 reads the packed
+// digit d is then dofs[d] + gsum[group][d] + toff[tile][d]. Pass 0 reads the caller's
 // keys; later passes read the digit bytes the previous scatter wrote beside its output.
 // Each thread counts 8 consecutive elements and adds each run of equal digits with one
 // shared-memory atomic (one per warp when the whole warp holds one digit), so a run of a
@@ -467,19 +480,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_sort_count(uint32_t j, uint32_t
     uint32_t dg[8];
     if (j == 0) {
         const uint32_t shift = 8u * P.digit[0];
-        const uint64_t* src = pass_src_keys(P, 0, sb);
-        if (nv == 8u) {
-            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(src + i0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const ulonglong2 v = p[k];
-                dg[2 * k] = (uint32_t)(v.x >> shift) & 255u;
-                dg[2 * k + 1] = (uint32_t)(v.y >> shift) & 255u;
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) dg[k] = (uint32_t)k < nv ? (uint32_t)(src[i0 + k] >> shift) & 255u : 0u;
-        }
+        query_digits(sb, i0, nv, shift, dg);
     } else {
         if (nv == 8u) {  // 8 digit bytes per thread: one 8-byte load
             const uint2 v = *reinterpret_cast<const uint2*>(sb.ndig + i0);
@@ -533,8 +534,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_scatter(uint32_t j, uint32
     const SortPlan& P = bm->plan;
     if (j >= P.npass) return;
     const uint32_t shift = 8u * P.digit[j];
-    const uint64_t* src_k = P.src[j] == 0 ? sb.in_k : (P.src[j] == 1 ? sb.a_k : sb.b_k);
-    const uint32_t* src_p = P.src[j] == 0 ? sb.in_p : (P.src[j] == 1 ? sb.a_p : sb.b_p);
+    const bool caller = P.src[j] == 0;  // the first pass reads the caller's queries
+    const uint64_t* src_k = P.src[j] == 1 ? sb.a_k : sb.b_k;
+    const uint32_t* src_p = P.src[j] == 1 ? sb.a_p : sb.b_p;
     uint64_t* dst_k = P.dst[j] == 1 ? sb.a_k : sb.b_k;
     uint32_t* dst_p = P.dst[j] == 1 ? sb.a_p : sb.b_p;
 
@@ -560,8 +562,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_scatter(uint32_t j, uint32
     for (int k = 0; k < kItems; ++k) {
         uint32_t li = warp * kWarpSpan + k * 32 + lane;
         bool v = li < tn;
-        key[k] = v ? src_k[tbase + li] : 0ull;
-        pay[k] = v ? src_p[tbase + li] : 0u;
+        key[k] = 0ull;
+        pay[k] = 0u;
+        if (v) {
+            if (caller) {
+                load_query(sb, tbase + li, key[k], pay[k]);
+            } else {
+                key[k] = src_k[tbase + li];
+                pay[k] = src_p[tbase + li];
+            }
+        }
         dig[k] = v ? (uint32_t)((key[k] >> shift) & 255u) : 256u;
     }
     warp_digit_ranks<kItems, 8>(dig, rank, s_whist[warp]);
@@ -1066,11 +1076,14 @@ static cudaError_t launch_count_passes(uint32_t n, const SortBuffers& sb, BatchM
     return cudaSuccess;
 }
 
-cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& sb,
+cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, const SortBuffers& buffers,
                         BatchMeta* bm, uint32_t* err, cudaStream_t s, int num_sms, int max_passes, bool* hist_clear,
                         bool long_too) {
     if (n == 0) return cudaSuccess;
     if (max_passes < 1 || max_passes > 8) return cudaErrorInvalidValue;
+    SortBuffers sb = buffers;
+    sb.ops = ops;
+    sb.keys = keys;
     const bool sweep = n <= kSweepMost, large = n >= kLargeTiles;
     const int grid = min((int)((n + 255) / 256), num_sms * 8);
     cudaError_t e = cudaSuccess;
@@ -1078,13 +1091,12 @@ cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, co
         if (!*hist_clear && (e = cudaMemsetAsync(sb.hist, 0, kSortHist * sizeof(uint32_t), s)) != cudaSuccess) return e;
         *hist_clear = false;
         const uint32_t tile = (uint32_t)kPassThreads * (large ? 8u : 4u), words = (n + tile - 1) / tile * 256u;
-        launch_dep(k_pack<true>, grid, 256, 0, s, ops, keys, n, sb.in_k, sb.in_p, sb.fixmap, sb.desc[0], words, sb.hist, bm);
+        launch_dep(k_scan<true>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.desc[0], words, sb.hist, bm);
         launch_dep(k_sort_plan<true>, min((int)((n + 2047) / 2048), num_sms * 4), 256, 0, s, n, sb, bm, (uint32_t)max_passes);
         g_launches += 2;
         e = large ? launch_passes<8>(n, sb, bm, err, s, max_passes) : launch_passes<4>(n, sb, bm, err, s, max_passes);
     } else {
-        launch_dep(k_pack<false>, grid, 256, 0, s, ops, keys, n, sb.in_k, sb.in_p, sb.fixmap, (uint32_t*)nullptr, 0u,
-                   (uint32_t*)nullptr, bm);
+        launch_dep(k_scan<false>, grid, 256, 0, s, ops, keys, n, sb.fixmap, (uint32_t*)nullptr, 0u, (uint32_t*)nullptr, bm);
         launch_dep(k_sort_plan<false>, 1, 256, 0, s, n, sb, bm, (uint32_t)max_passes);
         g_launches += 2;
         e = launch_count_passes(n, sb, bm, err, s, max_passes);

@@ -51,3 +51,24 @@ def test_sizes(orc_mod, kind, passes):
     assert idx.status() == 0
     idx.close()
     orc.close()
+
+
+@pytest.mark.parametrize("q", [5000, 70001, (1 << 20) + 6])
+@pytest.mark.parametrize("shift", [1, 3])
+def test_misaligned_arrays(orc_mod, q, shift):
+    """Views that start at odd elements: no 16-byte key loads, no word-wide op loads."""
+    import torch
+    from tests.parity import results_np, to_dev
+    n = 9000
+    keys = wl.distinct_keys(72, np.arange(n))
+    idx = make_index(keys, keys, 0.5, 5)
+    orc = orc_mod.Oracle(keys, keys, 0.5, 5)
+    s = wl.stream_seed(q, 73)
+    ops = wl.bounded(s, 0, q, 4).astype(np.uint8)
+    k = keys[wl.bounded(s, q, q, n)]
+    b = wl.Batch(ops, k, wl.u64_stream(s, 2 * q, q))
+    pad = lambda a, dt: to_dev(np.concatenate([np.zeros(shift, a.dtype), a]), dt)[shift:]  # noqa: E731
+    got = idx.execute(pad(b.ops, torch.uint8), pad(b.keys, torch.int64), pad(b.vals, torch.int64))
+    assert_results_equal(results_np(got), orc.execute(b.ops, b.keys, b.vals), f"q {q}")
+    idx.close()
+    orc.close()
