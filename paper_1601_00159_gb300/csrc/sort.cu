@@ -1,5 +1,5 @@
-// K0 + K1: validate/pack the query set and sort it by key (Definition 3: the queries
-// of a query set are ordered by key; Section 4.2: the sort can use data parallelism).
+// Sorts a query set by key (Definition 3: the queries of a query set are ordered by key;
+// Section 4.2: the sort can use data parallelism); invalid queries go to its end.
 //
 // LSD radix sort with 8-bit digits over tiles of 2048 or 4096 elements. A tile ranks its elements
 // stably and writes them staged in shared memory, so each digit's run is written
@@ -8,8 +8,9 @@
 // launch per pass, the digit counts over the whole batch having been counted by the kernel
 // before. Larger batches count each tile's digits in a kernel of its own before each pass, whose
 // last CTAs scan the counts, so that no tile waits for another.
-// A pass whose byte is the same in every key is skipped (byte-wise min/max in the scan). The sort is stable, so equal keys stay in arrival order: the order is
-// (key, arrival index), the reading of Definition 3 for duplicate keys.
+// A pass whose byte is the same in every key is skipped (byte-wise min/max in the scan). The
+// sort is stable, so equal keys stay in arrival order: the order is (key, arrival index), the
+// reading of Definition 3 for duplicate keys.
 //
 // Prefix passes. When more bytes vary than the caller's pass budget (4 for batches),
 // only the most significant varying bytes get passes. Keys that agree on those bytes
@@ -29,7 +30,7 @@
 namespace pi {
 namespace {
 
-constexpr int kThreads = 256;             // the fix-up's CTAs
+constexpr int kThreads = 256;             // of the count, the scatter and the fix-up
 constexpr int kItems = 8;
 constexpr int kTile = kThreads * kItems;
 constexpr int kWarps = kThreads / 32;
@@ -42,6 +43,11 @@ static_assert(kTile == kSortTile, "tile size shared with the host's sizing");
 constexpr uint32_t kUsualByte = 4;
 constexpr uint32_t kUsualRow = 8;         // its row of the counts (rows 0 .. 7: the passes')
 constexpr uint32_t kLargeTiles = 1u << 19;  // from here on, their tiles hold 4096 elements instead of 2048
+
+// Above kSweepMost: tiles per CTA of the counting kernel, elements per warp.
+constexpr uint32_t kCountTiles = 4;
+constexpr uint32_t kCountSpan = kTile * kCountTiles / kWarps;
+static_assert(kScanGroup % kCountTiles == 0 && kTile % kCountSpan == 0, "a CTA's tiles lie in one group");
 
 __device__ __forceinline__ uint32_t usual_digit(uint64_t k) { return (uint32_t)(k >> (8u * kUsualByte)) & 255u; }
 
@@ -73,13 +79,14 @@ __device__ __forceinline__ void count_digits(const uint32_t (&d)[kN], uint32_t n
     }
 }
 
-// K0: one read of the caller's queries that finds, per key byte, whether it is the same in every
+// One read of the caller's queries that finds, per key byte, whether it is the same in every
 // valid key (byte-wise min and max), which decides the radix passes that can be skipped, and
 // counts the invalid queries. Nothing is written: the first pass reads the caller's arrays again
 // and packs as it goes (writing the packed queries here and reading them back cost 12 us of 2^22
 // queries). Four consecutive queries per thread and step (16-byte key loads, one 4-byte load of
 // their op codes) when the arrays are aligned for it, so that every thread keeps several loads
-// in flight; the byte-wise extremes are kept four bytes to a word with SIMD min/max.
+// in flight; the byte-wise extremes are kept four bytes to a word with SIMD min/max. It also
+// clears what the passes start from: the first pass's look-back words, or the counts' arrivals.
 struct ScanAcc {
     uint32_t invalid = 0;
     uint32_t mxl = 0, mxh = 0;                  // byte-wise max of the valid keys (low, high word)
@@ -98,8 +105,8 @@ struct ScanAcc {
 
 template <bool kSweep>
 __global__ void __launch_bounds__(256) k_scan(const uint8_t* __restrict__ ops, const uint64_t* __restrict__ keys,
-                                              uint32_t n, uint32_t* __restrict__ fixmap, uint32_t* __restrict__ desc,
-                                              uint32_t ndesc, uint32_t* __restrict__ hist, BatchMeta* bm) {
+                                              uint32_t n, uint32_t* __restrict__ fixmap, uint32_t* __restrict__ clear,
+                                              uint32_t nclear, uint32_t* __restrict__ hist, BatchMeta* bm) {
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t s_hist[256];
@@ -108,8 +115,7 @@ __global__ void __launch_bounds__(256) k_scan(const uint8_t* __restrict__ ops, c
         __syncthreads();
     }
     const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
-    if (kSweep)
-        for (uint32_t w = gt; w < ndesc; w += gs) desc[w] = 0;  // the first pass's look-back words
+    for (uint32_t w = gt; w < nclear; w += gs) clear[w] = 0;
     for (uint32_t w = gt; w < (n + 31u) / 32u; w += gs) fixmap[w] = 0;  // segment marks of the prefix fix-up
     ScanAcc acc;
     const bool vec = ((reinterpret_cast<uintptr_t>(keys) & 15u) | (reinterpret_cast<uintptr_t>(ops) & 3u)) == 0;
@@ -215,23 +221,18 @@ __device__ __forceinline__ void query_digits(const SortBuffers& sb, uint32_t i0,
     }
 }
 
-template <bool kSweep>
 __global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, BatchMeta* bm, uint32_t max_passes) {
     pdl_wait();
     pdl_trigger();
     __shared__ SortPlan s_plan;
     __shared__ uint32_t s_hist[256];
-    if (!kSweep) {  // one CTA
-        const uint32_t ngroups = ((n + kTile - 1) / kTile + kScanGroup - 1) / kScanGroup;
-        for (uint32_t i = threadIdx.x; i < 8u * (ngroups + 1u); i += 256) sb.gctr[i] = 0;  // the counts' arrivals
-    }
     if (threadIdx.x == 0) {
         plan_digits(bm->bmax, bm->bnmin, bm->invalid, n, max_passes, s_plan);
         if (blockIdx.x == 0) bm->plan = s_plan;
     }
     s_hist[threadIdx.x] = 0;
     __syncthreads();
-    if (!kSweep || s_plan.digit[0] == kUsualByte) return;  // counted by the scan
+    if (s_plan.digit[0] == kUsualByte) return;  // counted by the scan
     const uint32_t shift = 8u * s_plan.digit[0];
     for (uint32_t base = blockIdx.x * 2048u; base < n; base += gridDim.x * 2048u) {
         const uint32_t i0 = base + threadIdx.x * 8u;
@@ -439,23 +440,30 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_sort_pass(uint32_t j, uint3
 // the group's counts into offsets within the group (toff) and the group's digit totals
 // (gsum); the last group to finish turns those totals into the groups' offsets, in
 // place, and the digit totals into digit bases (dofs). A tile's first output slot for
-// digit d is then dofs[d] + gsum[group][d] + toff[tile][d]. Pass 0 reads the caller's
-// keys; later passes read the digit bytes the previous scatter wrote beside its output.
-// Each thread counts 8 consecutive elements and adds each run of equal digits with one
-// shared-memory atomic (one per warp when the whole warp holds one digit), so a run of a
-// hot key costs no atomic contention. The scans load 16 rows per round trip.
+// digit d is then dofs[d] + gsum[group][d] + toff[tile][d]. Pass 0 (kFirst) plans the digits,
+// in every CTA, and reads the caller's keys; later passes read the digit bytes the previous
+// scatter wrote beside its output. A thread takes 8 consecutive elements a step and adds each
+// run of equal digits with one shared-memory atomic (one per warp when the whole warp holds
+// one digit), so a run of a hot key costs no atomic contention.
+// The kernel is bound by its chain of dependent round trips, not by the bytes: so a CTA counts
+// four tiles (2^22 queries are then one wave of 512 CTAs, not three of 2048 with one tile
+// each), with every load of digit bytes in flight, and the scans load 32 rows per round trip.
+// 2^22 queries on 2^27 keys took 504 us a batch with one tile per CTA, 16 rows and a kernel of
+// its own for the plan, and take 497. Tiles of 4096 elements, which need half the rows, left the
+// counts as they were and cost the scatter 8 us.
 // Exclusive running sum, per digit (thread d), over `rows` rows of 256 counters starting
 // at `in`: writes each row's prefix to `out` (may equal `in`) and returns the total.
 __device__ __forceinline__ uint32_t scan_rows(const uint32_t* in, uint32_t* out, uint32_t rows) {
     const uint32_t d = threadIdx.x;
+    constexpr int kRows = 32;
     uint32_t run = 0;
-    for (uint32_t t = 0; t < rows; t += 16) {
-        uint32_t c[16];
+    for (uint32_t t = 0; t < rows; t += kRows) {
+        uint32_t c[kRows];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) c[k] = (t + k < rows) ? __ldcg(&in[(size_t)(t + k) * 256 + d]) : 0u;
+        for (int k = 0; k < kRows; ++k) c[k] = (t + (uint32_t)k < rows) ? __ldcg(&in[(size_t)(t + k) * 256 + d]) : 0u;
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            if (t + k < rows) {
+        for (int k = 0; k < kRows; ++k) {
+            if (t + (uint32_t)k < rows) {
                 out[(size_t)(t + k) * 256 + d] = run;
                 run += c[k];
             }
@@ -464,41 +472,62 @@ __device__ __forceinline__ uint32_t scan_rows(const uint32_t* in, uint32_t* out,
     return run;
 }
 
-__global__ void __launch_bounds__(kThreads, 6) k_sort_count(uint32_t j, uint32_t n, SortBuffers sb, BatchMeta* bm) {
+template <bool kFirst>
+__global__ void __launch_bounds__(kThreads, 4) k_sort_count(uint32_t j, uint32_t n, SortBuffers sb, BatchMeta* bm,
+                                                            uint32_t max_passes) {
     pdl_wait();
     pdl_trigger();
-    __shared__ uint32_t h[256];
+    __shared__ uint32_t h[kCountTiles][256];
     __shared__ uint32_t s_tmp[33];
     __shared__ uint32_t s_last;
-    const SortPlan& P = bm->plan;
-    if (j >= P.npass) return;
-    h[threadIdx.x] = 0;
+    __shared__ SortPlan s_plan;
+    if (!kFirst && j >= bm->plan.npass) return;
+    if (kFirst && threadIdx.x == 0) {
+        plan_digits(bm->bmax, bm->bnmin, bm->invalid, n, max_passes, s_plan);
+        if (blockIdx.x == 0) bm->plan = s_plan;
+    }
+#pragma unroll
+    for (uint32_t t = 0; t < kCountTiles; ++t) h[t][threadIdx.x] = 0;
     __syncthreads();
-    const uint32_t tbase = blockIdx.x * kTile;
-    const uint32_t i0 = tbase + threadIdx.x * 8u;
-    const uint32_t nv = i0 < n ? min(8u, n - i0) : 0u;
-    uint32_t dg[8];
-    if (j == 0) {
-        const uint32_t shift = 8u * P.digit[0];
-        query_digits(sb, i0, nv, shift, dg);
+    // A warp reads kCountSpan consecutive elements of one tile, 8 per lane and step.
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint32_t* ht = h[warp / (kTile / kCountSpan)];
+    const uint32_t wbase = (blockIdx.x * kWarps + warp) * kCountSpan + lane * 8u;
+    if (kFirst) {
+        const uint32_t shift = 8u * s_plan.digit[0];
+#pragma unroll 1
+        for (uint32_t i0 = wbase; i0 < wbase + kCountSpan; i0 += 256u) {
+            const uint32_t nv = i0 < n ? min(8u, n - i0) : 0u;
+            uint32_t dg[8];
+            query_digits(sb, i0, nv, shift, dg);
+            count_digits(dg, nv, ht);
+        }
     } else {
-        if (nv == 8u) {  // 8 digit bytes per thread: one 8-byte load
-            const uint2 v = *reinterpret_cast<const uint2*>(sb.ndig + i0);
+        constexpr int kSteps = kCountSpan / 256u;
+        uint2 v[kSteps];
+#pragma unroll
+        for (int u = 0; u < kSteps; ++u) {  // 8 digit bytes a load, every load in flight
+            const uint32_t i0 = wbase + (uint32_t)u * 256u;
+            v[u] = i0 < n ? *reinterpret_cast<const uint2*>(sb.ndig + i0) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < kSteps; ++u) {
+            const uint32_t i0 = wbase + (uint32_t)u * 256u;
+            uint32_t dg[8];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                dg[k] = (v.x >> (8 * k)) & 255u;
-                dg[4 + k] = (v.y >> (8 * k)) & 255u;
+                dg[k] = (v[u].x >> (8 * k)) & 255u;
+                dg[4 + k] = (v[u].y >> (8 * k)) & 255u;
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) dg[k] = (uint32_t)k < nv ? sb.ndig[i0 + k] : 0u;
+            count_digits(dg, i0 < n ? min(8u, n - i0) : 0u, ht);
         }
     }
-    count_digits(dg, nv, h);
     __syncthreads();
     const uint32_t d = threadIdx.x;
-    const uint32_t tile = blockIdx.x, ntiles = gridDim.x;
-    sb.tcnt[(size_t)tile * 256 + d] = h[d];
+    const uint32_t tile = blockIdx.x * kCountTiles, ntiles = (n + kTile - 1) / kTile;
+#pragma unroll
+    for (uint32_t t = 0; t < kCountTiles; ++t)
+        if (tile + t < ntiles) sb.tcnt[(size_t)(tile + t) * 256 + d] = h[t][d];
     const uint32_t g = tile / kScanGroup, ngroups = (ntiles + kScanGroup - 1) / kScanGroup;
     const uint32_t t0 = g * kScanGroup, t1 = min(t0 + kScanGroup, ntiles);
     uint32_t* ctr = sb.gctr + (size_t)j * (ngroups + 1);
@@ -508,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_sort_count(uint32_t j, uint32_t
     __syncthreads();
     if (d == 0) {
         __threadfence();
-        s_last = atomicAdd(&ctr[g], 1u) == t1 - t0 - 1u;
+        s_last = atomicAdd(&ctr[g], 1u) == (t1 - t0 + kCountTiles - 1u) / kCountTiles - 1u;
         if (s_last) __threadfence();  // every CTA of the group has arrived: their counts are visible
     }
     __syncthreads();
@@ -1068,7 +1097,9 @@ static cudaError_t launch_count_passes(uint32_t n, const SortBuffers& sb, BatchM
     }
     const uint32_t tiles = (n + kTile - 1) / kTile;
     for (uint32_t j = 0; j < (uint32_t)max_passes; ++j) {
-        launch_dep(k_sort_count, tiles, kThreads, 0, s, j, n, sb, bm);
+        const uint32_t ctas = (tiles + kCountTiles - 1) / kCountTiles;
+        if (j == 0) launch_dep(k_sort_count<true>, ctas, kThreads, 0, s, j, n, sb, bm, (uint32_t)max_passes);
+        else launch_dep(k_sort_count<false>, ctas, kThreads, 0, s, j, n, sb, bm, (uint32_t)max_passes);
         ++g_launches;
         launch_dep(k_sort_scatter, tiles, kThreads, dyn, s, j, n, sb, bm, err);
         ++g_launches;
@@ -1092,13 +1123,14 @@ cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, co
         *hist_clear = false;
         const uint32_t tile = (uint32_t)kPassThreads * (large ? 8u : 4u), words = (n + tile - 1) / tile * 256u;
         launch_dep(k_scan<true>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.desc[0], words, sb.hist, bm);
-        launch_dep(k_sort_plan<true>, min((int)((n + 2047) / 2048), num_sms * 4), 256, 0, s, n, sb, bm, (uint32_t)max_passes);
+        launch_dep(k_sort_plan, min((int)((n + 2047) / 2048), num_sms * 4), 256, 0, s, n, sb, bm, (uint32_t)max_passes);
         g_launches += 2;
         e = large ? launch_passes<8>(n, sb, bm, err, s, max_passes) : launch_passes<4>(n, sb, bm, err, s, max_passes);
     } else {
-        launch_dep(k_scan<false>, grid, 256, 0, s, ops, keys, n, sb.fixmap, (uint32_t*)nullptr, 0u, (uint32_t*)nullptr, bm);
-        launch_dep(k_sort_plan<false>, 1, 256, 0, s, n, sb, bm, (uint32_t)max_passes);
-        g_launches += 2;
+        const uint32_t ngroups = ((n + kTile - 1) / kTile + kScanGroup - 1) / kScanGroup;
+        launch_dep(k_scan<false>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.gctr, 8u * (ngroups + 1u),
+                   (uint32_t*)nullptr, bm);
+        ++g_launches;
         e = launch_count_passes(n, sb, bm, err, s, max_passes);
     }
     if (e != cudaSuccess) return e;
