@@ -1,4 +1,4 @@
-// K4 + K5: single ownership and query execution (Algorithms 3 and 4, Section 3.2.4).
+// Single ownership and query execution (Algorithms 3 and 4, Section 3.2.4).
 //
 // In the paper each execution thread owns the storage nodes between its first
 // interception and the next thread's, handing queries over to its neighbour so that
@@ -18,8 +18,8 @@
 // The descent left the storage-layer state at each local run head (a query whose key differs
 // from the previous one, and the first query of every 128-query block) and each block's
 // largest e. A warp takes a block and scans it on its own: the nearest local head before a
-// query, by its number, has its state, and a block that continues a run looks back over the blocks' (then the
-// tiles') marks for the run's last write, 256 of them a step. So no warp waits for another
+// query, by its number, has its state, and a block that continues a run looks back over the
+// blocks' (then the tiles') marks for the run's last write, 256 of them a step. So no warp waits for another
 // until the counts of the tile: with block-wide scans, barriers were the largest stall.
 // New nodes, and the changes of built levels' membership, go to their places in key order in
 // the same pass: a tile's first place comes from a decoupled look-back over the tiles' counts,
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kApThreads, 4) k_apply(ApplyArgs a, uint32_t e
         uint64_t* desc = a.desc + (tid < 32 ? 0u : ntiles);
         if (c || (tile & 63u) == 0) {
             bool ok = true;
-            const uint32_t ex = lookback_warp_wide<false, 8>(desc, tile, epoch, c, a.err, &ok);
+            const uint32_t ex = lookback_warp_wide<8>(desc, tile, epoch, c, a.err, &ok);
             if (lane == 0) {
                 s_base[tid >> 5] = ex;
                 if (!ok) s_fail = 1;

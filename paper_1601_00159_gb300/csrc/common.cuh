@@ -122,7 +122,8 @@ __device__ __forceinline__ void plan_digits(const uint32_t* bmax, const uint32_t
             if (!((P.pmask >> (8 * d)) & 1u) && (varies[d] || differs[d])) P.rdig[P.nr++] = (uint32_t)d;
 }
 
-// Per-batch scratch counters, cleared by one memset at the start of every batch.
+// Per-batch scratch counters, zero when a batch starts: each batch clears the next one's at its
+// end (post_batch), and the host when that did not run.
 struct BatchMeta {
     uint32_t tile_ctr[24];       // dynamic tile counters, one per look-back kernel
     int32_t delta[kLevelSlots];  // change of n[l] in this batch
@@ -143,7 +144,7 @@ struct BatchMeta {
     uint32_t nchg;                    // packed membership changes
     uint32_t chg_hist[kLevelSlots];   // changes by height
     uint32_t inc;                     // 1: this batch's rebuild is incremental
-    uint32_t old_H, old_total;
+    uint32_t old_H;
     uint32_t old_n[kLevelSlots], old_base[kLevelSlots];
     uint32_t lst_off[kLevelSlots], lst_n[kLevelSlots];  // per-level change lists
 };
@@ -231,11 +232,6 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
     return m;
 }
-__device__ __forceinline__ uint32_t lanemask_le() {
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_le;" : "=r"(m));
-    return m;
-}
 
 // ---------------------------------------------------------------------------------
 // Decoupled look-back (Merrill and Garland, "Single-pass parallel prefix scan with
@@ -246,131 +242,28 @@ constexpr uint64_t kFlagAgg = 1ull << 30;
 constexpr uint64_t kFlagPrefix = 2ull << 30;
 constexpr uint32_t kValMask = (1u << 30) - 1u;
 
-template <bool kMax>
-__device__ __forceinline__ uint32_t lb_op(uint32_t a, uint32_t b) {
-    return kMax ? (a > b ? a : b) : a + b;
-}
-
-// Publishes `agg` for tile `tile` and returns the exclusive prefix of the tiles before
-// it (identity 0 for both sum and max). Sets *ok = false and records kErrTimeout if a
-// predecessor never published within the spin bound.
-template <bool kMax>
-__device__ uint32_t lookback(uint64_t* desc, size_t stride, uint32_t tile, uint32_t epoch,
-                             uint32_t agg, uint32_t* err, bool* ok) {
-    const uint64_t tag = (uint64_t)epoch << 32;
-    *ok = true;
-    if (tile == 0) {
-        publish(desc, tag | kFlagPrefix | (agg & kValMask));
-        return 0;
-    }
-    publish(desc + (size_t)tile * stride, tag | kFlagAgg | (agg & kValMask));
-    uint32_t excl = 0;
-    int64_t t = (int64_t)tile - 1;
-    uint32_t spins = 0;
-    while (t >= 0) {
-        uint64_t d = ld_relaxed(desc + (size_t)t * stride);
-        uint64_t flag = d & (3ull << 30);
-        if ((uint32_t)(d >> 32) != epoch || flag == 0) {
-            ++spins;
-            if (spins > kSpinLimit) {
-                atomicOr(err, kErrTimeout);
-                *ok = false;
-                return 0;
-            }
-            if ((spins & 1023u) == 0 && *(volatile uint32_t*)err) {  // another wait gave up
-                *ok = false;
-                return 0;
-            }
-            if (spins > 32) __nanosleep(100);
-            continue;
-        }
-        excl = lb_op<kMax>(excl, (uint32_t)(d & kValMask));
-        if (flag == kFlagPrefix) break;
-        --t;
-    }
-    publish(desc + (size_t)tile * stride, tag | kFlagPrefix | (lb_op<kMax>(excl, agg) & kValMask));
-    return excl;
-}
-
-// Per-thread variant that keeps kWin predecessor reads in flight per round trip
-// (one thread per digit in the radix sort, descriptors strided by `stride`).
-template <int kWin>
-__device__ __forceinline__ uint32_t lookback_sum_win(uint64_t* desc, size_t stride, uint32_t tile, uint32_t epoch, uint32_t agg,
-                                  uint32_t* err, bool* ok) {
-    const uint64_t tag = (uint64_t)epoch << 32;
-    *ok = true;
-    if (tile == 0) {
-        publish(desc, tag | kFlagPrefix | (agg & kValMask));
-        return 0;
-    }
-    publish(desc + (size_t)tile * stride, tag | kFlagAgg | (agg & kValMask));
-    uint32_t excl = 0, spins = 0;
-    int64_t t = (int64_t)tile - 1;
-    while (t >= 0) {
-        uint64_t d[kWin];
-#pragma unroll
-        for (int i = 0; i < kWin; ++i) d[i] = (t - i >= 0) ? ld_relaxed(desc + (size_t)(t - i) * stride) : (tag | kFlagPrefix);
-        int used = 0;
-        bool stop = false, stall = false;
-        uint32_t add = 0;
-#pragma unroll
-        for (int i = 0; i < kWin; ++i) {
-            if (stop || stall) continue;
-            const uint64_t flag = d[i] & (3ull << 30);
-            if ((uint32_t)(d[i] >> 32) != epoch || flag == 0) {
-                stall = true;
-                continue;
-            }
-            add += (uint32_t)(d[i] & kValMask);
-            ++used;
-            if (flag == kFlagPrefix) stop = true;
-        }
-        excl += add;
-        t -= used;
-        if (stop) break;
-        if (stall) {
-            ++spins;
-            if (spins > kSpinLimit) {
-                atomicOr(err, kErrTimeout);
-                *ok = false;
-                return 0;
-            }
-            if ((spins & 1023u) == 0 && *(volatile uint32_t*)err) {
-                *ok = false;
-                return 0;
-            }
-            if (spins > 32) __nanosleep(100);
-        }
-    }
-    publish(desc + (size_t)tile * stride, tag | kFlagPrefix | ((excl + agg) & kValMask));
-    return excl;
-}
-
-// First half of a look-back, for callers that publish their aggregate early and do
-// other work before waiting on their predecessors: tile 0 publishes its inclusive
-// prefix at once, every other tile its aggregate. One thread calls it.
+// For a tile that needs no prefix itself: tile 0 publishes its inclusive prefix, every other
+// tile its aggregate. One thread calls it.
 __device__ __forceinline__ void lookback_publish(uint64_t* desc, uint32_t tile, uint32_t epoch, uint32_t agg) {
     const uint64_t tag = (uint64_t)epoch << 32;
     publish(desc + tile, tag | (tile == 0 ? kFlagPrefix : kFlagAgg) | (agg & kValMask));
 }
 
-// Warp-wide variant, called by all 32 lanes of one warp: each round reads the
-// descriptors of 32 predecessors at once (lane i reads tile base - 1 - i), so a run of
-// predecessors that have published only their aggregates is crossed 32 tiles per
-// memory round trip instead of one. Returns the exclusive prefix in every lane.
-// With `published`, lookback_publish has already stored this tile's aggregate; `agg` must
-// still be that aggregate, since the inclusive prefix published at the end adds it.
-template <bool kMax>
-__device__ uint32_t lookback_warp(uint64_t* desc, uint32_t tile, uint32_t epoch, uint32_t agg, uint32_t* err,
-                                  bool* ok, bool published = false) {
+// Publishes `agg` for tile `tile` and returns the sum over the tiles before it, in every lane
+// of the one warp that calls it: each round reads the descriptors of 32 predecessors at once
+// (lane i reads tile base - 1 - i), so a run of predecessors that have published only their
+// aggregates is crossed 32 tiles per memory round trip. Sets *ok = false and records
+// kErrTimeout if a predecessor never published within the spin bound.
+__device__ inline uint32_t lookback_warp(uint64_t* desc, uint32_t tile, uint32_t epoch, uint32_t agg, uint32_t* err,
+                                  bool* ok) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t tag = (uint64_t)epoch << 32;
     *ok = true;
     if (tile == 0) {
-        if (lane == 0 && !published) publish(desc, tag | kFlagPrefix | (agg & kValMask));
+        if (lane == 0) publish(desc, tag | kFlagPrefix | (agg & kValMask));
         return 0;
     }
-    if (lane == 0 && !published) publish(desc + tile, tag | kFlagAgg | (agg & kValMask));
+    if (lane == 0) publish(desc + tile, tag | kFlagAgg | (agg & kValMask));
     uint32_t excl = 0;
     int64_t base = (int64_t)tile;
     uint32_t spins = 0;
@@ -397,25 +290,19 @@ __device__ uint32_t lookback_warp(uint64_t* desc, uint32_t tile, uint32_t epoch,
             if (spins > 32) __nanosleep(100);
             continue;
         }
-        uint32_t v = (lane <= stop) ? (uint32_t)(d & kValMask) : 0u;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const uint32_t y = __shfl_xor_sync(0xffffffffu, v, o);
-            v = lb_op<kMax>(v, y);
-        }
-        excl = lb_op<kMax>(excl, v);
+        excl += __reduce_add_sync(0xffffffffu, lane <= stop ? (uint32_t)(d & kValMask) : 0u);
         if (stop < 32u) break;
         base -= 32;
     }
-    if (lane == 0) publish(desc + tile, tag | kFlagPrefix | (lb_op<kMax>(excl, agg) & kValMask));
+    if (lane == 0) publish(desc + tile, tag | kFlagPrefix | ((excl + agg) & kValMask));
     return excl;
 }
 
-// Wider warp-wide variant: each lane reads kPer predecessors per round (lane i reads tile
+// Wider variant: each lane reads kPer predecessors per round (lane i reads tile
 // base - 1 - i - 32 k), so 32 kPer tiles are crossed per memory round trip. Kernels whose
 // first wave holds hundreds of tiles that all publish their aggregates at once use it:
 // the last tile of such a wave finds the nearest inclusive prefix in a few rounds.
-template <bool kMax, int kPer>
+template <int kPer>
 __device__ uint32_t lookback_warp_wide(uint64_t* desc, uint32_t tile, uint32_t epoch, uint32_t agg, uint32_t* err,
                                        bool* ok) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -468,13 +355,12 @@ __device__ uint32_t lookback_warp_wide(uint64_t* desc, uint32_t tile, uint32_t e
         uint32_t v = 0;
 #pragma unroll
         for (int k = 0; k < kPer; ++k)
-            if (lane + 32u * (uint32_t)k <= lim) v = lb_op<kMax>(v, (uint32_t)(d[k] & kValMask));
-        v = kMax ? __reduce_max_sync(0xffffffffu, v) : __reduce_add_sync(0xffffffffu, v);
-        excl = lb_op<kMax>(excl, v);
+            if (lane + 32u * (uint32_t)k <= lim) v += (uint32_t)(d[k] & kValMask);
+        excl += __reduce_add_sync(0xffffffffu, v);
         if (stop != 0xffffffffu) break;
         base -= 32 * kPer;
     }
-    if (lane == 0) publish(desc + tile, tag | kFlagPrefix | (lb_op<kMax>(excl, agg) & kValMask));
+    if (lane == 0) publish(desc + tile, tag | kFlagPrefix | ((excl + agg) & kValMask));
     return excl;
 }
 

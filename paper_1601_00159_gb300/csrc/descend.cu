@@ -1,4 +1,4 @@
-// K2 + K3: descend the index layer to each query's interception (Algorithm 2,
+// Descend the index layer to each query's interception (Algorithm 2,
 // Definition 4), then locate the query's key in the storage layer (Algorithm 4's
 // getNode), for every distinct key of the sorted batch.
 //

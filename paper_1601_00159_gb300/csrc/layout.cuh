@@ -39,7 +39,7 @@ __device__ __forceinline__ void level_layout(const RebuildArgs& a, bool merged) 
     const uint32_t chg = __ldcg(&bm->chg_hist[l]) + (l == 32u ? __ldcg(&bm->chg_hist[33]) : 0u);
     uint32_t tombs = (uint32_t)((int32_t)__ldcg(&m->tombs) + __ldcg(&bm->tomb_delta));
     uint32_t size = __ldcg(&m->size), cur = __ldcg(&m->cur), lcur = __ldcg(&m->lcur);
-    const uint32_t oH = __ldcg(&m->H), oLb = __ldcg(&m->Lb), old_total = __ldcg(&m->index_total);
+    const uint32_t oH = __ldcg(&m->H), oLb = __ldcg(&m->Lb);
     const uint32_t exact = __ldcg(&m->levels_exact), dirty = __ldcg(&bm->index_dirty);
     const uint32_t updates = __ldcg(&m->updates) + __ldcg(&bm->changes);
     const uint32_t newc = __ldcg(&bm->new_count), big = __ldcg(&bm->fix_big);
@@ -114,7 +114,6 @@ __device__ __forceinline__ void level_layout(const RebuildArgs& a, bool merged) 
     }
     if (lane == 0) {
         bm->old_H = oH;
-        bm->old_total = old_total;
         bm->inc = inc ? 1u : 0u;
         m->H = H;
         m->Lb = Lb;

@@ -1,9 +1,9 @@
 // Host side of the C ABI (include/pi.h): owns the device state of an index and
 // enqueues the batch pipeline of Algorithm 1 on the caller's stream:
-//   K0/K1 pack + radix sort  ->  K2/K3 descent + locate  ->  K4/K5 ownership + apply
-//   ->  K6 merge + level layout + rebuild  ->  async copy of the small device meta to
-//   a pinned mailbox (used only to tighten capacity bounds; never waited on, except
-//   when a bound could be exceeded).
+//   radix sort  ->  descent + locate  ->  ownership + apply
+//   ->  merge + level layout + rebuild; the batch's last step writes the small device
+//   meta to a pinned mailbox (used only to tighten capacity bounds; never waited on,
+//   except when a bound could be exceeded).
 
 #include <cstdio>
 #include <cstddef>

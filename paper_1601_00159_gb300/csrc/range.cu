@@ -10,8 +10,8 @@
 //   k_range_write  offsets[i] and, when the query's pairs fit in the caller's capacity,
 //                  its keys and values.
 // A lane per bound searches the index; sorting the bounds first, as a batch's keys are, took
-// twelve launches and gained nothing back: with 2^16 ranges on 2^24 keys 173 us a call against
-// 70, with 2^20 ranges 465 against 272.
+// twelve launches and gained nothing back: with 2^16 ranges on 2^24 keys 173 us of kernels
+// against 70, with 2^20 ranges 465 us a call against 272.
 // A warp takes up to 32 consecutive queries as one run of nodes, so that its lanes are busy
 // whatever the slices' lengths, its loads are consecutive nodes and its stores consecutive
 // pairs; fewer queries per warp when the queries would not fill the chip. (A warp per query, each

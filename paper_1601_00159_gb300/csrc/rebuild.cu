@@ -1,4 +1,4 @@
-// K6: storage-layer merge and index-layer rebuild (Sections 4.1 and 4.4.4), plus the
+// Storage-layer merge and index-layer rebuild (Sections 4.1 and 4.4.4), plus the
 // bulk build of a new index (Section 3.1) and the test-support export.
 //
 // Storage layer: contiguous sorted arrays keys / vals / meta (meta = height | F_del),
@@ -10,14 +10,14 @@
 // Rebuild: the paper's daemon scans the storage layer and puts the key of every
 // valid node of height > 1 into the index-layer arrays. Here one pass over the storage
 // layer does it for all levels at once: per tile of 4096 nodes, keys and meta arrive in
-// shared memory by TMA bulk copy; the tile counts its live nodes of height >= l for
-// every level l; one decoupled look-back per level (a warp, one lane per level) gives
-// the tile's offset in each level; then level by level the tile compacts its nodes of
-// height >= l (a prefix sum) and writes them with their down pointers.
+// shared memory by TMA bulk copy, and level by level the tile compacts its nodes of
+// height >= l (a prefix sum) and writes them with their down pointers, from the tile's offset
+// in the level on. The offsets are a scan of the tiles' counts, which the kernels that change
+// the nodes keep current.
 //
 // Level sizes are not counted by the rebuild: the apply kernel keeps them current as
-// deltas, so the layout (level bases, sentinels, staging split) is known before the
-// pass and the pass writes every entry exactly once.
+// deltas, so the layout (level bases, sentinels) is known before the pass and the pass writes
+// every entry exactly once.
 
 #include <cstddef>
 
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_merge(RebuildArgs a, uint32_t e
     if (warp == 0) {
         __threadfence();
         bool ok = true;
-        const uint32_t ex = lookback_warp_wide<false, 8>(a.desc, cta, epoch, live, a.err, &ok);
+        const uint32_t ex = lookback_warp_wide<8>(a.desc, cta, epoch, live, a.err, &ok);
         __threadfence();
         if (lane == 0) {
             s_pref = ex;
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(1024) k_rebuild_prep(RebuildArgs a, uint32_t e
     if (threadIdx.x < 32) {
         bool ok;
         // descriptors: one row of 64 chunks per level (level counts of 2^30 nodes fit)
-        const uint32_t ex = lookback_warp<false>(a.desc + (size_t)blockIdx.y * 64, chunk, epoch, tot, a.err, &ok);
+        const uint32_t ex = lookback_warp(a.desc + (size_t)blockIdx.y * 64, chunk, epoch, tot, a.err, &ok);
         if (threadIdx.x == 0) {
             s_prefix = ex;
             s_ok = ok ? 1 : 0;
@@ -733,7 +733,7 @@ __device__ __forceinline__ bool place_rows(Rows& R, uint64_t* desc, uint32_t epo
             x += c[k];
         }
         bool ok;
-        const uint32_t ex = lookback_warp_wide<false, 4>(desc, R.tile, epoch, tot, err, &ok);
+        const uint32_t ex = lookback_warp_wide<4>(desc, R.tile, epoch, tot, err, &ok);
         if (lane == 0) {
             R.prefix = ex;
             R.total = tot;
@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(kThreads) k_export_live(Storage st, const DevM
 // bounded look-back must give up, record kErrTimeout and return.
 __global__ void k_wait_selftest(uint64_t* desc, uint32_t* err) {
     bool ok = true;
-    lookback_warp<false>(desc, 1u, 1u, 0u, err, &ok);
+    lookback_warp(desc, 1u, 1u, 0u, err, &ok);
 }
 
 }  // namespace

@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_fix(uint32_t n, SortBuffers s
 // ---------------------------------------------------------------------------------
 // Small batches (at most kSmallSort queries): instead of the radix pipeline's chain of
 // dependent launches, every CTA sorts one tile of kRunTile consecutive queries by
-// (key, arrival) in shared memory and leaves it sorted in the packed buffers; the descent's
+// (key, arrival) in shared memory and leaves it sorted in in_k / in_p; the descent's
 // k_rank_locate then finds each query's place among the other tiles. Such a batch is bound
 // by launches and dependent latency, not by memory. A warp orders runs of 8 by counting,
 // then the runs merge pairwise: an element's place is its place in its own run plus the count
