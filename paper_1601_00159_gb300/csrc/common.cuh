@@ -201,6 +201,11 @@ __device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p) {
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ uint32_t ld_relaxed32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 // Publishes a look-back descriptor. An atomic exchange is performed at L2, where the
 // readers' relaxed loads look; a plain relaxed store was measured to take several
 // microseconds to become visible to them (a decoupled look-back waited 7.9 us per tile
@@ -757,9 +762,8 @@ inline cudaError_t launch_dep(void (*kernel)(KP...), dim3 grid, dim3 block, size
     return e;
 }
 
-cudaError_t launch_rebuild(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms);
-cudaError_t launch_rebuild_prep(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms);
-cudaError_t launch_rebuild_write(const RebuildArgs& a, cudaStream_t s, int num_sms);
+cudaError_t launch_rebuild_count(const RebuildArgs& a, cudaStream_t s, int num_sms);  // when forced
+cudaError_t launch_rebuild_write(const RebuildArgs& a, bool fused, uint32_t& epoch, cudaStream_t s, int num_sms);
 
 // Bulk build: sorted (key, payload) -> storage layer (last duplicate wins) + counts.
 struct CreateArgs {

@@ -886,9 +886,10 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     // the rebuild, in the background
     cudaStreamWaitEvent(x->rs, x->ev[slot], 0);
     prof_mark(x, 7, x->rs);
-    if ((e = launch_rebuild_prep(ra, ep, x->rs, x->num_sms)) != cudaSuccess) return map_cuda(e);
+    // the counts are recounted when the rebuild is forced (unless the batch merged)
+    if (ra.force_rebuild && (e = launch_rebuild_count(ra, x->rs, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 8, x->rs);
-    if ((e = launch_rebuild_write(ra, x->rs, x->num_sms)) != cudaSuccess) return map_cuda(e);
+    if ((e = launch_rebuild_write(ra, small, ep, x->rs, x->num_sms)) != cudaSuccess) return map_cuda(e);
     prof_mark(x, 9, x->rs);
     cudaEventRecord(x->ev_rebuilt, x->rs);
     x->rebuild_pending = true;
@@ -1082,7 +1083,8 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         RebuildArgs ra = rebuild_args(x, x->d_bm, (uint32_t)hm.size, 2u);
         uint32_t ep = next_epochs(x, 4, s);
         if ((e = launch_level_layout(ra, s)) != cudaSuccess) break;
-        if ((e = launch_rebuild(ra, ep, s, x->num_sms)) != cudaSuccess) break;
+        if ((e = launch_rebuild_count(ra, s, x->num_sms)) != cudaSuccess) break;
+        if ((e = launch_rebuild_write(ra, false, ep, s, x->num_sms)) != cudaSuccess) break;
         x->epoch = ep;
         if ((e = read_meta(x, s, &x->known)) != cudaSuccess) break;
         x->force_rebuild = false;

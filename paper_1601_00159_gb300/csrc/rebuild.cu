@@ -30,7 +30,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kNodes = 4096;             // storage nodes per tile
 constexpr int kPer = kNodes / kThreads;  // 16 per thread
-constexpr uint32_t kCtrMerge = 9, kCtrMergeDone = 10, kCtrCreate = 11;
+constexpr uint32_t kCtrMerge = 9, kCtrMergeDone = 10, kCtrCreate = 11, kCtrRebuild = 16, kCtrPrep = 17;
 
 // ---------------------------------------------------------------------------------
 // Merge: old live nodes + new nodes -> the other storage buffer, in key order. A new node with
@@ -451,55 +451,40 @@ __global__ void __launch_bounds__(256) k_rebuild_count(RebuildArgs a) {
     }
 }
 
-// Per built level, exclusive scan of the tile counts over tiles. Grid: (chunks, levels);
-// each CTA scans kScanChunk tiles (4 per thread) and gets the prefix of the chunks
-// before it by a warp-wide decoupled look-back (the chain is a few chunks long). The
-// level's last chunk checks the total against the level size. In an incremental rebuild
-// the first CTA of each row builds a level's change list instead.
-constexpr uint32_t kScanChunk = 4096;
-
-__global__ void __launch_bounds__(1024) k_rebuild_prep(RebuildArgs a, uint32_t epoch) {
-    pdl_wait();
-    pdl_trigger();
-    __shared__ uint32_t s_tmp[33];
+// Exclusive scan, over tiles, of the tile counts of level Lb + row, in chunks of kScanChunk tiles
+// (four per thread of a kB-thread CTA): a chunk gets the sum of the chunks before it by a look-back (the chain is a
+// few chunks long). The level's last chunk checks the total against the level size.
+template <int kB>
+__device__ void scan_counts(const RebuildArgs& a, uint32_t row, uint32_t chunk, uint32_t epoch, uint32_t* s_tmp) {
     __shared__ uint32_t s_prefix;
-    __shared__ int s_ok;
+    __shared__ int s_fine;
     const DevMeta* m = a.m;
-    if (!a.bm->rebuild) return;
-    if (block_sees_error(&m->error)) return;
-    if (a.bm->inc) {  // an incremental rebuild needs its change lists, not tile offsets
-        if (blockIdx.x == 0) relevel::lists(a, blockIdx.y, s_tmp);
-        return;
-    }
-    const uint32_t H = m->H, Lb = m->Lb, size = m->size;
-    const uint32_t l = Lb + blockIdx.y;
-    if (H < Lb || size == 0 || l > H) return;
-    const uint32_t ntiles = (size + kNodes - 1) / kNodes;
+    constexpr uint32_t kScanChunk = 4 * kB;
+    const uint32_t Lb = m->Lb, l = Lb + row;
+    const uint32_t ntiles = (m->size + kNodes - 1) / kNodes;
     const uint32_t nchunks = (ntiles + kScanChunk - 1) / kScanChunk;
-    const uint32_t chunk = blockIdx.x;
-    if (chunk >= nchunks) return;
     const uint32_t* c = a.lcnt + (size_t)(l - 2) * a.lstride;
-    uint32_t* o = a.loff + (size_t)(l - Lb) * ntiles;
+    uint32_t* o = a.loff + (size_t)row * ntiles;
     const uint32_t t0 = chunk * kScanChunk + threadIdx.x * 4u;
     uint32_t v[4], sum = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        v[k] = (t0 + k < ntiles) ? c[t0 + k] : 0u;
+        v[k] = t0 + k < ntiles ? c[t0 + k] : 0u;
         sum += v[k];
     }
     uint32_t tot;
-    uint32_t run = block_excl_sum<1024>(sum, s_tmp, &tot);
+    uint32_t run = block_excl_sum<kB>(sum, s_tmp, &tot);
     if (threadIdx.x < 32) {
         bool ok;
-        // descriptors: one row of 64 chunks per level (level counts of 2^30 nodes fit)
-        const uint32_t ex = lookback_warp(a.desc + (size_t)blockIdx.y * 64, chunk, epoch, tot, a.err, &ok);
+        // descriptors: a row of nchunks words per level
+        const uint32_t ex = lookback_warp(a.desc + (size_t)row * nchunks, chunk, epoch, tot, a.err, &ok);
         if (threadIdx.x == 0) {
             s_prefix = ex;
-            s_ok = ok ? 1 : 0;
+            s_fine = ok ? 1 : 0;
         }
     }
     __syncthreads();
-    if (!s_ok) return;
+    if (!s_fine) return;
     run += s_prefix;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -508,6 +493,71 @@ __global__ void __launch_bounds__(1024) k_rebuild_prep(RebuildArgs a, uint32_t e
     }
     if (chunk == nchunks - 1 && threadIdx.x == 0 && s_prefix + tot != m->n[l])
         atomicOr(a.err, kErrBounds);  // counts disagree with the level size
+}
+
+// What the writers need first: the scans of the tile counts, or, in an incremental rebuild, a
+// change list per level. CTAs of kB threads take these units in turn, each until none is left.
+// Returns how many there are.
+template <int kB>
+__device__ uint32_t prepare_units(const RebuildArgs& a, uint32_t epoch) {
+    __shared__ uint32_t s_tmp[33], s_unit;
+    const DevMeta* m = a.m;
+    BatchMeta* bm = a.bm;
+    const bool inc = bm->inc != 0;
+    const uint32_t Lb = m->Lb, H = inc && bm->old_H > m->H ? bm->old_H : m->H;
+    const uint32_t levels = H >= Lb && m->size ? H - Lb + 1u : 0u;
+    const uint32_t ntiles = (m->size + kNodes - 1) / kNodes;
+    const uint32_t units = inc ? levels : levels * ((ntiles + 4u * kB - 1u) / (4u * kB));
+    for (;;) {
+        if (threadIdx.x == 0) s_unit = atomicAdd(&bm->tile_ctr[kCtrRebuild], 1u);
+        __syncthreads();
+        const uint32_t u = s_unit;
+        if (u >= units) return units;
+        if (inc) relevel::lists<kB>(a, u, s_tmp);
+        else scan_counts<kB>(a, u % levels, u / levels, epoch, s_tmp);  // a level's chunks in order
+        __syncthreads();  // the barrier and thread 0's fence release the unit's results
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(&bm->tile_ctr[kCtrPrep], 1u);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_rebuild_prep(RebuildArgs a, uint32_t epoch) {
+    pdl_wait();
+    pdl_trigger();
+    if (!a.bm->rebuild) return;
+    if (block_sees_error(&a.m->error)) return;
+    prepare_units<1024>(a, epoch);
+}
+
+// The same inside the writer (kFused): every CTA waits until all units are done, only for units
+// that running CTAs have taken, so the wait ends however many CTAs fit the chip at once. It is
+// bounded all the same, and an error ends it.
+// For small batches, which are bound by their launches: one less (28.1 -> 27.0 us a batch of 1000
+// look-ups, 47.7 -> 40.4 of 6000 mixed queries), with a grid that leaves half of each SM to the
+// next batch. Larger batches keep k_rebuild_prep: the waiting CTAs would hold the SMs that the
+// next batch's sort runs on (2^20 queries on 2^24 keys 359 -> 368 us a batch, 2^22 on 2^27 2% more).
+__device__ bool prepare_write(const RebuildArgs& a, uint32_t epoch) {
+    __shared__ int s_ready;
+    const uint32_t units = prepare_units<kThreads>(a, epoch);
+    if (threadIdx.x == 0) {
+        uint32_t spins = 0;
+        bool ok = true;
+        while (ok && ld_relaxed32(&a.bm->tile_ctr[kCtrPrep]) < units) {
+            ++spins;
+            if (spins > kSpinLimit) {
+                atomicOr(a.err, kErrTimeout);
+                ok = false;
+            }
+            if ((spins & 1023u) == 0 && *(volatile uint32_t*)a.err) ok = false;
+            if (spins > 32) __nanosleep(100);
+        }
+        __threadfence();  // the results are visible to the CTA past the barrier
+        s_ready = ok ? 1 : 0;
+    }
+    __syncthreads();
+    return s_ready != 0;
 }
 
 // Byte-wise arithmetic on a meta word holding four nodes (height in bits 0-5, delete
@@ -540,8 +590,7 @@ constexpr uint32_t kWarpNodes = kNodes / 8;  // 512 nodes per warp
 //     levels repeat step 3 on the shrinking list.
 // An incremental rebuild writes from the previous levels instead (relevel.cuh). One kernel
 // for both, since the host cannot know which a batch needs and a launch that only exits costs
-// it 3 us (the rebuild was five launches: 1000 lookups 47.6 -> 40.4 us a batch, 6000 mixed
-// queries 55.6 -> 50.7). Six CTAs per SM at 40 registers measured best over both kinds.
+// it 3 us. Six CTAs per SM at 40 registers measured best over both kinds.
 union WriteSmem {
     struct {
         uint8_t meta[kMetaBytes];
@@ -551,7 +600,8 @@ union WriteSmem {
     relevel::WriteSmem inc;
 };
 
-__global__ void __launch_bounds__(kThreads, 6) k_rebuild_write(RebuildArgs a) {
+template <bool kFused>
+__global__ void __launch_bounds__(kThreads, 6) k_rebuild_write(RebuildArgs a, uint32_t epoch) {
     pdl_wait();
     pdl_trigger();
     __shared__ __align__(16) WriteSmem s_u;
@@ -563,6 +613,8 @@ __global__ void __launch_bounds__(kThreads, 6) k_rebuild_write(RebuildArgs a) {
     const DevMeta* m = a.m;
     if (!a.bm->rebuild) return;
     if (block_sees_error(&m->error)) return;
+    if (!a.bm->inc && (m->H < m->Lb || m->size == 0)) return;
+    if (kFused && !prepare_write(a, epoch)) return;
     if (a.bm->inc) {
         relevel::write(a, blockIdx.x, gridDim.x, s_u.inc);
         return;
@@ -571,7 +623,6 @@ __global__ void __launch_bounds__(kThreads, 6) k_rebuild_write(RebuildArgs a) {
     uint32_t* s_list = s_u.full.list;
     auto& s_wcnt = s_u.full.wcnt;
     const uint32_t H = m->H, Lb = m->Lb, size = m->size, cur = m->cur;
-    if (H < Lb || size == 0) return;
     uint64_t* LK = m->lcur ? a.lkeys1 : a.lkeys;  // the index layer's buffer in use
     uint32_t* LD = m->lcur ? a.ldown1 : a.ldown;
     const uint32_t ntiles = (size + kNodes - 1) / kNodes;
@@ -885,32 +936,31 @@ cudaError_t launch_level_layout(const RebuildArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_rebuild_prep(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms) {
+cudaError_t launch_rebuild_count(const RebuildArgs& a, cudaStream_t s, int num_sms) {
     const uint32_t tiles = (a.size_ub + kNodes - 1) / kNodes + 1;
-    if (a.force_rebuild) {  // the counts are recounted (unless the batch merged)
-        const uint32_t cb = (tiles + 7) / 8, ccap = (uint32_t)num_sms * 4u;
-        launch_dep(k_rebuild_count, cb < ccap ? cb : ccap, 256, 0, s, a);
-        ++g_launches;
-    }
-    const uint32_t chunks = (tiles + kScanChunk - 1) / kScanChunk;
-    launch_dep(k_rebuild_prep, dim3(chunks, kLevelSlots - 2), 1024, 0, s, a, ++epoch);
+    const uint32_t cb = (tiles + 7) / 8, ccap = (uint32_t)num_sms * 4u;
+    launch_dep(k_rebuild_count, cb < ccap ? cb : ccap, 256, 0, s, a);
     ++g_launches;
     return cudaGetLastError();
 }
 
-cudaError_t launch_rebuild_write(const RebuildArgs& a, cudaStream_t s, int num_sms) {
-    const uint32_t cap = (uint32_t)num_sms * 6u;  // the CTAs resident at once
+cudaError_t launch_rebuild_write(const RebuildArgs& a, bool fused, uint32_t& epoch, cudaStream_t s, int num_sms) {
     // per tile of the storage layer, or of the levels and their changes (fewer but for change
-    // lists, which a batch's queries bound)
-    const uint32_t tiles = (a.size_ub + kNodes - 1) / kNodes + 1 + a.lst_cap / (2u * 256u) + kLevelSlots;
-    launch_dep(k_rebuild_write, tiles < cap ? tiles : cap, kThreads, 0, s, a);
+    // lists, which a batch's queries bound); at most the CTAs resident at once
+    const uint32_t nodes = (a.size_ub + kNodes - 1) / kNodes + 1;
+    const uint32_t tiles = nodes + a.lst_cap / (2u * 256u) + kLevelSlots, cap = (uint32_t)num_sms * (fused ? 3u : 6u);
+    const uint32_t grid = tiles < cap ? tiles : cap;
+    ++epoch;
+    if (fused) {
+        launch_dep(k_rebuild_write<true>, grid, kThreads, 0, s, a, epoch);
+    } else {
+        const uint32_t units = (nodes + 4095) / 4096 * (kLevelSlots - 2), most = (uint32_t)num_sms;
+        launch_dep(k_rebuild_prep, units < most ? units : most, 1024, 0, s, a, epoch);
+        ++g_launches;
+        launch_dep(k_rebuild_write<false>, grid, kThreads, 0, s, a, epoch);
+    }
     ++g_launches;
     return cudaGetLastError();
-}
-
-cudaError_t launch_rebuild(const RebuildArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms) {
-    cudaError_t e = launch_rebuild_prep(a, epoch, s, num_sms);
-    return e != cudaSuccess ? e : launch_rebuild_write(a, s, num_sms);
 }
 
 cudaError_t launch_create_storage(const CreateArgs& a, uint32_t& epoch, cudaStream_t s, int num_sms) {

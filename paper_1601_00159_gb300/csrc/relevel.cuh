@@ -4,9 +4,9 @@
 // lowest built level; every other key keeps its storage position. The rebuild then reads
 // the old levels (the buffer not in use after the layout step flipped DevMeta::lcur) and
 // writes the new ones, instead of scanning the storage layer and gathering member keys:
-//   lists (k_rebuild_prep)   one CTA per level l: the batch's changes of height >= l, in key
+//   lists   one CTA per level l: the batch's changes of height >= l, in key
 //                     order, with the running count (inserts - deletes) before each;
-//   write (k_rebuild_write)  every old entry moves by the running count of its level's list
+//   write   every old entry moves by the running count of its level's list
 //                     before its key (or goes, if deleted); its down pointer into level
 //                     l - 1 moves by that level's running count; every insert lands at
 //                     (old entries below its key) + (running count before it).
@@ -62,7 +62,8 @@ __device__ __forceinline__ uint32_t lb_keys(const uint64_t* K, uint32_t n, uint6
     return lo;
 }
 
-// Level Lb + row's change list, by a CTA of 1024 threads.
+// Level Lb + row's change list, by a CTA of kB threads.
+template <int kB>
 __device__ void lists(const RebuildArgs& a, uint32_t row, uint32_t* s_tmp) {
     __shared__ uint32_t s_off;
     const DevMeta* m = a.m;
@@ -80,7 +81,7 @@ __device__ void lists(const RebuildArgs& a, uint32_t row, uint32_t* s_tmp) {
     const uint32_t off = s_off, nchg = bm->nchg;
     constexpr uint32_t kPer = 8;  // consecutive changes per thread
     uint32_t carry = 0, icarry = 0;
-    for (uint32_t c0 = 0; c0 < nchg; c0 += 1024u * kPer) {
+    for (uint32_t c0 = 0; c0 < nchg; c0 += (uint32_t)kB * kPer) {
         const uint32_t i0 = c0 + threadIdx.x * kPer;
         uint32_t sm = 0, im = 0;
 #pragma unroll
@@ -93,8 +94,8 @@ __device__ void lists(const RebuildArgs& a, uint32_t row, uint32_t* s_tmp) {
             }
         }
         uint32_t tot, itot;
-        uint32_t j = carry + block_excl_sum<1024>((uint32_t)__popc(sm), s_tmp, &tot);
-        uint32_t ib = icarry + block_excl_sum<1024>((uint32_t)__popc(im), s_tmp, &itot);
+        uint32_t j = carry + block_excl_sum<kB>((uint32_t)__popc(sm), s_tmp, &tot);
+        uint32_t ib = icarry + block_excl_sum<kB>((uint32_t)__popc(im), s_tmp, &itot);
 #pragma unroll
         for (uint32_t k = 0; k < kPer; ++k) {
             if (!((sm >> k) & 1u)) continue;

@@ -250,12 +250,6 @@ __global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, B
 // next pass, and the scan those of the first.
 constexpr uint32_t kWordAgg = 1u << 30, kWordPrefix = 2u << 30, kWordMask = kWordAgg - 1u;
 
-__device__ __forceinline__ uint32_t ld_relaxed32(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // Sum of one digit's counts over the tiles before `tile`: 16 tiles' words per round, which the
 // threads of the digits read as rows. A wait that gives up records kErrTimeout and returns
 // false.
