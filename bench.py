@@ -4,7 +4,7 @@
 Default workload: the skewed configuration -- 2^27 distinct uniform uint64 keys with
 value = splitmix64(key), promotion p = 1/4, batches of 2^22 queries with Zipf(0.99)
 keys over the key set, 90% search / 5% insert / 5% delete, index layer rebuilt after
-every batch that changes it. One "step" = one pi_execute_batch: pack + sort, descent,
+every batch that changes it. One "step" = one pi_execute_batch: sort, descent and locate,
 ownership + apply, merge, layout, rebuild.
 
 Inputs are synthetic and seeded (paper_1601_00159_gb300/workloads.py), generated on

@@ -84,8 +84,8 @@ typedef struct {
                                     the lowest level l whose expected storage gap (1/P)^(l-1)
                                     is at least 32 nodes (4 for P = 1/4), since on the GPU the
                                     storage search interpolates within a gap and reads about
-                                    one 64-byte line of it, while every built level costs a
-                                    rebuild pass and a descent step. 2 builds every level, as
+                                    one 64-byte line of it, while every built level costs
+                                    rebuild work and descent probes. 2 builds every level, as
                                     the paper does. Levels below it still count in
                                     pi_info's level sizes; pi_export_level reports them as
                                     PI_ERR_NOT_BUILT. */
@@ -104,10 +104,10 @@ typedef struct {
                                     runs as one launch, the batching form's pipeline on a
                                     thread-block cluster of 16 CTAs of 16 warps (8 where 16
                                     do not fit), with the same results. Measured on a
-                                    GB300 it is about as fast as the default for such
-                                    batches (98 against 99 us for 2^14 searches on 2^16
-                                    keys; faster on the smallest batches, slower on 2^12
-                                    queries on 2^18 keys). Not taken while profiling, with
+                                    GB300 it is slower than the default (2^14 searches on
+                                    2^16 keys 90 against 26 us, 2^10 queries on 2^16 keys
+                                    74 against 26, 2^12 on 2^18 114 against 27): one launch
+                                    on 16 SMs against six on all. Not taken while profiling, with
                                     test_flags or with the deferred rebuild policy. */
 } pi_config_t;
 
