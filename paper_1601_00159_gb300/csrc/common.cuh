@@ -683,7 +683,7 @@ struct MultiArgs {
     uint64_t stride;
     uint32_t qcap;            // queries per batch the scratch holds
     uint32_t pad_;
-    DevMeta* mirror;          // copy of every processed index's meta, by index (may be null)
+    DevMeta* mirror;          // copy of every processed index's meta, by index, in pinned host memory (may be null)
 };
 
 // Range search of n queries.

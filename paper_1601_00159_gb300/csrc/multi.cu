@@ -1009,29 +1009,39 @@ __device__ void m_sentinels(const DevMeta& m, uint64_t* LK, uint32_t* LD) {
     }
 }
 
-// Publishes the index's new state (one thread).
+// Publishes the index's new state, and its copy for the host, by one warp: a call of small items
+// ends with this, a hundred words one after another on one thread. (17 indices of up to 20,000
+// keys: 75 us a call on one thread with the copy on the device, 67 so.)
 __device__ void m_publish(const MultiArgs& a, const MItem& it, const MIndex& X, const DevMeta& m) {
+    const uint32_t lane = threadIdx.x & 31u;
     DevMeta* gm = X.m;
-    gm->cur = m.cur;
-    gm->size = m.size;
-    gm->tombs = m.tombs;
-    gm->H = m.H;
-    gm->Lb = m.Lb;
-    gm->Ls = m.Ls;
-    gm->smem_entries = m.smem_entries;
-    gm->index_total = m.index_total;
-    gm->index_need = m.index_need;
-    gm->grow_request = m.grow_request;
-    gm->updates = m.updates;
-    gm->rebuilds = m.rebuilds;
-    gm->levels_exact = m.levels_exact;
-    gm->batches = m.batches;
-    for (int l = 0; l < kLevelSlots; ++l) {
+    if (lane == 0) {
+        gm->cur = m.cur;
+        gm->size = m.size;
+        gm->tombs = m.tombs;
+        gm->H = m.H;
+        gm->Lb = m.Lb;
+        gm->Ls = m.Ls;
+        gm->smem_entries = m.smem_entries;
+        gm->index_total = m.index_total;
+        gm->index_need = m.index_need;
+        gm->grow_request = m.grow_request;
+        gm->updates = m.updates;
+        gm->rebuilds = m.rebuilds;
+        gm->levels_exact = m.levels_exact;
+        gm->batches = m.batches;
+    }
+    for (int l = (int)lane; l < kLevelSlots; l += 32) {
         gm->cnt[l] = m.cnt[l];
         gm->n[l] = m.n[l];
         gm->base[l] = m.base[l];
     }
-    if (a.mirror) a.mirror[it.index] = *gm;  // the host reads the set's sizes from one copy
+    __syncwarp();
+    if (!a.mirror) return;
+    constexpr uint32_t kWords = sizeof(DevMeta) / 4;  // the host reads the set's sizes from one copy
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(gm);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(a.mirror + it.index);
+    for (uint32_t w = lane; w < kWords; w += 32u) dst[w] = src[w];
 }
 
 // Per-item shared state reset (every CTA that works on the item).
@@ -1445,7 +1455,7 @@ __device__ void m_item(const MultiArgs& a, const MItem& it, const MScratchPtrs& 
     }
 
     // ---- publish the index's new state
-    if (tid == 0) m_publish(a, it, X, sh.m);
+    if (tid < 32) m_publish(a, it, X, sh.m);
     __syncthreads();
 }
 
@@ -1804,7 +1814,7 @@ __device__ void m_item_cl(const cg::cluster_group& cl, const MultiArgs& a, const
     }
     if (me == 0) {
         __syncthreads();
-        if (tid == 0) m_publish(a, it, X, sh.m);
+        if (tid < 32) m_publish(a, it, X, sh.m);
     }
     __syncthreads();
 }

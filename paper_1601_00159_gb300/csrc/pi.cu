@@ -1520,9 +1520,9 @@ struct pi_multi {
     std::vector<MIndex> h_idx;
     pi_multi_config_t cfg{};
     MIndex* d_idx = nullptr;
-    // The indices' metas as the last call left them, and pinned copies of them per call parity,
-    // with the operation that the call was for each of its indices
-    DevMeta* d_mirror = nullptr;
+    // The indices' metas as the last call of each parity left them (pinned, written by its
+    // kernels: no copy at the call's end), with the operation that the call was for each of
+    // its indices
     DevMeta* h_mirror[2] = {};
     std::vector<std::pair<uint32_t, uint64_t>> call_ops[2];
     uint8_t* d_q = nullptr;
@@ -1592,7 +1592,6 @@ void multi_destroy(pi_multi* mx) {
     if (mx->ev_done) cudaEventDestroy(mx->ev_done);
     multi_free_graphs(mx);
     dfree(mx->d_idx);
-    dfree(mx->d_mirror);
     dfree(mx->d_q);
     for (auto& h : mx->h_q)
         if (h) cudaFreeHost(h);
@@ -1643,7 +1642,7 @@ cudaError_t multi_build_graphs(pi_multi* mx) {
             a.scratch = mx->scratch[c];
             a.stride = mx->stride[c];
             a.qcap = mx->qcap[c];
-            a.mirror = mx->d_mirror;
+            a.mirror = mx->h_mirror[p];
             const pi_multi_class_t& q = mx->cfg.cls[c];
             cudaError_t r =
                 launch_multi(a, (int)q.warps, (int)q.radix_bits, (int)q.cluster, mx->grid[c], mx->ls[c]);
@@ -1651,7 +1650,6 @@ cudaError_t multi_build_graphs(pi_multi* mx) {
             cudaEventRecord(mx->evj[c], mx->ls[c]);
             cudaStreamWaitEvent(mx->cs, mx->evj[c], 0);
         }
-        cudaMemcpyAsync(mx->h_mirror[p], mx->d_mirror, count * sizeof(DevMeta), cudaMemcpyDeviceToHost, mx->cs);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(mx->cs, &g);
         if (e == cudaSuccess && le != cudaSuccess) e = le;
@@ -1734,13 +1732,13 @@ pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi
         if ((e = cudaMemcpy(mx->d_idx, mx->h_idx.data(), count * sizeof(MIndex), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
             break;
-        if ((e = dalloc(&mx->d_mirror, count)) != cudaSuccess) break;
         mx->q_bytes = kQHeader + (uint64_t)PI_MULTI_MAX_CLASSES * count * sizeof(MItem);
         if ((e = dalloc(&mx->d_q, mx->q_bytes)) != cudaSuccess) break;
         for (int p = 0; p < 2; ++p) {
             if ((e = cudaMallocHost(reinterpret_cast<void**>(&mx->h_q[p]), mx->q_bytes)) != cudaSuccess) break;
             std::memset(mx->h_q[p], 0, mx->q_bytes);
             if ((e = cudaMallocHost(reinterpret_cast<void**>(&mx->h_mirror[p]), count * sizeof(DevMeta))) != cudaSuccess) break;
+            std::memset(static_cast<void*>(mx->h_mirror[p]), 0, count * sizeof(DevMeta));
             if ((e = cudaEventCreateWithFlags(&mx->q_free[p], cudaEventDisableTiming)) != cudaSuccess) break;
         }
         if (e != cudaSuccess) break;
