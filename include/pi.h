@@ -262,6 +262,9 @@ int pi_size(pi_index_t* idx, uint64_t* size_out_host, pi_stream_t stream);
  * pi_test_fail_allocations: the next `count` device allocations the library makes on the
  *   calling host thread fail as if the device were out of memory (0 clears). The call
  *   that hits one returns PI_ERR_OOM and leaves the index as it was.
+ * pi_test_set_error: records the error bits (1: a bounded wait gave up, 2: an internal bound
+ *   check refused an access) in the index's sticky device error word, as a kernel would.
+ *   Synchronises `stream`; the host learns of it as it would of a kernel's.
  * pi_selftest_wait: launches one CTA that waits, through the bounded look-back the batch
  *   kernels use, for a predecessor that never publishes. The wait gives up after its
  *   spin bound (on a GB300 about 1.4 s), records the timeout in a scratch error word, which
@@ -269,6 +272,7 @@ int pi_size(pi_index_t* idx, uint64_t* size_out_host, pi_stream_t stream);
  *   bound worked. Allocates and frees 516 B of device memory; synchronises `stream`.
  */
 void pi_test_fail_allocations(uint32_t count);
+int pi_test_set_error(pi_index_t* idx, uint32_t bits, pi_stream_t stream);
 int pi_selftest_wait(uint32_t* err_word_host, pi_stream_t stream);
 
 /* H, the number of levels (Definition 1: level 1 is the storage layer, so H = 1 when no

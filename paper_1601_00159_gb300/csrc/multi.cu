@@ -1009,6 +1009,25 @@ __device__ void m_sentinels(const DevMeta& m, uint64_t* LK, uint32_t* LD) {
     }
 }
 
+// The host's copy of an index's meta, by one warp. The host takes it for the state after the call,
+// so every batch of the call leaves one, also a batch that the index's error word refuses. Read
+// past L1: other SMs may have set error bits.
+__device__ __forceinline__ void m_mirror(const MultiArgs& a, const MItem& it, const DevMeta* gm) {
+    __syncwarp();
+    if (!a.mirror) return;
+    constexpr uint32_t kWords = sizeof(DevMeta) / 4;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(gm);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(a.mirror + it.index);
+    for (uint32_t w = threadIdx.x & 31u; w < kWords; w += 32u) dst[w] = __ldcg(&src[w]);
+}
+
+// A batch larger than the scratch holds (the host never queues one), by one warp.
+__device__ __forceinline__ void m_refuse(const MultiArgs& a, const MItem& it) {
+    DevMeta* gm = a.idx[it.index].m;
+    if ((threadIdx.x & 31u) == 0) atomicOr(&gm->error, kErrBounds);
+    m_mirror(a, it, gm);
+}
+
 // Publishes the index's new state, and its copy for the host, by one warp: a call of small items
 // ends with this, a hundred words one after another on one thread. (17 indices of up to 20,000
 // keys: 75 us a call on one thread with the copy on the device, 67 so.)
@@ -1036,12 +1055,7 @@ __device__ void m_publish(const MultiArgs& a, const MItem& it, const MIndex& X, 
         gm->n[l] = m.n[l];
         gm->base[l] = m.base[l];
     }
-    __syncwarp();
-    if (!a.mirror) return;
-    constexpr uint32_t kWords = sizeof(DevMeta) / 4;  // the host reads the set's sizes from one copy
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(gm);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(a.mirror + it.index);
-    for (uint32_t w = lane; w < kWords; w += 32u) dst[w] = src[w];
+    m_mirror(a, it, gm);
 }
 
 // Per-item shared state reset (every CTA that works on the item).
@@ -1357,7 +1371,10 @@ __device__ void m_item(const MultiArgs& a, const MItem& it, const MScratchPtrs& 
     uint32_t* err = &X.m->error;
 
     m_begin<kT>(X, sh);
-    if (sh.m.error || n == 0) return;
+    if (sh.m.error || n == 0) {
+        if (tid < 32) m_mirror(a, it, X.m);
+        return;
+    }
     const uint32_t cur = sh.m.cur;
     uint64_t* SK = X.st.keys[cur];
     uint64_t* SV = X.st.vals[cur];
@@ -1564,7 +1581,10 @@ __device__ void m_item_cl(const cg::cluster_group& cl, const MultiArgs& a, const
     // Every CTA reads the index's meta before the first cluster barrier; no CTA of the
     // cluster writes it before that barrier, so all start from the same copy.
     m_begin<kT>(X, sh);
-    if (sh.m.error || n == 0) return;
+    if (sh.m.error || n == 0) {
+        if (me == 0 && tid < 32) m_mirror(a, it, X.m);
+        return;
+    }
     const uint32_t cur = sh.m.cur;
     uint64_t* SK = X.st.keys[cur];
     uint64_t* SV = X.st.vals[cur];
@@ -1834,7 +1854,7 @@ __global__ void __launch_bounds__(kW * 32) k_multi(MultiArgs a) {
         if (item >= nitems) break;
         const MItem it = a.items[item];
         if (it.n <= a.qcap) m_item<kT, kBits>(a, it, s, dsm, sh);
-        else if (threadIdx.x == 0) atomicOr(&a.idx[it.index].m->error, kErrBounds);
+        else if (threadIdx.x < 32) m_refuse(a, it);
         __syncthreads();
     }
 }
@@ -1858,7 +1878,7 @@ __global__ void __launch_bounds__(kW * 32) k_multi_cl(MultiArgs a) {
         if (item >= nitems) break;
         const MItem it = a.items[item];
         if (it.n <= a.qcap) m_item_cl<kT, kBits>(cl, a, it, s, dsm, sh, cx);
-        else if (me == 0 && threadIdx.x == 0) atomicOr(&a.idx[it.index].m->error, kErrBounds);
+        else if (me == 0 && threadIdx.x < 32) m_refuse(a, it);
         cl.sync();  // rank 0 takes the next slot only after every CTA has read this one
     }
     cl.sync();  // no CTA leaves while another may still read its shared memory

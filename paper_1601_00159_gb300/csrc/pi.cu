@@ -1395,6 +1395,16 @@ int pi_info(pi_index_t* x, pi_info_t* out, pi_stream_t stream) {
 
 void pi_test_fail_allocations(uint32_t count) { g_fail_allocs = count; }
 
+int pi_test_set_error(pi_index_t* x, uint32_t bits, pi_stream_t stream) {
+    if (!x) return PI_ERR_INVALID_ARG;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    order_after_last(x, s);
+    wait_rebuild(x, s);
+    cudaError_t e = cudaMemcpyAsync(&x->d_meta->error, &bits, sizeof(bits), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return map_cuda(e);
+}
+
 int pi_selftest_wait(uint32_t* err_word_host, pi_stream_t stream) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     uint64_t* desc = nullptr;
