@@ -653,8 +653,10 @@ cudaError_t grow_index(pi_index* x, uint64_t need, cudaStream_t s) {
         cudaMemcpyAsync(na.k0, ok, used * 8, cudaMemcpyDeviceToDevice, s);
         cudaMemcpyAsync(na.d0, od, used * 4, cudaMemcpyDeviceToDevice, s);
     }
-    const uint32_t zero = 0;
-    cudaMemcpyAsync(&x->d_meta->lcur, &zero, sizeof(zero), cudaMemcpyHostToDevice, s);
+    cudaMemsetAsync(&x->d_meta->lcur, 0, sizeof(uint32_t), s);
+    // granted: the next states that the device reports must not ask again (a batching-form call
+    // lays the levels out anew only when they change)
+    cudaMemsetAsync(&x->d_meta->grow_request, 0, sizeof(uint32_t), s);
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         dfree(na.k0);
