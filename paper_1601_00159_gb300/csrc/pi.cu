@@ -263,7 +263,10 @@ uint64_t desc_need(uint64_t q, uint64_t s) {
     return (m > c ? m : c) + 64;
 }
 
-cudaError_t ensure_desc(pi_index* x, uint64_t words) {
+// Clears of new arrays go to the stream whose work uses them next (`s`): the legacy stream's
+// order says nothing about the library's own streams, which do not block on it, and a clear that
+// it holds back behind other work would wipe what has been written meanwhile.
+cudaError_t ensure_desc(pi_index* x, uint64_t words, cudaStream_t s) {
     if (words <= x->desc_words) return cudaSuccess;
     dfree(x->desc);
     cudaError_t e = dalloc(&x->desc, words);
@@ -271,32 +274,32 @@ cudaError_t ensure_desc(pi_index* x, uint64_t words) {
         x->desc_words = 0;
         return e;
     }
-    e = cudaMemset(x->desc, 0, words * sizeof(uint64_t));
+    e = cudaMemsetAsync(x->desc, 0, words * sizeof(uint64_t), s);
     x->desc_words = words;
     return e;
 }
 
 // Per-level per-tile counts are rows of (storage capacity / 4096 + 2) tiles; a new
 // capacity reallocates them and the next rebuild recounts (force_rebuild).
-cudaError_t ensure_tile_cnt(pi_index* x, uint64_t st_cap) {
+cudaError_t ensure_tile_cnt(pi_index* x, uint64_t st_cap, cudaStream_t s) {
     const uint64_t stride = st_cap / 4096 + 2;
     if (stride <= x->lstride) return cudaSuccess;
     dfree(x->lcnt);
     cudaError_t e = dalloc(&x->lcnt, 64 * stride);  // the offsets follow the counts
     x->loff = e == cudaSuccess ? x->lcnt + 32 * stride : nullptr;
-    if (e == cudaSuccess) e = cudaMemset(x->lcnt, 0, 32 * stride * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemsetAsync(x->lcnt, 0, 32 * stride * sizeof(uint32_t), s);
     x->lstride = (e == cudaSuccess) ? (uint32_t)stride : 0u;
     x->force_rebuild = true;
     return e;
 }
 
 // PI_TEST_OWNER_CHECK: one zeroed write counter per storage node.
-cudaError_t ensure_wcount(pi_index* x, uint64_t st_cap) {
+cudaError_t ensure_wcount(pi_index* x, uint64_t st_cap, cudaStream_t s) {
     if (!(x->test_flags & PI_TEST_OWNER_CHECK) || x->wcap >= st_cap) return cudaSuccess;
     dfree(x->wcount);
     x->wcap = 0;
     cudaError_t e = dalloc(&x->wcount, st_cap + 1);
-    if (e == cudaSuccess) e = cudaMemset(x->wcount, 0, (st_cap + 1) * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemsetAsync(x->wcount, 0, (st_cap + 1) * sizeof(uint32_t), s);
     if (e == cudaSuccess) x->wcap = st_cap;
     return e;
 }
@@ -412,7 +415,7 @@ void free_storage(Storage& st) {
     st = Storage{};
 }
 
-cudaError_t alloc_storage(Storage& st, uint64_t cap) {
+cudaError_t alloc_storage(Storage& st, uint64_t cap, cudaStream_t s) {
     const uint64_t c = storage_alloc(cap);
     uint8_t* slab = nullptr;
     cudaError_t e = dalloc(&slab, 4 * al256(c * 8) + 2 * al256(c));
@@ -423,7 +426,7 @@ cudaError_t alloc_storage(Storage& st, uint64_t cap) {
         v.take(st.vals[i], c * 8);
     }
     for (int i = 0; i < 2; ++i) v.take(st.meta[i], c);
-    e = cudaMemset(st.meta[0], 0, 2 * al256(c));
+    e = cudaMemsetAsync(st.meta[0], 0, 2 * al256(c), s);
     if (e != cudaSuccess) free_storage(st);
     return e;
 }
@@ -618,7 +621,7 @@ cudaError_t grow_storage(pi_index* x, uint64_t need, cudaStream_t s) {
     uint64_t cap = need + need / 2 + kMinStorage;
     if (cap > PI_MAX_KEYS) cap = PI_MAX_KEYS;
     Storage ns{};
-    cudaError_t e = alloc_storage(ns, cap);
+    cudaError_t e = alloc_storage(ns, cap, s);
     if (e != cudaSuccess) return e;
     const uint32_t cur = x->known.cur;
     const uint64_t cnt = (uint64_t)x->known.size + 1;  // with the sentinel
@@ -635,9 +638,9 @@ cudaError_t grow_storage(pi_index* x, uint64_t need, cudaStream_t s) {
     x->st = ns;
     x->st_cap = cap;
     x->known.cur = 0;
-    if ((e = ensure_tile_cnt(x, cap)) != cudaSuccess) return e;
-    if ((e = ensure_wcount(x, cap)) != cudaSuccess) return e;
-    return ensure_desc(x, desc_need(x->sc.cap, cap));
+    if ((e = ensure_tile_cnt(x, cap, s)) != cudaSuccess) return e;
+    if ((e = ensure_wcount(x, cap, s)) != cudaSuccess) return e;
+    return ensure_desc(x, desc_need(x->sc.cap, cap), s);
 }
 
 cudaError_t grow_index(pi_index* x, uint64_t need, cudaStream_t s) {
@@ -682,7 +685,7 @@ cudaError_t grow_scratch(pi_index* x, uint64_t n, cudaStream_t s) {
     q = std::min<uint64_t>(std::max<uint64_t>(q, 4096), std::max<uint64_t>(n, PI_MAX_BATCH));
     free_scratch(x->sc);
     if ((e = alloc_scratch(x->sc, q)) != cudaSuccess) return e;
-    return ensure_desc(x, desc_need(q, x->st_cap));
+    return ensure_desc(x, desc_need(q, x->st_cap), s);
 }
 
 // Whether a batch's descent takes windows of the lowest built level, by the host's last view of
@@ -1020,11 +1023,11 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         if ((e = cudaEventCreateWithFlags(&x->ev_last, cudaEventDisableTiming)) != cudaSuccess) break;
         cudaMemsetAsync(x->d_meta, 0, sizeof(DevMeta), s);
         cudaMemsetAsync(x->d_bm, 0, 2 * sizeof(BatchMeta), s);
-        if ((e = alloc_storage(x->st, st_cap)) != cudaSuccess) break;
+        if ((e = alloc_storage(x->st, st_cap, s)) != cudaSuccess) break;
         x->st_cap = st_cap;
-        if ((e = ensure_tile_cnt(x, st_cap)) != cudaSuccess) break;
-        if ((e = ensure_wcount(x, st_cap)) != cudaSuccess) break;
-        if ((e = ensure_desc(x, desc_need(n, st_cap))) != cudaSuccess) break;
+        if ((e = ensure_tile_cnt(x, st_cap, s)) != cudaSuccess) break;
+        if ((e = ensure_wcount(x, st_cap, s)) != cudaSuccess) break;
+        if ((e = ensure_desc(x, desc_need(n, st_cap), s)) != cudaSuccess) break;
         // 1. sort (key, arrival) and keep the last of every key run
         if (n > 0) {
             if ((e = alloc_sort_scratch(tmp, n)) != cudaSuccess) break;
