@@ -261,7 +261,8 @@ int pi_size(pi_index_t* idx, uint64_t* size_out_host, pi_stream_t stream);
  * Failure-path support (no counterpart in the paper).
  * pi_test_fail_allocations: the next `count` device allocations the library makes on the
  *   calling host thread fail as if the device were out of memory (0 clears). The call
- *   that hits one returns PI_ERR_OOM and leaves the index as it was.
+ *   that hits one returns PI_ERR_OOM and leaves the index as it was, or does without.
+ *   pi_test_skip_allocations, called after it: the next `count` succeed before those.
  * pi_test_set_error: records the error bits (1: a bounded wait gave up, 2: an internal bound
  *   check refused an access) in the index's sticky device error word, as a kernel would.
  *   Synchronises `stream`; the host learns of it as it would of a kernel's.
@@ -272,6 +273,7 @@ int pi_size(pi_index_t* idx, uint64_t* size_out_host, pi_stream_t stream);
  *   bound worked. Allocates and frees 516 B of device memory; synchronises `stream`.
  */
 void pi_test_fail_allocations(uint32_t count);
+void pi_test_skip_allocations(uint32_t count);
 int pi_test_set_error(pi_index_t* idx, uint32_t bits, pi_stream_t stream);
 int pi_selftest_wait(uint32_t* err_word_host, pi_stream_t stream);
 

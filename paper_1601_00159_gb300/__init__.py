@@ -20,7 +20,8 @@ PI_MAX_BATCH = 1 << 28
 PI_MAX_KEYS = (1 << 30) - 2
 
 EXPORTED = ["pi_create", "pi_create_ex", "pi_execute_batch", "pi_execute_batch_host", "pi_destroy",
-            "pi_last_error", "pi_status", "pi_info", "pi_size", "pi_test_fail_allocations", "pi_test_set_error",
+            "pi_last_error", "pi_status", "pi_info", "pi_size", "pi_test_fail_allocations",
+            "pi_test_skip_allocations", "pi_test_set_error",
             "pi_selftest_wait", "pi_num_levels", "pi_export", "pi_export_level", "pi_export_storage", "pi_profile",
             "pi_profile_read", "pi_profile_kernels", "pi_execute_batch_noalloc", "pi_flush",
             "pi_range_search", "pi_multi_create", "pi_multi_execute", "pi_multi_destroy", "pi_multi_kernels_per_call",
@@ -129,6 +130,8 @@ def load_library(path: str = LIB_PATH):
     lib.pi_info.argtypes = [vp, ctypes.POINTER(PiInfo), vp]
     lib.pi_test_fail_allocations.restype = None
     lib.pi_test_fail_allocations.argtypes = [ctypes.c_uint32]
+    lib.pi_test_skip_allocations.restype = None
+    lib.pi_test_skip_allocations.argtypes = [ctypes.c_uint32]
     lib.pi_test_set_error.restype = i32
     lib.pi_test_set_error.argtypes = [vp, ctypes.c_uint32, vp]
     lib.pi_selftest_wait.restype = i32
@@ -222,10 +225,11 @@ def _chk(rc: int, what: str):
         raise PiError(rc, what)
 
 
-def test_fail_allocations(count: int) -> None:
-    """The next `count` device allocations of the library on this thread fail as out of
-    memory (pi_test_fail_allocations)."""
+def test_fail_allocations(count: int, skip: int = 0) -> None:
+    """After `skip` more, the next `count` device allocations of the library on this thread fail
+    as out of memory (pi_test_fail_allocations, pi_test_skip_allocations)."""
     load_library().pi_test_fail_allocations(count)
+    load_library().pi_test_skip_allocations(skip)
 
 
 def test_set_error(index, bits: int, stream=None) -> None:

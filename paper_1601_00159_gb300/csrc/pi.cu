@@ -214,18 +214,27 @@ struct pi_index {
 
 namespace {
 
-// pi_test_fail_allocations: device allocations of this host thread still to fail.
-thread_local uint32_t g_fail_allocs = 0;
+// pi_test_fail_allocations, pi_test_skip_allocations: device allocations of this host thread still to
+// fail, and those that succeed before them.
+thread_local uint32_t g_fail_allocs = 0, g_skip_allocs = 0;
 
 template <typename T>
 cudaError_t dalloc(T** p, uint64_t count) {
     *p = nullptr;
-    if (g_fail_allocs > 0) {  // injected failure, as if the device were out of memory
-        --g_fail_allocs;
-        return cudaErrorMemoryAllocation;
-    }
     if (count == 0) count = 1;
-    return cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T));
+    uint64_t bytes = count * sizeof(T);
+    if (g_skip_allocs > 0) {
+        --g_skip_allocs;
+    } else if (g_fail_allocs > 0) {  // injected failure: more than any device has
+        --g_fail_allocs;
+        bytes = 1ull << 60;
+    }
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();  // the caller reports it, or does without: the launches after it are not at fault
+    }
+    return e;
 }
 
 template <typename T>
@@ -263,45 +272,69 @@ uint64_t desc_need(uint64_t q, uint64_t s) {
     return (m > c ? m : c) + 64;
 }
 
-// Clears of new arrays go to the stream whose work uses them next (`s`): the legacy stream's
-// order says nothing about the library's own streams, which do not block on it, and a clear that
-// it holds back behind other work would wipe what has been written meanwhile.
-cudaError_t ensure_desc(pi_index* x, uint64_t words, cudaStream_t s) {
-    if (words <= x->desc_words) return cudaSuccess;
-    dfree(x->desc);
-    cudaError_t e = dalloc(&x->desc, words);
-    if (e != cudaSuccess) {
-        x->desc_words = 0;
-        return e;
+// The arrays beside the storage layer whose sizes follow the capacities.
+struct SideArrays {
+    uint64_t* desc = nullptr;    // look-back words
+    uint32_t* lcnt = nullptr;    // per-level per-tile counts: rows of (storage capacity / 4096 + 2) tiles
+    uint32_t* wcount = nullptr;  // PI_TEST_OWNER_CHECK: one write counter per storage node
+    uint64_t words = 0, stride = 0, wcap = 0;
+};
+
+void free_side(SideArrays& n) {
+    dfree(n.desc);
+    dfree(n.lcnt);
+    dfree(n.wcount);
+    n = SideArrays{};
+}
+
+// Allocates and clears those that are too small for batches of q queries and st_cap nodes. Nothing
+// of the index changes before use_side, so a growth allocates all that it needs first and leaves
+// the index as it was when some of it cannot be had. Clears go to the stream whose work uses the
+// arrays next: the legacy stream's order says nothing about the library's own streams, which do
+// not block on it, and a clear that it holds back behind other work would wipe what has been
+// written meanwhile.
+cudaError_t alloc_side(const pi_index* x, uint64_t q, uint64_t st_cap, cudaStream_t s, SideArrays& n) {
+    const uint64_t words = desc_need(q, st_cap), stride = st_cap / 4096 + 2;
+    cudaError_t e = cudaSuccess;
+    if (words > x->desc_words) {
+        n.words = words;
+        e = dalloc(&n.desc, words);
+        if (e == cudaSuccess) e = cudaMemsetAsync(n.desc, 0, words * sizeof(uint64_t), s);
     }
-    e = cudaMemsetAsync(x->desc, 0, words * sizeof(uint64_t), s);
-    x->desc_words = words;
+    if (e == cudaSuccess && stride > x->lstride) {
+        n.stride = stride;
+        e = dalloc(&n.lcnt, 64 * stride);  // the offsets follow the counts
+        if (e == cudaSuccess) e = cudaMemsetAsync(n.lcnt, 0, 32 * stride * sizeof(uint32_t), s);
+    }
+    if (e == cudaSuccess && (x->test_flags & PI_TEST_OWNER_CHECK) && x->wcap < st_cap) {
+        n.wcap = st_cap;
+        e = dalloc(&n.wcount, st_cap + 1);
+        if (e == cudaSuccess) e = cudaMemsetAsync(n.wcount, 0, (st_cap + 1) * sizeof(uint32_t), s);
+    }
+    if (e != cudaSuccess) free_side(n);
     return e;
 }
 
-// Per-level per-tile counts are rows of (storage capacity / 4096 + 2) tiles; a new
-// capacity reallocates them and the next rebuild recounts (force_rebuild).
-cudaError_t ensure_tile_cnt(pi_index* x, uint64_t st_cap, cudaStream_t s) {
-    const uint64_t stride = st_cap / 4096 + 2;
-    if (stride <= x->lstride) return cudaSuccess;
-    dfree(x->lcnt);
-    cudaError_t e = dalloc(&x->lcnt, 64 * stride);  // the offsets follow the counts
-    x->loff = e == cudaSuccess ? x->lcnt + 32 * stride : nullptr;
-    if (e == cudaSuccess) e = cudaMemsetAsync(x->lcnt, 0, 32 * stride * sizeof(uint32_t), s);
-    x->lstride = (e == cudaSuccess) ? (uint32_t)stride : 0u;
-    x->force_rebuild = true;
-    return e;
-}
-
-// PI_TEST_OWNER_CHECK: one zeroed write counter per storage node.
-cudaError_t ensure_wcount(pi_index* x, uint64_t st_cap, cudaStream_t s) {
-    if (!(x->test_flags & PI_TEST_OWNER_CHECK) || x->wcap >= st_cap) return cudaSuccess;
-    dfree(x->wcount);
-    x->wcap = 0;
-    cudaError_t e = dalloc(&x->wcount, st_cap + 1);
-    if (e == cudaSuccess) e = cudaMemsetAsync(x->wcount, 0, (st_cap + 1) * sizeof(uint32_t), s);
-    if (e == cudaSuccess) x->wcap = st_cap;
-    return e;
+// Puts them in use in place of the index's (no work of the index is in flight).
+void use_side(pi_index* x, SideArrays& n) {
+    if (n.desc) {
+        dfree(x->desc);
+        x->desc = n.desc;
+        x->desc_words = n.words;
+    }
+    if (n.lcnt) {
+        dfree(x->lcnt);
+        x->lcnt = n.lcnt;
+        x->loff = n.lcnt + 32 * n.stride;
+        x->lstride = (uint32_t)n.stride;
+        x->force_rebuild = true;  // the next rebuild recounts
+    }
+    if (n.wcount) {
+        dfree(x->wcount);
+        x->wcount = n.wcount;
+        x->wcap = n.wcap;
+    }
+    n = SideArrays{};
 }
 
 uint32_t next_epochs(pi_index* x, uint32_t count, cudaStream_t s) {
@@ -617,12 +650,18 @@ int sticky_error(const DevMeta& m) {
     return PI_OK;
 }
 
+// Called with `known` current. The index stays as it is unless all of the growth succeeds.
 cudaError_t grow_storage(pi_index* x, uint64_t need, cudaStream_t s) {
     uint64_t cap = need + need / 2 + kMinStorage;
     if (cap > PI_MAX_KEYS) cap = PI_MAX_KEYS;
     Storage ns{};
+    SideArrays side;
     cudaError_t e = alloc_storage(ns, cap, s);
     if (e != cudaSuccess) return e;
+    if ((e = alloc_side(x, x->sc.cap, cap, s, side)) != cudaSuccess) {
+        free_storage(ns);
+        return e;
+    }
     const uint32_t cur = x->known.cur;
     const uint64_t cnt = (uint64_t)x->known.size + 1;  // with the sentinel
     cudaMemcpyAsync(ns.keys[0], x->st.keys[cur], cnt * 8, cudaMemcpyDeviceToDevice, s);
@@ -632,15 +671,15 @@ cudaError_t grow_storage(pi_index* x, uint64_t need, cudaStream_t s) {
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         free_storage(ns);
+        free_side(side);
         return e;
     }
     free_storage(x->st);
     x->st = ns;
     x->st_cap = cap;
     x->known.cur = 0;
-    if ((e = ensure_tile_cnt(x, cap, s)) != cudaSuccess) return e;
-    if ((e = ensure_wcount(x, cap, s)) != cudaSuccess) return e;
-    return ensure_desc(x, desc_need(x->sc.cap, cap), s);
+    use_side(x, side);
+    return cudaSuccess;
 }
 
 cudaError_t grow_index(pi_index* x, uint64_t need, cudaStream_t s) {
@@ -683,9 +722,12 @@ cudaError_t grow_scratch(pi_index* x, uint64_t n, cudaStream_t s) {
     x->rebuild_pending = false;
     uint64_t q = std::max<uint64_t>(n, x->sc.cap + x->sc.cap / 2);
     q = std::min<uint64_t>(std::max<uint64_t>(q, 4096), std::max<uint64_t>(n, PI_MAX_BATCH));
+    // the look-back words first: a scratch in use means that they suffice for its batches
+    SideArrays side;
+    if ((e = alloc_side(x, q, x->st_cap, s, side)) != cudaSuccess) return e;
+    use_side(x, side);
     free_scratch(x->sc);
-    if ((e = alloc_scratch(x->sc, q)) != cudaSuccess) return e;
-    return ensure_desc(x, desc_need(q, x->st_cap), s);
+    return alloc_scratch(x->sc, q);
 }
 
 // Whether a batch's descent takes windows of the lowest built level, by the host's last view of
@@ -1025,9 +1067,9 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
         cudaMemsetAsync(x->d_bm, 0, 2 * sizeof(BatchMeta), s);
         if ((e = alloc_storage(x->st, st_cap, s)) != cudaSuccess) break;
         x->st_cap = st_cap;
-        if ((e = ensure_tile_cnt(x, st_cap, s)) != cudaSuccess) break;
-        if ((e = ensure_wcount(x, st_cap, s)) != cudaSuccess) break;
-        if ((e = ensure_desc(x, desc_need(n, st_cap), s)) != cudaSuccess) break;
+        SideArrays side;
+        if ((e = alloc_side(x, n, st_cap, s, side)) != cudaSuccess) break;
+        use_side(x, side);
         // 1. sort (key, arrival) and keep the last of every key run
         if (n > 0) {
             if ((e = alloc_sort_scratch(tmp, n)) != cudaSuccess) break;
@@ -1398,7 +1440,12 @@ int pi_info(pi_index_t* x, pi_info_t* out, pi_stream_t stream) {
     return sticky_error(m);
 }
 
-void pi_test_fail_allocations(uint32_t count) { g_fail_allocs = count; }
+void pi_test_fail_allocations(uint32_t count) {
+    g_fail_allocs = count;
+    g_skip_allocs = 0;
+}
+
+void pi_test_skip_allocations(uint32_t count) { g_skip_allocs = count; }
 
 int pi_test_set_error(pi_index_t* x, uint32_t bits, pi_stream_t stream) {
     if (!x) return PI_ERR_INVALID_ARG;
@@ -1842,7 +1889,11 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
             size_ub = (uint64_t)x->known.size + n;
             if (size_ub > PI_MAX_KEYS) return PI_ERR_INVALID_ARG;
             const uint64_t room = std::min<uint64_t>(size_ub + 2 * n, PI_MAX_KEYS);
-            if (room > x->st_cap && (e = grow_storage(x, room, s)) != cudaSuccess && size_ub > x->st_cap) return map_cuda(e);
+            if (room > x->st_cap && (e = grow_storage(x, room, s)) != cudaSuccess) {
+                // no memory for that much: what this batch needs decides
+                if (e == cudaErrorMemoryAllocation) e = size_ub > x->st_cap ? grow_storage(x, size_ub, s) : cudaSuccess;
+                if (e != cudaSuccess) return map_cuda(e);
+            }
             if (x->known.grow_request && x->known.index_need + 64ull > x->idx_cap) {
                 if ((e = grow_index(x, x->known.index_need, s)) != cudaSuccess) return map_cuda(e);
             }

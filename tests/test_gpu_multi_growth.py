@@ -64,3 +64,71 @@ def test_index_layer_grows_once(orc_mod):
     assert_state_equal(idx, orc)
     idx.close()
     orc.close()
+
+
+def mixed(keys, seed, q, inserts):
+    s = wl.stream_seed(seed, 96)
+    k = np.concatenate([keys[wl.bounded(s, 0, q - inserts, len(keys))], wl.u64_stream(s, q, inserts) >> np.uint64(1)])
+    return wl.Batch(np.repeat(np.array([0, 1], np.uint8), [q - inserts, inserts]), k, wl.u64_stream(s, 2 * q, q))
+
+
+@pytest.mark.parametrize("fails", [1, 2])
+@pytest.mark.parametrize("skip", [0, 1, 2])
+@pytest.mark.parametrize("needed", [False, True])
+def test_growth_that_fails_part_way(orc_mod, needed, skip, fails):
+    """An index that comes near its capacity gets more room than the call needs. Whichever of that
+    growth's allocations fails, the call does without the room when it does not need it, and
+    takes just what it needs when it does; only a failure of that refuses it. The set and the plain
+    path are right afterwards."""
+    import torch
+    import paper_1601_00159_gb300 as pkg
+    n, q = 70_000, 50_000
+    keys = wl.distinct_keys(96, np.arange(n))
+    idx = make_index(keys, wl.splitmix64(keys), 0.25, 13)
+    orc = orc_mod.Oracle(keys, wl.splitmix64(keys), 0.25, 13)
+    ms = pkg.MultiSet([idx])
+    cap = idx.info()["storage_capacity"]
+
+    def check(b, dev, what):
+        torch.cuda.synchronize()
+        assert_results_equal(results_np(dev[3]), orc.execute(b.ops, b.keys, b.vals), what)
+
+    calls = [mixed(keys, 1, q, 0), mixed(keys, 2, 20_000, 20_000 if needed else 0),
+             mixed(keys, 3, q, q if needed else 1000)]
+    devs = [dev_batch(b) for b in calls]
+    ms.execute([(0, *devs[0])])  # the class's scratch
+    check(calls[0], devs[0], "call 0")
+    torch.cuda._sleep(100_000_000)  # call 1 stays in flight: its queries count as possible nodes
+    ms.execute([(0, *devs[1])])
+    assert (n + len(calls[1]) + q > cap) and (needed == (n + int(calls[1].ops.sum()) + q > cap))
+    pkg.test_fail_allocations(fails, skip)
+    try:
+        refused = False
+        try:
+            ms.execute([(0, *devs[2])])
+        except pkg.PiError as e:
+            assert e.code == pkg.PI_ERR_OOM
+            refused = True
+    finally:
+        pkg.test_fail_allocations(0)
+    # the first failure is the room's; a second one meets what the batch needs, if it needs any
+    assert refused == (needed and fails == 2)
+    check(calls[1], devs[1], "call 1")
+    if refused:
+        assert idx.info()["storage_capacity"] == cap
+        ms.execute([(0, *devs[2])])
+    check(calls[2], devs[2], "call 2")
+    assert (idx.info()["storage_capacity"] > cap) == needed
+    for i in range(2):
+        b = mixed(keys, 20 + i, 60_000, 40_000)
+        dev = dev_batch(b)
+        idx.execute(*dev)
+        check(b, dev, f"plain {i}")
+        b = mixed(keys, 30 + i, q, 30_000)
+        dev = dev_batch(b)
+        ms.execute([(0, *dev)])
+        check(b, dev, f"set {i}")
+    ms.close()
+    assert_state_equal(idx, orc)
+    idx.close()
+    orc.close()
