@@ -1049,6 +1049,7 @@ pi_index_t* pi_create_ex(const uint64_t* keys, const uint64_t* values, uint64_t 
             if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) break;
         if (e != cudaSuccess) break;
         if ((e = cudaMallocHost(reinterpret_cast<void**>(&x->h_mbox), kRing * sizeof(DevMeta))) != cudaSuccess) break;
+        std::memset(static_cast<void*>(x->h_mbox), 0, kRing * sizeof(DevMeta));
         {  // the small device state, one allocation that starts at d_meta
             uint8_t* slab = nullptr;
             if ((e = dalloc(&slab, al256(sizeof(DevMeta)) + al256(2 * sizeof(BatchMeta)) + al256((kSortHist + 256) * 4) + 256)) !=

@@ -101,8 +101,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_merge(RebuildArgs a, uint32_t e
         for (int k = 0; k < kStages; ++k) mbar_init(&s_bar[k], 1);
     }
     if (tid < 2 * kLevelSlots) (&s_cnt[0][0])[tid] = 0;
+    // A CTA that stops for an error is not counted as finished, so no other may be the last: each
+    // of them posts, or the host would read whatever the slot held before.
     if (block_sees_error(&m->error)) {
-        if (blockIdx.x == 0 && warp == 0) post_batch(a);
+        if (warp == 0) post_batch(a);
         return;
     }
     const uint32_t size = m->size, src = m->cur, dst = src ^ 1u;
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_merge(RebuildArgs a, uint32_t e
     }
     __syncthreads();
     flush();
-    if (s_fail) {  // this CTA will not arrive, so the batch has no last one; its copies land first
+    if (s_fail) {  // nor is this one; its copies land first
         if (tid == 0)
             for (uint32_t k = 0; k < (uint32_t)kStages && c0 + landed + k < c1; ++k) {
                 const uint32_t f = landed + k;
