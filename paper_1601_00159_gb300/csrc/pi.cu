@@ -1583,6 +1583,7 @@ struct pi_multi {
     std::vector<MIndex> h_idx;
     pi_multi_config_t cfg{};
     MIndex* d_idx = nullptr;
+    bool idx_stale = true;  // d_idx lags h_idx: the next call that runs brings it up to date
     // The indices' metas as the last call of each parity left them (pinned, written by its
     // kernels: no copy at the call's end), with the operation that the call was for each of
     // its indices
@@ -1792,9 +1793,6 @@ pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi
     do {
         for (auto* x : v) mx->h_idx.push_back(mindex_of(x));
         if ((e = dalloc(&mx->d_idx, count)) != cudaSuccess) break;
-        if ((e = cudaMemcpy(mx->d_idx, mx->h_idx.data(), count * sizeof(MIndex), cudaMemcpyHostToDevice)) !=
-            cudaSuccess)
-            break;
         mx->q_bytes = kQHeader + (uint64_t)PI_MULTI_MAX_CLASSES * count * sizeof(MItem);
         if ((e = dalloc(&mx->d_q, mx->q_bytes)) != cudaSuccess) break;
         for (int p = 0; p < 2; ++p) {
@@ -1877,7 +1875,6 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
     // kernel. Growing (rare) synchronises the stream, as in pi_execute_batch; an index that
     // comes near gets room for the calls that may be in flight, so that the next calls need
     // no synchronisation to be sure of it.
-    bool idx_changed = false;
     for (uint32_t i = 0; i < nb; ++i) {
         pi_index* x = mx->idx[b[i].index];
         refresh_known(x);
@@ -1907,14 +1904,16 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
         const MIndex now = mindex_of(x);
         if (std::memcmp(&now, &mx->h_idx[b[i].index], sizeof(MIndex)) != 0) {
             mx->h_idx[b[i].index] = now;
-            idx_changed = true;
+            mx->idx_stale = true;  // also for the calls after this one, should it be refused below
         }
         wait_rebuild(x, s);
     }
-    if (idx_changed &&
-        (e = cudaMemcpyAsync(mx->d_idx, mx->h_idx.data(), mx->h_idx.size() * sizeof(MIndex),
-                             cudaMemcpyHostToDevice, s)) != cudaSuccess)
-        return map_cuda(e);
+    if (mx->idx_stale) {
+        if ((e = cudaMemcpyAsync(mx->d_idx, mx->h_idx.data(), mx->h_idx.size() * sizeof(MIndex), cudaMemcpyHostToDevice,
+                                 s)) != cudaSuccess)
+            return map_cuda(e);
+        mx->idx_stale = false;
+    }
     // the queue: per class, largest estimated work first (longest-processing-time order)
     std::vector<std::vector<std::pair<uint64_t, uint32_t>>> per(mx->cfg.num_classes);
     uint32_t need_q[PI_MULTI_MAX_CLASSES] = {};

@@ -132,3 +132,44 @@ def test_growth_that_fails_part_way(orc_mod, needed, skip, fails):
     assert_state_equal(idx, orc)
     idx.close()
     orc.close()
+
+
+@pytest.mark.parametrize("alone", [True, False])
+def test_call_refused_after_an_index_grew(orc_mod, alone):
+    """A call in which one index grows and the next cannot is refused. The set's later calls, on the
+    first index alone or on both, work on its new arrays."""
+    import torch
+    import paper_1601_00159_gb300 as pkg
+    n, q = 70_000, 100_000
+    keys = [wl.distinct_keys(102 + i, np.arange(n)) for i in range(2)]
+    idx = [make_index(k, wl.splitmix64(k), 0.25, i) for i, k in enumerate(keys)]
+    orc = [orc_mod.Oracle(k, wl.splitmix64(k), 0.25, i) for i, k in enumerate(keys)]
+    ms = pkg.MultiSet(idx)
+    caps = [x.info()["storage_capacity"] for x in idx]
+    assert n + q > max(caps)
+
+    def call(bs):
+        devs = [dev_batch(b) for b in bs]
+        ms.execute([(i, *d) for i, d in enumerate(devs)])
+        torch.cuda.synchronize()
+        for i, (b, d) in enumerate(zip(bs, devs)):
+            assert_results_equal(results_np(d[3]), orc[i].execute(b.ops, b.keys, b.vals), f"index {i}")
+
+    call([mixed(k, 1, n // 2, 0) for k in keys])
+    bs = [mixed(k, 2 + i, q, q) for i, k in enumerate(keys)]
+    pkg.test_fail_allocations(2, 3)  # the first index's storage, look-back words and counts succeed
+    try:
+        with pytest.raises(pkg.PiError) as ei:
+            ms.execute([(i, *dev_batch(b)) for i, b in enumerate(bs)])
+    finally:
+        pkg.test_fail_allocations(0)
+    assert ei.value.code == pkg.PI_ERR_OOM
+    grown = [x.info()["storage_capacity"] for x in idx]
+    assert grown[0] > caps[0] and grown[1] == caps[1]
+    call(bs[:1] if alone else bs)
+    call([mixed(k, 7 + i, q, q // 2) for i, k in enumerate(keys)])
+    ms.close()
+    for x, o in zip(idx, orc):
+        assert_state_equal(x, o)
+        x.close()
+        o.close()
