@@ -1594,6 +1594,7 @@ struct pi_multi {
     uint64_t q_bytes = 0;
     cudaEvent_t q_free[2] = {};
     uint64_t calls = 0;
+    cudaStream_t last_stream = nullptr;  // of the last call
     uint64_t launches = 0;  // kernels per graph launch
     uint32_t grid[PI_MULTI_MAX_CLASSES] = {};
     uint32_t qcap[PI_MULTI_MAX_CLASSES] = {};
@@ -1871,6 +1872,10 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
     if ((e = cudaEventSynchronize(mx->q_free[p])) != cudaSuccess) return map_cuda(e);
     multi_adopt(mx, p);
     if (cudaEventQuery(mx->q_free[p ^ 1]) == cudaSuccess) multi_adopt(mx, p ^ 1);
+    // The queue, the table of indices and the scratch on the device are the set's: a call on
+    // another stream comes after the last one, also when they have no index in common.
+    if (mx->calls && mx->last_stream != s && (e = cudaStreamWaitEvent(s, mx->q_free[p ^ 1], 0)) != cudaSuccess)
+        return map_cuda(e);
     // Capacities: every index must hold its batch's new keys without growing in the
     // kernel. Growing (rare) synchronises the stream, as in pi_execute_batch; an index that
     // comes near gets room for the calls that may be in flight, so that the next calls need
@@ -1969,6 +1974,7 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
     if ((e = cudaGraphLaunch(mx->gx[p], s)) != cudaSuccess) return map_cuda(e);
     if ((e = cudaEventRecord(mx->q_free[p], s)) != cudaSuccess) return map_cuda(e);
     mx->calls++;
+    mx->last_stream = s;
     g_launches += mx->launches;
     if (single) {
         pi_index* x = single;
