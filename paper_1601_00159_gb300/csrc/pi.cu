@@ -8,12 +8,12 @@
 #include <cstdio>
 #include <cstddef>
 #include <cstring>
-#include <deque>
 #include <mutex>
 #include <string>
 #include <new>
 #include <algorithm>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -179,7 +179,7 @@ struct pi_index {
     struct Op {
         uint64_t id, n;
     };
-    std::deque<Op> ops;      // those after known_op
+    std::vector<Op> ops;     // those after known_op, a few dozen at most (a vector: making it cannot throw)
     uint64_t op_count = 0, known_op = 0;
     uint64_t pending_n = 0;  // their queries
     bool force_rebuild = false;
@@ -584,9 +584,16 @@ cudaError_t read_meta(pi_index* x, cudaStream_t s, DevMeta* out) {
 
 constexpr uint64_t kRing = 64;
 
-// Numbers an operation of n queries that is being issued.
-uint64_t note_op(pi_index* x, uint64_t n) {
-    x->ops.push_back({++x->op_count, n});
+// Numbers an operation of n queries that is being issued. Without memory to list it, its queries
+// stay counted as pending until the next sync_known: the host then synchronises earlier than it
+// would have to. (Nothing may be thrown here: the work is on the stream, and the callers are
+// C entries.)
+uint64_t note_op(pi_index* x, uint64_t n) noexcept {
+    ++x->op_count;
+    try {
+        x->ops.push_back({x->op_count, n});
+    } catch (...) {
+    }
     x->pending_n += n;
     return x->op_count;
 }
@@ -596,10 +603,9 @@ void adopt(pi_index* x, const DevMeta& m, uint64_t op) {
     if (op <= x->known_op) return;
     x->known = m;
     x->known_op = op;
-    while (!x->ops.empty() && x->ops.front().id <= op) {
-        x->pending_n -= x->ops.front().n;
-        x->ops.pop_front();
-    }
+    size_t done = 0;
+    for (; done < x->ops.size() && x->ops[done].id <= op; ++done) x->pending_n -= x->ops[done].n;
+    x->ops.erase(x->ops.begin(), x->ops.begin() + (ptrdiff_t)done);
 }
 
 // Non-blocking: adopt the newest completed batch's mailbox. Batches complete in order, so the
@@ -1736,7 +1742,7 @@ cudaError_t multi_build_graphs(pi_multi* mx) {
 
 extern "C" {
 
-pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi_multi_config_t* cfg) {
+pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi_multi_config_t* cfg) try {
     g_last_error = PI_OK;
     if (!indices || count == 0) {
         g_last_error = PI_ERR_INVALID_ARG;
@@ -1785,14 +1791,22 @@ pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi
         g_last_error = PI_ERR_OOM;
         return nullptr;
     }
+    try {  // all that the set's lists will hold
+        mx->h_idx.reserve(count);
+        for (auto& ops : mx->call_ops) ops.reserve(count);
+    } catch (...) {
+        delete mx;
+        g_last_error = PI_ERR_OOM;
+        return nullptr;
+    }
     mx->device = v[0]->device;
     mx->num_sms = v[0]->num_sms;
-    mx->idx = v;
+    mx->idx = std::move(v);
     mx->cfg = c;
     cudaSetDevice(mx->device);
     cudaError_t e = cudaSuccess;
     do {
-        for (auto* x : v) mx->h_idx.push_back(mindex_of(x));
+        for (auto* x : mx->idx) mx->h_idx.push_back(mindex_of(x));
         if ((e = dalloc(&mx->d_idx, count)) != cudaSuccess) break;
         mx->q_bytes = kQHeader + (uint64_t)PI_MULTI_MAX_CLASSES * count * sizeof(MItem);
         if ((e = dalloc(&mx->d_q, mx->q_bytes)) != cudaSuccess) break;
@@ -1826,6 +1840,9 @@ pi_multi_t* pi_multi_create(pi_index_t* const* indices, uint32_t count, const pi
         return nullptr;
     }
     return mx;
+} catch (...) {  // no memory for the checks
+    g_last_error = PI_ERR_OOM;
+    return nullptr;
 }
 
 }  // extern "C"
@@ -1853,7 +1870,7 @@ namespace {
 // call is that index's batch for pi_execute_batch, which has already checked the
 // capacities; its bookkeeping is then a plain batch's (the mailbox ring and the index's
 // last-operation event) so the host's view of the sizes stays current without a sync.
-int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStream_t s, pi_index* single) {
+int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStream_t s, pi_index* single) try {
     if (nb == 0) return PI_OK;
     const uint32_t count = (uint32_t)mx->idx.size();
     if (!b || nb > count) return PI_ERR_INVALID_ARG;
@@ -2004,6 +2021,8 @@ int multi_execute(pi_multi* mx, const pi_multi_batch_t* b, uint32_t nb, cudaStre
     }
     cudaEventRecord(mx->ev_done, s);
     return PI_OK;
+} catch (...) {  // no host memory for the queue: nothing has been enqueued
+    return PI_ERR_OOM;
 }
 
 constexpr uint64_t kSmallBatch = 1ull << 16;  // queries
