@@ -125,6 +125,9 @@ typedef struct {
  * a sticky error (pi_status then returns PI_ERR_CUDA), and pi_info's
  * owner_checked_writes sums the writes checked. The batching form is not checked. */
 #define PI_TEST_OWNER_CHECK 0x100u
+/* test_flags bit: a range search copies the slices of a warp's queries one at a time from 64 nodes
+ * on (2^31 in use, where they overlap many times over). */
+#define PI_TEST_SHORT_RUNS 0x200u
 
 /*
  * pi_create -- bulk-build an index from n (key, value) pairs (Section 3.1: the index

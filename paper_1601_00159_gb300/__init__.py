@@ -33,6 +33,7 @@ PI_NOALLOC_MAX_BATCH = 1 << 16
 PI_TEST_WALK_LEVELS = 1
 PI_TEST_SORT_FULL = 2
 PI_TEST_OWNER_CHECK = 0x100
+PI_TEST_SHORT_RUNS = 0x200
 
 
 def PI_TEST_SORT_PREFIX(k: int) -> int:

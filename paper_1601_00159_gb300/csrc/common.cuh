@@ -705,6 +705,7 @@ struct RangeArgs {
     uint64_t* keys_out;       // [cap] output (caller's)
     uint64_t* vals_out;
     uint64_t cap;
+    uint64_t run_most;        // a warp's slices of that many nodes together are copied one at a time
     uint32_t n;
     uint32_t* err;
 };

@@ -1296,6 +1296,7 @@ int pi_range_search(pi_index_t* x, const uint64_t* lo, const uint64_t* hi, uint6
     ra.keys_out = keys_out;
     ra.vals_out = vals_out;
     ra.cap = cap;
+    ra.run_most = x->test_flags & PI_TEST_SHORT_RUNS ? 64ull : 1ull << 31;
     ra.n = (uint32_t)n;
     ra.err = &x->d_meta->error;
     e = launch_range(ra, s, x->num_sms);

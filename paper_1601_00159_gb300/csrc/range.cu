@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kThreads) k_range_write(RangeArgs a, uint32_t 
     const uint64_t* SK = a.st.keys[cur];
     const uint64_t* SV = a.st.vals[cur];
     const uint8_t* SM = a.st.meta[cur];
-    if (total < (1ull << 31)) {
+    if (total < a.run_most) {
         copy_run(a, SK, SV, SM, s, (uint32_t)pre, (uint32_t)total, wbase);
     } else {  // slices that overlap many times over: one at a time
         uint64_t o = wbase;
