@@ -9,10 +9,9 @@ entry of the lowest level spans), and writes the fastest per class to multi_tuni
 beside it, which bench.py and MultiSet callers pass to pi_multi_create / pi_create_ex.
 
 Plain path (--plain): for each index size of the skewed workload (batches of 2^22 Zipf
-queries), the fan-out (lowest built level) together with the entries pinned in shared
-memory, then the radix passes per batch with the fastest of those; every variant's
-results and final key/value set must equal the default configuration's, bit for bit.
-Writes plain_tuning.json beside this file, which bench.py reads.
+queries), the fan-out (lowest built level), then the radix passes per batch with the
+fastest of those; every variant's results and final key/value set must equal the default
+configuration's, bit for bit. Writes plain_tuning.json beside this file, which bench.py reads.
 
     python -m paper_1601_00159_gb300.autotune [--calls 8]
     python -m paper_1601_00159_gb300.autotune --plain [--sizes 24 26 27] [--calls 6]
@@ -101,12 +100,12 @@ def tune_plain(args):
         timings, shapes = {}, {}
         ms, info = run({})
         timings["default"] = ms
-        shapes["default"] = {"lowest_built": info["bottom_built"], "pinned_from_level": info["smem_low_level"]}
-        fan = [{"lowest_level": lo, "smem_top_entries": sm} for lo in (2, 3, 4) for sm in (2048, 12288)]
+        shapes["default"] = {"lowest_built": info["bottom_built"]}
+        fan = [{"lowest_level": lo} for lo in (2, 3, 4)]
         for cfg in fan:
             ms, info = run(cfg)
             timings[variant_name(cfg)] = ms
-            shapes[variant_name(cfg)] = {"lowest_built": info["bottom_built"], "pinned_from_level": info["smem_low_level"]}
+            shapes[variant_name(cfg)] = {"lowest_built": info["bottom_built"]}
             print(f"2^{logn}: {variant_name(cfg)}: {ms:.4f} ms per batch", flush=True)
         best_fan = min(fan, key=lambda c: timings[variant_name(c)])
         for sp in (3, 4, 8):
