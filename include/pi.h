@@ -107,7 +107,7 @@ typedef struct {
                                     GB300 it is slower than the default (2^14 searches on
                                     2^16 keys 90 against 26 us, 2^10 queries on 2^16 keys
                                     74 against 26, 2^12 on 2^18 114 against 27): one launch
-                                    on 16 SMs against six on all. Not taken while profiling, with
+                                    on 16 SMs against five on all. Not taken while profiling, with
                                     test_flags or with the deferred rebuild policy. */
 } pi_config_t;
 

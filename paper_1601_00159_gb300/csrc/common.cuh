@@ -12,14 +12,14 @@ constexpr uint64_t kMaxKey = ~0ull;  // reserved key: level and storage sentinel
 constexpr int kLevelSlots = 34;      // per-level arrays are indexed by level 0..33
 constexpr uint8_t kTomb = 0x80;      // meta bit 7: the delete flag F_del (Algorithm 4)
 constexpr uint8_t kHeightMask = 0x3F;
-constexpr uint32_t kSmemTopMax = 12288;  // index entries staged in shared memory (148 KB with their downs)
+constexpr uint32_t kSmemTopMax = 12288;  // largest smem_top_entries (see pi_config_t)
 constexpr uint32_t kPad = 64;           // readable entries past every array's end
 constexpr uint32_t kSortTile = 2048;    // elements per radix-sort tile (the smaller of two sizes)
 constexpr uint32_t kSortHist = 9 * 256; // digit counts of a radix sort
 constexpr uint32_t kSweepMost = 1u << 20;  // largest batch whose radix passes look back (see k_sort_count)
 constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the count kernel's scan
 constexpr uint32_t kCtrApply = 15;      // BatchMeta::tile_ctr slot: the apply kernel's tile counter
-constexpr uint32_t kApplyTile = 2048;   // sorted queries per apply tile
+constexpr uint32_t kApplyTile = 2048;   // sorted queries per tile of the descent with windows, and of its marks
 constexpr uint32_t kApplyBlock = 128;   // sorted queries per apply warp
 constexpr uint32_t kRunTile = 1024;     // queries per tile of the small batches' sort
 // Largest batch sorted that way. A query is ranked in every other tile, so the ranking's work
@@ -44,8 +44,8 @@ struct DevMeta {
     // layout of the index layer as last built
     uint32_t H;            // top built level (1: no index level)
     uint32_t Lb;           // lowest materialised index level
-    uint32_t Ls;           // lowest level staged in shared memory (> H: none)
-    uint32_t smem_entries; // entries [0, smem_entries) are staged
+    uint32_t Ls;           // lowest level whose entries and those above fit smem_top (> H: none); pi_info's
+    uint32_t smem_entries; // those entries
     uint32_t index_total;  // entries in use (sentinels included)
     uint32_t index_need;   // entries a full build needs
     uint32_t grow_request; // 1 when levels were dropped for lack of capacity
@@ -635,7 +635,7 @@ struct RebuildArgs {
     uint32_t threshold_pct;
     uint32_t force_rebuild;  // 1: rebuild regardless; 2: initial build (not a batch)
     uint32_t st_cap;         // storage capacity (nodes, padding excluded)
-    uint32_t smem_top;       // cap on pinned entries (<= kSmemTopMax)
+    uint32_t smem_top;       // cap on the entries that count for DevMeta::Ls
     uint32_t min_lb;         // lowest index level to build (>= 2)
     uint32_t* err;
     LevelChanges chg;        // the batch's level membership changes (key order)
@@ -660,7 +660,7 @@ struct MIndex {           // one index of the set: its own arrays and device met
     uint32_t* ldown1;
     uint32_t st_cap;      // storage nodes per buffer
     uint32_t idx_cap;     // index-layer entries
-    uint32_t smem_top;    // the plain descent's pinned-entry cap (kept in DevMeta::Ls)
+    uint32_t smem_top;    // cap on the entries that count for DevMeta::Ls
     uint32_t min_lb;      // lowest index level to build (>= 2)
     HashParams hp;
 };

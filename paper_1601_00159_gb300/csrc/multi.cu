@@ -2,7 +2,7 @@
 // persistent launch (Algorithm 1 applied to every index of a set at once).
 //
 // Small indices and small batches leave the level-synchronous whole-GPU pipeline of a
-// single index (tens of launches, each spread over all SMs) launch-bound. Here a CTA
+// single index (at least five launches, each spread over all SMs) launch-bound. Here a CTA
 // runs the whole pipeline of one index's batch by itself, and the CTAs of a persistent
 // launch take batches from a device-side work queue, largest first:
 //   sort        stable LSD radix sort of (key, arrival) over the varying key bytes,
@@ -620,7 +620,7 @@ __device__ uint32_t m_apply_span(const MItem& it, const MIndex& X, const MScratc
 
 // The new level layout from the live counts (one thread; before the merge, which may
 // write the lowest level): levels that do not fit the index layer's capacity are
-// dropped from the bottom, and the pinned-entry prefix is recomputed.
+// dropped from the bottom, and DevMeta::Ls is recomputed.
 __device__ void m_layout(const MIndex& X, DevMeta& m) {
     uint32_t H = 1;
     for (int l = 2; l < kLevelSlots; ++l)

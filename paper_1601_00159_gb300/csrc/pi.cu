@@ -125,7 +125,7 @@ struct pi_index {
     int num_sms = 0;
     HashParams hp{};
     uint32_t rebuild_policy = 0, threshold_pct = 15;
-    uint32_t smem_top = kSmemTopMax;  // pinned-entry cap
+    uint32_t smem_top = kSmemTopMax;  // pi_config_t.smem_top_entries
     uint32_t min_lb = 2;              // lowest index level built
     uint32_t test_flags = 0;
     uint32_t sort_cfg = 0;            // pi_config_t.sort_passes
@@ -186,7 +186,7 @@ struct pi_index {
     bool bm_clear = false;   // the next batch's counters are zero (the last batch cleared them)
     // With small_mode 1, small batches (Q <= kSmallBatch on at most kSmallIndex nodes) run
     // through a one-index batching set whose batch takes a thread-block cluster: one
-    // launch instead of the level-synchronous pipeline's tens. Created on first use.
+    // launch instead of the level-synchronous pipeline's five or more. Created on first use.
     pi_multi* small = nullptr;
     uint32_t small_mode = 0;
     uint64_t routed = 0;  // batches that took the route
@@ -264,12 +264,9 @@ int map_cuda(cudaError_t e) {
 
 // Look-back descriptors needed for q queries and a storage capacity of s nodes.
 uint64_t desc_need(uint64_t q, uint64_t s) {
-    uint64_t a = 0;                                    // (the sort needs none)
-    uint64_t b = 2 * ((q + 1023) / 1024);    // apply
-    uint64_t c = (s / 4096 + 2) * 32;        // merge, export
-    if (c < 32 * 64) c = 32 * 64;            // rebuild level scan: 64 chunks x 32 levels
-    uint64_t m = a > b ? a : b;
-    return (m > c ? m : c) + 64;
+    const uint64_t a = 2 * ((q + 1023) / 1024);                            // apply: two words a tile
+    const uint64_t b = std::max<uint64_t>((s / 4096 + 2) * 32, 32 * 64);  // merge, export, build, level scans
+    return std::max(a, b) + 64;
 }
 
 // The arrays beside the storage layer whose sizes follow the capacities.
@@ -490,8 +487,8 @@ void use_index(pi_index* x, const IndexArrays& n) {
 
 constexpr uint32_t kProfSlots = 2048;
 // Per batch: 0 start, 1 after sort, 2 after waiting for the previous rebuild, 3 after
-// descent, 4 after apply, 5 after merge, 6 after layout, 7 rebuild start, 8 before the
-// rebuild's writer kernel, 9 rebuild end, 10 before the storage locate.
+// descent, 4 after apply, 5 and 6 after the merge and the level layout (one kernel), 7 rebuild
+// start, 8 before its preparing and writing kernels, 9 rebuild end, 10 before the descent's kernel.
 constexpr int kProfEvents = 11;
 
 void prof_fold(pi_index* x) {

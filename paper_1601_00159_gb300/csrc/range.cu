@@ -16,7 +16,7 @@
 // whatever the slices' lengths, its loads are consecutive nodes and its stores consecutive
 // pairs; fewer queries per warp when the queries would not fill the chip. (A warp per query, each
 // lane copying 16 consecutive nodes, took 182 us for 2^16 ranges of 100 keys, a call 399 us; the
-// call now takes 119.) The CSR offsets fix every query's output place, so no query waits for
+// call now takes 110.) The CSR offsets fix every query's output place, so no query waits for
 // another.
 
 #include "search.cuh"

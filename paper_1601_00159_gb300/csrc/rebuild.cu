@@ -9,10 +9,10 @@
 //
 // Rebuild: the paper's daemon scans the storage layer and puts the key of every
 // valid node of height > 1 into the index-layer arrays. Here one pass over the storage
-// layer does it for all levels at once: per tile of 4096 nodes, keys and meta arrive in
+// layer does it for all levels at once: per tile of 4096 nodes, the state bytes arrive in
 // shared memory by TMA bulk copy, and level by level the tile compacts its nodes of
-// height >= l (a prefix sum) and writes them with their down pointers, from the tile's offset
-// in the level on. The offsets are a scan of the tiles' counts, which the kernels that change
+// height >= l (a prefix sum), gathers their keys and writes them with their down pointers, from
+// the tile's offset in the level on. The offsets are a scan of the tiles' counts, which the kernels that change
 // the nodes keep current.
 //
 // Level sizes are not counted by the rebuild: the apply kernel keeps them current as
@@ -44,7 +44,7 @@ constexpr uint32_t kCtrMerge = 9, kCtrMergeDone = 10, kCtrCreate = 11, kCtrRebui
 //   1. its cuts, all at once by its warps, and the live nodes among its old ones (no read when
 //      nothing is delete-flagged); a look-back over the CTAs, numbered in the order they
 //      start, gives its first output place;
-//   2. per chunk, whose old nodes arrive in shared memory by TMA bulk copies two chunks ahead,
+//   2. per chunk, whose old nodes arrive in shared memory by TMA bulk copies one chunk ahead,
 //      a blocked pass over the state bytes and the new nodes' insertion points gives every
 //      position its output offset, and a striped pass writes the live nodes, coalesced.
 // The pass also counts, per output tile, the nodes of each built level (the rebuild's offsets
@@ -404,16 +404,11 @@ __global__ void __launch_bounds__(32) k_level_layout(RebuildArgs a) {
 // Index-layer rebuild over tiles of 4096 storage nodes.
 //   lcnt[(l - 2) * stride + tile] = live nodes of height >= l in the tile, for every
 //   level l >= 2. The apply kernel keeps these counts current (its owners add or
-//   remove one node per liveness change), so they are recounted from meta only after
-//   the storage layer was re-laid-out (merge), at create, or after a capacity change.
-//   scan:  per level, the exclusive prefix of the counts over tiles (one CTA/level)
-//          into loff[(l - Lb) * ntiles + tile];
-//   write: per tile, keys and meta arrive in shared memory by TMA bulk copy. Warp w
-//          owns nodes [512 w, 512 w + 512) of the tile: it counts its nodes per level
-//          (one ballot per level per 32 nodes), the warps' counts are prefixed across
-//          the tile (one barrier), then the warp sweeps its nodes again and every node
-//          of height >= l writes its key and down pointer to level l at the position
-//          given by the same ballots.
+//   remove one node per liveness change) and a merge counts what it writes, so they are
+//   recounted from the state bytes only at create or after a capacity change;
+//   prep:  per level, the exclusive prefix of the counts over tiles, in chunks, into
+//          loff[(l - Lb) * ntiles + tile] (scan_counts);
+//   write: the levels (k_rebuild_write).
 __global__ void __launch_bounds__(256) k_rebuild_count(RebuildArgs a) {
     pdl_wait();
     pdl_trigger();

@@ -175,7 +175,7 @@ __device__ __forceinline__ uint32_t slice_rank(const uint64_t* sk, uint32_t len,
     return lo;
 }
 
-// The shared memory of the writer, in the rebuild kernel's dynamic block.
+// The shared memory of the writer, a part of the rebuild kernel's.
 struct WriteSmem {
     uint64_t k0[kSlice], k1[kSlice];
     int32_t p0[kSlice + 1], p1[kSlice + 1];

@@ -178,15 +178,6 @@ __global__ void __launch_bounds__(256) k_scan(const uint8_t* __restrict__ ops, c
     else if (threadIdx.x == 16 && s_red[16]) atomicAdd(&bm->invalid, s_red[16]);
 }
 
-// Pass plan. The digit bytes D are the bytes that vary among the valid keys. Invalid
-// queries carry the sort key 2^64-1 and must follow every valid key: when there are
-// some, D also holds the highest byte p whose maximum over the valid keys is below 0xFF
-// (every invalid key is larger there; with no such byte D is every byte). Passes
-// ping-pong so that the last one writes buffer A.
-// With more than max_passes bytes in D, the passes take the most significant
-// max_passes of them (the prefix). The fix-up then orders each segment of equal prefix
-// bytes by the full key; its long-segment path sorts by every other byte that can
-// differ inside a segment (rdig).
 // Query i of the caller, as the sort takes it: invalid queries get the key 2^64-1.
 __device__ __forceinline__ void load_query(const SortBuffers& sb, uint32_t i, uint64_t& key, uint32_t& pay) {
     const uint32_t op = sb.ops ? sb.ops[i] : 0u;
@@ -221,6 +212,17 @@ __device__ __forceinline__ void query_digits(const SortBuffers& sb, uint32_t i0,
     }
 }
 
+// Pass plan. The digit bytes D are the bytes that vary among the valid keys. Invalid
+// queries carry the sort key 2^64-1 and must follow every valid key: when there are
+// some, D also holds the highest byte p whose maximum over the valid keys is below 0xFF
+// (every invalid key is larger there; with no such byte D is every byte). Passes
+// ping-pong so that the last one writes buffer A.
+// With more than max_passes bytes in D, the passes take the most significant
+// max_passes of them (the prefix). The fix-up then orders each segment of equal prefix
+// bytes by the full key; its long-segment path sorts by every other byte that can
+// differ inside a segment (rdig).
+// This kernel plans for the passes with a look-back, and counts the first pass's digits when they are
+// not those that the scan has counted.
 __global__ void __launch_bounds__(256) k_sort_plan(uint32_t n, SortBuffers sb, BatchMeta* bm, uint32_t max_passes) {
     pdl_wait();
     pdl_trigger();
@@ -429,22 +431,6 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_sort_pass(uint32_t j, uint3
 // 2^22 queries on 2^27 keys took 571 us a batch with k_sort_pass and 544 with these two; at 2^20
 // queries k_sort_pass is ahead (428 against 432), and at 10^5 by 21 of 99 us.
 
-// Digit histogram of every tile for pass j, then its scan, by the CTAs that finish
-// last (no CTA waits for another): the last CTA of each group of kScanGroup tiles turns
-// the group's counts into offsets within the group (toff) and the group's digit totals
-// (gsum); the last group to finish turns those totals into the groups' offsets, in
-// place, and the digit totals into digit bases (dofs). A tile's first output slot for
-// digit d is then dofs[d] + gsum[group][d] + toff[tile][d]. Pass 0 (kFirst) plans the digits,
-// in every CTA, and reads the caller's keys; later passes read the digit bytes the previous
-// scatter wrote beside its output. A thread takes 8 consecutive elements a step and adds each
-// run of equal digits with one shared-memory atomic (one per warp when the whole warp holds
-// one digit), so a run of a hot key costs no atomic contention.
-// The kernel is bound by its chain of dependent round trips, not by the bytes: so a CTA counts
-// four tiles (2^22 queries are then one wave of 512 CTAs, not three of 2048 with one tile
-// each), with every load of digit bytes in flight, and the scans load 32 rows per round trip.
-// 2^22 queries on 2^27 keys took 504 us a batch with one tile per CTA, 16 rows and a kernel of
-// its own for the plan, and take 497. Tiles of 4096 elements, which need half the rows, left the
-// counts as they were and cost the scatter 8 us.
 // Exclusive running sum, per digit (thread d), over `rows` rows of 256 counters starting
 // at `in`: writes each row's prefix to `out` (may equal `in`) and returns the total.
 __device__ __forceinline__ uint32_t scan_rows(const uint32_t* in, uint32_t* out, uint32_t rows) {
@@ -466,6 +452,22 @@ __device__ __forceinline__ uint32_t scan_rows(const uint32_t* in, uint32_t* out,
     return run;
 }
 
+// Digit histogram of every tile for pass j, then its scan, by the CTAs that finish
+// last (no CTA waits for another): the last CTA of each group of kScanGroup tiles turns
+// the group's counts into offsets within the group (toff) and the group's digit totals
+// (gsum); the last group to finish turns those totals into the groups' offsets, in
+// place, and the digit totals into digit bases (dofs). A tile's first output slot for
+// digit d is then dofs[d] + gsum[group][d] + toff[tile][d]. Pass 0 (kFirst) plans the digits,
+// in every CTA, and reads the caller's keys; later passes read the digit bytes the previous
+// scatter wrote beside its output. A thread takes 8 consecutive elements a step and adds each
+// run of equal digits with one shared-memory atomic (one per warp when the whole warp holds
+// one digit), so a run of a hot key costs no atomic contention.
+// The kernel is bound by its chain of dependent round trips, not by the bytes: so a CTA counts
+// four tiles (2^22 queries are then one wave of 512 CTAs, not three of 2048 with one tile
+// each), with every load of digit bytes in flight, and the scans load 32 rows per round trip.
+// 2^22 queries on 2^27 keys took 504 us a batch with one tile per CTA, 16 rows and a kernel of
+// its own for the plan, and take 497. Tiles of 4096 elements, which need half the rows, left the
+// counts as they were and cost the scatter 8 us.
 template <bool kFirst>
 __global__ void __launch_bounds__(kThreads, 4) k_sort_count(uint32_t j, uint32_t n, SortBuffers sb, BatchMeta* bm,
                                                             uint32_t max_passes) {
@@ -952,8 +954,8 @@ __global__ void __launch_bounds__(kThreads) k_sort_fix(uint32_t n, SortBuffers s
 // (a probe is a load, a 64-bit compare and an add), the levels inside a warp's 64 elements need
 // no block barrier, and a tile that is not full stops merging at its length.
 // Measured, 2^14 searches on 2^16 keys: sort and look-up took 15 launches and 89 us between
-// events (98 us a batch); as two launches 29 us (56 us a batch). 2^10 queries on 50,021 keys:
-// 92 to 54 us a batch.
+// events, as two launches 29; the batch went from 98 to 56 us by this (28 with the launches and
+// host work around it cut since). 2^10 queries on 50,021 keys: 92 to 54 us a batch (26 since).
 constexpr int kRunThreads = kRunTile / 2;  // two elements per thread, 64 consecutive ones per warp
 
 // Keys of the sorted run[0, kLen) below x.
