@@ -18,9 +18,10 @@
 // The descent left the storage-layer state at each local run head (a query whose key differs
 // from the previous one, and the first query of every 128-query block) and each block's
 // largest e. A warp takes a block and scans it on its own: the nearest local head before a
-// query, by its number, has its state, and a block that continues a run looks back over the
-// blocks' (then the tiles') marks for the run's last write, 256 of them a step. So no warp waits for another
-// until the counts of the tile: with block-wide scans, barriers were the largest stall.
+// query, by its number, has its state, and a block that continues a run looks back over 256
+// blocks' marks, then the groups', for the run's last write: two steps or three however long the
+// run is. (Over the blocks' marks alone, a batch that is one key's run took time with the square of its
+// length: 2^23 searches 1043 us, now 336.) So no warp waits for another until the counts of the tile: with block-wide scans, barriers were the largest stall.
 // New nodes, and the changes of built levels' membership, go to their places in key order in
 // the same pass: a tile's first place comes from a decoupled look-back over the tiles' counts,
 // which only tiles that have some wait for. Half of the kernel's time is its scattered 16-byte
@@ -73,34 +74,29 @@ __device__ uint32_t marker_before_tile(const ApplyArgs& a, uint32_t tb, uint32_t
     return 0;
 }
 
-// The nearest nonzero of marks[0, n), from the end, by a whole warp; *seen is how many entries
-// were looked at when it gave up after `steps` steps.
-__device__ __forceinline__ uint32_t last_mark(const uint32_t* marks, uint32_t n, uint32_t steps, uint32_t* seen) {
-    constexpr int kPer = 8;
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t done = 0;
-    for (uint32_t st = 0; st < steps && done < n; ++st, done += 32u * kPer) {
-        uint32_t most = 0;  // markers grow with their place, so the largest is the nearest
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const uint32_t x = done + 32u * (uint32_t)u + lane;
-            most = max(most, x < n ? marks[n - 1u - x] : 0u);
-        }
-        most = __reduce_max_sync(0xffffffffu, most);
-        if (most) return most;
+// The nearest nonzero of the last kMarkBlocks of marks[0, n), by a whole warp (four loads at a time:
+// with all eight in flight the kernel spilled 44 bytes a thread instead of 12).
+__device__ __forceinline__ uint32_t last_mark(const uint32_t* marks, uint32_t n) {
+    uint32_t most = 0;  // markers grow with their place, so the largest is the nearest
+#pragma unroll 4
+    for (uint32_t u = 0; u < kMarkBlocks / 32u; ++u) {
+        const uint32_t x = 32u * u + (threadIdx.x & 31u);
+        most = max(most, x < n ? marks[n - 1u - x] : 0u);
     }
-    *seen = min(done, n);
-    return 0;
+    return __reduce_max_sync(0xffffffffu, most);
 }
 
-// Largest marker before block blk, which continues the run before it.
+// Largest marker before block blk, which continues the run before it: of the blocks before it, or,
+// when the first step finds none, of the groups. Those start with the group of the last block not
+// looked at: the blocks of it that come after that one were looked at, and hold none. The block
+// that is sought is filled up to its end by the run, as is the next one, so its group has its marker.
 __device__ __forceinline__ uint32_t marker_before_block(const ApplyArgs& a, uint32_t blk) {
-    uint32_t seen = 0;
-    const uint32_t mk = last_mark(a.blk_mark, blk, a.tile_mark ? 1u : 0xffffffffu, &seen);
-    if (mk || !a.tile_mark) return mk;
-    // the tile of the last block not looked at, and all before it (a tile's other blocks hold none)
-    const uint32_t left = blk - seen;
-    return last_mark(a.tile_mark, (left + kApplyTile / kApplyBlock - 1u) / (kApplyTile / kApplyBlock), 0xffffffffu, &seen);
+    uint32_t mk = last_mark(a.blk_mark, blk);
+    if (mk || blk <= kMarkBlocks) return mk;
+#pragma unroll 1
+    for (uint32_t n = (blk - 1u) / kMarkBlocks; mk == 0u && n; n = n > kMarkBlocks ? n - kMarkBlocks : 0u)
+        mk = last_mark(a.grp_mark, n);
+    return mk;
 }
 
 // kSmall: a batch from k_rank_locate, whose storage-layer state is kept at every query, and which
@@ -203,7 +199,7 @@ __global__ void __launch_bounds__(kApThreads, 4) k_apply(ApplyArgs a, uint32_t e
         }
         x = __shfl_up_sync(0xffffffffu, x, 1);
         M = lane ? max(mark, x) : mark;
-        const uint32_t dtile = a.tile_mark ? kApplyTile : kDescendTile;
+        const uint32_t dtile = a.windows ? kApplyTile : kDescendTile;
         h += head0 + base / dtile * dtile - heads - 1u;  // (wraps for a block past the valid queries: not used)
 #pragma unroll
         for (int k = 0; k < kItems; ++k) dres[k] += h;

@@ -19,8 +19,10 @@ constexpr uint32_t kSortHist = 9 * 256; // digit counts of a radix sort
 constexpr uint32_t kSweepMost = 1u << 20;  // largest batch whose radix passes look back (see k_sort_count)
 constexpr uint32_t kScanGroup = 64;     // radix-sort tiles per group of the count kernel's scan
 constexpr uint32_t kCtrApply = 15;      // BatchMeta::tile_ctr slot: the apply kernel's tile counter
-constexpr uint32_t kApplyTile = 2048;   // sorted queries per tile of the descent with windows, and of its marks
+constexpr uint32_t kApplyTile = 2048;   // sorted queries per tile of the descent with windows
 constexpr uint32_t kApplyBlock = 128;   // sorted queries per apply warp
+constexpr uint32_t kMarkBlocks = 256;   // such blocks per group of the run markers
+constexpr uint32_t kMarkGroup = kMarkBlocks * kApplyBlock;  // sorted queries per group
 constexpr uint32_t kRunTile = 1024;     // queries per tile of the small batches' sort
 // Largest batch sorted that way. A query is ranked in every other tile, so the ranking's work
 // grows with the square of the batch; the radix passes' chain of launches does not grow.
@@ -531,6 +533,7 @@ struct SortBuffers {
     uint32_t* gctr;      // [8][groups + 1] arrival counters of the count kernel's CTAs
     uint8_t* ndig;       // next pass's digit of every element, in the current pass's output order
     uint32_t* fixmap;    // [ceil(n / 32)] bit per position: start of a segment to reorder
+    uint32_t* grp_mark;  // the descent's, per group of queries: cleared by the sort (null: none)
 };
 
 // Radix sort of (key, payload) pairs: result in a_k / a_p, stable, by key.
@@ -555,7 +558,8 @@ struct DescendArgs {
     const uint32_t* sp;  // sorted payload (op << 30 | arrival index)
     uint32_t* blk_head;  // per 128-query block: its first local run head's number in the descent's tile
     uint32_t* blk_mark;  // per block: the largest run marker e_i in it (0: none)
-    uint32_t* tile_mark; // per apply tile; null: the batch takes no windows, and there are none
+    uint32_t* grp_mark;  // per group of blocks: the largest of those that a run leaves into a full block (zero before)
+    bool windows;        // the batch takes windows of the lowest built level
     const DevMeta* m;
     BatchMeta* bm;
     const uint64_t* lkeys;   // index-layer buffer 0 (DevMeta::lcur picks the one in use)
@@ -596,7 +600,8 @@ struct ApplyArgs {
     uint64_t* desc;            // look-back descriptors: 2 words per tile
     const uint32_t* blk_head;  // from the descent (not for small batches)
     const uint32_t* blk_mark;
-    const uint32_t* tile_mark;
+    const uint32_t* grp_mark;
+    bool windows;              // the descent's
     LevelChanges chg;          // level membership changes, in key order
     uint32_t* lcnt;  // per-level per-tile live counts (see RebuildArgs)
     uint32_t lstride;

@@ -15,8 +15,10 @@
 // previous one, or the first query of a 128-query block), finds each head's place on the lowest
 // built level (which holds every key of the levels above it) and, in the gap below, the storage
 // node with the largest key <= q and its state, which it leaves in the tile's part of the state
-// arrays, head after head. It also leaves each block's first head's number and largest ownership
-// marker for k_apply. No tile waits for another.
+// arrays, head after head. No tile waits for another. For k_apply it also leaves each block's first
+// head's number and largest ownership marker, and, per group of blocks, the largest marker of those
+// whose last key fills the next block too: a look-back that has come past blocks without a marker
+// ends at such a block. (The largest of every block cost 2^18 queries 4 us of contended atomics.)
 // Large batches take windows: the keys of a tile are neighbours, so their places lie in one
 // stretch of the level, which the CTA reads into shared memory once, with coalesced loads, and
 // searches there; the level is then read about once per batch instead of a few random sectors
@@ -117,6 +119,7 @@ __global__ void __launch_bounds__(kWin ? kThreads + 64 : kThreads, kWin ? 4 : 6)
     extern __shared__ __align__(16) uint8_t s_dyn[];
     LocateSmem<kWin>& S = *reinterpret_cast<LocateSmem<kWin>*>(s_dyn);
     __shared__ uint32_t s_cnt[kWarps], s_half[kWarps], s_max[kWarps], s_c[2];
+    __shared__ bool s_more[kWarps];
     const DevMeta* m = a.m;
     if (block_sees_error(&m->error)) return;
     note_sizes(a);
@@ -136,6 +139,8 @@ __global__ void __launch_bounds__(kWin ? kThreads + 64 : kThreads, kWin ? 4 : 6)
             op[k] = i < qv ? (a.sp[i] >> 30) : 0u;
         }
         uint64_t carry = (w0 > 0 && w0 - 1 < qv) ? a.sk[w0 - 1] : kMaxKey;  // key before the element
+        const uint32_t beyond = w0 + 32u * kR - 1u + kApplyBlock;  // a block past the warp's last query
+        const uint64_t kb = beyond < qv ? a.sk[beyond] : 0ull;
         uint32_t nq = 0, half = 0, most = 0;
 #pragma unroll
         for (int k = 0; k < kR; ++k) {
@@ -156,14 +161,21 @@ __global__ void __launch_bounds__(kWin ? kThreads + 64 : kThreads, kWin ? 4 : 6)
             if (kWin && (k + 1) % (int)(kApplyBlock / 32u) == 0) {  // a block ends
                 const uint32_t mk = __reduce_max_sync(0xffffffffu, most);
                 const uint32_t bs = i / kApplyBlock * kApplyBlock;
-                if (lane == 0 && bs < n) a.blk_mark[bs / kApplyBlock] = mk >= 2u * bs + 2u ? mk : 0u;
+                const uint64_t kn = k + 1 < kR ? __shfl_sync(0xffffffffu, kk[kR - 1], 31) : kb;
+                if (lane == 0 && bs < n) {
+                    const bool any = mk >= 2u * bs + 2u;
+                    a.blk_mark[bs / kApplyBlock] = any ? mk : 0u;
+                    if (any && bs + 2u * kApplyBlock - 1u < qv && kn == carry) atomicMax(&a.grp_mark[bs / kMarkGroup], mk);
+                }
             }
         }
         const uint32_t mk = __reduce_max_sync(0xffffffffu, most);
+        const bool more = beyond < qv && kb == carry;
         if (lane == 0) {
             s_cnt[warp] = nq;
             s_half[warp] = half;
             s_max[warp] = mk;
+            s_more[warp] = more;
         }
     } else if (tb < qv) {  // the places of the tile's first and last key
         const uint32_t last = min(tb + kT, qv) - 1u;
@@ -172,12 +184,6 @@ __global__ void __launch_bounds__(kWin ? kThreads + 64 : kThreads, kWin ? 4 : 6)
     }
     __syncthreads();
     if (kWin) {
-        if (tid == 0) {
-            uint32_t mk = 0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) mk = max(mk, s_max[w]);
-            a.tile_mark[blockIdx.x] = mk;
-        }
         if (tid < kWarps) {  // a warp's two blocks
             uint32_t h = 0;
             for (int w = 0; w < tid; ++w) h += s_cnt[w];
@@ -192,6 +198,7 @@ __global__ void __launch_bounds__(kWin ? kThreads + 64 : kThreads, kWin ? 4 : 6)
         if (tb + (uint32_t)tid * kApplyBlock < n) {
             a.blk_mark[tb / kApplyBlock + (uint32_t)tid] = mk;
             a.blk_head[tb / kApplyBlock + (uint32_t)tid] = h;
+            if (mk && s_more[(tid + 1) * (int)(kApplyBlock / 32u) - 1]) atomicMax(&a.grp_mark[tb / kMarkGroup], mk);
         }
     }
     if (tb >= qv) return;
@@ -388,7 +395,7 @@ bool descend_windows(uint64_t n, uint64_t entries) {
 
 cudaError_t launch_descend(const DescendArgs& a, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
-    if (a.tile_mark) {
+    if (a.windows) {
         static bool attr_set = false;
         constexpr int smem = (int)sizeof(LocateSmem<true>);
         if (!attr_set) {

@@ -56,8 +56,8 @@ struct Scratch {
     uint8_t* lst_ins = nullptr;
     uint64_t lst_cap = 0;
     uint32_t* blk_head = nullptr;   // descent: per 128-query block, its first head's number
-    uint32_t* blk_mark = nullptr;   // descent: markers per block and per apply tile
-    uint32_t* tile_mark = nullptr;
+    uint32_t* blk_mark = nullptr;   // descent: markers per block and per group of blocks
+    uint32_t* grp_mark = nullptr;
 };
 
 // pi_profile level 2: the two events around every kernel launch of the batch entry
@@ -365,7 +365,7 @@ constexpr uint64_t scratch_bytes(uint64_t q) {
            + 2 * al256(c * 8) + al256(c * 4) + al256(c)            // new nodes
            + al256(c * 8) + al256(c * 4) + al256(c)                // level changes
            + al256((2 * c + 64) * 8) + 2 * al256((2 * c + 64) * 4) + al256(2 * c + 64)  // lists
-           + 2 * al256(tiles * (kApplyTile / kApplyBlock) * 4) + al256(tiles * 4);      // heads, marks
+           + 2 * al256(tiles * (kApplyTile / kApplyBlock) * 4) + al256((q / kMarkGroup + 1) * 4);  // heads, marks
 }
 
 struct Carver {
@@ -402,7 +402,7 @@ uint64_t carve_scratch(uint8_t* base, uint64_t q, Scratch& s) {
     v.take(s.lst_keys, s.lst_cap * 8); v.take(s.lst_pos, s.lst_cap * 4); v.take(s.lst_pref, s.lst_cap * 4);
     v.take(s.lst_ins, s.lst_cap);
     v.take(s.blk_head, tiles * (kApplyTile / kApplyBlock) * 4); v.take(s.blk_mark, tiles * (kApplyTile / kApplyBlock) * 4);
-    v.take(s.tile_mark, tiles * 4);
+    v.take(s.grp_mark, (q / kMarkGroup + 1) * 4);
     s.cap = q;
     return v.off;
 }
@@ -569,6 +569,7 @@ SortBuffers sort_buffers(pi_index* x, const Scratch& s) {
     sb.gctr = s.gctr;
     sb.ndig = s.ndig;
     sb.fixmap = s.fixmap;
+    sb.grp_mark = s.grp_mark;
     return sb;
 }
 
@@ -870,7 +871,8 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     da.sp = sc.a_p;
     da.blk_head = sc.blk_head;
     da.blk_mark = sc.blk_mark;
-    da.tile_mark = windows_for(x, n) ? sc.tile_mark : nullptr;
+    da.grp_mark = sc.grp_mark;
+    da.windows = windows_for(x, n);
     da.m = x->d_meta;
     da.bm = bm;
     da.lkeys = x->lkeys;
@@ -902,7 +904,8 @@ int enqueue_batch_body(pi_index* x, const Scratch& sc, const uint8_t* ops, const
     aa.desc = x->desc;
     aa.blk_head = sc.blk_head;
     aa.blk_mark = sc.blk_mark;
-    aa.tile_mark = da.tile_mark;
+    aa.grp_mark = sc.grp_mark;
+    aa.windows = da.windows;
     aa.chg = sc.chg;
     aa.lcnt = x->lcnt;
     aa.lstride = x->lstride;

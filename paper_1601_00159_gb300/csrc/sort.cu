@@ -86,7 +86,8 @@ __device__ __forceinline__ void count_digits(const uint32_t (&d)[kN], uint32_t n
 // queries). Four consecutive queries per thread and step (16-byte key loads, one 4-byte load of
 // their op codes) when the arrays are aligned for it, so that every thread keeps several loads
 // in flight; the byte-wise extremes are kept four bytes to a word with SIMD min/max. It also
-// clears what the passes start from: the first pass's look-back words, or the counts' arrivals.
+// clears what the passes start from, the first pass's look-back words or the counts' arrivals, and the
+// descent's group marks.
 struct ScanAcc {
     uint32_t invalid = 0;
     uint32_t mxl = 0, mxh = 0;                  // byte-wise max of the valid keys (low, high word)
@@ -106,7 +107,8 @@ struct ScanAcc {
 template <bool kSweep>
 __global__ void __launch_bounds__(256) k_scan(const uint8_t* __restrict__ ops, const uint64_t* __restrict__ keys,
                                               uint32_t n, uint32_t* __restrict__ fixmap, uint32_t* __restrict__ clear,
-                                              uint32_t nclear, uint32_t* __restrict__ hist, BatchMeta* bm) {
+                                              uint32_t nclear, uint32_t* __restrict__ marks, uint32_t nmarks,
+                                              uint32_t* __restrict__ hist, BatchMeta* bm) {
     pdl_wait();
     pdl_trigger();
     __shared__ uint32_t s_hist[256];
@@ -116,6 +118,7 @@ __global__ void __launch_bounds__(256) k_scan(const uint8_t* __restrict__ ops, c
     }
     const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
     for (uint32_t w = gt; w < nclear; w += gs) clear[w] = 0;
+    for (uint32_t w = gt; w < nmarks; w += gs) marks[w] = 0;
     for (uint32_t w = gt; w < (n + 31u) / 32u; w += gs) fixmap[w] = 0;  // segment marks of the prefix fix-up
     ScanAcc acc;
     const bool vec = ((reinterpret_cast<uintptr_t>(keys) & 15u) | (reinterpret_cast<uintptr_t>(ops) & 3u)) == 0;
@@ -1113,19 +1116,20 @@ cudaError_t launch_sort(const uint8_t* ops, const uint64_t* keys, uint32_t n, co
     sb.keys = keys;
     const bool sweep = n <= kSweepMost, large = n >= kLargeTiles;
     const int grid = min((int)((n + 255) / 256), num_sms * 8);
+    const uint32_t nmarks = sb.grp_mark ? (n + kMarkGroup - 1) / kMarkGroup : 0u;
     cudaError_t e = cudaSuccess;
     if (sweep) {
         if (!*hist_clear && (e = cudaMemsetAsync(sb.hist, 0, kSortHist * sizeof(uint32_t), s)) != cudaSuccess) return e;
         *hist_clear = false;
         const uint32_t tile = (uint32_t)kPassThreads * (large ? 8u : 4u), words = (n + tile - 1) / tile * 256u;
-        launch_dep(k_scan<true>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.desc[0], words, sb.hist, bm);
+        launch_dep(k_scan<true>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.desc[0], words, sb.grp_mark, nmarks, sb.hist, bm);
         launch_dep(k_sort_plan, min((int)((n + 2047) / 2048), num_sms * 4), 256, 0, s, n, sb, bm, (uint32_t)max_passes);
         g_launches += 2;
         e = large ? launch_passes<8>(n, sb, bm, err, s, max_passes) : launch_passes<4>(n, sb, bm, err, s, max_passes);
     } else {
         const uint32_t ngroups = ((n + kTile - 1) / kTile + kScanGroup - 1) / kScanGroup;
-        launch_dep(k_scan<false>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.gctr, 8u * (ngroups + 1u),
-                   (uint32_t*)nullptr, bm);
+        launch_dep(k_scan<false>, grid, 256, 0, s, ops, keys, n, sb.fixmap, sb.gctr, 8u * (ngroups + 1u), sb.grp_mark,
+                   nmarks, (uint32_t*)nullptr, bm);
         ++g_launches;
         e = launch_count_passes(n, sb, bm, err, s, max_passes);
     }

@@ -41,7 +41,7 @@ def check(orc_mod, keys, p, batches, cfg=None, **state):
 
 @pytest.mark.parametrize("q,hot", [((1 << 20) + 77, 300_000), (1 << 20, 33_000), (1 << 18, 100_000)])
 @pytest.mark.parametrize("write", ["none", "first", "last"])
-@pytest.mark.parametrize("flags", [0, 1])  # 1: without windows, so without the tiles' marks
+@pytest.mark.parametrize("flags", [0, 1])  # 1: without windows
 def test_long_run_of_searches(orc_mod, q, hot, write, flags):
     keys = wl.distinct_keys(120, np.arange(60_000))
     s = wl.stream_seed(q, 121)
@@ -58,6 +58,33 @@ def test_long_run_of_searches(orc_mod, q, hot, write, flags):
     gone = wl.Batch(np.where(k == hk, 2, 0).astype(np.uint8), k, b.vals)  # one delete, then searches
     gone.ops[at[1:]] = 0
     check(orc_mod, keys, 0.25, [b, gone, b], {"test_flags": flags} if flags else None)
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+@pytest.mark.parametrize("write", [None, 1000, 5_000_000])
+def test_batch_of_one_key(write, flags):
+    """A run over more groups of marks than one step of the look-back takes."""
+    import torch
+    n, q = 1 << 20, (1 << 24) + 33
+    keys = wl.distinct_keys(128, np.arange(n))
+    idx = make_index(keys, wl.splitmix64(keys), 0.25, 23, {"test_flags": flags} if flags else None)
+    old = int(wl.splitmix64(keys[7:8]).view(np.int64)[0])
+    ops = torch.zeros(q, dtype=torch.uint8, device="cuda")
+    k = to_dev(keys[7:8], torch.int64).expand(q).contiguous()
+    vals = torch.full((q,), 4711, dtype=torch.int64, device="cuda")
+    want = torch.full((q,), old, dtype=torch.int64, device="cuda")
+    if write is not None:
+        ops[write] = 1
+        want[write + 1:] = 4711
+    r = idx.execute(ops, k, vals)
+    assert torch.equal(r[:, 0], want) and bool((r[:, 1] == 1).all())
+    if write is not None:  # then a delete, after which the key is absent
+        ops[write] = 2
+        r = idx.execute(ops, k, vals)
+        assert bool((r[: write + 1, 0] == 4711).all()) and bool((r[: write + 1, 1] == 1).all())
+        assert not bool(r[write + 1:].any())
+    assert idx.status() == 0
+    idx.close()
 
 
 @pytest.mark.parametrize("q", [1 << 19, (1 << 20) + 5])
