@@ -21,7 +21,8 @@
 // query, by its number, has its state, and a block that continues a run looks back over 256
 // blocks' marks, then the groups', for the run's last write: two steps or three however long the
 // run is. (Over the blocks' marks alone, a batch that is one key's run took time with the square of its
-// length: 2^23 searches 1043 us, now 336.) So no warp waits for another until the counts of the tile: with block-wide scans, barriers were the largest stall.
+// length: 2^23 searches 1043 us, now 336.) So no warp waits for another until the counts of the
+// tile: with block-wide scans, barriers were the largest stall.
 // New nodes, and the changes of built levels' membership, go to their places in key order in
 // the same pass: a tile's first place comes from a decoupled look-back over the tiles' counts,
 // which only tiles that have some wait for. Half of the kernel's time is its scattered 16-byte

@@ -1,7 +1,7 @@
 """Branches that only large or lopsided shapes take: a run of equal keys longer than the nearest blocks'
 marks reach, tiles whose stretch of the lowest built level does not fit a window, windows over the
-storage layer itself, merges of so many nodes that a CTA finds its cuts in groups, and range
-slices copied one at a time. Everything is compared with the oracle, or, at 2^28 keys, with the
+storage layer itself, merges of so many nodes that a CTA finds its cuts in groups, range slices
+copied one at a time, and slices long enough to be counted by a whole warp. Everything is compared with the oracle, or, at 2^28 keys, with the
 same update done by sorting."""
 import numpy as np
 import pytest
@@ -185,6 +185,36 @@ def test_range_slices_one_at_a_time(orc_mod, q):
         assert np.array_equal(offs.cpu().numpy().view(np.uint64), eo)
         assert np.array_equal(got[0, :fit], ek[:fit]) and np.array_equal(got[1, :fit], ev[:fit])
         assert (out[:, fit:] == -7).all()
+    assert idx.status() == 0
+    idx.close()
+    orc.close()
+
+
+@pytest.mark.parametrize("q", [1, 40, 5000, 160_000])
+def test_long_range_slices_with_deleted_nodes(orc_mod, q):
+    """Slices of 255 to some thousand 16-byte chunks of state bytes, from any node to any node, among
+    short and empty ones."""
+    import torch
+    n = 60_000
+    keys = np.sort(wl.distinct_keys(129, np.arange(n)))
+    idx = make_index(keys, wl.splitmix64(keys), 0.25, 3)
+    orc = orc_mod.Oracle(keys, wl.splitmix64(keys), 0.25, 3)
+    gone = keys[wl.bounded(wl.stream_seed(130, 0), 0, n // 10, n)]
+    b = wl.Batch(np.full(len(gone), 2, np.uint8), gone, gone)
+    assert_results_equal(run_batch(idx, b), orc.execute(b.ops, b.keys, b.vals))
+    s = wl.stream_seed(q, 131)
+    at = wl.bounded(s, 0, q, n).astype(np.int64)
+    kind = wl.bounded(s, q, q, max(q // 40, 1))  # some forty long ones
+    span = np.where(kind == 0, 4000 + wl.bounded(s, 2 * q, q, 50_000).astype(np.int64),
+                    wl.bounded(s, 3 * q, q, 30).astype(np.int64))
+    edge = kind == 1  # at the limit, from every offset
+    span = np.where(edge, 255 * 16 - 20 + wl.bounded(s, 4 * q, q, 40).astype(np.int64), span)
+    lo, hi = keys[at], keys[np.minimum(at + span, n - 1)]
+    eo, ek, ev = orc.range(lo, hi)
+    offs, k, v = idx.range_search(to_dev(lo, torch.int64), to_dev(hi, torch.int64), cap=int(eo[-1]))
+    assert np.array_equal(offs.cpu().numpy().view(np.uint64), eo)
+    assert np.array_equal(k.cpu().numpy().view(np.uint64), ek)
+    assert np.array_equal(v.cpu().numpy().view(np.uint64), ev)
     assert idx.status() == 0
     idx.close()
     orc.close()
