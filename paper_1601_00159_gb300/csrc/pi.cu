@@ -580,6 +580,14 @@ cudaError_t read_meta(pi_index* x, cudaStream_t s, DevMeta* out) {
     return e;
 }
 
+// The highest level that holds a live key (1: only the storage layer). DevMeta::H is the highest
+// level as last laid out, and a change of keys below the lowest built level lays nothing out.
+int top_level(const DevMeta& m) {
+    int l = kLevelSlots - 1;
+    while (l > 1 && m.cnt[l] == 0) --l;
+    return l;
+}
+
 constexpr uint64_t kRing = 64;
 
 // Numbers an operation of n queries that is being issued. Without memory to list it, its queries
@@ -1432,7 +1440,7 @@ int pi_info(pi_index_t* x, pi_info_t* out, pi_stream_t stream) {
     out->size = m.size;
     out->live = m.cnt[1];
     out->tombstones = m.tombs;
-    out->top_level = m.H;
+    out->top_level = (uint32_t)top_level(m);
     out->bottom_built = m.Lb;
     out->smem_low_level = m.Ls;
     out->promote_shift = (uint32_t)x->hp.b;
@@ -1498,7 +1506,7 @@ int pi_num_levels(pi_index_t* x, pi_stream_t stream) {
     cudaError_t e = sync_known(x, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return map_cuda(e);
     if (int rc = sticky_error(x->known)) return rc;
-    return (int)x->known.H;
+    return top_level(x->known);
 }
 
 int pi_export(pi_index_t* x, uint64_t* keys_out, uint64_t* vals_out, uint64_t cap, uint64_t* n_out_host,
