@@ -269,6 +269,8 @@ int pi_size(pi_index_t* idx, uint64_t* size_out_host, pi_stream_t stream);
  * pi_test_set_error: records the error bits (1: a bounded wait gave up, 2: an internal bound
  *   check refused an access) in the index's sticky device error word, as a kernel would.
  *   Synchronises `stream`; the host learns of it as it would of a kernel's.
+ * pi_test_set_epoch: moves the count that tags the look-backs of the index's launches forward to
+ *   `epoch` (PI_ERR_INVALID_ARG for a smaller one), so that a test can take it past 2^32.
  * pi_selftest_wait: launches one CTA that waits, through the bounded look-back the batch
  *   kernels use, for a predecessor that never publishes. The wait gives up after its
  *   spin bound (on a GB300 about 1.4 s), records the timeout in a scratch error word, which
@@ -277,6 +279,7 @@ int pi_size(pi_index_t* idx, uint64_t* size_out_host, pi_stream_t stream);
  */
 void pi_test_fail_allocations(uint32_t count);
 void pi_test_skip_allocations(uint32_t count);
+int pi_test_set_epoch(pi_index_t* idx, uint32_t epoch);
 int pi_test_set_error(pi_index_t* idx, uint32_t bits, pi_stream_t stream);
 int pi_selftest_wait(uint32_t* err_word_host, pi_stream_t stream);
 

@@ -21,7 +21,7 @@ PI_MAX_KEYS = (1 << 30) - 2
 
 EXPORTED = ["pi_create", "pi_create_ex", "pi_execute_batch", "pi_execute_batch_host", "pi_destroy",
             "pi_last_error", "pi_status", "pi_info", "pi_size", "pi_test_fail_allocations",
-            "pi_test_skip_allocations", "pi_test_set_error",
+            "pi_test_skip_allocations", "pi_test_set_error", "pi_test_set_epoch",
             "pi_selftest_wait", "pi_num_levels", "pi_export", "pi_export_level", "pi_export_storage", "pi_profile",
             "pi_profile_read", "pi_profile_kernels", "pi_execute_batch_noalloc", "pi_flush",
             "pi_range_search", "pi_multi_create", "pi_multi_execute", "pi_multi_destroy", "pi_multi_kernels_per_call",
@@ -135,6 +135,8 @@ def load_library(path: str = LIB_PATH):
     lib.pi_test_skip_allocations.argtypes = [ctypes.c_uint32]
     lib.pi_test_set_error.restype = i32
     lib.pi_test_set_error.argtypes = [vp, ctypes.c_uint32, vp]
+    lib.pi_test_set_epoch.restype = i32
+    lib.pi_test_set_epoch.argtypes = [vp, ctypes.c_uint32]
     lib.pi_selftest_wait.restype = i32
     lib.pi_selftest_wait.argtypes = [ctypes.POINTER(ctypes.c_uint32), vp]
     lib.pi_size.restype = i32
@@ -236,6 +238,11 @@ def test_fail_allocations(count: int, skip: int = 0) -> None:
 def test_set_error(index, bits: int, stream=None) -> None:
     """Records error bits in the index's sticky device error word (pi_test_set_error)."""
     _chk(index.lib.pi_test_set_error(index._h, bits, _stream_handle(stream)), "pi_test_set_error")
+
+
+def test_set_epoch(index, epoch: int) -> None:
+    """Moves the index's look-back epoch forward (pi_test_set_epoch)."""
+    _chk(index.lib.pi_test_set_epoch(index._h, epoch), "pi_test_set_epoch")
 
 
 def selftest_wait(stream=None):

@@ -334,10 +334,14 @@ void use_side(pi_index* x, SideArrays& n) {
     n = SideArrays{};
 }
 
+void wait_rebuild(pi_index* x, cudaStream_t s);
+
 uint32_t next_epochs(pi_index* x, uint32_t count, cudaStream_t s) {
     // Epochs tag look-back descriptors; on wrap-around clear them so no stale word can
-    // carry a reused epoch.
+    // carry a reused epoch. The last batch's rebuild, on its own stream, may still be looking
+    // back over them.
     if (x->epoch > 0xFFFFFFFFu - count - 64u) {
+        wait_rebuild(x, s);
         cudaMemsetAsync(x->desc, 0, x->desc_words * sizeof(uint64_t), s);
         x->epoch = 1;
     }
@@ -1462,6 +1466,12 @@ void pi_test_fail_allocations(uint32_t count) {
 }
 
 void pi_test_skip_allocations(uint32_t count) { g_skip_allocs = count; }
+
+int pi_test_set_epoch(pi_index_t* x, uint32_t epoch) {
+    if (!x || epoch < x->epoch) return PI_ERR_INVALID_ARG;
+    x->epoch = epoch;
+    return PI_OK;
+}
 
 int pi_test_set_error(pi_index_t* x, uint32_t bits, pi_stream_t stream) {
     if (!x) return PI_ERR_INVALID_ARG;
